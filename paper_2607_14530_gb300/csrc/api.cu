@@ -167,6 +167,7 @@ Layout make_layout(const Dims& d, int64_t T) {
         L.hpost[q] = o; o = al(o + t * d.k * d.K[q] * 4);
     }
     L.hres = o; o = al(o + t * d.k * d.k * 4);
+    L.wsum = o; o = al(o + (size_t)d.N * 4);
     for (int q = 0; q < d.G; ++q)
         if (d.K[q] > 1 && d.gs) { L.gram[q] = o; o = al(o + t * NGRAM * 8); }
     L.saved_total = o;
@@ -203,7 +204,7 @@ Layout make_layout(const Dims& d, int64_t T) {
     o = al(o + std::max((size_t)L.splits_full * d.nfull, (size_t)L.splits_act * nact_max) * t * 4);
     L.pstats = o; o = al(o + (size_t)std::max(L.splits_full, L.splits_act) * t * 2 * 4);
     L.astat = o; o = al(o + (size_t)stream_warps(d.C) * t * 2 * 4);
-    L.wsum = o; o = al(o + (size_t)d.N * 4);
+    L.wsump = o; o = al(o + (size_t)COLSUM_PARTS * d.N * 4);
     L.rsum = o; o = al(o + (size_t)d.N * 4);
     L.base = o; o = al(o + (size_t)(d.G - 1) * t * d.C * 2);
     L.red = o; o = al(o + t * L.nslice * NRED * 4);
@@ -214,7 +215,8 @@ Layout make_layout(const Dims& d, int64_t T) {
     L.dhpre = o; o = al(o + t * d.G * d.N * 4);
     L.tokmat = o; o = al(o + t * TOKMAT * 4);
     L.dz = o; o = al(o + t * std::max(d.nfull, nact_max) * 4);
-    L.tokgrad = o; o = al(o + t * NTG * 4);
+    L.scal = o; o = al(o + t * 2 * 4);
+    L.colp = o; o = al(o + (size_t)((T + 3) / 4) * NCOLP * 4);   // blocks of at least 4 tokens
     L.wpart = o;
     {
         size_t w1 = std::max((size_t)ts_full * d.N * d.C * d.nfull, (size_t)ts_act * d.k * d.C * nact_max);
@@ -222,7 +224,6 @@ Layout make_layout(const Dims& d, int64_t T) {
         o = al(o + std::max(w1, w2) * 4);
     }
     L.cpart = o; o = al(o + (size_t)L.ntiles * d.kapsum * d.C * 4);
-    L.colscr = o; o = al(o + (size_t)64 * 256 * 4);
     L.ws_total = o;
     return L;
 }
@@ -586,14 +587,12 @@ ConvPtrs conv_of(const Dims& d, const xhc_params* P, int slot) {
     return c;
 }
 
-// above this many split-K partial slots the coefficient kernels get them pre-summed
-constexpr int SLOT_SUM_MIN = 8;
-
 // Active-state mapping generation of one slot (Eq. param_post, Eq. param_res).
 xhc_status active_maps(const Ctx& c, int slot, const xhc_params* P) {
     const Dims& d = c.d;
     const WSegs wa = act_segs(d, P, slot);
-    int splits = c.L.splits_act, ssplits = c.L.splits_act;
+    SlotPlan sp = slots_of(c.L.splits_act);
+    int ssplits = c.L.splits_act;
     float* pstats = c.W<float>(c.L.pstats);
     if (c.T < 128 || d.k * d.C < 64) {
         XHC_K("rowproj_active", c.st, launch_rowproj(c.xact(slot), (int64_t)d.k * d.C, d.k * d.C, c.T, wa,
@@ -601,7 +600,7 @@ xhc_status active_maps(const Ctx& c, int slot, const xhc_params* P) {
                                                      c.W<float>(c.L.pstats), c.st));
     } else {
         ProjTcPlan pl = plan_proj_tc(c.T, d.k * d.C, d.nact[slot], device_sms(), true);
-        splits = pl.nseg;
+        sp = slots_of(pl);
         XHC_K("pack_w", c.st, launch_pack_w(wa, d.nact[slot], pl.NB, d.k * d.C,
                                             c.W<uint16_t>(c.L.wpack), c.st));
         // the norm statistics come from the read / input pass that produced x_act
@@ -611,16 +610,8 @@ xhc_status active_maps(const Ctx& c, int slot, const xhc_params* P) {
         pstats = c.W<float>(c.L.astat);
         ssplits = stream_warps(d.C);
     }
-    if (splits > SLOT_SUM_MIN) {
-        XHC_K("slot_sum", c.st, launch_slot_sum(c.W<float>(c.L.part), splits, (long long)c.T * d.nact[slot], c.st));
-        splits = 1;
-    }
-    if (ssplits > SLOT_SUM_MIN && pstats == c.W<float>(c.L.pstats)) {
-        XHC_K("slot_sum", c.st, launch_slot_sum(pstats, ssplits, (long long)c.T * 2, c.st));
-        ssplits = 1;
-    }
     XHC_K("coef_act", c.st, launch_coef_act(d, slot, c.T, c.W<float>(c.L.part), pstats, ssplits,
-                             splits, P->alpha_post, P->b_post[slot], P->alpha_res, P->b_res,
+                             sp, P->alpha_post, P->b_post[slot], P->alpha_res, P->b_res,
                              c.S<float>(c.L.zact[slot]), c.S<float>(c.L.rs[slot]),
                              c.S<float>(c.L.hpost[slot]), c.S<float>(c.L.hres), c.st));
     return XHC_OK;
@@ -641,33 +632,26 @@ xhc_status xhc_pre_fwd(const xhc_handle* h, int slot, int64_t T, const xhc_param
     const Dims& d = c.d;
     if (slot == 0) {
         if (d.hr)
-            XHC_K("colsum", c.st, launch_colsum(P->W_r, d.N * d.C, d.N, d.N, c.W<float>(c.L.wsum), 0,
-                                   c.W<float>(c.L.colscr), c.st));
+            XHC_K("colsum", c.st, launch_colsum(P->W_r, d.N * d.C, d.N, c.W<float>(c.L.wsump), c.st));
         const WSegs wf = full_segs(d, P);
-        // partial slots written (and summed by coef_full): the split count of the path taken
-        int fsplits = c.L.splits_full;
+        // partial slots written (and summed by coef_full): those of the path taken
+        SlotPlan sp = slots_of(c.L.splits_full);
         if (c.T < 128 || d.N * d.C < 64) {
             // smaller than one tensor-core tile: fp32 CUDA-core projection
             XHC_K("rowproj_full", c.st, launch_rowproj(X, (int64_t)d.N * d.C, d.N * d.C, c.T, wf,
                                                        d.nfull, c.L.splits_full, c.W<float>(c.L.part),
                                                        c.W<float>(c.L.pstats), c.st));
         } else {
-        fsplits = c.L.tc.nseg;
+        sp = slots_of(c.L.tc);
         XHC_K("pack_w", c.st, launch_pack_w(wf, d.nfull, c.L.tc.NB, d.N * d.C,
                                             c.W<uint16_t>(c.L.wpack), c.st));
         XHC_K("proj_tc", c.st, launch_proj_tc(X, c.T, d.N * d.C, c.W<uint16_t>(c.L.wpack), d.nfull,
                                               c.L.tc, c.W<float>(c.L.part), c.W<float>(c.L.pstats),
                                               c.W<int>(c.L.err), c.st));
         }
-        if (fsplits > SLOT_SUM_MIN) {
-            // few tokens, many split-K slots: summed in parallel first
-            XHC_K("slot_sum", c.st, launch_slot_sum(c.W<float>(c.L.part), fsplits, (long long)c.T * d.nfull, c.st));
-            XHC_K("slot_sum", c.st, launch_slot_sum(c.W<float>(c.L.pstats), fsplits, (long long)c.T * 2, c.st));
-            fsplits = 1;
-        }
         XHC_K("coef_full", c.st, launch_coef_full(d, c.T, c.W<float>(c.L.part), c.W<float>(c.L.pstats),
-                                  fsplits, c.W<float>(c.L.wsum), P->alpha_pre, P->b_pre,
-                                  c.S<float>(c.L.zfull), c.S<float>(c.L.stats),
+                                  sp, c.W<float>(c.L.wsump), COLSUM_PARTS, P->alpha_pre, P->b_pre,
+                                  c.S<float>(c.L.zfull), c.S<float>(c.L.stats), c.S<float>(c.L.wsum),
                                   c.S<float>(c.L.hpre), c.S<int>(c.L.I), c.S<float>(c.L.p), c.st));
         XHC_K("read", c.st, launch_read(d, c.T, X, c.S<float>(c.L.hpre), c.S<int>(c.L.I), input,
                              c.W<uint16_t>(c.L.base), c.xact(0), c.W<float>(c.L.astat), c.st));
@@ -839,10 +823,8 @@ xhc_status post_bwd_impl(const xhc_handle* h, int slot, int64_t T, const xhc_par
     const int K = d.K[slot], n = d.nact[slot];
     float* red = c.W<float>(c.L.red);
     float* dxact = c.W<float>(c.L.dxact);
-    if (last) {
-        XHC_CUDA(cudaMemsetAsync(c.W<float>(c.L.dp), 0, (size_t)T32 * d.k * 4, c.st));
+    if (last)
         XHC_K("restore", c.st, launch_restore(d, T32, c.xact(0), c.S<int>(c.L.I), X, c.st));
-    }
     const int bslices = wb_bred_slices(d, slot);
     if (K == 1) {
         // no conv: reductions and apply in one pass (the apply coefficients are forward values)
@@ -853,13 +835,13 @@ xhc_status post_bwd_impl(const xhc_handle* h, int slot, int64_t T, const xhc_par
         XHC_K("wb_bred", c.st, launch_wb_bred(d, slot, T32, out, cw, dX, c.S<int>(c.L.I), dxact, c.xact(slot),
                                               bslices, red, c.st));
     }
+    int nblk = 0;
     XHC_K("bwd_coef", c.st, launch_bwd_coef(d, slot, T32, red, bslices, c.S<float>(c.L.zact[slot]),
                              c.S<float>(c.L.rs[slot]), c.S<float>(c.L.p),
                              c.S<float>(c.L.hpost[slot]),
                              (d.K[slot] > 1 && d.gs) ? c.S<double>(c.L.gram[slot]) : nullptr,
-                             P->alpha_post, P->b_post[slot],
-                             P->alpha_res, P->b_res, c.W<float>(c.L.tokmat), c.W<float>(c.L.dz),
-                             c.W<float>(c.L.dp), c.W<float>(c.L.tokgrad), c.st));
+                             P->alpha_post, P->alpha_res, P->b_res, c.W<float>(c.L.tokmat),
+                             c.W<float>(c.L.dz), c.W<float>(c.L.dp), c.W<float>(c.L.colp), &nblk, c.st));
     // weight gradient of the post/res projections and the alpha / b column sums need only dZ_act
     // and the per-token contributions: side stream, overlapping the apply kernel
     const cudaStream_t sd = fork_from(c.st);
@@ -867,23 +849,21 @@ xhc_status post_bwd_impl(const xhc_handle* h, int slot, int64_t T, const xhc_par
         const int ts = std::min(c.L.tsplits, pick_tsplits(d.k * d.C, T32));
         XHC_K("wgrad_active", sd, launch_wgrad(c.xact(slot), (int64_t)d.k * d.C, d.k * d.C, T32,
                                                c.W<float>(c.L.dz), n, n, ts, c.W<float>(c.L.wpart),
-                                               act_segs_g(d, g, slot), sd));
+                                               act_segs_g(d, g, slot), nullptr, sd));
     } else {
         ProjTcPlan pl = plan_proj_tc(d.k * d.C, T32, n, device_sms(), false);
         XHC_K("wgrad_tc_active", sd, launch_wgrad_tc(c.xact(slot), T32, d.k * d.C, c.W<float>(c.L.dz), n, n,
                                                      c.W<uint16_t>(c.L.dzpack), pl, c.W<float>(c.L.wpart),
                                                      c.W<int>(c.L.err), sd));
-        XHC_K("wgrad_reduce", sd, launch_wgrad_reduce(c.W<float>(c.L.wpart), pl.nseg, d.k * d.C, n,
-                                                      act_segs_g(d, g, slot), sd));
+        XHC_K("wgrad_reduce", sd, launch_wgrad_reduce(c.W<float>(c.L.wpart), slots_of(pl), d.k * d.C, n,
+                                                      act_segs_g(d, g, slot), nullptr, sd));
     }
-    float* tg = c.W<float>(c.L.tokgrad);
-    float* scr = c.W<float>(c.L.colscr);
-    XHC_K("colsum", sd, launch_colsum(tg, T32, NTG, d.k * K, g->b_post[slot], 1, scr, sd));
-    XHC_K("colsum", sd, launch_colsum(tg + d.k * K, T32, NTG, 1, g->alpha_post + slot, 1, scr, sd));
-    if (last) {
-        XHC_K("colsum", sd, launch_colsum(tg + d.k * K + 1, T32, NTG, d.k * d.k, g->b_res, 1, scr, sd));
-        XHC_K("colsum", sd, launch_colsum(tg + d.k * K + 1 + d.k * d.k, T32, NTG, 1, g->alpha_res, 1, scr, sd));
-    }
+    const int kK = d.k * K, kk = d.k * d.k;
+    const ColOut co = {{g->b_post[slot], g->alpha_post + slot, last ? g->b_res : nullptr, last ? g->alpha_res : nullptr},
+                       {0, kK, kK + 1, kK + 1 + kk},
+                       {kK, 1, last ? kk : 0, last ? 1 : 0},
+                       {0, 0, 0, 0}};
+    XHC_K("colsum_out", sd, launch_colsum_out(c.W<float>(c.L.colp), nblk, kK + 1 + (last ? kk + 1 : 0), co, sd));
     // d_out, conv weight-gradient partials and (last slot) the mixed active gradient; the
     // active gradient of earlier slots is read in place and completed by pre_bwd(slot)
     if (K > 1)
@@ -953,49 +933,45 @@ xhc_status xhc_pre_bwd(const xhc_handle* h, int slot, int64_t T, const xhc_param
                                     c.W<float>(c.L.dhpre), dinput, c.W<float>(c.L.tokmat), c.st));
     }
     if (slot != 0) return XHC_OK;
-    if (d.hr)
-        XHC_K("colsum", c.st, launch_colsum(P->W_r, d.N * d.C, d.N, d.N, c.W<float>(c.L.wsum), 0,
-                               c.W<float>(c.L.colscr), c.st));
     XHC_K("full_dots", c.st, launch_full_dots(d, T32, X, dinput, c.S<int>(c.L.I), c.W<float>(c.L.dhpre), c.st));
+    int nblk = 0;
     XHC_K("full_coef", c.st, launch_full_coef(d, T32, c.W<float>(c.L.dhpre), c.S<float>(c.L.hpre),
-                              c.S<float>(c.L.zfull), c.S<float>(c.L.stats), c.W<float>(c.L.wsum),
+                              c.S<float>(c.L.zfull), c.S<float>(c.L.stats), c.S<float>(c.L.wsum),
                               c.S<int>(c.L.I), c.W<float>(c.L.dp), P->alpha_pre,
-                              c.W<float>(c.L.dz), c.W<float>(c.L.tokgrad), c.st));
+                              c.W<float>(c.L.dz), c.W<float>(c.L.scal), c.W<float>(c.L.colp), &nblk, c.st));
     // the full-state weight gradient and the pre-map / router column sums need only dZ and the
     // per-token contributions: side stream, overlapping the full-state dX
     const cudaStream_t sd = fork_from(c.st);
+    const int GN = d.G * d.N;
+    float* rsum = d.hr ? c.W<float>(c.L.rsum) : nullptr;
+    const ColOut co = {{g->b_pre, g->alpha_pre, rsum, nullptr},
+                       {0, GN, GN + d.G, 0},
+                       {GN, d.G, d.hr ? d.N : 0, 0},
+                       {0, 0, 1, 0}};
+    XHC_K("colsum_out", sd, launch_colsum_out(c.W<float>(c.L.colp), nblk, GN + d.G + (d.hr ? d.N : 0), co, sd));
     if (T32 < 64 || d.N * d.C < 128) {
         const int ts = std::min(c.L.tsplits, pick_tsplits(d.N * d.C, T32));
         XHC_K("wgrad_full", sd, launch_wgrad(X, (int64_t)d.N * d.C, d.N * d.C, T32, c.W<float>(c.L.dz),
                                                d.nfull, d.nfull, ts, c.W<float>(c.L.wpart),
-                                               full_segs_g(d, g), sd));
+                                               full_segs_g(d, g), rsum, sd));
     } else {
         const ProjTcPlan& pl = c.L.twf;
         XHC_K("wgrad_tc_full", sd, launch_wgrad_tc(X, T32, d.N * d.C, c.W<float>(c.L.dz), d.nfull, d.nfull,
                                                      c.W<uint16_t>(c.L.dzpack), pl, c.W<float>(c.L.wpart),
                                                      c.W<int>(c.L.err), sd));
-        XHC_K("wgrad_reduce", sd, launch_wgrad_reduce(c.W<float>(c.L.wpart), pl.nseg, d.N * d.C, d.nfull,
-                                                        full_segs_g(d, g), sd));
-    }
-    float* tg = c.W<float>(c.L.tokgrad);
-    float* scr = c.W<float>(c.L.colscr);
-    XHC_K("colsum", sd, launch_colsum(tg + 2, T32, NTG, d.G * d.N, g->b_pre, 1, scr, sd));
-    XHC_K("colsum", sd, launch_colsum(tg + 2 + d.G * d.N, T32, NTG, d.G, g->alpha_pre, 1, scr, sd));
-    if (d.hr) {
-        float* rsum = c.W<float>(c.L.rsum);
-        XHC_K("colsum", sd, launch_colsum(tg + 2 + d.G * d.N + d.G, T32, NTG, d.N, rsum, 0, scr, sd));
-        XHC_K("sub_rows", sd, launch_sub_rows(g->W_r, d.N * d.C, d.N, rsum, sd));
+        XHC_K("wgrad_reduce", sd, launch_wgrad_reduce(c.W<float>(c.L.wpart), slots_of(pl), d.N * d.C, d.nfull,
+                                                        full_segs_g(d, g), rsum, sd));
     }
     const WSegs wf = full_segs(d, P);
     if (dx_tc_ok(T32, d.N, d.C, d.nfull, d.G)) {
         XHC_K("dx_tc", c.st, launch_dx_tc(d, T32, c.W<float>(c.L.dz), wf, c.W<uint16_t>(c.L.dz16),
                                           c.W<uint16_t>(c.L.w16), X, dinput, c.S<float>(c.L.hpre),
-                                          c.S<int>(c.L.I), c.W<float>(c.L.dxact), c.W<float>(c.L.tokgrad),
-                                          NTG, dX, c.W<int>(c.L.err), c.st));
+                                          c.S<int>(c.L.I), c.W<float>(c.L.dxact), c.W<float>(c.L.scal),
+                                          2, dX, c.W<int>(c.L.err), c.st));
     } else {
         XHC_K("full_dx", c.st, launch_full_dx(d, T32, c.W<float>(c.L.dz), wf, X, dinput, c.S<float>(c.L.hpre),
                                               c.S<int>(c.L.I), c.W<float>(c.L.dxact),
-                                              c.W<float>(c.L.tokgrad), dX, c.st));
+                                              c.W<float>(c.L.scal), dX, c.st));
     }
     return join_into(c.st, sd);
 }

@@ -1,4 +1,4 @@
-// Per-token coefficient kernels (one thread per token, fp32):
+// Per-token coefficient kernels (fp32; the Gram-Schmidt part in fp64):
 //   coef_full  norm statistics -> router scores, TopK routing, pre-maps
 //              (Eq. fused_normalized_projection, Eq. router, Eq. router_topk, Eq. param_pre)
 //   coef_act   active RMS -> post-map, Sinkhorn residual map + row clamp
@@ -7,335 +7,331 @@
 //              write-back contraction (Eq. sparse_write_delta)
 //   full_coef  reverse of coef_full (norm corrections, pre-map sigmoid, router through the
 //              selected routed scores only)
+//   colsum_out the alpha / b gradients from the column sums that bwd_coef's and full_coef's blocks leave
+//
+// A block takes a few consecutive tokens.  What it reads of the projections (every partial slot of a
+// split reduction: no separate pass sums them) is read with neighbouring threads on neighbouring
+// columns and kept in shared memory; the maps are computed with one thread per entry, the Sinkhorn
+// iterations with one lane per matrix row.  These kernels are bound by latency, not by bytes: with one
+// thread per token, which walked its row of slots alone, and the sums over slots and over tokens in
+// passes of their own, a training step of one N = 16, k = 4, C = 256 MLP sublayer of 512 tokens spent
+// 0.28 ms in them (bwd_coef 0.10, column sums 0.09, coef_act 0.034) and now 0.09 ms (bwd_coef 0.022);
+// at 16384 tokens and C = 2048 bwd_coef went from 0.12 to 0.056 ms.
 #include <algorithm>
 
 #include "xhc_internal.cuh"
 
 namespace xhc {
 
+namespace {
+
 // ---------------------------------------------------------------------------------------------
-// Sinkhorn of Eq. mhc_sinkhorn on a k x k block (k <= KM), with the App. A row clamp.
+// number of partial slots of 128-row tile m: the persistent CTAs of the stream-K plan that cover it
+
+template <class U>
+__device__ __forceinline__ U cta_of(U W, U P, U x) {
+    U c = x * P / W;
+    while (c > 0 && W * c / P > x) --c;
+    while (W * (c + 1) / P <= x) ++c;
+    return c;
+}
+template <class U>
+__device__ __forceinline__ int tile_slots(U W, U P, U KB, U m) {
+    return (int)(cta_of<U>(W, P, (m + 1) * KB - 1) - cta_of<U>(W, P, m * KB)) + 1;
+}
+__device__ __forceinline__ int slot_count(const SlotPlan& s, int m) {
+    if (s.n > 0) return s.n;
+    // 32-bit division where the products fit
+    if ((unsigned long long)s.W * (unsigned)(s.P + 1) < (1ull << 32))
+        return tile_slots<uint32_t>((uint32_t)s.W, (uint32_t)s.P, (uint32_t)s.KB, (uint32_t)m);
+    return tile_slots<unsigned long long>((unsigned long long)s.W, (unsigned long long)s.P,
+                                          (unsigned long long)s.KB, (unsigned long long)m);
+}
+
+// sum over `cnt` slots of p, `stride` apart, starting at slot q0 in steps of dq
+__device__ __forceinline__ float slot_sum(const float* p, long long stride, int cnt, int q0, int dq) {
+    float s = 0.f;
+    int q = q0;
+    for (; q + 7 * dq < cnt; q += 8 * dq) {
+        float v[8];   // eight loads in flight, added in slot order
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = p[(q + u * dq) * stride];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) s += v[u];
+    }
+    for (; q < cnt; q += dq) s += p[q * stride];
+    return s;
+}
+
+// Two arrays of slot sums into shared memory: dst[0, n0) = sums of p0 + e, dst[n0, n0 + n1) = sums of
+// p1 + e * step1.  With fewer elements than threads, groups of threads take interleaved slots and
+// their sums are added in group order (scr: one float per thread).  Ends with a block barrier.
+__device__ __forceinline__ void slot_sums(const float* __restrict__ p0, long long stride0, int cnt0, int n0,
+                                          const float* __restrict__ p1, long long stride1, int cnt1, int n1,
+                                          int step1, float* dst, float* scr) {
+    const int n = n0 + n1, nt = blockDim.x, tid = threadIdx.x;
+    const int ng = nt / n;
+    if (ng > 1) {
+        const int g = tid / n, e = tid - g * n;
+        if (g < ng)
+            scr[tid] = (e < n0) ? slot_sum(p0 + e, stride0, cnt0, g, ng)
+                                : slot_sum(p1 + (long long)(e - n0) * step1, stride1, cnt1, g, ng);
+        __syncthreads();
+        if (tid < n) {
+            float s = 0.f;
+            for (int q = 0; q < ng; ++q) s += scr[q * n + tid];
+            dst[tid] = s;
+        }
+    } else {
+        for (int e = tid; e < n; e += nt)
+            dst[e] = (e < n0) ? slot_sum(p0 + e, stride0, cnt0, 0, 1)
+                              : slot_sum(p1 + (long long)(e - n0) * step1, stride1, cnt1, 0, 1);
+    }
+    __syncthreads();
+}
+
+// ---------------------------------------------------------------------------------------------
+// Sinkhorn of Eq. mhc_sinkhorn on a k x k block (k <= KM), with the App. A row clamp.  KM neighbouring
+// lanes hold one matrix, lane a its row a; columns are summed over the lanes by shuffles.
 // exp(M - rowmax): the first row normalisation removes any per-row scale, so this equals exp(M).
 
 template <int KM>
-__device__ __forceinline__ void sk_init(const float (&M)[KM][KM], int k, float (&A)[KM][KM]) {
+__device__ __forceinline__ void sk_init(const float (&M)[KM], int a, int k, float (&A)[KM]) {
+    float mx = -INFINITY;
 #pragma unroll
-    for (int a = 0; a < KM; ++a) {
-        float mx = -INFINITY;
+    for (int b = 0; b < KM; ++b)
+        if (b < k) mx = fmaxf(mx, M[b]);
 #pragma unroll
-        for (int b = 0; b < KM; ++b)
-            if (a < k && b < k) mx = fmaxf(mx, M[a][b]);
-#pragma unroll
-        for (int b = 0; b < KM; ++b) A[a][b] = (a < k && b < k) ? expf(M[a][b] - mx) : 0.f;
-    }
+    for (int b = 0; b < KM; ++b) A[b] = (a < k && b < k) ? expf(M[b] - mx) : 0.f;
 }
 
-// one half-step: h even = row normalisation, h odd = column normalisation (one reciprocal per
-// row or column, then products)
+// row normalisation; returns the factor (0 for a row outside the matrix)
 template <int KM>
-__device__ __forceinline__ void sk_half(float (&A)[KM][KM], int k, int h) {
-    if ((h & 1) == 0) {
+__device__ __forceinline__ float sk_row(float (&A)[KM], int a, int k) {
+    float s = 0.f;
 #pragma unroll
-        for (int a = 0; a < KM; ++a) {
-            if (a >= k) continue;
-            float s = 0.f;
+    for (int b = 0; b < KM; ++b) s += A[b];
+    const float r = (a < k) ? 1.0f / s : 0.f;
 #pragma unroll
-            for (int b = 0; b < KM; ++b) s += A[a][b];
-            const float r = 1.0f / s;
-#pragma unroll
-            for (int b = 0; b < KM; ++b) A[a][b] = A[a][b] * r;
-        }
-    } else {
-#pragma unroll
-        for (int b = 0; b < KM; ++b) {
-            if (b >= k) continue;
-            float s = 0.f;
-#pragma unroll
-            for (int a = 0; a < KM; ++a) s += A[a][b];
-            const float r = 1.0f / s;
-#pragma unroll
-            for (int a = 0; a < KM; ++a) A[a][b] = A[a][b] * r;
-        }
-    }
+    for (int b = 0; b < KM; ++b) A[b] *= r;
+    return r;
 }
 
 template <int KM>
-__device__ __forceinline__ void sinkhorn_fwd(const float (&M)[KM][KM], int k, int iters,
-                                             float (&H)[KM][KM]) {
-    sk_init<KM>(M, k, H);
-    for (int h = 0; h < 2 * iters; ++h) sk_half<KM>(H, k, h);
+__device__ __forceinline__ void sum_rows(float (&v)[KM]) {
 #pragma unroll
-    for (int a = 0; a < KM; ++a) {
-        float s = 0.f;
+    for (int o = 1; o < KM; o <<= 1)
 #pragma unroll
-        for (int b = 0; b < KM; ++b) s += H[a][b];
-        if (s > 1.f) {
+        for (int b = 0; b < KM; ++b) v[b] += __shfl_xor_sync(0xffffffffu, v[b], o);
+}
+
+// column normalisation with factors r
+template <int KM>
+__device__ __forceinline__ void sk_col(float (&A)[KM], int k, float (&r)[KM]) {
 #pragma unroll
-            for (int b = 0; b < KM; ++b) H[a][b] = H[a][b] / s;
-        }
+    for (int b = 0; b < KM; ++b) r[b] = A[b];
+    sum_rows<KM>(r);
+#pragma unroll
+    for (int b = 0; b < KM; ++b) {
+        r[b] = (b < k) ? 1.0f / r[b] : 0.f;
+        A[b] *= r[b];
     }
 }
 
-// Reverse mode of sinkhorn_fwd: given dH returns dM (and H).  The forward iterates are rebuilt
-// from checkpoints: the matrix entering every L-th half-step is kept in shared memory (ck, laid
-// out [segment][entry][thread] with stride nth), and the half-steps of a segment are replayed
-// from its checkpoint, so the reverse sweep costs O(iters * L) half-steps instead of O(iters^2).
-// The replayed values are bit-identical to the forward ones.
 template <int KM>
-__device__ void sinkhorn_bwd(const float (&M)[KM][KM], int k, int iters, int L, float* ck, int nth,
-                             const float (&dH)[KM][KM], float (&H)[KM][KM], float (&dM)[KM][KM]) {
-    const int nh = 2 * iters;
-    float A[KM][KM], dA[KM][KM];
-    sk_init<KM>(M, k, A);
-    for (int h = 0; h < nh; ++h) {
-        if (h % L == 0) {
-            float* c = ck + (size_t)(h / L) * KM * KM * nth;
+__device__ __forceinline__ float row_total(const float (&A)[KM]) {
+    float s = 0.f;
 #pragma unroll
-            for (int a = 0; a < KM; ++a)
-#pragma unroll
-                for (int b = 0; b < KM; ++b) c[(a * KM + b) * nth] = A[a][b];
-        }
-        sk_half<KM>(A, k, h);
-    }
-    // clamp
-#pragma unroll
-    for (int a = 0; a < KM; ++a) {
-        float s = 0.f;
-#pragma unroll
-        for (int b = 0; b < KM; ++b) s += A[a][b];
-        if (s > 1.f) {
-            float dot = 0.f;
-#pragma unroll
-            for (int b = 0; b < KM; ++b) {
-                H[a][b] = A[a][b] / s;
-                dot += dH[a][b] * H[a][b];
-            }
-#pragma unroll
-            for (int b = 0; b < KM; ++b) dA[a][b] = (dH[a][b] - dot) / s;
-        } else {
-#pragma unroll
-            for (int b = 0; b < KM; ++b) {
-                H[a][b] = A[a][b];
-                dA[a][b] = dH[a][b];
-            }
-        }
-    }
-    // half-steps in reverse; the input of step h is replayed from its segment's checkpoint
-    for (int h = nh - 1; h >= 0; --h) {
-        const int h0 = (h / L) * L;
-        float In[KM][KM];
-        const float* c = ck + (size_t)(h / L) * KM * KM * nth;
-#pragma unroll
-        for (int a = 0; a < KM; ++a)
-#pragma unroll
-            for (int b = 0; b < KM; ++b) In[a][b] = c[(a * KM + b) * nth];
-        for (int q = h0; q < h; ++q) sk_half<KM>(In, k, q);
-        // output of step h
-        float Out[KM][KM];
-#pragma unroll
-        for (int a = 0; a < KM; ++a)
-#pragma unroll
-            for (int b = 0; b < KM; ++b) Out[a][b] = In[a][b];
-        sk_half<KM>(Out, k, h);
-        if ((h & 1) == 0) {
-#pragma unroll
-            for (int a = 0; a < KM; ++a) {
-                if (a >= k) continue;
-                float s = 0.f, dot = 0.f;
-#pragma unroll
-                for (int b = 0; b < KM; ++b) {
-                    s += In[a][b];
-                    dot += dA[a][b] * Out[a][b];
-                }
-#pragma unroll
-                for (int b = 0; b < KM; ++b) dA[a][b] = (dA[a][b] - dot) * (1.0f / s);
-            }
-        } else {
-#pragma unroll
-            for (int b = 0; b < KM; ++b) {
-                if (b >= k) continue;
-                float s = 0.f, dot = 0.f;
-#pragma unroll
-                for (int a = 0; a < KM; ++a) {
-                    s += In[a][b];
-                    dot += dA[a][b] * Out[a][b];
-                }
-#pragma unroll
-                for (int a = 0; a < KM; ++a) dA[a][b] = (dA[a][b] - dot) * (1.0f / s);
-            }
-        }
-    }
-    float A0[KM][KM];
-    sk_init<KM>(M, k, A0);
-#pragma unroll
-    for (int a = 0; a < KM; ++a)
-#pragma unroll
-        for (int b = 0; b < KM; ++b) dM[a][b] = (a < k && b < k) ? dA[a][b] * A0[a][b] : 0.f;
+    for (int b = 0; b < KM; ++b) s += A[b];
+    return s;
 }
 
 // ---------------------------------------------------------------------------------------------
-// slot_sum: x[e] = sum_q x[q * n + e] over the split-K partial slots, in slot order (the order
-// in which the coefficient kernels sum them, so a summed buffer read as one slot gives the same
-// bits), into slot 0.  Used when there are many slots (few tokens): one thread per element
-// instead of one thread per token walking every slot.
+// coef_full: a block of TB tokens (inside one 128-token tile of the projection)
 
-__global__ void k_slot_sum(float* __restrict__ x, int nslots, long long n) {
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-         e += (long long)gridDim.x * blockDim.x) {
+constexpr int CF_NT = 512;
+
+__global__ void __launch_bounds__(CF_NT) k_coef_full(Dims d, int T, int TB, const float* __restrict__ part,
+                                                     const float* __restrict__ pstats, SlotPlan sp,
+                                                     const float* __restrict__ wsum, int nws,
+                                                     const float* __restrict__ alpha_pre,
+                                                     const float* __restrict__ b_pre, float* __restrict__ zfull,
+                                                     float* __restrict__ stats, float* __restrict__ wsum_out,
+                                                     float* __restrict__ hpre, int* __restrict__ I,
+                                                     float* __restrict__ p) {
+    extern __shared__ float sm[];   // [TB][n] projections, [TB][2] statistics
+    __shared__ float scr[CF_NT], scw[CF_NT], ws[MAXN];
+    const int tid = threadIdx.x, lane = tid & 31, N = d.N, n = d.nfull;
+    const long long t0 = (long long)blockIdx.x * TB;
+    const int ntok = (int)min((long long)TB, T - t0);
+    // column sums of W_r: groups of N threads over the partials
+    const int gw = CF_NT / N;
+    if (d.hr && tid < gw * N) {
         float s = 0.f;
-        for (int q = 0; q < nslots; ++q) s += x[(long long)q * n + e];
-        x[e] = s;
+        for (int q = tid / N; q < nws; q += gw) s += wsum[q * N + tid % N];
+        scw[tid] = s;
     }
-}
-
-cudaError_t launch_slot_sum(float* x, int nslots, long long n, cudaStream_t st) {
-    const int blocks = (int)std::min<long long>((n + 255) / 256, 4096);
-    k_slot_sum<<<blocks, 256, 0, st>>>(x, nslots, n); note_launch();
-    return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------------------------
-// coef_full
-
-__global__ void k_coef_full(Dims d, int T, const float* __restrict__ part,
-                            const float* __restrict__ pstats, int splits,
-                            const float* __restrict__ wsum, const float* __restrict__ alpha_pre,
-                            const float* __restrict__ b_pre, float* __restrict__ zfull,
-                            float* __restrict__ stats, float* __restrict__ hpre,
-                            int* __restrict__ I, float* __restrict__ p) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= T) return;
-    const int n = d.nfull;
-    const float inv_nc = 1.0f / (float)(d.N * d.C);
-    float s1 = 0.f, s2 = 0.f;
-    for (int q = 0; q < splits; ++q) {
-        s1 += pstats[((int64_t)q * T + t) * 2 + 0];
-        s2 += pstats[((int64_t)q * T + t) * 2 + 1];
+    const int nsl = slot_count(sp, (int)(t0 >> 7));
+    float* zs = sm;
+    float* st = sm + ntok * n;
+    slot_sums(part + t0 * n, (long long)T * n, nsl, ntok * n, pstats + t0 * 2, (long long)T * 2, nsl, ntok * 2, 1,
+              zs, scr);
+    if (d.hr && tid < N) {
+        float s = 0.f;
+        for (int q = 0; q < gw; ++q) s += scw[q * N + tid];
+        ws[tid] = s;
+        if (blockIdx.x == 0) wsum_out[tid] = s;
     }
-    const float mu = s1 * inv_nc, nu = s2 * inv_nc;
-    stats[(int64_t)t * 2 + 0] = mu;
-    stats[(int64_t)t * 2 + 1] = nu;
-    const float rstd = 1.0f / sqrtf(nu + d.eps);
-    float zr[MAXN];
-    for (int o = 0; o < n; ++o) {
-        float z = 0.f;
-        for (int q = 0; q < splits; ++q) z += part[((int64_t)q * T + t) * n + o];
-        zfull[(int64_t)t * n + o] = z;
-        if (d.hr && o < d.N) {
-            zr[o] = z;
-        } else {
-            const int qo = o - (d.hr ? d.N : 0);
-            const int slot = qo / d.N, i = qo - slot * d.N;
-            hpre[((int64_t)t * d.G + slot) * d.N + i] =
-                sigm(alpha_pre[slot] * (z * rstd) + b_pre[slot * d.N + i]);
+    const float inv_nc = 1.0f / (float)(N * d.C);
+    if (tid < ntok * 2) stats[t0 * 2 + tid] = st[tid] * inv_nc;
+    const int roff = d.hr ? N : 0, GN = d.G * N;
+    for (int e = tid; e < ntok * n; e += CF_NT) {
+        const int tt = e / n, o = e - tt * n;
+        const float z = zs[e];
+        zfull[t0 * n + e] = z;
+        if (o >= roff) {
+            const int qo = o - roff, slot = qo / N;
+            const float rstd = 1.0f / sqrtf(st[tt * 2 + 1] * inv_nc + d.eps);
+            hpre[(t0 + tt) * GN + qo] = sigm(alpha_pre[slot] * (z * rstd) + b_pre[qo]);
         }
     }
-    // Eq. router_topk: fixed streams 0..m-1 (p = 1), then TopK over i >= m by router logit
-    // (sigmoid and softmax are both monotone in the logit), descending, ties to the lower
-    // stream index.
-    for (int j = 0; j < d.m; ++j) {
-        I[(int64_t)t * d.k + j] = j;
-        p[(int64_t)t * d.k + j] = 1.0f;
-    }
-    if (d.hr) {
+    __syncthreads();
+    // Eq. router_topk, a warp per token with a lane per stream: fixed streams 0..m-1 (p = 1), then TopK
+    // over i >= m by router logit (sigmoid and softmax are both monotone in the logit), descending,
+    // ties to the lower stream index.
+    for (int tt = tid >> 5; tt < ntok; tt += CF_NT / 32) {
+        const long long tk = (t0 + tt) * d.k;
+        if (lane < d.m) {
+            I[tk + lane] = lane;
+            p[tk + lane] = 1.0f;
+        }
+        if (!d.hr) continue;
+        const float mu = st[tt * 2] * inv_nc, nu = st[tt * 2 + 1] * inv_nc;
         const float lstd = 1.0f / sqrtf(nu - mu * mu + d.eps);
-        float zmax = -INFINITY;
-        for (int i = 0; i < d.N; ++i) {
-            zr[i] = (zr[i] - mu * wsum[i]) * lstd;
-            zmax = fmaxf(zmax, zr[i]);
+        const float z = (lane < N) ? (zs[tt * n + lane] - mu * ws[lane]) * lstd : -INFINITY;
+        float zmax = z, den = 0.f;
+        if (d.softmax) {
+            // softmax router: s_i = exp(z_i) / sum over all N logits (the fixed streams' included)
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
+            den = warp_sum(lane < N ? expf(z - zmax) : 0.f);
         }
-        // softmax router: s_i = exp(z_i) / sum over all N logits (the fixed streams' included)
-        float den = 0.f;
-        if (d.softmax)
-            for (int i = 0; i < d.N; ++i) den += expf(zr[i] - zmax);
-        uint32_t taken = 0u;
+        bool open = lane >= d.m && lane < N;
         for (int j = d.m; j < d.k; ++j) {
-            int best = -1;
-            float bv = 0.f;
-            for (int i = d.m; i < d.N; ++i) {
-                if (taken & (1u << i)) continue;
-                if (best < 0 || zr[i] > bv) {
-                    best = i;
-                    bv = zr[i];
+            // the first open stream wins over a NaN logit of a later one, and with a NaN of its own
+            const unsigned om = __ballot_sync(0xffffffffu, open);
+            float key = z;
+            if (z != z) key = (lane == __ffs(om) - 1) ? INFINITY : -INFINITY;
+            int best = open ? lane : 64;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float ko = __shfl_xor_sync(0xffffffffu, key, o);
+                const int bo = __shfl_xor_sync(0xffffffffu, best, o);
+                if (bo < 64 && (best >= 64 || ko > key || (ko == key && bo < best))) {
+                    key = ko;
+                    best = bo;
                 }
             }
-            taken |= 1u << best;
-            I[(int64_t)t * d.k + j] = best;
-            p[(int64_t)t * d.k + j] = d.softmax ? expf(bv - zmax) / den : sigm(bv);
+            if (lane == best) {
+                open = false;
+                I[tk + j] = lane;
+                p[tk + j] = d.softmax ? expf(z - zmax) / den : sigm(z);
+            }
         }
     }
-}
-
-cudaError_t launch_coef_full(const Dims& d, int T, const float* part, const float* pstats,
-                             int splits, const float* wsum, const float* alpha_pre,
-                             const float* b_pre, float* zfull, float* stats, float* hpre,
-                             int* I, float* p, cudaStream_t st) {
-    k_coef_full<<<(T + 127) / 128, 128, 0, st>>>(d, T, part, pstats, splits, wsum, alpha_pre,
-                                                  b_pre, zfull, stats, hpre, I, p); note_launch();
-    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------------------------
 // coef_act
 
 template <int KM>
-__global__ void k_coef_act(Dims d, int slot, int T, const float* __restrict__ part,
-                           const float* __restrict__ pstats, int ssplits, int splits,
-                           const float* __restrict__ alpha_post, const float* __restrict__ b_post,
-                           const float* __restrict__ alpha_res, const float* __restrict__ b_res,
-                           float* __restrict__ zact, float* __restrict__ rs,
-                           float* __restrict__ hpost, float* __restrict__ hres) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= T) return;
-    const int k = d.k, K = d.K[slot], n = d.nact[slot];
-    const bool last = (slot == d.G - 1);
-    float s2 = 0.f;
-    for (int q = 0; q < ssplits; ++q) s2 += pstats[((int64_t)q * T + t) * 2 + 1];
-    const float r = 1.0f / sqrtf(s2 / (float)(k * d.C) + d.eps);
-    rs[t] = r;
+__global__ void __launch_bounds__(CF_NT) k_coef_act(Dims d, int slot, int T, int TB, const float* __restrict__ part,
+                                                    const float* __restrict__ pstats, int ssplits, SlotPlan sp,
+                                                    const float* __restrict__ alpha_post,
+                                                    const float* __restrict__ b_post,
+                                                    const float* __restrict__ alpha_res,
+                                                    const float* __restrict__ b_res, float* __restrict__ zact,
+                                                    float* __restrict__ rs, float* __restrict__ hpost,
+                                                    float* __restrict__ hres) {
+    extern __shared__ float sm[];   // [TB][n] projections, [TB] sums of squares
+    __shared__ float scr[CF_NT];
+    const int tid = threadIdx.x, k = d.k, kK = d.k * d.K[slot], n = d.nact[slot];
+    const long long t0 = (long long)blockIdx.x * TB;
+    const int ntok = (int)min((long long)TB, T - t0);
+    const int nsl = slot_count(sp, (int)(t0 >> 7));
+    float* zs = sm;
+    float* st = sm + ntok * n;
+    slot_sums(part + t0 * n, (long long)T * n, nsl, ntok * n, pstats + t0 * 2 + 1, (long long)T * 2, ssplits, ntok, 2,
+              zs, scr);
+    const float inv = 1.0f / (float)(k * d.C);
+    if (tid < ntok) rs[t0 + tid] = 1.0f / sqrtf(st[tid] * inv + d.eps);
     const float ap = alpha_post[slot];
-    float M[KM][KM];
-#pragma unroll
-    for (int a = 0; a < KM; ++a)
-#pragma unroll
-        for (int b = 0; b < KM; ++b) M[a][b] = 0.f;
-    const float ar = last ? alpha_res[0] : 0.f;
-    for (int o = 0; o < n; ++o) {
-        float z = 0.f;
-        for (int q = 0; q < splits; ++q) z += part[((int64_t)q * T + t) * n + o];
-        zact[(int64_t)t * n + o] = z;
-        if (o < k * K) {
-            hpost[(int64_t)t * k * K + o] = 2.0f * sigm(ap * (z * r) + b_post[o]);
-        } else {
-            const int q = o - k * K, a = q / k, b = q - a * k;
-#pragma unroll
-            for (int aa = 0; aa < KM; ++aa)
-#pragma unroll
-                for (int bb = 0; bb < KM; ++bb)
-                    if (aa == a && bb == b) M[aa][bb] = ar * (z * r) + b_res[q];
+    for (int e = tid; e < ntok * n; e += CF_NT) {
+        const int tt = e / n, o = e - tt * n;
+        const float z = zs[e];
+        zact[t0 * n + e] = z;
+        if (o < kK) {
+            const float r = 1.0f / sqrtf(st[tt] * inv + d.eps);
+            hpost[(t0 + tt) * kK + o] = 2.0f * sigm(ap * (z * r) + b_post[o]);
         }
     }
-    if (last) {
-        float H[KM][KM];
-        sinkhorn_fwd<KM>(M, k, d.iters, H);
+    if (slot != d.G - 1 || (tid & ~31) >= TB * KM) return;
+    // whole warps run the iterations (lanes past the last token repeat it)
+    const int tq = tid / KM, a = tid - tq * KM;
+    const int tt = min(tq, ntok - 1);
+    const float ar = alpha_res[0], r = 1.0f / sqrtf(st[tt] * inv + d.eps);
+    float M[KM], H[KM], cr[KM];
 #pragma unroll
-        for (int a = 0; a < KM; ++a)
+    for (int b = 0; b < KM; ++b)
+        M[b] = (a < k && b < k) ? ar * (zs[tt * n + kK + a * k + b] * r) + b_res[a * k + b] : 0.f;
+    sk_init<KM>(M, a, k, H);
+    for (int it = 0; it < d.iters; ++it) {
+        sk_row<KM>(H, a, k);
+        sk_col<KM>(H, k, cr);
+    }
+    const float s = row_total<KM>(H);
+    if (tq < ntok && a < k) {
+        float* dst = hres + (t0 + tt) * k * k + a * k;
 #pragma unroll
-            for (int b = 0; b < KM; ++b)
-                if (a < k && b < k) hres[(int64_t)t * k * k + a * k + b] = H[a][b];
+        for (int b = 0; b < KM; ++b)
+            if (b < k) dst[b] = (s > 1.f) ? H[b] / s : H[b];
     }
 }
 
+// tokens per block: enough blocks for the GPU at few tokens, whole warps of matrix rows at many; a
+// power of two up to 32, so that a block lies in one 128-token tile
+int coef_tokens(int T) {
+    int tb = 1;
+    while (tb < 32 && T / (2 * tb) >= 2 * device_sms()) tb *= 2;
+    return tb;
+}
+
+}  // namespace
+
+cudaError_t launch_coef_full(const Dims& d, int T, const float* part, const float* pstats,
+                             const SlotPlan& sp, const float* wsum, int nws, const float* alpha_pre,
+                             const float* b_pre, float* zfull, float* stats, float* wsum_out, float* hpre,
+                             int* I, float* p, cudaStream_t st) {
+    const int TB = coef_tokens(T);
+    const size_t sm = (size_t)TB * (d.nfull + 2) * 4;
+    k_coef_full<<<(T + TB - 1) / TB, CF_NT, sm, st>>>(d, T, TB, part, pstats, sp, wsum, nws, alpha_pre, b_pre,
+                                                      zfull, stats, wsum_out, hpre, I, p); note_launch();
+    return cudaGetLastError();
+}
+
 cudaError_t launch_coef_act(const Dims& d, int slot, int T, const float* part,
-                            const float* pstats, int ssplits, int splits, const float* alpha_post,
+                            const float* pstats, int ssplits, const SlotPlan& sp, const float* alpha_post,
                             const float* b_post, const float* alpha_res, const float* b_res,
                             float* zact, float* rs, float* hpost, float* hres, cudaStream_t st) {
+    const int TB = coef_tokens(T);
+    const size_t sm = (size_t)TB * (d.nact[slot] + 1) * 4;
+    const unsigned grid = (unsigned)((T + TB - 1) / TB);
     if (d.k <= 4) {
-        k_coef_act<4><<<(T + 127) / 128, 128, 0, st>>>(d, slot, T, part, pstats, ssplits, splits, alpha_post,
-                                                        b_post, alpha_res, b_res, zact, rs, hpost, hres); note_launch();
+        k_coef_act<4><<<grid, CF_NT, sm, st>>>(d, slot, T, TB, part, pstats, ssplits, sp, alpha_post, b_post,
+                                               alpha_res, b_res, zact, rs, hpost, hres); note_launch();
     } else {
-        k_coef_act<8><<<(T + 127) / 128, 128, 0, st>>>(d, slot, T, part, pstats, ssplits, splits, alpha_post,
-                                                        b_post, alpha_res, b_res, zact, rs, hpost, hres); note_launch();
+        k_coef_act<8><<<grid, CF_NT, sm, st>>>(d, slot, T, TB, part, pstats, ssplits, sp, alpha_post, b_post,
+                                               alpha_res, b_res, zact, rs, hpost, hres); note_launch();
     }
     return cudaGetLastError();
 }
@@ -344,307 +340,544 @@ cudaError_t launch_coef_act(const Dims& d, int slot, int T, const float* part,
 // bwd_coef: per token, from the reductions
 //   P[j][a] = <dXn_j, u_a>   Q[j][i] = <dXn_j, x_act_i> (last slot)   Gm[a][b] = <u_a, u_b> (GS)
 // produce E[j][a] = p_j sum_q Hpost[j][q] B[q][a], D = dG + dG^T, H_res, the scaled projection
-// gradient dZs = dz * r, the RMS coefficient cx, dp (+=) and the alpha/b contributions.
+// gradient dZs = dz * r, the RMS coefficient cx, dp and the alpha / b contributions (summed over the
+// block's tokens).
+//
+// A block takes TB tokens: its first warp the post-map and Gram-Schmidt reverse of token `lane`, its
+// other warps (last slot) the Sinkhorn reverse with one lane per matrix row.  The matrix entering every
+// iteration is kept in shared memory, so the reverse sweep rebuilds one half-step an iteration.
+
+namespace {
 
 template <int KM>
-__global__ void k_bwd_coef(Dims d, int slot, int T, const float* __restrict__ red, int nslice,
-                           const float* __restrict__ zact, const float* __restrict__ rs,
-                           const float* __restrict__ p, const float* __restrict__ hpost,
-                           const double* __restrict__ gram, int skL,
-                           const float* __restrict__ alpha_post, const float* __restrict__ b_post,
-                           const float* __restrict__ alpha_res, const float* __restrict__ b_res,
-                           float* __restrict__ tokmat, float* __restrict__ dzs,
-                           float* __restrict__ dp, float* __restrict__ tokgrad) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= T) return;
-    const int k = d.k, K = d.K[slot], n = d.nact[slot];
-    const bool last = (slot == d.G - 1);
-    const bool gs = (K > 1) && d.gs;
-    // reduction slots per token (see wb_bred): P at j*4 + a, Q at KM*4 + j*KM + i; the Gram
-    // matrix of the components comes from the forward (lower triangle packed, fp64)
-    const int offQ = KM * 4;
-    float Pm[KM][MAXCOMP], Q[KM][KM];
-    double Gm[MAXCOMP][MAXCOMP];
+__device__ void sinkhorn_bwd(const float (&M)[KM], int a, int k, int iters, float* ck, int stride,
+                             const float (&dH)[KM], float (&H)[KM], float (&dM)[KM]) {
+    float A[KM], A0[KM], rc[KM], dA[KM];
+    sk_init<KM>(M, a, k, A);
 #pragma unroll
-    for (int j = 0; j < KM; ++j) {
+    for (int b = 0; b < KM; ++b) A0[b] = A[b];
+    for (int it = 0; it < iters; ++it) {
 #pragma unroll
-        for (int a = 0; a < MAXCOMP; ++a) Pm[j][a] = 0.f;
-#pragma unroll
-        for (int i = 0; i < KM; ++i) Q[j][i] = 0.f;
+        for (int b = 0; b < KM; ++b) ck[(it * KM + b) * stride] = A[b];
+        sk_row<KM>(A, a, k);
+        sk_col<KM>(A, k, rc);
     }
-    // loops to MAXCOMP / KM with guards on K / k: compile-time indices, registers only
+    // clamp
+    const float s = row_total<KM>(A);
+    if (s > 1.f) {
+        float dot = 0.f;
 #pragma unroll
-    for (int a = 0; a < MAXCOMP; ++a)
-#pragma unroll
-        for (int b = 0; b < MAXCOMP; ++b) Gm[a][b] = 0.0;
-    for (int s = 0; s < nslice; ++s) {
-        const float* rp = red + ((int64_t)t * nslice + s) * NRED;
-#pragma unroll
-        for (int j = 0; j < KM; ++j)
-#pragma unroll
-            for (int a = 0; a < MAXCOMP; ++a)
-                if (j < k && a < K) Pm[j][a] += rp[j * 4 + a];
-        if (last) {
-#pragma unroll
-            for (int j = 0; j < KM; ++j)
-#pragma unroll
-                for (int i = 0; i < KM; ++i)
-                    if (j < k && i < k) Q[j][i] += rp[offQ + j * KM + i];
+        for (int b = 0; b < KM; ++b) {
+            H[b] = A[b] / s;
+            dot += dH[b] * H[b];
         }
-    }
-    if (gs) {
 #pragma unroll
-        for (int a = 0; a < MAXCOMP; ++a)
-#pragma unroll
-            for (int b = 0; b <= a; ++b)
-                if (a < K) Gm[a][b] = gram[(int64_t)t * NGRAM + a * (a + 1) / 2 + b];
-    }
-#pragma unroll
-    for (int a = 0; a < MAXCOMP; ++a)
-#pragma unroll
-        for (int b = a + 1; b < MAXCOMP; ++b)
-            if (b < K) Gm[a][b] = Gm[b][a];
-    double B[MAXCOMP][MAXCOMP], cc[MAXCOMP][MAXCOMP], vv[MAXCOMP];
-    if (gs) {
-        gs_coef(Gm, K, (double)d.eps_gs, B, cc, vv);
+        for (int b = 0; b < KM; ++b) dA[b] = (dH[b] - dot) / s;
     } else {
 #pragma unroll
-        for (int a = 0; a < MAXCOMP; ++a)
-#pragma unroll
-            for (int b = 0; b < MAXCOMP; ++b) B[a][b] = (a == b) ? 1.0 : 0.0;
+        for (int b = 0; b < KM; ++b) {
+            H[b] = A[b];
+            dA[b] = dH[b];
+        }
     }
-    float* tm = tokmat + (int64_t)t * TOKMAT;
-    float* tg = tokgrad + (int64_t)t * NTG;
-    const float r = rs[t];
-    const float* za = zact + (int64_t)t * n;
-    const float ap = alpha_post[slot];
-    // the scaled map-logit gradients go straight to dzs (dz * r); sdz = sum_o dz_o zact_o feeds
-    // the RMS coefficient cx
-    float* dzr = dzs + (int64_t)t * n;
-    float sdz = 0.f;
-    double dB[MAXCOMP][MAXCOMP];
+    for (int it = iters - 1; it >= 0; --it) {
+        // R: after the row step; A: after the column step
+        float R[KM], dot[KM];
 #pragma unroll
-    for (int a = 0; a < MAXCOMP; ++a)
+        for (int b = 0; b < KM; ++b) R[b] = ck[(it * KM + b) * stride];
+        const float rr = sk_row<KM>(R, a, k);
 #pragma unroll
-        for (int b = 0; b < MAXCOMP; ++b) dB[a][b] = 0.0;
-    float dap = 0.f;
+        for (int b = 0; b < KM; ++b) A[b] = R[b];
+        sk_col<KM>(A, k, rc);
 #pragma unroll
-    for (int j = 0; j < KM; ++j) {
-        if (j >= k) continue;
-        const float pj = p[(int64_t)t * k + j];
-        float dpj = 0.f;
+        for (int b = 0; b < KM; ++b) dot[b] = dA[b] * A[b];
+        sum_rows<KM>(dot);
+        float rdot = 0.f;
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            float e = 0.f;
-            if (a < K) {
+        for (int b = 0; b < KM; ++b) {
+            dA[b] = (dA[b] - dot[b]) * rc[b];
+            rdot += dA[b] * R[b];
+        }
+#pragma unroll
+        for (int b = 0; b < KM; ++b) dA[b] = (dA[b] - rdot) * rr;
+    }
+#pragma unroll
+    for (int b = 0; b < KM; ++b) dM[b] = (a < k && b < k) ? dA[b] * A0[b] : 0.f;
+}
+
+// shared memory of one token, in floats: reductions, E, D, H_res, scaled gradients, column terms and
+// the two parts of sum_o dz_o zact_o
+template <int KM>
+struct BwdTok {
+    static constexpr int R = 0;                       // [KM*4] P, [KM*KM] Q
+    static constexpr int E = R + KM * 4 + KM * KM;    // [KM*4]
+    static constexpr int D = E + KM * 4;              // [16]
+    static constexpr int H = D + 16;                  // [KM*KM]
+    static constexpr int DZ = H + KM * KM;            // [KM*4 + KM*KM]
+    static constexpr int TG = DZ + KM * 4 + KM * KM;  // [KM*4 + 1 + KM*KM + 1]
+    static constexpr int S = TG + KM * 4 + KM * KM + 2;
+    static constexpr int ROW = (S + KM + 1) | 1;      // odd: a lane per token hits different banks
+};
+
+template <int KM>
+__global__ void __launch_bounds__(160) k_bwd_coef(Dims d, int slot, int T, int TB, const float* __restrict__ red,
+                                                  int nslice, const float* __restrict__ zact,
+                                                  const float* __restrict__ rs, const float* __restrict__ p,
+                                                  const float* __restrict__ hpost, const double* __restrict__ gram,
+                                                  const float* __restrict__ alpha_post,
+                                                  const float* __restrict__ alpha_res,
+                                                  const float* __restrict__ b_res, float* __restrict__ tokmat,
+                                                  float* __restrict__ dzs, float* __restrict__ dp,
+                                                  float* __restrict__ colp) {
+    using L = BwdTok<KM>;
+    extern __shared__ float sm[];   // [TB][ROW], then the Sinkhorn iterates
+    const int tid = threadIdx.x, lane = tid & 31, nt = blockDim.x;
+    const int k = d.k, K = d.K[slot], kK = k * K, n = d.nact[slot];
+    const bool last = (slot == d.G - 1);
+    const bool gs = (K > 1) && d.gs;
+    const long long t0 = (long long)blockIdx.x * TB;
+    const int ntok = (int)min((long long)TB, T - t0);
+    // reduction slots per token (see wb_bred): P at j*4 + a, Q at KM*4 + j*KM + i
+    {
+        const int nv = last ? KM * 4 + KM * KM : KM * 4;
+        for (int e = tid; e < ntok * nv; e += nt) {
+            const int tt = e / nv, q = e - tt * nv;
+            bool used;
+            if (q < KM * 4) used = (q >> 2) < k && (q & 3) < K;
+            else used = (q - KM * 4) / KM < k && (q - KM * 4) % KM < k;
+            float s = 0.f;
+            if (used) s = slot_sum(red + (t0 + tt) * nslice * NRED + q, NRED, nslice, 0, 1);
+            sm[tt * L::ROW + L::R + q] = s;
+        }
+    }
+    __syncthreads();
+    const float ar = last ? alpha_res[0] : 0.f;
+    if (tid < 32) {
+        if (lane < ntok) {
+            const long long t = t0 + lane;
+            float* row = sm + lane * L::ROW;
+            const float r = rs[t], ap = alpha_post[slot];
+            const float* za = zact + t * n;
+            float B[MAXCOMP][MAXCOMP];
+            double Gm[NGRAM];
+            GramSchmidt G;
+            if (gs) {
+#pragma unroll
+                for (int q = 0; q < NGRAM; ++q) Gm[q] = 0.0;
+#pragma unroll
+                for (int a = 0; a < MAXCOMP; ++a)
+#pragma unroll
+                    for (int b = 0; b <= a; ++b)
+                        if (a < K) Gm[a * (a + 1) / 2 + b] = gram[t * NGRAM + a * (a + 1) / 2 + b];
+                G.forward(Gm, (double)d.eps_gs);
+                G.coef(B);
+            } else {
 #pragma unroll
                 for (int q = 0; q < MAXCOMP; ++q)
-                    if (q < K) e += hpost[((int64_t)t * k + j) * K + q] * (float)B[q][a];
+#pragma unroll
+                    for (int a = 0; a < MAXCOMP; ++a) B[q][a] = (q == a) ? 1.f : 0.f;
             }
-            tm[j * 4 + a] = pj * e;
-        }
+            double d10 = 0.0, d20 = 0.0, d21 = 0.0, d30 = 0.0, d31 = 0.0, d32 = 0.0;
+            float dap = 0.f, sdz = 0.f;
 #pragma unroll
-        for (int q = 0; q < MAXCOMP; ++q) {
-            if (q >= K) continue;
-            float pb = 0.f;
+            for (int j = 0; j < KM; ++j) {
+                if (j >= k) continue;
+                const float pj = p[t * k + j];
+                float h[MAXCOMP], P[MAXCOMP], dpj = 0.f;
 #pragma unroll
-            for (int a = 0; a < MAXCOMP; ++a)
-                if (a < K) pb += Pm[j][a] * (float)B[q][a];
-            const float h = hpost[((int64_t)t * k + j) * K + q];
-            const float dh = pj * pb;
-            dpj += h * pb;
+                for (int q = 0; q < MAXCOMP; ++q) {
+                    h[q] = (q < K) ? hpost[(t * k + j) * K + q] : 0.f;
+                    P[q] = row[L::R + j * 4 + q];
+                }
 #pragma unroll
-            for (int a = 0; a < MAXCOMP; ++a)
-                if (a < K) dB[q][a] += (double)(pj * h) * (double)Pm[j][a];
-            // H = 2 sigma(y): dy = dH * H * (1 - H / 2)
-            const float dy = dh * h * (1.0f - 0.5f * h);
-            const int o = j * K + q;
-            const float dzo = ap * dy;
-            dap += dy * (za[o] * r);
-            tg[o] = dy;
-            sdz += dzo * za[o];
-            dzr[o] = dzo * r;
-        }
-        dp[(int64_t)t * k + j] += dpj;
-    }
-    tg[k * K] = dap;
-    // D = dG + dG^T (symmetric Gram entries)
+                for (int a = 0; a < MAXCOMP; ++a) {
+                    float e = 0.f;
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+                    for (int q = a; q < MAXCOMP; ++q) e += h[q] * B[q][a];
+                    row[L::E + j * 4 + a] = pj * e;
+                }
 #pragma unroll
-        for (int b = 0; b < 4; ++b) tm[32 + a * 4 + b] = 0.f;
-    if (gs) {
-        double dG[MAXCOMP][MAXCOMP];
-        gs_coef_bwd(Gm, K, B, cc, vv, dB, dG);
+                for (int q = 0; q < MAXCOMP; ++q) {
+                    if (q >= K) continue;
+                    float pb = 0.f;
 #pragma unroll
-        for (int a = 0; a < MAXCOMP; ++a)
-#pragma unroll
-            for (int b = 0; b < MAXCOMP; ++b)
-                if (a < K && b < K) tm[32 + a * 4 + b] = (float)(dG[a][b] + dG[b][a]);
-    }
-    if (last) {
-        float M[KM][KM], dH[KM][KM], H[KM][KM], dM[KM][KM];
-        const float ar = alpha_res[0];
-#pragma unroll
-        for (int a = 0; a < KM; ++a)
-#pragma unroll
-            for (int b = 0; b < KM; ++b) {
-                const bool v = (a < k && b < k);
-                M[a][b] = v ? ar * (za[k * K + a * k + b] * r) + b_res[a * k + b] : 0.f;
-                dH[a][b] = v ? Q[a][b] : 0.f;
+                    for (int a = 0; a <= q; ++a) pb += P[a] * B[q][a];
+                    dpj += h[q] * pb;
+                    // H = 2 sigma(y): dy = dH * H * (1 - H / 2)
+                    const float dy = pj * pb * h[q] * (1.0f - 0.5f * h[q]);
+                    const int o = j * K + q;
+                    const float z = za[o], dzo = ap * dy;
+                    dap += dy * (z * r);
+                    sdz += dzo * z;
+                    row[L::TG + o] = dy;
+                    row[L::DZ + o] = dzo * r;
+                }
+                if (gs) {
+                    // dB[q][a] = sum_j p_j H_post[j][q] P[j][a], below the diagonal
+                    const double p0 = (double)P[0], p1 = (double)P[1], p2 = (double)P[2];
+                    const double h1 = (double)(pj * h[1]), h2 = (double)(pj * h[2]), h3 = (double)(pj * h[3]);
+                    d10 = fma(h1, p0, d10);
+                    d20 = fma(h2, p0, d20);
+                    d21 = fma(h2, p1, d21);
+                    d30 = fma(h3, p0, d30);
+                    d31 = fma(h3, p1, d31);
+                    d32 = fma(h3, p2, d32);
+                }
+                // slots run from the last to the first: the last one stores, the others add
+                dp[t * k + j] = last ? dpj : dp[t * k + j] + dpj;
             }
-        extern __shared__ float sk_ck[];
-        sinkhorn_bwd<KM>(M, k, d.iters, skL, sk_ck + threadIdx.x, blockDim.x, dH, H, dM);
-        float dar = 0.f;
+            row[L::TG + kK] = dap;
+            row[L::S + KM] = sdz;
+            double D[NGRAM];
 #pragma unroll
-        for (int a = 0; a < KM; ++a)
+            for (int q = 0; q < NGRAM; ++q) D[q] = 0.0;
+            if (gs) G.reverse(Gm, d10, d20, d21, d30, d31, d32, D);
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b)
+                    row[L::D + a * 4 + b] = (float)D[a >= b ? a * (a + 1) / 2 + b : b * (b + 1) / 2 + a];
+        }
+    } else if (last) {
+        const int tq = (tid - 32) / KM, a = (tid - 32) - tq * KM;
+        const int tt = min(tq, ntok - 1);
+        const long long t = t0 + tt;
+        float* row = sm + tt * L::ROW;
+        const float r = rs[t];
+        float M[KM], z[KM], dH[KM], H[KM], dM[KM];
+#pragma unroll
+        for (int b = 0; b < KM; ++b) {
+            const bool v = (a < k && b < k);
+            z[b] = v ? zact[t * n + kK + a * k + b] : 0.f;
+            M[b] = v ? ar * (z[b] * r) + b_res[a * k + b] : 0.f;
+            dH[b] = v ? row[L::R + KM * 4 + a * KM + b] : 0.f;
+        }
+        sinkhorn_bwd<KM>(M, a, k, d.iters, sm + TB * L::ROW + (tid - 32), TB * KM, dH, H, dM);
+        if (tq < ntok) {
+            float sdz = 0.f, dar = 0.f;
 #pragma unroll
             for (int b = 0; b < KM; ++b) {
                 if (a >= k || b >= k) continue;
-                const int o = k * K + a * k + b;
-                const float dzo = ar * dM[a][b];
-                dar += dM[a][b] * (za[o] * r);
-                tg[k * K + 1 + a * k + b] = dM[a][b];
-                tm[48 + a * 8 + b] = H[a][b];
-                sdz += dzo * za[o];
-                dzr[o] = dzo * r;
+                const int o = kK + a * k + b;
+                const float dzo = ar * dM[b];
+                dar += dM[b] * (z[b] * r);
+                sdz += dzo * z[b];
+                row[L::TG + kK + 1 + a * k + b] = dM[b];
+                row[L::DZ + o] = dzo * r;
+                row[L::H + a * KM + b] = H[b];
             }
-        tg[k * K + 1 + k * k] = dar;
+            row[L::S + a] = sdz;
+            // this row's share of d alpha_res: the reductions of the row are read by no one any more
+            row[L::R + KM * 4 + a * KM] = dar;
+        }
     }
-    // active RMS: z_o = r * zraw_o, r = (sum x^2 / kC + eps)^(-1/2)
-    tm[112] = r * r * r / (float)(k * d.C) * sdz;
+    __syncthreads();
+    // per-token matrices and gradients, neighbouring threads on neighbouring words
+    for (int e = tid; e < ntok * (KM * 4 + 16); e += nt) {
+        const int tt = e / (KM * 4 + 16), q = e - tt * (KM * 4 + 16);
+        const float v = sm[tt * L::ROW + L::E + q];
+        if (q >= KM * 4) tokmat[(t0 + tt) * TOKMAT + 32 + q - KM * 4] = v;
+        else if ((q >> 2) < k) tokmat[(t0 + tt) * TOKMAT + q] = v;
+    }
+    if (last)
+        for (int e = tid; e < ntok * KM * KM; e += nt) {
+            const int tt = e / (KM * KM), q = e - tt * KM * KM, a = q / KM, b = q - a * KM;
+            if (a < k && b < k) tokmat[(t0 + tt) * TOKMAT + 48 + a * 8 + b] = sm[tt * L::ROW + L::H + q];
+        }
+    for (int e = tid; e < ntok * n; e += nt) {
+        const int tt = e / n, o = e - tt * n;
+        dzs[t0 * n + e] = sm[tt * L::ROW + L::DZ + o];
+    }
+    if (tid < ntok) {
+        // active RMS: z_o = r * zraw_o, r = (sum x^2 / kC + eps)^(-1/2)
+        const float* row = sm + tid * L::ROW;
+        const float r = rs[t0 + tid];
+        float sdz = row[L::S + KM];
+        if (last)
+            for (int a = 0; a < k; ++a) sdz += row[L::S + a];
+        tokmat[(t0 + tid) * TOKMAT + 112] = r * r * r / (float)(k * d.C) * sdz;
+    }
+    // column sums over the block's tokens: [dy (k K) | d alpha_post | dM (k k) | d alpha_res]
+    const int ncol = kK + 1 + (last ? k * k + 1 : 0);
+    for (int c = tid; c < ncol; c += nt) {
+        float s = 0.f;
+        if (c <= kK + k * k) {
+            for (int tt = 0; tt < ntok; ++tt) s += sm[tt * L::ROW + L::TG + c];
+        } else {
+            for (int tt = 0; tt < ntok; ++tt)
+                for (int a = 0; a < k; ++a) s += sm[tt * L::ROW + L::R + KM * 4 + a * KM];
+        }
+        colp[(long long)blockIdx.x * ncol + c] = s;
+    }
 }
+
+template <int KM>
+cudaError_t bwd_coef_km(const Dims& d, int slot, int T, const float* red, int nslice, const float* zact,
+                        const float* rs, const float* p, const float* hpost, const double* gram,
+                        const float* alpha_post, const float* alpha_res, const float* b_res, float* tokmat,
+                        float* dz, float* dp, float* colp, int* nblk, cudaStream_t st) {
+    // 32 tokens a block (k <= 4) fill the fp64 warp, which is what bounds the kernel at many tokens;
+    // a quarter of that at few, for more blocks.  (k > 4: 16 and 4.)  The iterates of a long Sinkhorn
+    // run (k > 4, more than 50 iterations) only fit with the small block.
+    const bool last = (slot == d.G - 1);
+    auto smem = [&](int tb) {
+        return (size_t)tb * BwdTok<KM>::ROW * 4 + (last ? (size_t)d.iters * KM * tb * KM * 4 : 0);
+    };
+    int TB = 128 / KM;
+    if (T < TB * 2 * device_sms() || smem(TB) > 200 * 1024) TB = 32 / KM;
+    const size_t sm = smem(TB);
+    const cudaError_t e =
+        cudaFuncSetAttribute((const void*)k_bwd_coef<KM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    *nblk = (T + TB - 1) / TB;
+    k_bwd_coef<KM><<<*nblk, 32 + TB * KM, sm, st>>>(d, slot, T, TB, red, nslice, zact, rs, p, hpost, gram,
+                                                   alpha_post, alpha_res, b_res, tokmat, dz, dp, colp);
+    note_launch();
+    return cudaGetLastError();
+}
+
+}  // namespace
 
 cudaError_t launch_bwd_coef(const Dims& d, int slot, int T, const float* red, int nslice,
                             const float* zact, const float* rs, const float* p,
                             const float* hpost, const double* gram, const float* alpha_post,
-                            const float* b_post, const float* alpha_res, const float* b_res,
-                            float* tokmat, float* dz, float* dp, float* tokgrad, cudaStream_t st) {
-    (void)b_post;
-    // Sinkhorn checkpoints (last slot): segments of L half-steps, at most ~96 KB per block
-    const int KMv = d.k <= 4 ? 4 : 8, nth = 64;
-    const int nh = 2 * d.iters;
-    const int segmax = std::max(1, (96 * 1024) / (KMv * KMv * 4 * nth));
-    const int L = std::max(8, (nh + segmax - 1) / segmax);
-    const int nseg = std::max(1, (nh + L - 1) / L);
-    const size_t sm = (slot == d.G - 1) ? (size_t)nseg * KMv * KMv * 4 * nth : 0;
-    cudaError_t e;
-    if (d.k <= 4) {
-        if ((e = cudaFuncSetAttribute((const void*)k_bwd_coef<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)std::max<size_t>(sm, 1))) != cudaSuccess)
-            return e;
-        k_bwd_coef<4><<<(T + nth - 1) / nth, nth, sm, st>>>(d, slot, T, red, nslice, zact, rs, p, hpost, gram,
-                                                            L, alpha_post, b_post, alpha_res, b_res, tokmat,
-                                                            dz, dp, tokgrad); note_launch();
-    } else {
-        if ((e = cudaFuncSetAttribute((const void*)k_bwd_coef<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)std::max<size_t>(sm, 1))) != cudaSuccess)
-            return e;
-        k_bwd_coef<8><<<(T + nth - 1) / nth, nth, sm, st>>>(d, slot, T, red, nslice, zact, rs, p, hpost, gram,
-                                                            L, alpha_post, b_post, alpha_res, b_res, tokmat,
-                                                            dz, dp, tokgrad); note_launch();
-    }
-    return cudaGetLastError();
+                            const float* alpha_res, const float* b_res,
+                            float* tokmat, float* dz, float* dp, float* colp, int* nblk, cudaStream_t st) {
+    if (d.k <= 4)
+        return bwd_coef_km<4>(d, slot, T, red, nslice, zact, rs, p, hpost, gram, alpha_post, alpha_res, b_res,
+                              tokmat, dz, dp, colp, nblk, st);
+    return bwd_coef_km<8>(d, slot, T, red, nslice, zact, rs, p, hpost, gram, alpha_post, alpha_res, b_res,
+                          tokmat, dz, dp, colp, nblk, st);
 }
 
 // ---------------------------------------------------------------------------------------------
-// full_coef: reverse of coef_full for one token.  dz columns follow zfull: [router | pre_0..].
-// tokgrad: [0] = d mu / NC, [1] = 2 d nu / NC, [2 + q*N + i] = db_pre, [2 + G*N + q] = dalpha_pre,
-// [2 + G*N + G + o] = mu * dZ_r[o]: the router logit subtracts mu * colsum(W_r), so every row of
-// dW_r also receives -sum_t mu_t dZ_r[t][o].
+// full_coef: reverse of coef_full.  dz columns follow zfull: [router | pre_0..].  A warp takes a token
+// at a time with a lane per column, and keeps the column sums of its tokens in registers:
+// [dy (G N) | dy * z * rstd (G N), summed over a slot's N columns: d alpha_pre (G) | mu dZ_r (N): the
+// router logit subtracts mu * colsum(W_r), so every row of dW_r also receives -sum_t mu_t dZ_r[t]].
+// scal: (d mu / NC, 2 d nu / NC), the per-token scalars of the full-state dX.
 
-__global__ void k_full_coef(Dims d, int T, const float* __restrict__ dhpre,
-                            const float* __restrict__ hpre, const float* __restrict__ zfull,
-                            const float* __restrict__ stats, const float* __restrict__ wsum,
-                            const int* __restrict__ I, const float* __restrict__ dp,
-                            const float* __restrict__ alpha_pre, float* __restrict__ dz,
-                            float* __restrict__ tokgrad) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= T) return;
-    const int N = d.N, G = d.G, n = d.nfull;
-    const int roff = d.hr ? N : 0;
-    const float mu = stats[(int64_t)t * 2], nu = stats[(int64_t)t * 2 + 1];
-    const float rstd = 1.0f / sqrtf(nu + d.eps);
-    const float* zf = zfull + (int64_t)t * n;
-    float* dzt = dz + (int64_t)t * n;
-    float* tg = tokgrad + (int64_t)t * NTG;
-    float drstd = 0.f;
-    for (int q = 0; q < G; ++q) {
-        const float a = alpha_pre[q];
-        float da = 0.f;
-        for (int i = 0; i < N; ++i) {
-            const float h = hpre[((int64_t)t * G + q) * N + i];
-            const float dy = dhpre[((int64_t)t * G + q) * N + i] * h * (1.0f - h);
-            const float zraw = zf[roff + q * N + i];
-            dzt[roff + q * N + i] = a * dy * rstd;
-            drstd += a * dy * zraw;
-            da += dy * (zraw * rstd);
-            tg[2 + q * N + i] = dy;
-        }
-        tg[2 + G * N + q] = da;
-    }
-    float dmu = 0.f;
-    float dnu = -0.5f * drstd * rstd * rstd * rstd;
-    if (d.hr) {
-        const float lstd = 1.0f / sqrtf(nu - mu * mu + d.eps);
-        float dlstd = 0.f;
-        for (int i = 0; i < N; ++i) {
-            dzt[i] = 0.f;
-            tg[2 + G * N + G + i] = 0.f;
-        }
-        if (!d.softmax) {
-            // sigmoid scores: only the selected routed streams' logits receive a gradient
-            for (int j = d.m; j < d.k; ++j) {
-                const int i = I[(int64_t)t * d.k + j];
-                const float zc = zf[i] - mu * wsum[i];
-                const float s = sigm(zc * lstd);
-                const float dzr = dp[(int64_t)t * d.k + j] * s * (1.0f - s);
-                dzt[i] = dzr * lstd;
-                tg[2 + G * N + G + i] = mu * dzr * lstd;
-                dmu -= dzr * lstd * wsum[i];
-                dlstd += dzr * zc;
-            }
-        } else {
-            // softmax scores s = softmax(z): dz_l = s_l (g_l - sum_j dp_j s_{I_j}), g_l = dp_j
-            // where l = I_j is a selected routed stream, 0 elsewhere; every logit receives one
-            float zmax = -INFINITY;
-            for (int i = 0; i < N; ++i) zmax = fmaxf(zmax, (zf[i] - mu * wsum[i]) * lstd);
-            float den = 0.f;
-            for (int i = 0; i < N; ++i) den += expf((zf[i] - mu * wsum[i]) * lstd - zmax);
-            float gs[MAXN];
-            for (int i = 0; i < N; ++i) gs[i] = 0.f;
-            float dot = 0.f;
-            for (int j = d.m; j < d.k; ++j) {
-                const int i = I[(int64_t)t * d.k + j];
-                const float s = expf((zf[i] - mu * wsum[i]) * lstd - zmax) / den;
-                gs[i] = dp[(int64_t)t * d.k + j];
-                dot += gs[i] * s;
-            }
-            for (int i = 0; i < N; ++i) {
-                const float zc = zf[i] - mu * wsum[i];
-                const float s = expf(zc * lstd - zmax) / den;
-                const float dzr = s * (gs[i] - dot);
-                dzt[i] = dzr * lstd;
-                tg[2 + G * N + G + i] = mu * dzr * lstd;
-                dmu -= dzr * lstd * wsum[i];
-                dlstd += dzr * zc;
-            }
-        }
-        const float l3 = lstd * lstd * lstd;
-        dnu += -0.5f * dlstd * l3;
-        dmu += dlstd * mu * l3;
-    }
+namespace {
+
+constexpr int FC_NT = 256;
+constexpr int FC_R = 4;   // pre-map columns per lane: G N <= 128
+
+__global__ void __launch_bounds__(FC_NT) k_full_coef(Dims d, int T, int TB, const float* __restrict__ dhpre,
+                                                     const float* __restrict__ hpre,
+                                                     const float* __restrict__ zfull,
+                                                     const float* __restrict__ stats,
+                                                     const float* __restrict__ wsum, const int* __restrict__ I,
+                                                     const float* __restrict__ dp,
+                                                     const float* __restrict__ alpha_pre, float* __restrict__ dz,
+                                                     float* __restrict__ scal, float* __restrict__ colp) {
+    __shared__ float sh[FC_NT / 32][NCOLP];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int N = d.N, GN = d.G * d.N, n = d.nfull, roff = d.hr ? N : 0;
+    const long long t0 = (long long)blockIdx.x * TB;
+    const int ntok = (int)min((long long)TB, T - t0);
     const float inv_nc = 1.0f / (float)(N * d.C);
-    tg[0] = dmu * inv_nc;
-    tg[1] = 2.0f * dnu * inv_nc;
+    const float ws = (d.hr && lane < N) ? wsum[lane] : 0.f;
+    float al[FC_R], sdy[FC_R], sda[FC_R], srt = 0.f;
+#pragma unroll
+    for (int q = 0; q < FC_R; ++q) {
+        const int e = lane + 32 * q;
+        al[q] = (e < GN) ? alpha_pre[e / N] : 0.f;
+        sdy[q] = sda[q] = 0.f;
+    }
+    for (int tt = warp; tt < ntok; tt += FC_NT / 32) {
+        const long long t = t0 + tt;
+        const float mu = stats[t * 2], nu = stats[t * 2 + 1];
+        const float rstd = 1.0f / sqrtf(nu + d.eps);
+        const float* zf = zfull + t * n;
+        float drstd = 0.f;
+#pragma unroll
+        for (int q = 0; q < FC_R; ++q) {
+            const int e = lane + 32 * q;
+            if (e >= GN) continue;
+            const float h = hpre[t * GN + e];
+            const float dy = dhpre[t * GN + e] * h * (1.0f - h);
+            const float z = zf[roff + e];
+            dz[t * n + roff + e] = al[q] * dy * rstd;
+            drstd += al[q] * dy * z;
+            sdy[q] += dy;
+            sda[q] += dy * (z * rstd);
+        }
+        drstd = warp_sum(drstd);
+        float dmu = 0.f;
+        float dnu = -0.5f * drstd * rstd * rstd * rstd;
+        if (d.hr) {
+            const float lstd = 1.0f / sqrtf(nu - mu * mu + d.eps);
+            const float zc = (lane < N) ? zf[lane] - mu * ws : 0.f;
+            // the routed stream of lane j, and its routing-weight gradient
+            const bool rj = lane >= d.m && lane < d.k;
+            const int Ij = rj ? I[t * d.k + lane] : -1;
+            const float dj = rj ? dp[t * d.k + lane] : 0.f;
+            float g = 0.f;
+            bool sel = false;
+            for (int j = d.m; j < d.k; ++j) {
+                const int ij = __shfl_sync(0xffffffffu, Ij, j);
+                const float gj = __shfl_sync(0xffffffffu, dj, j);
+                if (ij == lane) {
+                    g = gj;
+                    sel = true;
+                }
+            }
+            float dzr = 0.f;
+            if (!d.softmax) {
+                // sigmoid scores: only the selected routed streams' logits receive a gradient
+                if (sel) {
+                    const float s = sigm(zc * lstd);
+                    dzr = g * s * (1.0f - s);
+                }
+            } else {
+                // softmax scores s = softmax(z): dz_l = s_l (g_l - sum_j dp_j s_{I_j}), g_l = dp_j
+                // where l = I_j is a selected routed stream, 0 elsewhere; every logit receives one
+                const float zl = (lane < N) ? zc * lstd : -INFINITY;
+                float zmax = zl;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
+                const float ex = (lane < N) ? expf(zl - zmax) : 0.f;
+                const float s = ex / warp_sum(ex);
+                dzr = s * (g - warp_sum(g * s));
+            }
+            if (lane < N) dz[t * n + lane] = dzr * lstd;
+            srt += mu * dzr * lstd;
+            dmu = -warp_sum(dzr * lstd * ws);
+            const float dlstd = warp_sum(dzr * zc);
+            const float l3 = lstd * lstd * lstd;
+            dnu += -0.5f * dlstd * l3;
+            dmu += dlstd * mu * l3;
+        }
+        if (lane == 0) {
+            scal[t * 2] = dmu * inv_nc;
+            scal[t * 2 + 1] = 2.0f * dnu * inv_nc;
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < FC_R; ++q) {
+        const int e = lane + 32 * q;
+        if (e < GN) {
+            sh[warp][e] = sdy[q];
+            sh[warp][GN + e] = sda[q];
+        }
+    }
+    if (d.hr && lane < N) sh[warp][2 * GN + lane] = srt;
+    __syncthreads();
+    for (int c = tid; c < 2 * GN + roff; c += FC_NT) {
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < FC_NT / 32; ++w) s += sh[w][c];
+        sh[0][c] = s;   // column c is this thread's alone
+    }
+    __syncthreads();
+    const int ncol = GN + d.G + roff;
+    for (int c = tid; c < ncol; c += FC_NT) {
+        float s;
+        if (c < GN) {
+            s = sh[0][c];
+        } else if (c < GN + d.G) {
+            s = 0.f;
+            for (int i = 0; i < N; ++i) s += sh[0][GN + (c - GN) * N + i];
+        } else {
+            s = sh[0][GN - d.G + c];
+        }
+        colp[(long long)blockIdx.x * ncol + c] = s;
+    }
 }
+
+}  // namespace
 
 cudaError_t launch_full_coef(const Dims& d, int T, const float* dhpre, const float* hpre,
                              const float* zfull, const float* stats, const float* wsum,
                              const int* I, const float* dp, const float* alpha_pre, float* dz,
-                             float* tokgrad, cudaStream_t st) {
-    k_full_coef<<<(T + 127) / 128, 128, 0, st>>>(d, T, dhpre, hpre, zfull, stats, wsum, I, dp,
-                                                  alpha_pre, dz, tokgrad); note_launch();
+                             float* scal, float* colp, int* nblk, cudaStream_t st) {
+    // 8 tokens a block (a token per warp) at few tokens, 32 at many
+    const int TB = (T >= 32 * 2 * device_sms()) ? 32 : 8;
+    *nblk = (T + TB - 1) / TB;
+    k_full_coef<<<*nblk, FC_NT, 0, st>>>(d, T, TB, dhpre, hpre, zfull, stats, wsum, I, dp, alpha_pre, dz, scal,
+                                         colp); note_launch();
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------------------------
+// colsum_out: the block partials' column sums into their targets; a block per output
+
+namespace {
+
+__global__ void __launch_bounds__(128) k_colsum_out(const float* __restrict__ colp, int nblk, int ncol, ColOut out) {
+    __shared__ float sh[4];
+    int o = blockIdx.x;
+    // the target of output o, selected with static indices
+    float* ptr = nullptr;
+    int off = 0, set = 0;
+    bool found = false;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if (!found) {
+            if (o < out.n[q]) {
+                ptr = out.ptr[q] + o;
+                off = out.off[q] + o;
+                set = out.set[q];
+                found = true;
+            } else {
+                o -= out.n[q];
+            }
+        }
+    }
+    float s = warp_sum(slot_sum(colp + off, ncol, nblk, threadIdx.x, 128));
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const float v = (sh[0] + sh[1]) + (sh[2] + sh[3]);
+        *ptr = set ? v : *ptr + v;
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_colsum_out(const float* colp, int nblk, int ncol, const ColOut& out, cudaStream_t st) {
+    int n = 0;
+    for (int q = 0; q < 4; ++q) n += out.n[q];
+    k_colsum_out<<<n, 128, 0, st>>>(colp, nblk, ncol, out); note_launch();
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------------------------
+// wgrad_reduce: G[e][o] += sum over the slots of wpart[slot][e][o].  A block column takes one 128-row
+// tile of the plan, so the number of slots is found once per block.
+
+namespace {
+
+__global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ wpart, SlotPlan sp, int E, int n,
+                                                      WSegsOut G, const float* __restrict__ sub) {
+    const int e0 = blockIdx.y * 128, ne = min(128, E - e0) * n;
+    const int nsl = slot_count(sp, blockIdx.y);
+    for (int idx = blockIdx.x * 256 + threadIdx.x; idx < ne; idx += gridDim.x * 256) {
+        float s = slot_sum(wpart + (long long)e0 * n + idx, (long long)E * n, nsl, 0, 1);
+        const int e = e0 + idx / n, o = idx % n;
+        // the segment of column o, selected with static indices (no local copy of the parameter)
+        float* p = G.ptr[0];
+        int width = G.width[0], off = G.off[0];
+        if (sub != nullptr && o < G.off[1]) s -= sub[o];
+#pragma unroll
+        for (int q = 1; q < MAXSEG; ++q)
+            if (q < G.n && o >= G.off[q]) {
+                p = G.ptr[q];
+                width = G.width[q];
+                off = G.off[q];
+            }
+        p[(long long)e * width + (o - off)] += s;
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_wgrad_reduce(const float* wpart, const SlotPlan& sp, int E, int n, const WSegsOut& G,
+                                const float* sub, cudaStream_t st) {
+    // a few elements a thread where there are many tiles (the slot count costs a division)
+    const int tiles = (E + 127) / 128, per = (128 * n + 255) / 256;
+    const dim3 grid((unsigned)std::max(1, tiles >= 256 ? per / 8 : per), (unsigned)tiles);
+    k_wgrad_reduce<<<grid, 256, 0, st>>>(wpart, sp, E, n, G, sub); note_launch();
     return cudaGetLastError();
 }
 

@@ -4,7 +4,7 @@
 //   gemm_dzw  dX_act += dZ W^T (backward of the active projection)
 //   full_dx   dX = dX_base + dZ W^T + a + b x (backward of the full-state projection and norms)
 //   wgrad     dW += A^T dZ, reduced over tokens in a fixed order
-//   colsum    fixed-order column sums (per-token parameter-gradient contributions, W_r sums)
+//   colsum    fixed-order partial column sums of W_r
 #include "xhc_internal.cuh"
 
 namespace xhc {
@@ -115,61 +115,37 @@ cudaError_t launch_rowproj(const uint16_t* A, int64_t lda, int K, int T, const W
 }
 
 // ---------------------------------------------------------------------------------------------
-// colsum: out[o] (+)= sum_r in[r * ld + o], fixed order: each of 8 threads per column sums a
-// strided subset of the row chunk, then a fixed tree; long columns go through a second stage.
+// colsum: partial column sums of in [rows][n] (n <= MAXN), a block per chunk of rows: the threads walk
+// the chunk in memory order, each on one column, then a fixed tree
 
-__global__ void __launch_bounds__(256) k_colsum(const float* __restrict__ in, int rows, int ld, int n,
-                                                int rchunk, float* __restrict__ out, int out_ld,
-                                                int accumulate) {
-    __shared__ float sh[8][33];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int o = blockIdx.x * 32 + tx;
-    const int r0 = blockIdx.y * rchunk, r1 = min(rows, r0 + rchunk);
+constexpr int CS_NT = 1024;
+
+__global__ void __launch_bounds__(CS_NT) k_colsum(const float* __restrict__ in, int rows, int n, int rchunk,
+                                                  float* __restrict__ out) {
+    __shared__ float sh[CS_NT];
+    const int tid = threadIdx.x, nr = CS_NT / n;   // rows taken at a time
+    const int r0 = blockIdx.x * rchunk, r1 = min(rows, r0 + rchunk);
     float s = 0.f;
-    if (o < n)
-        for (int r = r0 + ty; r < r1; r += 8) s += in[(int64_t)r * ld + o];
-    sh[ty][tx] = s;
+    if (tid < nr * n) {
+        const int o = tid % n;
+#pragma unroll 8
+        for (int r = r0 + tid / n; r < r1; r += nr) s += in[(int64_t)r * n + o];
+    }
+    sh[tid] = s;
     __syncthreads();
-    if (ty == 0 && o < n) {
-        float t = 0.f;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) t += sh[q][tx];
-        float* dst = out + (int64_t)blockIdx.y * out_ld + o;
-        *dst = accumulate ? *dst + t : t;
+    // rows of the table folded in halves
+    for (int m = nr; m > 1;) {
+        const int h = (m + 1) / 2;
+        if (tid < (m - h) * n) sh[tid] += sh[h * n + tid];
+        __syncthreads();
+        m = h;
     }
+    if (tid < n) out[blockIdx.x * n + tid] = sh[tid];
 }
 
-// scratch holds up to 64 x 256 floats (n <= 256)
-cudaError_t launch_colsum(const float* in, int rows, int ld, int n, float* out, int accumulate,
-                          float* scratch, cudaStream_t st) {
-    if (n <= 0 || rows <= 0) return cudaSuccess;
-    if (rows <= 4096 || scratch == nullptr || n > 256) {
-        dim3 grid((n + 31) / 32, 1);
-        k_colsum<<<grid, 256, 0, st>>>(in, rows, ld, n, rows, out, n, accumulate); note_launch();
-        return cudaGetLastError();
-    }
-    int rchunk = (rows + 63) / 64;
-    const int nch = (rows + rchunk - 1) / rchunk;
-    dim3 g1((n + 31) / 32, nch);
-    k_colsum<<<g1, 256, 0, st>>>(in, rows, ld, n, rchunk, scratch, n, 0); note_launch();
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    dim3 g2((n + 31) / 32, 1);
-    k_colsum<<<g2, 256, 0, st>>>(scratch, nch, n, n, nch, out, n, accumulate); note_launch();
-    return cudaGetLastError();
-}
-
-// sub_rows: G[e][o] -= v[o] for every row e (the mean term of the router LayerNorm)
-
-__global__ void k_sub_rows(float* __restrict__ G, int rows, int n, const float* __restrict__ v) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)rows * n) return;
-    G[idx] -= v[idx % n];
-}
-
-cudaError_t launch_sub_rows(float* G, int rows, int n, const float* v, cudaStream_t st) {
-    const int64_t tot = (int64_t)rows * n;
-    k_sub_rows<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(G, rows, n, v); note_launch();
+cudaError_t launch_colsum(const float* in, int rows, int n, float* out, cudaStream_t st) {
+    const int rchunk = (rows + COLSUM_PARTS - 1) / COLSUM_PARTS;
+    k_colsum<<<COLSUM_PARTS, CS_NT, 0, st>>>(in, rows, n, rchunk, out); note_launch();
     return cudaGetLastError();
 }
 
@@ -314,7 +290,7 @@ __global__ void __launch_bounds__(256) k_full_dx(Dims d, int T, const float* __r
                 v[3] = fmaf(h, __uint_as_float(g.y & 0xffff0000u), v[3]);
             }
         }
-        const float a = scal[(int64_t)t * NTG + 0], b = scal[(int64_t)t * NTG + 1];
+        const float a = scal[(int64_t)t * 2], b = scal[(int64_t)t * 2 + 1];
         const uint2 xu = *reinterpret_cast<const uint2*>(X + (int64_t)t * E + e);
         const float xv[4] = {__uint_as_float(xu.x << 16), __uint_as_float(xu.x & 0xffff0000u),
                              __uint_as_float(xu.y << 16), __uint_as_float(xu.y & 0xffff0000u)};
@@ -404,56 +380,29 @@ __global__ void __launch_bounds__(256) k_wgrad(const uint16_t* __restrict__ A, i
     }
 }
 
-__global__ void k_wgrad_reduce(const float* __restrict__ wpart, int splits, int E, int n,
-                               WSegsOut G) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)E * n) return;
-    const int e = (int)(idx / n), o = (int)(idx - (int64_t)e * n);
-    float s = 0.f;
-    for (int q = 0; q < splits; ++q) s += wpart[(int64_t)q * E * n + idx];
-    // the segment of column o, selected with static indices (no local copy of the parameter)
-    float* p = G.ptr[0];
-    int width = G.width[0], off = G.off[0];
-#pragma unroll
-    for (int q = 1; q < MAXSEG; ++q)
-        if (q < G.n && o >= G.off[q]) {
-            p = G.ptr[q];
-            width = G.width[q];
-            off = G.off[q];
-        }
-    p[(int64_t)e * width + (o - off)] += s;
-}
-
-cudaError_t launch_wgrad_reduce(const float* wpart, int splits, int E, int n, const WSegsOut& G,
-                                cudaStream_t st) {
-    const int64_t tot = (int64_t)E * n;
-    k_wgrad_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(wpart, splits, E, n, G); note_launch();
-    return cudaGetLastError();
-}
-
 template <int NT>
 static cudaError_t wgrad_nt(const uint16_t* A, int64_t lda, int E, int T, const float* dz, int ldz,
-                            int n, int tsplits, float* wpart, const WSegsOut& G, cudaStream_t st) {
+                            int n, int tsplits, float* wpart, const WSegsOut& G, const float* sub,
+                            cudaStream_t st) {
     const int tchunk = ((T + tsplits - 1) / tsplits + 31) / 32 * 32;
     const int splits = (T + tchunk - 1) / tchunk;
     dim3 grid((E + 63) / 64, splits);
     k_wgrad<NT><<<grid, 256, 0, st>>>(A, lda, E, T, dz, ldz, n, tchunk, wpart); note_launch();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int64_t tot = (int64_t)E * n;
-    k_wgrad_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(wpart, splits, E, n, G); note_launch();
-    return cudaGetLastError();
+    return launch_wgrad_reduce(wpart, slots_of(splits), E, n, G, sub, st);
 }
 
 cudaError_t launch_wgrad(const uint16_t* A, int64_t lda, int E, int T, const float* dz, int ldz,
-                         int n, int tsplits, float* wpart, const WSegsOut& G, cudaStream_t st) {
+                         int n, int tsplits, float* wpart, const WSegsOut& G, const float* sub,
+                         cudaStream_t st) {
     const int nt = (n + 15) / 16;
-    if (nt <= 1) return wgrad_nt<1>(A, lda, E, T, dz, ldz, n, tsplits, wpart, G, st);
-    if (nt <= 2) return wgrad_nt<2>(A, lda, E, T, dz, ldz, n, tsplits, wpart, G, st);
-    if (nt <= 4) return wgrad_nt<4>(A, lda, E, T, dz, ldz, n, tsplits, wpart, G, st);
-    if (nt <= 6) return wgrad_nt<6>(A, lda, E, T, dz, ldz, n, tsplits, wpart, G, st);
-    if (nt <= 8) return wgrad_nt<8>(A, lda, E, T, dz, ldz, n, tsplits, wpart, G, st);
-    if (nt <= 10) return wgrad_nt<10>(A, lda, E, T, dz, ldz, n, tsplits, wpart, G, st);
+    if (nt <= 1) return wgrad_nt<1>(A, lda, E, T, dz, ldz, n, tsplits, wpart, G, sub, st);
+    if (nt <= 2) return wgrad_nt<2>(A, lda, E, T, dz, ldz, n, tsplits, wpart, G, sub, st);
+    if (nt <= 4) return wgrad_nt<4>(A, lda, E, T, dz, ldz, n, tsplits, wpart, G, sub, st);
+    if (nt <= 6) return wgrad_nt<6>(A, lda, E, T, dz, ldz, n, tsplits, wpart, G, sub, st);
+    if (nt <= 8) return wgrad_nt<8>(A, lda, E, T, dz, ldz, n, tsplits, wpart, G, sub, st);
+    if (nt <= 10) return wgrad_nt<10>(A, lda, E, T, dz, ldz, n, tsplits, wpart, G, sub, st);
     return cudaErrorInvalidValue;
 }
 

@@ -584,14 +584,8 @@ cudaError_t launch_proj_tc(const uint16_t* X, int T, int K, const uint16_t* Wpac
     if (!make_map(&ma, X, (uint64_t)K, (uint64_t)T, BM)) return cudaErrorInvalidValue;
     if (!make_map(&mb, Wpack, (uint64_t)K, (uint64_t)p.NB, (uint32_t)(p.NB / p.nchunk)))
         return cudaErrorInvalidValue;
-    cudaError_t e = cudaMemsetAsync(part, 0, (size_t)p.nseg * T * nfull * sizeof(float), st);
-    if (e != cudaSuccess) return e;
-    if (pstats) {
-        e = cudaMemsetAsync(pstats, 0, (size_t)p.nseg * T * 2 * sizeof(float), st);
-        if (e != cudaSuccess) return e;
-    }
     const size_t sm = proj_tc_smem(p);
-    e = cudaFuncSetAttribute((const void*)k_proj_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = cudaFuncSetAttribute((const void*)k_proj_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     ProjTcArgs a;
     a.T = T;
@@ -645,8 +639,6 @@ cudaError_t launch_wgrad_tc(const uint16_t* A, int T, int E, const float* dz, in
     if (!make_map_box(&mb, dzpack, (uint64_t)T, (uint64_t)p.NB, BK, (uint32_t)(p.NB / p.nchunk),
                       (uint64_t)Tp * 2))
         return cudaErrorInvalidValue;
-    e = cudaMemsetAsync(part, 0, (size_t)p.nseg * E * n * sizeof(float), st);
-    if (e != cudaSuccess) return e;
     const size_t sm = proj_tc_smem(p);
     e = cudaFuncSetAttribute((const void*)k_proj_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;

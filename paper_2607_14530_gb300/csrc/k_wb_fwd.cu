@@ -5,65 +5,62 @@ namespace xhc {
 namespace {
 
 // ---------------------------------------------------------------------------------------------
-// wb_coef: one thread per token.  With Gram-Schmidt, the slice partials of the Gram matrix are
-// summed in fp64, kept in `gram` for the backward and turned into the coefficients B of Eq. gs
-// (orthogonalised component q = sum_a B[q][a] u_a), so that the write-back of active slot j is
-// sum_a E[j][a] u_a with E[j][a] = p_j sum_q H_post[j][q] B[q][a]; without it B is the
-// identity.  E goes to the per-token matrix buffer (rows j < k, four entries each).
+// wb_coef: with Gram-Schmidt, the slice partials of the Gram matrix are summed in fp64, kept in `gram`
+// for the backward and turned into the coefficients B of Eq. gs (orthogonalised component q = sum_a
+// B[q][a] u_a), so that the write-back of active slot j is sum_a E[j][a] u_a with E[j][a] = p_j sum_q
+// H_post[j][q] B[q][a]; without it B is the identity.  E goes to the per-token matrix buffer (rows
+// j < k, four entries each).  A block takes TB <= 32 tokens: a thread per (token, Gram entry) for the
+// sums, a lane per token for the coefficients, a thread per (token, entry of E).
 
-__global__ void __launch_bounds__(64) k_wb_coef(Dims d, int slot, int T, const float* __restrict__ red,
-                                                int nslice, const float* __restrict__ p,
-                                                const float* __restrict__ hpost,
-                                                double* __restrict__ gram, float* __restrict__ emat) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= T) return;
-    const int k = d.k, K = d.K[slot];
+constexpr int WC_NT = 128;
+
+__global__ void __launch_bounds__(WC_NT) k_wb_coef(Dims d, int slot, int T, int TB, const float* __restrict__ red,
+                                                   int nslice, const float* __restrict__ p,
+                                                   const float* __restrict__ hpost,
+                                                   double* __restrict__ gram, float* __restrict__ emat) {
+    __shared__ double Gs[32][NGRAM + 1];
+    __shared__ float Bs[32][MAXCOMP * MAXCOMP + 1];
+    const int tid = threadIdx.x, k = d.k, K = d.K[slot];
     const bool gs = (K > 1) && d.gs;
-    // loops to MAXCOMP with guards on K: compile-time indices, the arrays stay in registers
-    double B[MAXCOMP][MAXCOMP];
-#pragma unroll
-    for (int a = 0; a < MAXCOMP; ++a)
-#pragma unroll
-        for (int b = 0; b < MAXCOMP; ++b) B[a][b] = (a == b) ? 1.0 : 0.0;
+    const long long t0 = (long long)blockIdx.x * TB;
+    const int ntok = (int)min((long long)TB, T - t0);
     if (gs) {
-        double Gm[MAXCOMP][MAXCOMP], cc[MAXCOMP][MAXCOMP], vv[MAXCOMP];
-#pragma unroll
-        for (int a = 0; a < MAXCOMP; ++a)
-#pragma unroll
-            for (int b = 0; b < MAXCOMP; ++b) Gm[a][b] = 0.0;
-        for (int sl = 0; sl < nslice; ++sl) {
-            const float* rp = red + ((int64_t)t * nslice + sl) * NRED;
-#pragma unroll
-            for (int a = 0; a < MAXCOMP; ++a)
-#pragma unroll
-                for (int b = 0; b <= a; ++b)
-                    if (a < K) Gm[a][b] += (double)rp[a * (a + 1) / 2 + b];
-        }
-#pragma unroll
-        for (int a = 0; a < MAXCOMP; ++a)
-#pragma unroll
-            for (int b = 0; b <= a; ++b)
-                if (a < K) gram[(int64_t)t * NGRAM + a * (a + 1) / 2 + b] = Gm[a][b];
-#pragma unroll
-        for (int a = 0; a < MAXCOMP; ++a)
-#pragma unroll
-            for (int b = a + 1; b < MAXCOMP; ++b)
-                if (b < K) Gm[a][b] = Gm[b][a];
-        gs_coef(Gm, K, (double)d.eps_gs, B, cc, vv);
-    }
-    float* em = emat + (int64_t)t * TOKMAT;
-    for (int j = 0; j < k; ++j) {
-        const float pj = p[(int64_t)t * k + j];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            float e = 0.f;
-            if (a < K) {
-#pragma unroll
-                for (int q = 0; q < MAXCOMP; ++q)
-                    if (q < K) e += hpost[((int64_t)t * k + j) * K + q] * (float)B[q][a];
+        const int nq = K * (K + 1) / 2;
+        for (int e = tid; e < ntok * NGRAM; e += WC_NT) {
+            const int tt = e / NGRAM, q = e - tt * NGRAM;
+            const float* rp = red + (t0 + tt) * nslice * NRED + q;
+            double s = 0.0;
+            if (q < nq) {
+#pragma unroll 8
+                for (int sl = 0; sl < nslice; ++sl) s += (double)rp[sl * NRED];
+                gram[t0 * NGRAM + e] = s;
             }
-            em[j * 4 + a] = pj * e;
+            Gs[tt][q] = s;
         }
+        __syncthreads();
+    }
+    if (tid < ntok) {
+        float B[MAXCOMP][MAXCOMP];
+        if (gs) {
+            double Gm[NGRAM];
+#pragma unroll
+            for (int q = 0; q < NGRAM; ++q) Gm[q] = Gs[tid][q];
+            GramSchmidt G;
+            G.forward(Gm, (double)d.eps_gs);
+            G.coef(B);
+        }
+#pragma unroll
+        for (int q = 0; q < MAXCOMP; ++q)
+#pragma unroll
+            for (int a = 0; a < MAXCOMP; ++a) Bs[tid][q * MAXCOMP + a] = gs ? B[q][a] : (q == a ? 1.f : 0.f);
+    }
+    __syncthreads();
+    for (int e = tid; e < ntok * k * 4; e += WC_NT) {
+        const int tt = e / (k * 4), q4 = e - tt * k * 4, j = q4 >> 2, a = q4 & 3;
+        const long long tj = (t0 + tt) * k + j;
+        float v = 0.f;
+        for (int q = a; q < K; ++q) v += hpost[tj * K + q] * Bs[tt][q * MAXCOMP + a];
+        emat[(t0 + tt) * TOKMAT + q4] = p[tj] * v;
     }
 }
 
@@ -132,7 +129,9 @@ cudaError_t launch_wb_gram(const Dims& d, int slot, int T, const uint16_t* out, 
 
 cudaError_t launch_wb_coef(const Dims& d, int slot, int T, const float* red, int nslice, const float* p,
                            const float* hpost, double* gram, float* emat, cudaStream_t st) {
-    k_wb_coef<<<(T + 63) / 64, 64, 0, st>>>(d, slot, T, red, nslice, p, hpost, gram, emat); note_launch();
+    // full fp64 warps at many tokens, more blocks at few
+    const int TB = (T >= 32 * device_sms()) ? 32 : 8;
+    k_wb_coef<<<(T + TB - 1) / TB, WC_NT, 0, st>>>(d, slot, T, TB, red, nslice, p, hpost, gram, emat); note_launch();
     return cudaGetLastError();
 }
 

@@ -51,7 +51,7 @@ extern "C" xhc_status xhc_route_noalloc(const xhc_handle* hh, int64_t T, const x
     const size_t o_part = o;  o = al256(o + (size_t)splits * t * d.nfull * 4);
     const size_t o_pst = o;   o = al256(o + (size_t)splits * t * 2 * 4);
     const size_t o_wsum = o;  o = al256(o + (size_t)d.N * 4);
-    const size_t o_scr = o;   o = al256(o + (size_t)64 * 256 * 4);
+    const size_t o_wsump = o; o = al256(o + (size_t)64 * 256 * 4);   // partial column sums of W_r
     const size_t o_zf = o;    o = al256(o + t * d.nfull * 4);
     const size_t o_st = o;    o = al256(o + t * 2 * 4);
     if (o > (size_t)XHC_NOALLOC_SCRATCH_BYTES) return XHC_ERR_UNSUPPORTED;
@@ -74,10 +74,10 @@ extern "C" xhc_status xhc_route_noalloc(const xhc_handle* hh, int64_t T, const x
     float* part = (float*)(base + o_part);
     float* pst = (float*)(base + o_pst);
     float* wsum = (float*)(base + o_wsum);
-    float* scr = (float*)(base + o_scr);
+    float* wsump = (float*)(base + o_wsump);
     // every scratch word read below is first written by this call (split-K partials, column
     // sums, statistics), so no clearing is needed
-    if (d.hr && launch_colsum(P->W_r, d.N * d.C, d.N, d.N, wsum, 0, scr, st) != cudaSuccess)
+    if (d.hr && launch_colsum(P->W_r, d.N * d.C, d.N, wsump, st) != cudaSuccess)
         return XHC_ERR_CUDA;
     WSegs w;
     memset(&w, 0, sizeof(w));
@@ -92,8 +92,8 @@ extern "C" xhc_status xhc_route_noalloc(const xhc_handle* hh, int64_t T, const x
     if (launch_rowproj(X, (int64_t)d.N * d.C, d.N * d.C, (int)T, w, d.nfull, splits, part, pst, st) !=
         cudaSuccess)
         return XHC_ERR_CUDA;
-    if (launch_coef_full(d, (int)T, part, pst, splits, wsum, P->alpha_pre, P->b_pre,
-                         (float*)(base + o_zf), (float*)(base + o_st), hpre, I, p, st) != cudaSuccess)
+    if (launch_coef_full(d, (int)T, part, pst, slots_of(splits), wsump, COLSUM_PARTS, P->alpha_pre, P->b_pre,
+                         (float*)(base + o_zf), (float*)(base + o_st), wsum, hpre, I, p, st) != cudaSuccess)
         return XHC_ERR_CUDA;
     return XHC_OK;
 }

@@ -65,6 +65,15 @@ struct ProjTcPlan {
 ProjTcPlan plan_proj_tc(int T, int K, int nfull, int nsm, bool proj);  // proj: A = X rows (else weight gradient)
 int device_sms();
 
+// Partial slots of a split reduction: `n` of them for every row, or (n == 0) those of a stream-K plan,
+// whose persistent CTAs cover each 128-row tile with a number of segments of its own.
+struct SlotPlan {
+    long long W;
+    int P, KB, n;
+};
+inline SlotPlan slots_of(const ProjTcPlan& p) { return SlotPlan{p.W, p.P, p.KB, 0}; }
+inline SlotPlan slots_of(int n) { return SlotPlan{0, 0, 0, n}; }
+
 // Byte offsets of the per-group buffers for a given T (all 256-byte aligned).
 struct Layout {
     // saved
@@ -78,6 +87,7 @@ struct Layout {
     size_t rs[4];           // f32 [T]: active rstd
     size_t hpost[4];        // f32 [T][k*K_t]
     size_t hres;            // f32 [T][k*k]
+    size_t wsum;            // f32 [N]: column sums of W_r (left by the forward for the backward)
     size_t gram[4];         // f64 [T][NGRAM]: Gram matrix of the write-back components (lower
                             // triangle), slots with a temporal conv and Gram-Schmidt
     size_t saved_total;
@@ -88,7 +98,7 @@ struct Layout {
     size_t pstats;          // f32 [splits][T][2]
     size_t astat;           // f32 [stream_warps(C)][T][2]: per-warp partial sums of squares (at 1;
                             // 0 is not written) of the active state being mapped
-    size_t wsum;            // f32 [N]: column sums of W_r
+    size_t wsump;           // f32 [64][N]: partial column sums of W_r
     size_t rsum;            // f32 [N]: sum_t mu_t dZ_r[t] (router mean-term gradient)
     size_t base;            // bf16 [G-1][T][C]: non-active base readouts of slots 1..G-1
     size_t red;             // f32 [T][nslice][NRED]: per-slice reduction partials
@@ -99,10 +109,10 @@ struct Layout {
     size_t dhpre;           // f32 [T][G][N]
     size_t tokmat;          // f32 [T][TOKMAT]: per-token matrices (E, D, H_res, scalars)
     size_t dz;              // f32 [T][max(nfull, nact)]: projection-output gradients
-    size_t tokgrad;         // f32 [T][NTG]: per-token alpha / b gradient contributions
+    size_t scal;            // f32 [T][2]: per-token scalars of the full-state dX (d mu / NC, 2 d nu / NC)
+    size_t colp;            // f32 [blocks][ncol]: per-block column sums of the alpha / b gradients
     size_t wpart;           // f32 [tsplits][rows * n]: weight-gradient partials
     size_t cpart;           // f32 [ntiles][kapsum][C]: conv weight-gradient partials
-    size_t colscr;          // f32 [64][256]: column-sum scratch
     size_t ws_total;
     int splits_full, splits_act, nslice, tsplits, ntiles;
     ProjTcPlan tc;          // full-state projection: rows T, K = N*C
@@ -114,10 +124,10 @@ struct Layout {
     size_t w16;             // bf16 [N*C][ld]: full-state projection weight rows
 };
 
-constexpr int NGRAM = 10;    // lower triangle of the 4 x 4 component Gram matrix
+constexpr int NGRAM = 10;    // lower triangle of the 4 x 4 component Gram matrix, (a, b) at a (a + 1) / 2 + b
 constexpr int NRED = 112;    // per-token reduction slots (>= k*K + k*k + K*K)
 constexpr int TOKMAT = 176;  // E[k][4] + D[4][4] + Hres[k][k] + dX_act mix + scalars (k<=8)
-constexpr int NTG = 208;     // per-token alpha/b gradient contributions
+constexpr int NCOLP = 320;   // column sums a coefficient kernel's block leaves (full: 2 G N + N)
 
 // Conv taps of one MLP slot (by value into kernels): w[j] is [kappa_j, C].  For a call on a
 // later chunk of its sequences (sequence split), halo [B][R][C] bf16 holds the R = max(kappa) - 1
@@ -216,85 +226,101 @@ __device__ __forceinline__ float seg_elem(const WSegs& w, long long r, int o) {
 // Gram-Schmidt of Eq. gs expressed on the Gram matrix of u = [out, g_1, ..., g_r]:
 // v_j = sum_a B[j][a] u_a, B unit lower-triangular.  Denominators <v_i, v_i> + eps.
 
-// The loops run to MAXCOMP with guards on K (the same operations in the same order as loops to
-// K), so every array index is a compile-time constant and the arrays stay in registers.
-__device__ inline void gs_coef(const double (&G)[MAXCOMP][MAXCOMP], int K, double eps,
-                        double (&B)[MAXCOMP][MAXCOMP], double (&c)[MAXCOMP][MAXCOMP],
-                        double (&vv)[MAXCOMP]) {
-#pragma unroll
-    for (int j = 0; j < MAXCOMP; ++j)
-#pragma unroll
-        for (int a = 0; a < MAXCOMP; ++a) {
-            B[j][a] = (j == a) ? 1.0 : 0.0;
-            c[j][a] = 0.0;
-        }
-#pragma unroll
-    for (int j = 0; j < MAXCOMP; ++j) {
-        if (j >= K) break;
-#pragma unroll
-        for (int i = 0; i < j; ++i) {
-            double num = 0.0;
-#pragma unroll
-            for (int a = 0; a <= i; ++a) num += B[i][a] * G[j][a];
-            c[j][i] = num / vv[i];
-        }
-#pragma unroll
-        for (int i = 0; i < j; ++i)
-#pragma unroll
-            for (int a = 0; a <= i; ++a) B[j][a] -= c[j][i] * B[i][a];
-        double q = 0.0;
-#pragma unroll
-        for (int a = 0; a <= j; ++a)
-#pragma unroll
-            for (int b = 0; b <= j; ++b) q += B[j][a] * B[j][b] * G[a][b];
-        vv[j] = q + eps;
-    }
-}
+// Gm is the lower triangle (a, b) at a (a + 1) / 2 + b; rows of absent components (a >= K) are zero,
+// which makes their coefficients zero (the denominators are at least eps > 0).  The products
+// y_i = Gm B[i] serve the numerators <g_j, v_i> = y_i[j], the norms <v_i, v_i> = <B[i], y_i> and the
+// reverse mode, and each denominator is inverted once: about 60 fp64 operations forward and 60 in
+// reverse (the literal sums took 150 and 250).  fp64 runs at two FMAs per clock and SM here, so
+// these counts are what bounds the per-token kernels at many tokens, and their dependent chain (three
+// reciprocals) at few.
+struct GramSchmidt {
+    double c10, c20, c30, c21, c31, c32;      // c[j][i] = <g_j, v_i> / (<v_i, v_i> + eps)
+    double b10, b20, b21, b30, b31, b32;      // B below its unit diagonal
+    double iv0, iv1, iv2;                     // 1 / (<v_i, v_i> + eps)
+    double y10, y11, y20, y21, y22;           // y_i[a], a <= i
 
-// Reverse of gs_coef: dB (modified in place) -> dG (full, not symmetrised).
-__device__ inline void gs_coef_bwd(const double (&G)[MAXCOMP][MAXCOMP], int K,
-                            const double (&B)[MAXCOMP][MAXCOMP], const double (&c)[MAXCOMP][MAXCOMP],
-                            const double (&vv)[MAXCOMP], double (&dB)[MAXCOMP][MAXCOMP],
-                            double (&dG)[MAXCOMP][MAXCOMP]) {
-    double dvv[MAXCOMP] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-    for (int a = 0; a < MAXCOMP; ++a)
-#pragma unroll
-        for (int b = 0; b < MAXCOMP; ++b) dG[a][b] = 0.0;
-#pragma unroll
-    for (int j = MAXCOMP - 1; j >= 0; --j) {
-        if (j >= K) continue;
-        // vv[j] = B[j]^T G B[j] + eps
-        if (dvv[j] != 0.0) {
-#pragma unroll
-            for (int a = 0; a <= j; ++a) {
-                double s = 0.0;
-#pragma unroll
-                for (int b = 0; b <= j; ++b) s += (G[a][b] + G[b][a]) * B[j][b];
-                dB[j][a] += dvv[j] * s;
-#pragma unroll
-                for (int b = 0; b <= j; ++b) dG[a][b] += dvv[j] * B[j][a] * B[j][b];
-            }
-        }
-        // B[j] = e_j - sum_i c[j][i] B[i];  c[j][i] = num / vv[i];  num = sum_a B[i][a] G[j][a]
-#pragma unroll
-        for (int i = j - 1; i >= 0; --i) {
-            double dc = 0.0;
-#pragma unroll
-            for (int a = 0; a <= i; ++a) {
-                dc -= dB[j][a] * B[i][a];
-                dB[i][a] -= c[j][i] * dB[j][a];
-            }
-            const double dnum = dc / vv[i];
-            dvv[i] -= dc * c[j][i] / vv[i];
-#pragma unroll
-            for (int a = 0; a <= i; ++a) {
-                dB[i][a] += dnum * G[j][a];
-                dG[j][a] += dnum * B[i][a];
-            }
-        }
+    __device__ __forceinline__ void forward(const double (&g)[NGRAM], double eps) {
+        iv0 = 1.0 / (g[0] + eps);
+        c10 = g[1] * iv0;
+        c20 = g[3] * iv0;
+        c30 = g[6] * iv0;
+        b10 = -c10;
+        y10 = fma(g[0], b10, g[1]);
+        y11 = fma(g[1], b10, g[2]);
+        iv1 = 1.0 / (fma(b10, y10, y11) + eps);
+        c21 = fma(g[3], b10, g[4]) * iv1;
+        c31 = fma(g[6], b10, g[7]) * iv1;
+        b20 = fma(-c21, b10, -c20);
+        b21 = -c21;
+        y20 = fma(g[0], b20, fma(g[1], b21, g[3]));
+        y21 = fma(g[1], b20, fma(g[2], b21, g[4]));
+        y22 = fma(g[3], b20, fma(g[4], b21, g[5]));
+        iv2 = 1.0 / (fma(b20, y20, fma(b21, y21, y22)) + eps);
+        c32 = fma(g[6], b20, fma(g[7], b21, g[8])) * iv2;
+        b30 = fma(-c32, b20, fma(-c31, b10, -c30));
+        b31 = fma(-c32, b21, -c31);
+        b32 = -c32;
     }
-}
+
+    // B[q][a] as fp32 (zero above the diagonal)
+    __device__ __forceinline__ void coef(float (&B)[MAXCOMP][MAXCOMP]) const {
+#pragma unroll
+        for (int q = 0; q < MAXCOMP; ++q)
+#pragma unroll
+            for (int a = 0; a < MAXCOMP; ++a) B[q][a] = (q == a) ? 1.f : 0.f;
+        B[1][0] = (float)b10;
+        B[2][0] = (float)b20;
+        B[2][1] = (float)b21;
+        B[3][0] = (float)b30;
+        B[3][1] = (float)b31;
+        B[3][2] = (float)b32;
+    }
+
+    // D = dG + dG^T (lower triangle) from dB below the diagonal (d10, d20, d21, d30, d31, d32)
+    __device__ __forceinline__ void reverse(const double (&g)[NGRAM], double d10, double d20, double d21,
+                                            double d30, double d31, double d32, double (&D)[NGRAM]) const {
+        // row 3: B[3] = e_3 - sum_i c[3][i] B[i]
+        double dn = -fma(d30, b20, fma(d31, b21, d32)) * iv2;   // d<g_3, v_2>
+        double v2 = -dn * c32;                                   // d(<v_2, v_2> + eps)
+        d20 = fma(dn, g[6], fma(-c32, d30, d20));
+        d21 = fma(dn, g[7], fma(-c32, d31, d21));
+        D[6] = dn * b20;
+        D[7] = dn * b21;
+        D[8] = dn;
+        dn = -fma(d30, b10, d31) * iv1;
+        double v1 = -dn * c31;
+        d10 = fma(dn, g[6], fma(-c31, d30, d10));
+        D[6] = fma(dn, b10, D[6]);
+        D[7] += dn;
+        dn = -d30 * iv0;
+        double v0 = -dn * c30;
+        D[6] += dn;
+        // row 2
+        d20 = fma(2.0 * v2, y20, d20);
+        d21 = fma(2.0 * v2, y21, d21);
+        dn = -fma(d20, b10, d21) * iv1;
+        v1 = fma(-dn, c21, v1);
+        d10 = fma(dn, g[3], fma(-c21, d20, d10));
+        D[3] = dn * b10;
+        D[4] = dn;
+        dn = -d20 * iv0;
+        v0 = fma(-dn, c20, v0);
+        D[3] += dn;
+        // row 1
+        d10 = fma(2.0 * v1, y10, d10);
+        dn = -d10 * iv0;
+        v0 = fma(-dn, c10, v0);
+        // the norms' own terms, v_i B[i] B[i]^T, counted from both triangles
+        const double w2 = 2.0 * v2, w1 = 2.0 * v1;
+        D[0] = fma(w2 * b20, b20, fma(w1 * b10, b10, 2.0 * v0));
+        D[1] = fma(w2 * b20, b21, fma(w1, b10, dn));
+        D[2] = fma(w2 * b21, b21, w1);
+        D[3] = fma(w2, b20, D[3]);
+        D[4] = fma(w2, b21, D[4]);
+        D[5] = w2;
+        D[9] = 0.0;
+    }
+};
 
 // ---------------------------------------------------------------------------------------------
 // launch accounting and tracing (host side)
@@ -375,19 +401,20 @@ cudaError_t launch_wb_bapp(const Dims& d, int slot, int T, const uint16_t* out, 
                            const uint16_t* dX, const int* I, const float* dn_in,
                            const float* tokmat, float* dxact_out, uint16_t* d_out, float* cpart,
                            cudaStream_t st);
-cudaError_t launch_wgrad_reduce(const float* wpart, int splits, int E, int n, const WSegsOut& G,
-                                cudaStream_t st);
-cudaError_t launch_colsum(const float* in, int rows, int ld, int n, float* out, int accumulate,
-                          float* scratch, cudaStream_t st);
-cudaError_t launch_sub_rows(float* G, int rows, int n, const float* v, cudaStream_t st);
-// sum of split-K partial slots into slot 0, in slot order ([nslots][n] -> [n])
-cudaError_t launch_slot_sum(float* x, int nslots, long long n, cudaStream_t st);
+// G[e][o] += sum of the slots of wpart[slot][e][o], less sub[o] on the first segment's columns (sub
+// null: nothing is subtracted)
+cudaError_t launch_wgrad_reduce(const float* wpart, const SlotPlan& sp, int E, int n, const WSegsOut& G,
+                                const float* sub, cudaStream_t st);
+// partial column sums of in [rows][n]: out [nparts][n], part q over the rows of chunk q
+constexpr int COLSUM_PARTS = 64;
+cudaError_t launch_colsum(const float* in, int rows, int n, float* out, cudaStream_t st);
+// wsum: [nws][N] partial column sums of W_r; their sum is left in wsum_out [N]
 cudaError_t launch_coef_full(const Dims& d, int T, const float* part, const float* pstats,
-                             int splits, const float* wsum, const float* alpha_pre,
-                             const float* b_pre, float* zfull, float* stats, float* hpre,
+                             const SlotPlan& sp, const float* wsum, int nws, const float* alpha_pre,
+                             const float* b_pre, float* zfull, float* stats, float* wsum_out, float* hpre,
                              int* I, float* p, cudaStream_t st);
 cudaError_t launch_coef_act(const Dims& d, int slot, int T, const float* part,
-                            const float* pstats, int ssplits, int splits, const float* alpha_post,
+                            const float* pstats, int ssplits, const SlotPlan& sp, const float* alpha_post,
                             const float* b_post, const float* alpha_res, const float* b_res,
                             float* zact, float* rs, float* hpost, float* hres, cudaStream_t st);
 int stream_warps(int C);  // warps per block of the one-block-per-token stream kernels
@@ -400,14 +427,23 @@ cudaError_t launch_restore(const Dims& d, int T, const uint16_t* xact0, const in
 cudaError_t launch_bwd_coef(const Dims& d, int slot, int T, const float* red, int nslice,
                             const float* zact, const float* rs, const float* p,
                             const float* hpost, const double* gram, const float* alpha_post,
-                            const float* b_post, const float* alpha_res, const float* b_res,
-                            float* tokmat, float* dz, float* dp, float* tokgrad, cudaStream_t st);
+                            const float* alpha_res, const float* b_res,
+                            float* tokmat, float* dz, float* dp, float* colp, int* nblk, cudaStream_t st);
+// adds the column sums over the blocks' partials colp [nblk][ncol] to up to four targets: target q
+// takes columns off[q] .. off[q] + n[q] - 1
+struct ColOut {
+    float* ptr[4];
+    int off[4], n[4];
+    int set[4];   // 1: stored instead of added
+};
+cudaError_t launch_colsum_out(const float* colp, int nblk, int ncol, const ColOut& out, cudaStream_t st);
 cudaError_t launch_gemm_dzw(const Dims& d, int T, const float* dz, int ldz, int n,
                             const WSegs& W, int E, float* dxact, cudaStream_t st);
 cudaError_t launch_conv_wgrad_reduce(const Dims& d, int slot, const float* cpart, int ntiles,
                                      ConvGradPtrs gconv, cudaStream_t st);
 cudaError_t launch_wgrad(const uint16_t* A, int64_t lda, int E, int T, const float* dz, int ldz,
-                         int n, int tsplits, float* wpart, const WSegsOut& G, cudaStream_t st);
+                         int n, int tsplits, float* wpart, const WSegsOut& G, const float* sub,
+                         cudaStream_t st);
 cudaError_t launch_dinput_act(const Dims& d, int slot, int T, int add_dx, const uint16_t* d_input,
                               const uint16_t* xact, const float* hpre, const int* I,
                               float* dxact, float* dhpre, uint16_t* dinput_copy,
@@ -417,10 +453,10 @@ cudaError_t launch_full_dots(const Dims& d, int T, const uint16_t* X, const uint
 cudaError_t launch_full_coef(const Dims& d, int T, const float* dhpre, const float* hpre,
                              const float* zfull, const float* stats, const float* wsum,
                              const int* I, const float* dp, const float* alpha_pre, float* dz,
-                             float* tokgrad, cudaStream_t st);
+                             float* scal, float* colp, int* nblk, cudaStream_t st);
 cudaError_t launch_full_dx(const Dims& d, int T, const float* dz, const WSegs& W,
                            const uint16_t* X, const uint16_t* dinput, const float* hpre,
-                           const int* I, const float* dxact, const float* tokgrad_scal,
+                           const int* I, const float* dxact, const float* scal,
                            uint16_t* dX, cudaStream_t st);
 
 }  // namespace xhc
