@@ -650,7 +650,7 @@ xhc_status xhc_pre_fwd(const xhc_handle* h, int slot, int64_t T, const xhc_param
                                               c.W<int>(c.L.err), c.st));
         }
         XHC_K("coef_full", c.st, launch_coef_full(d, c.T, c.W<float>(c.L.part), c.W<float>(c.L.pstats),
-                                  sp, c.W<float>(c.L.wsump), COLSUM_PARTS, P->alpha_pre, P->b_pre,
+                                  sp, c.W<float>(c.L.wsump), colsum_parts(d.N * d.C), P->alpha_pre, P->b_pre,
                                   c.S<float>(c.L.zfull), c.S<float>(c.L.stats), c.S<float>(c.L.wsum),
                                   c.S<float>(c.L.hpre), c.S<int>(c.L.I), c.S<float>(c.L.p), c.st));
         XHC_K("read", c.st, launch_read(d, c.T, X, c.S<float>(c.L.hpre), c.S<int>(c.L.I), input,

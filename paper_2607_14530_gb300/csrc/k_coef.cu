@@ -48,34 +48,39 @@ __device__ __forceinline__ int slot_count(const SlotPlan& s, int m) {
                                           (unsigned long long)s.KB, (unsigned long long)m);
 }
 
-// sum over `cnt` slots of p, `stride` apart, starting at slot q0 in steps of dq
-__device__ __forceinline__ float slot_sum(const float* p, long long stride, int cnt, int q0, int dq) {
+// sum over `cnt` slots of p, `stride` apart, starting at slot q0 in steps of dq, added in slot order with
+// U loads in flight
+template <int U>
+__device__ __forceinline__ float slot_sum(const float* __restrict__ p, long long stride, int cnt, int q0, int dq) {
     float s = 0.f;
     int q = q0;
-    for (; q + 7 * dq < cnt; q += 8 * dq) {
-        float v[8];   // eight loads in flight, added in slot order
+    for (; q + (U - 1) * dq < cnt; q += U * dq) {
+        float v[U];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = p[(q + u * dq) * stride];
+        for (int u = 0; u < U; ++u) v[u] = p[(q + u * dq) * stride];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) s += v[u];
+        for (int u = 0; u < U; ++u) s += v[u];
     }
+#pragma unroll 4
     for (; q < cnt; q += dq) s += p[q * stride];
     return s;
 }
 
 // Two arrays of slot sums into shared memory: dst[0, n0) = sums of p0 + e, dst[n0, n0 + n1) = sums of
-// p1 + e * step1.  With fewer elements than threads, groups of threads take interleaved slots and
-// their sums are added in group order (scr: one float per thread).  Ends with a block barrier.
-__device__ __forceinline__ void slot_sums(const float* __restrict__ p0, long long stride0, int cnt0, int n0,
-                                          const float* __restrict__ p1, long long stride1, int cnt1, int n1,
+// p1 + e * step1.  The slots of a stream-K plan are added in slot order (any number of tokens gives
+// the same bits for a token, and so the same routing); those of an even split, of which there are
+// many on few tokens, by groups of threads that take interleaved slots (scr: one float per thread).
+// Ends with a block barrier.
+__device__ __forceinline__ void slot_sums(bool ordered, const float* __restrict__ p0, long long stride0, int cnt0,
+                                          int n0, const float* __restrict__ p1, long long stride1, int cnt1, int n1,
                                           int step1, float* dst, float* scr) {
     const int n = n0 + n1, nt = blockDim.x, tid = threadIdx.x;
-    const int ng = nt / n;
+    const int ng = ordered ? 1 : nt / n;
     if (ng > 1) {
         const int g = tid / n, e = tid - g * n;
         if (g < ng)
-            scr[tid] = (e < n0) ? slot_sum(p0 + e, stride0, cnt0, g, ng)
-                                : slot_sum(p1 + (long long)(e - n0) * step1, stride1, cnt1, g, ng);
+            scr[tid] = (e < n0) ? slot_sum<8>(p0 + e, stride0, cnt0, g, ng)
+                                : slot_sum<8>(p1 + (long long)(e - n0) * step1, stride1, cnt1, g, ng);
         __syncthreads();
         if (tid < n) {
             float s = 0.f;
@@ -84,15 +89,16 @@ __device__ __forceinline__ void slot_sums(const float* __restrict__ p0, long lon
         }
     } else {
         for (int e = tid; e < n; e += nt)
-            dst[e] = (e < n0) ? slot_sum(p0 + e, stride0, cnt0, 0, 1)
-                              : slot_sum(p1 + (long long)(e - n0) * step1, stride1, cnt1, 0, 1);
+            dst[e] = (e < n0) ? slot_sum<16>(p0 + e, stride0, cnt0, 0, 1)
+                              : slot_sum<16>(p1 + (long long)(e - n0) * step1, stride1, cnt1, 0, 1);
     }
     __syncthreads();
 }
 
 // ---------------------------------------------------------------------------------------------
 // Sinkhorn of Eq. mhc_sinkhorn on a k x k block (k <= KM), with the App. A row clamp.  KM neighbouring
-// lanes hold one matrix, lane a its row a; columns are summed over the lanes by shuffles.
+// lanes hold one matrix, lane a its row a; columns are normalised as rows of the transposed matrix
+// (log2 KM exchanges between the lanes: one division a lane and half-step, sums in index order).
 // exp(M - rowmax): the first row normalisation removes any per-row scale, so this equals exp(M).
 
 template <int KM>
@@ -105,9 +111,26 @@ __device__ __forceinline__ void sk_init(const float (&M)[KM], int a, int k, floa
     for (int b = 0; b < KM; ++b) A[b] = (a < k && b < k) ? expf(M[b] - mx) : 0.f;
 }
 
-// row normalisation; returns the factor (0 for a row outside the matrix)
+// the lanes' KM x KM matrix transposed
 template <int KM>
-__device__ __forceinline__ float sk_row(float (&A)[KM], int a, int k) {
+__device__ __forceinline__ void transpose(float (&A)[KM], int a) {
+#pragma unroll
+    for (int o = 1; o < KM; o <<= 1) {
+        const bool up = (a & o) != 0;
+#pragma unroll
+        for (int b = 0; b < KM; ++b) {
+            if (b & o) continue;
+            const float got = __shfl_xor_sync(0xffffffffu, up ? A[b] : A[b | o], o);
+            if (up) A[b] = got;
+            else A[b | o] = got;
+        }
+    }
+}
+
+// normalisation of the lane's row (or column, of the transposed matrix); returns the factor, 0 outside
+// the matrix
+template <int KM>
+__device__ __forceinline__ float sk_half(float (&A)[KM], int a, int k) {
     float s = 0.f;
 #pragma unroll
     for (int b = 0; b < KM; ++b) s += A[b];
@@ -118,24 +141,11 @@ __device__ __forceinline__ float sk_row(float (&A)[KM], int a, int k) {
 }
 
 template <int KM>
-__device__ __forceinline__ void sum_rows(float (&v)[KM]) {
-#pragma unroll
-    for (int o = 1; o < KM; o <<= 1)
-#pragma unroll
-        for (int b = 0; b < KM; ++b) v[b] += __shfl_xor_sync(0xffffffffu, v[b], o);
-}
-
-// column normalisation with factors r
-template <int KM>
-__device__ __forceinline__ void sk_col(float (&A)[KM], int k, float (&r)[KM]) {
-#pragma unroll
-    for (int b = 0; b < KM; ++b) r[b] = A[b];
-    sum_rows<KM>(r);
-#pragma unroll
-    for (int b = 0; b < KM; ++b) {
-        r[b] = (b < k) ? 1.0f / r[b] : 0.f;
-        A[b] *= r[b];
-    }
+__device__ __forceinline__ void sk_iter(float (&A)[KM], int a, int k) {
+    sk_half<KM>(A, a, k);
+    transpose<KM>(A, a);
+    sk_half<KM>(A, a, k);
+    transpose<KM>(A, a);
 }
 
 template <int KM>
@@ -160,30 +170,32 @@ __global__ void __launch_bounds__(CF_NT) k_coef_full(Dims d, int T, int TB, cons
                                                      float* __restrict__ hpre, int* __restrict__ I,
                                                      float* __restrict__ p) {
     extern __shared__ float sm[];   // [TB][n] projections, [TB][2] statistics
-    __shared__ float scr[CF_NT], scw[CF_NT], ws[MAXN];
+    __shared__ float scr[CF_NT], scw[8 * MAXN], ws[MAXN];
     const int tid = threadIdx.x, lane = tid & 31, N = d.N, n = d.nfull;
     const long long t0 = (long long)blockIdx.x * TB;
     const int ntok = (int)min((long long)TB, T - t0);
-    // column sums of W_r: groups of N threads over the partials
-    const int gw = CF_NT / N;
-    if (d.hr && tid < gw * N) {
-        float s = 0.f;
-        for (int q = tid / N; q < nws; q += gw) s += wsum[q * N + tid % N];
-        scw[tid] = s;
-    }
+    // column sums of W_r from the partials: eight threads a column, then their sum
+    if (d.hr && tid < 8 * N) scw[tid] = slot_sum<8>(wsum + tid % N, N, nws, tid / N, 8);
     const int nsl = slot_count(sp, (int)(t0 >> 7));
     float* zs = sm;
     float* st = sm + ntok * n;
-    slot_sums(part + t0 * n, (long long)T * n, nsl, ntok * n, pstats + t0 * 2, (long long)T * 2, nsl, ntok * 2, 1,
-              zs, scr);
+    slot_sums(sp.n == 0, part + t0 * n, (long long)T * n, nsl, ntok * n, pstats + t0 * 2, (long long)T * 2, nsl,
+              ntok * 2, 1, zs, scr);
     if (d.hr && tid < N) {
         float s = 0.f;
-        for (int q = 0; q < gw; ++q) s += scw[q * N + tid];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) s += scw[q * N + tid];
         ws[tid] = s;
         if (blockIdx.x == 0) wsum_out[tid] = s;
     }
     const float inv_nc = 1.0f / (float)(N * d.C);
-    if (tid < ntok * 2) stats[t0 * 2 + tid] = st[tid] * inv_nc;
+    for (int e = tid; e < ntok * 2; e += CF_NT) {
+        // mean and mean square, rounded here: what follows is not to be contracted with the product
+        const float v = __fmul_rn(st[e], inv_nc);
+        st[e] = v;
+        stats[t0 * 2 + e] = v;
+    }
+    __syncthreads();
     const int roff = d.hr ? N : 0, GN = d.G * N;
     for (int e = tid; e < ntok * n; e += CF_NT) {
         const int tt = e / n, o = e - tt * n;
@@ -191,7 +203,7 @@ __global__ void __launch_bounds__(CF_NT) k_coef_full(Dims d, int T, int TB, cons
         zfull[t0 * n + e] = z;
         if (o >= roff) {
             const int qo = o - roff, slot = qo / N;
-            const float rstd = 1.0f / sqrtf(st[tt * 2 + 1] * inv_nc + d.eps);
+            const float rstd = 1.0f / sqrtf(st[tt * 2 + 1] + d.eps);
             hpre[(t0 + tt) * GN + qo] = sigm(alpha_pre[slot] * (z * rstd) + b_pre[qo]);
         }
     }
@@ -206,7 +218,7 @@ __global__ void __launch_bounds__(CF_NT) k_coef_full(Dims d, int T, int TB, cons
             p[tk + lane] = 1.0f;
         }
         if (!d.hr) continue;
-        const float mu = st[tt * 2] * inv_nc, nu = st[tt * 2 + 1] * inv_nc;
+        const float mu = st[tt * 2], nu = st[tt * 2 + 1];
         const float lstd = 1.0f / sqrtf(nu - mu * mu + d.eps);
         const float z = (lane < N) ? (zs[tt * n + lane] - mu * ws[lane]) * lstd : -INFINITY;
         float zmax = z, den = 0.f;
@@ -261,34 +273,34 @@ __global__ void __launch_bounds__(CF_NT) k_coef_act(Dims d, int slot, int T, int
     const int nsl = slot_count(sp, (int)(t0 >> 7));
     float* zs = sm;
     float* st = sm + ntok * n;
-    slot_sums(part + t0 * n, (long long)T * n, nsl, ntok * n, pstats + t0 * 2 + 1, (long long)T * 2, ssplits, ntok, 2,
-              zs, scr);
-    const float inv = 1.0f / (float)(k * d.C);
-    if (tid < ntok) rs[t0 + tid] = 1.0f / sqrtf(st[tid] * inv + d.eps);
+    slot_sums(sp.n == 0, part + t0 * n, (long long)T * n, nsl, ntok * n, pstats + t0 * 2 + 1, (long long)T * 2,
+              ssplits, ntok, 2, zs, scr);
+    if (tid < ntok) {
+        const float r = 1.0f / sqrtf(st[tid] / (float)(k * d.C) + d.eps);
+        st[tid] = r;
+        rs[t0 + tid] = r;
+    }
+    __syncthreads();
     const float ap = alpha_post[slot];
     for (int e = tid; e < ntok * n; e += CF_NT) {
         const int tt = e / n, o = e - tt * n;
         const float z = zs[e];
         zact[t0 * n + e] = z;
         if (o < kK) {
-            const float r = 1.0f / sqrtf(st[tt] * inv + d.eps);
-            hpost[(t0 + tt) * kK + o] = 2.0f * sigm(ap * (z * r) + b_post[o]);
+            hpost[(t0 + tt) * kK + o] = 2.0f * sigm(ap * (z * st[tt]) + b_post[o]);
         }
     }
     if (slot != d.G - 1 || (tid & ~31) >= TB * KM) return;
     // whole warps run the iterations (lanes past the last token repeat it)
     const int tq = tid / KM, a = tid - tq * KM;
     const int tt = min(tq, ntok - 1);
-    const float ar = alpha_res[0], r = 1.0f / sqrtf(st[tt] * inv + d.eps);
-    float M[KM], H[KM], cr[KM];
+    const float ar = alpha_res[0], r = st[tt];
+    float M[KM], H[KM];
 #pragma unroll
     for (int b = 0; b < KM; ++b)
         M[b] = (a < k && b < k) ? ar * (zs[tt * n + kK + a * k + b] * r) + b_res[a * k + b] : 0.f;
     sk_init<KM>(M, a, k, H);
-    for (int it = 0; it < d.iters; ++it) {
-        sk_row<KM>(H, a, k);
-        sk_col<KM>(H, k, cr);
-    }
+    for (int it = 0; it < d.iters; ++it) sk_iter<KM>(H, a, k);
     const float s = row_total<KM>(H);
     if (tq < ntok && a < k) {
         float* dst = hres + (t0 + tt) * k * k + a * k;
@@ -352,15 +364,14 @@ namespace {
 template <int KM>
 __device__ void sinkhorn_bwd(const float (&M)[KM], int a, int k, int iters, float* ck, int stride,
                              const float (&dH)[KM], float (&H)[KM], float (&dM)[KM]) {
-    float A[KM], A0[KM], rc[KM], dA[KM];
+    float A[KM], A0[KM], dA[KM];
     sk_init<KM>(M, a, k, A);
 #pragma unroll
     for (int b = 0; b < KM; ++b) A0[b] = A[b];
     for (int it = 0; it < iters; ++it) {
 #pragma unroll
         for (int b = 0; b < KM; ++b) ck[(it * KM + b) * stride] = A[b];
-        sk_row<KM>(A, a, k);
-        sk_col<KM>(A, k, rc);
+        sk_iter<KM>(A, a, k);
     }
     // clamp
     const float s = row_total<KM>(A);
@@ -381,25 +392,27 @@ __device__ void sinkhorn_bwd(const float (&M)[KM], int a, int k, int iters, floa
         }
     }
     for (int it = iters - 1; it >= 0; --it) {
-        // R: after the row step; A: after the column step
-        float R[KM], dot[KM];
+        // R: after the row step; A: its transpose after the column step; dA follows
+        float R[KM];
 #pragma unroll
         for (int b = 0; b < KM; ++b) R[b] = ck[(it * KM + b) * stride];
-        const float rr = sk_row<KM>(R, a, k);
+        const float rr = sk_half<KM>(R, a, k);
 #pragma unroll
         for (int b = 0; b < KM; ++b) A[b] = R[b];
-        sk_col<KM>(A, k, rc);
+        transpose<KM>(A, a);
+        const float rc = sk_half<KM>(A, a, k);
+        transpose<KM>(dA, a);
+        float dot = 0.f;
 #pragma unroll
-        for (int b = 0; b < KM; ++b) dot[b] = dA[b] * A[b];
-        sum_rows<KM>(dot);
-        float rdot = 0.f;
+        for (int b = 0; b < KM; ++b) dot += dA[b] * A[b];
 #pragma unroll
-        for (int b = 0; b < KM; ++b) {
-            dA[b] = (dA[b] - dot[b]) * rc[b];
-            rdot += dA[b] * R[b];
-        }
+        for (int b = 0; b < KM; ++b) dA[b] = (dA[b] - dot) * rc;
+        transpose<KM>(dA, a);
+        dot = 0.f;
 #pragma unroll
-        for (int b = 0; b < KM; ++b) dA[b] = (dA[b] - rdot) * rr;
+        for (int b = 0; b < KM; ++b) dot += dA[b] * R[b];
+#pragma unroll
+        for (int b = 0; b < KM; ++b) dA[b] = (dA[b] - dot) * rr;
     }
 #pragma unroll
     for (int b = 0; b < KM; ++b) dM[b] = (a < k && b < k) ? dA[b] * A0[b] : 0.f;
@@ -446,7 +459,7 @@ __global__ void __launch_bounds__(160) k_bwd_coef(Dims d, int slot, int T, int T
             if (q < KM * 4) used = (q >> 2) < k && (q & 3) < K;
             else used = (q - KM * 4) / KM < k && (q - KM * 4) % KM < k;
             float s = 0.f;
-            if (used) s = slot_sum(red + (t0 + tt) * nslice * NRED + q, NRED, nslice, 0, 1);
+            if (used) s = slot_sum<8>(red + (t0 + tt) * nslice * NRED + q, NRED, nslice, 0, 1);
             sm[tt * L::ROW + L::R + q] = s;
         }
     }
@@ -824,7 +837,7 @@ __global__ void __launch_bounds__(128) k_colsum_out(const float* __restrict__ co
             }
         }
     }
-    float s = warp_sum(slot_sum(colp + off, ncol, nblk, threadIdx.x, 128));
+    float s = warp_sum(slot_sum<8>(colp + off, ncol, nblk, threadIdx.x, 128));
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -853,7 +866,7 @@ __global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ 
     const int e0 = blockIdx.y * 128, ne = min(128, E - e0) * n;
     const int nsl = slot_count(sp, blockIdx.y);
     for (int idx = blockIdx.x * 256 + threadIdx.x; idx < ne; idx += gridDim.x * 256) {
-        float s = slot_sum(wpart + (long long)e0 * n + idx, (long long)E * n, nsl, 0, 1);
+        float s = slot_sum<4>(wpart + (long long)e0 * n + idx, (long long)E * n, nsl, 0, 1);
         const int e = e0 + idx / n, o = idx % n;
         // the segment of column o, selected with static indices (no local copy of the parameter)
         float* p = G.ptr[0];

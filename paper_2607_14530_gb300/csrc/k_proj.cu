@@ -115,37 +115,46 @@ cudaError_t launch_rowproj(const uint16_t* A, int64_t lda, int K, int T, const W
 }
 
 // ---------------------------------------------------------------------------------------------
-// colsum: partial column sums of in [rows][n] (n <= MAXN), a block per chunk of rows: the threads walk
-// the chunk in memory order, each on one column, then a fixed tree
+// colsum: partial column sums of in [rows][n] (n <= MAXN), a block per chunk of rows, eight threads a
+// column over interleaved rows (16 loads each in flight), then their sum in order
 
-constexpr int CS_NT = 1024;
-
-__global__ void __launch_bounds__(CS_NT) k_colsum(const float* __restrict__ in, int rows, int n, int rchunk,
-                                                  float* __restrict__ out) {
-    __shared__ float sh[CS_NT];
-    const int tid = threadIdx.x, nr = CS_NT / n;   // rows taken at a time
+__global__ void __launch_bounds__(8 * MAXN) k_colsum(const float* __restrict__ in, int rows, int n, int rchunk,
+                                                     float* __restrict__ out) {
+    __shared__ float sh[8 * MAXN];
+    const int o = threadIdx.x % n, ty = threadIdx.x / n;
     const int r0 = blockIdx.x * rchunk, r1 = min(rows, r0 + rchunk);
     float s = 0.f;
-    if (tid < nr * n) {
-        const int o = tid % n;
-#pragma unroll 8
-        for (int r = r0 + tid / n; r < r1; r += nr) s += in[(int64_t)r * n + o];
+    int r = r0 + ty;
+    for (; r + 120 < r1; r += 128) {
+        float v[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) v[u] = in[(int64_t)(r + 8 * u) * n + o];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) s += v[u];
     }
-    sh[tid] = s;
+#pragma unroll 4
+    for (; r < r1; r += 8) s += in[(int64_t)r * n + o];
+    sh[threadIdx.x] = s;
     __syncthreads();
-    // rows of the table folded in halves
-    for (int m = nr; m > 1;) {
-        const int h = (m + 1) / 2;
-        if (tid < (m - h) * n) sh[tid] += sh[h * n + tid];
-        __syncthreads();
-        m = h;
+    if (ty == 0) {
+        float t = 0.f;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) t += sh[q * n + o];
+        out[blockIdx.x * n + o] = t;
     }
-    if (tid < n) out[blockIdx.x * n + tid] = sh[tid];
+}
+
+// a single chunk up to 4096 rows; returns the number of partials
+int colsum_parts(int rows) {
+    if (rows <= 4096) return 1;
+    const int rchunk = (rows + COLSUM_PARTS - 1) / COLSUM_PARTS;
+    return (rows + rchunk - 1) / rchunk;
 }
 
 cudaError_t launch_colsum(const float* in, int rows, int n, float* out, cudaStream_t st) {
-    const int rchunk = (rows + COLSUM_PARTS - 1) / COLSUM_PARTS;
-    k_colsum<<<COLSUM_PARTS, CS_NT, 0, st>>>(in, rows, n, rchunk, out); note_launch();
+    const int parts = colsum_parts(rows);
+    const int rchunk = parts == 1 ? rows : (rows + COLSUM_PARTS - 1) / COLSUM_PARTS;
+    k_colsum<<<parts, 8 * n, 0, st>>>(in, rows, n, rchunk, out); note_launch();
     return cudaGetLastError();
 }
 

@@ -22,6 +22,8 @@
 //   wb_fwd8, wb_b8   the same for slots without conv (K = 1), 8 channels per thread; wb_b8 does
 //             the backward reductions and apply in one pass
 #pragma once
+#include <algorithm>
+
 #include "xhc_internal.cuh"
 
 namespace xhc {
@@ -1419,24 +1421,45 @@ inline bool paper_kaps(const Dims& d) {
     return d.nconv == 3 && d.kap[0] == 4 && d.kap[1] == 8 && d.kap[2] == 12;
 }
 
-inline int run_len(int KW, int per) {  // tokens per CTA run: a multiple of KW near `per`
-    const int u = KW > 0 ? KW : 4;
-    int r = (per / u) * u;
-    return r < u ? u : r;
-}
-
 // number of runs of TB tokens (with a conv: runs inside each sequence of S tokens)
-inline long long n_runs(const Dims& d, int T, int TB, bool conv) {
-    if (!conv || d.S <= 0) return ((long long)T + TB - 1) / TB;
+inline long long n_runs(const Dims& d, int64_t T, int TB, bool conv) {
+    if (!conv || d.S <= 0) return (T + TB - 1) / TB;
     const long long rps = (d.S + TB - 1) / TB;
     const long long rem = T % d.S;
     return (T / d.S) * rps + (rem + TB - 1) / TB;
 }
 
-// tokens per run of the backward apply (longer runs amortise the KW - 1 recomputed tokens)
-// tokens per run of the backward apply (with a conv: any length works with the block ring; 296
-// measured best at S = 4096, C = 4096 among 240 / 256 / 296 — fewer, fuller waves of CTAs)
-inline int bapp_run(int KW) { return KW > 0 ? 296 : 64; }
+// Tokens per run.  A run costs its tokens plus `extra` token steps (tables, taps and ring to load,
+// recomputed tokens of the backward apply); with `slices` x runs CTAs on `per_sm` of them per SM, the
+// call takes about (waves of CTAs) x (run + extra) steps.  The longest run that this allows wins, so
+// many tokens keep the `longest` one (measured best at 32768 tokens); few tokens get shorter runs
+// that fill the GPU: 512 tokens of C = 256 took 141 us in the backward apply as two runs of 296 tokens
+// and 16 us as 128 of 4 (forward apply 53 -> 11, reductions 39 -> 10).  Runs are multiples of 4 (the block ring).
+inline int pick_run(const Dims& d, int64_t T, bool conv, int slices, int per_sm, int extra, int longest) {
+    const long long cap = (long long)per_sm * device_sms();
+    const long long S = (conv && d.S > 0) ? d.S : T;
+    auto cost = [&](int tb) {
+        const long long ctas = slices * n_runs(d, T, tb, conv);
+        return ((ctas + cap - 1) / cap) * (std::min<long long>(tb, S) + extra);
+    };
+    if (slices * n_runs(d, T, longest, conv) >= 4 * cap) return longest;
+    int best = longest;
+    long long least = cost(longest);
+    for (int tb = longest - 4; tb >= 4; tb -= 4) {
+        const long long c = cost(tb);
+        if (c < least) {
+            least = c;
+            best = tb;
+        }
+    }
+    return best;
+}
+
+// tokens per run of the backward apply: long runs amortise the KW - 1 recomputed tokens (296 measured
+// best at S = 4096, C = 4096 among 240 / 256 / 296: fewer, fuller waves of CTAs)
+inline int bapp_run(const Dims& d, int64_t T) {
+    return pick_run(d, T, true, wb_nslice(d.C), 2, kw_of(d) + 5, 296);
+}
 
 inline cudaError_t smem_attr(const void* fn, size_t bytes) {
     if (bytes <= 48 * 1024) return cudaSuccess;

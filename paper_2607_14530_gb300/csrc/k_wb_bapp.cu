@@ -8,7 +8,7 @@ template <int KM, int KW, int KS, bool HALO = false>
 cudaError_t bapp_kw(const Dims& d, int slot, int T, const uint16_t* out, ConvPtrs cw, const uint16_t* dX,
                     const int* I, const float* dn_in, const float* tokmat, float* dxact_out,
                     uint16_t* d_out, float* cpart, int nslice, cudaStream_t st) {
-    const int TB = bapp_run(KW);
+    const int TB = bapp_run(d, T);
     const int TH = TB + (KW > 0 ? KW - 1 : 0);
     const size_t sm = sizeof(ARing<KM>) + (size_t)TH * (KM * 4 + 16 + KM * KM + KM) * 4;
     cudaError_t e = smem_attr((const void*)k_wb_bapp<KM, KW, KS, HALO>, sm);

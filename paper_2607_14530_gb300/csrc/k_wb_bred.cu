@@ -9,7 +9,8 @@ cudaError_t bred_kw(const Dims& d, int slot, int T, const uint16_t* out, ConvPtr
                     const int* I, const float* dxact, const uint16_t* xact, int nslice, float* red,
                     cudaStream_t st) {
     constexpr int NVP = NV < 32 ? 16 : NV;
-    int TB = KW > 0 ? 64 : run_len(KW, 48);   // 64 measured faster than 48 with the block ring
+    // 64 measured faster than 48 with the block ring
+    int TB = pick_run(d, T, true, nslice, KM == 4 ? 3 : 2, 12, 64);
     while (TB > 4 && (size_t)TB * (WT / 32) * NVP * 4 > 96 * 1024) TB -= 4;
     const size_t sm = sizeof(BRing<KM>) + (size_t)TB * KM * 4 + (size_t)TB * (WT / 32) * NVP * sizeof(float);
     cudaError_t e = smem_attr((const void*)k_wb_bred<KM, KW, NV, KS>, sm);
@@ -24,7 +25,7 @@ cudaError_t bred2_kw(const Dims& d, int slot, int T, const uint16_t* out, ConvPt
                      const int* I, const float* dxact, const uint16_t* xact, int nslice, float* red,
                      cudaStream_t st) {
     constexpr int NVP = NV < 32 ? 16 : NV;
-    const int TB = 64;
+    const int TB = pick_run(d, T, true, d.C / WSL2, 2, 12, 64);
     const size_t sm = sizeof(BRing2<KM>) + (size_t)TB * KM * 4 + (size_t)TB * (WT / 32) * NVP * sizeof(float);
     cudaError_t e = smem_attr((const void*)k_wb_bred2<KM, NV>, sm);
     if (e != cudaSuccess) return e;
@@ -43,7 +44,7 @@ cudaError_t b8_kw(const Dims& d, int slot, int T, const uint16_t* out, const uin
                   cudaStream_t st) {
     constexpr int NQ = KM + KM * KM;
     constexpr int NV = NQ <= 32 ? 32 : 96;
-    const int TB = 32;
+    const int TB = pick_run(d, T, false, (d.C + W8 - 1) / W8, KM == 4 ? 3 : 2, 4, 32);
     const size_t sm = (size_t)TB * (2 * KM + KM * KM) * 4 + (size_t)TB * (WT / 32) * NV * 4;
     cudaError_t e = smem_attr((const void*)k_wb_b8<KM>, sm);
     if (e != cudaSuccess) return e;

@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(WC_NT) k_wb_coef(Dims d, int slot, int T, int 
 template <int KW, int KS>
 cudaError_t gram_kw(const Dims& d, int slot, int T, const uint16_t* out, ConvPtrs cw, int nslice,
                     float* red, cudaStream_t st) {
-    const int TB = run_len(KW, 64);
+    const int TB = pick_run(d, T, true, nslice, 4, 12, 64);
     const size_t sm = (size_t)TB * (WT / 32) * 16 * sizeof(float);
     cudaError_t e = smem_attr((const void*)k_wb_gram<KW, KS>, sm);
     if (e != cudaSuccess) return e;
@@ -80,7 +80,8 @@ template <int KM, int KW, int KS>
 cudaError_t fwd_kw(const Dims& d, int slot, int T, const uint16_t* out, ConvPtrs cw, const float* emat,
                    int nslice, const uint16_t* xact, const int* I, const float* hres,
                    uint16_t* xact_next, uint16_t* X, cudaStream_t st) {
-    const int TB = KW > 0 ? 128 : run_len(KW, 96);   // 128 measured faster than 96 with the block ring
+    // 128 measured faster than 96 with the block ring
+    const int TB = pick_run(d, T, true, nslice, KM == 4 ? 4 : 3, 12, 128);
     const size_t sm = sizeof(FRing<KM>) + (size_t)TB * (KM * 4 + KM * KM + KM) * 4;
     cudaError_t e = smem_attr((const void*)k_wb_fwd<KM, KW, KS>, sm);
     if (e != cudaSuccess) return e;
@@ -94,7 +95,7 @@ template <int KM>
 cudaError_t fwd8_kw(const Dims& d, int slot, int T, const uint16_t* out, const float* emat,
                     const uint16_t* xact, const int* I, const float* hres, uint16_t* xact_next,
                     uint16_t* X, cudaStream_t st) {
-    const int TB = 32;
+    const int TB = pick_run(d, T, false, (d.C + W8 - 1) / W8, KM == 4 ? 6 : 3, 4, 32);
     const size_t sm = (size_t)TB * (KM + KM * KM + KM) * 4;
     dim3 grid((d.C + W8 - 1) / W8, (T + TB - 1) / TB);
     k_wb_fwd8<KM><<<grid, WT, sm, st>>>(d, slot, T, TB, out, emat, xact, I, hres, xact_next, X); note_launch();
@@ -105,8 +106,7 @@ cudaError_t fwd8_kw(const Dims& d, int slot, int T, const uint16_t* out, const f
 
 int wb_nslice(int C) { return (C + WSL - 1) / WSL; }
 int wb_conv_runs(const Dims& d, int64_t T) {
-    const int KW = kw_of(d);
-    return (int)n_runs(d, (int)T, bapp_run(KW), true);
+    return (int)n_runs(d, T, bapp_run(d, T), true);
 }
 
 // the two-pair Gram kernel: the (4, 8, 12) taps and C a multiple of WSL2
@@ -118,7 +118,7 @@ int wb_gram_slices(const Dims& d) { return gram2_ok(d) ? d.C / WSL2 : wb_nslice(
 cudaError_t launch_wb_gram(const Dims& d, int slot, int T, const uint16_t* out, ConvPtrs cw,
                            int nslice, float* red, cudaStream_t st) {
     if (gram2_ok(d)) {
-        const int TB = 64;
+        const int TB = pick_run(d, T, true, d.C / WSL2, 2, 12, 64);
         const size_t sm = (size_t)TB * (WT / 32) * 16 * sizeof(float);
         dim3 grid(d.C / WSL2, (unsigned)n_runs(d, T, TB, true));
         k_wb_gram2<<<grid, WT, sm, st>>>(d, slot, T, TB, out, cw, nslice, red); note_launch();

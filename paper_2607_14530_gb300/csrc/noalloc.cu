@@ -92,7 +92,7 @@ extern "C" xhc_status xhc_route_noalloc(const xhc_handle* hh, int64_t T, const x
     if (launch_rowproj(X, (int64_t)d.N * d.C, d.N * d.C, (int)T, w, d.nfull, splits, part, pst, st) !=
         cudaSuccess)
         return XHC_ERR_CUDA;
-    if (launch_coef_full(d, (int)T, part, pst, slots_of(splits), wsump, COLSUM_PARTS, P->alpha_pre, P->b_pre,
+    if (launch_coef_full(d, (int)T, part, pst, slots_of(splits), wsump, colsum_parts(d.N * d.C), P->alpha_pre, P->b_pre,
                          (float*)(base + o_zf), (float*)(base + o_st), wsum, hpre, I, p, st) != cudaSuccess)
         return XHC_ERR_CUDA;
     return XHC_OK;

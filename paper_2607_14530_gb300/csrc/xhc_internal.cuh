@@ -405,8 +405,9 @@ cudaError_t launch_wb_bapp(const Dims& d, int slot, int T, const uint16_t* out, 
 // null: nothing is subtracted)
 cudaError_t launch_wgrad_reduce(const float* wpart, const SlotPlan& sp, int E, int n, const WSegsOut& G,
                                 const float* sub, cudaStream_t st);
-// partial column sums of in [rows][n]: out [nparts][n], part q over the rows of chunk q
-constexpr int COLSUM_PARTS = 64;
+// partial column sums of in [rows][n]: out [colsum_parts(rows)][n], part q over the rows of chunk q
+constexpr int COLSUM_PARTS = 64;   // at most
+int colsum_parts(int rows);
 cudaError_t launch_colsum(const float* in, int rows, int n, float* out, cudaStream_t st);
 // wsum: [nws][N] partial column sums of W_r; their sum is left in wsum_out [N]
 cudaError_t launch_coef_full(const Dims& d, int T, const float* part, const float* pstats,
