@@ -591,13 +591,14 @@ ConvPtrs conv_of(const Dims& d, const xhc_params* P, int slot) {
 xhc_status active_maps(const Ctx& c, int slot, const xhc_params* P) {
     const Dims& d = c.d;
     const WSegs wa = act_segs(d, P, slot);
-    SlotPlan sp = slots_of(c.L.splits_act);
+    SlotPlan sp;
     int ssplits = c.L.splits_act;
     float* pstats = c.W<float>(c.L.pstats);
     if (c.T < 128 || d.k * d.C < 64) {
         XHC_K("rowproj_active", c.st, launch_rowproj(c.xact(slot), (int64_t)d.k * d.C, d.k * d.C, c.T, wa,
-                                                     d.nact[slot], c.L.splits_act, c.W<float>(c.L.part),
+                                                     d.nact[slot], &ssplits, c.W<float>(c.L.part),
                                                      c.W<float>(c.L.pstats), c.st));
+        sp = slots_of(ssplits);
     } else {
         ProjTcPlan pl = plan_proj_tc(c.T, d.k * d.C, d.nact[slot], device_sms(), true);
         sp = slots_of(pl);
@@ -635,12 +636,14 @@ xhc_status xhc_pre_fwd(const xhc_handle* h, int slot, int64_t T, const xhc_param
             XHC_K("colsum", c.st, launch_colsum(P->W_r, d.N * d.C, d.N, c.W<float>(c.L.wsump), c.st));
         const WSegs wf = full_segs(d, P);
         // partial slots written (and summed by coef_full): those of the path taken
-        SlotPlan sp = slots_of(c.L.splits_full);
+        SlotPlan sp;
         if (c.T < 128 || d.N * d.C < 64) {
             // smaller than one tensor-core tile: fp32 CUDA-core projection
+            int nslots = c.L.splits_full;
             XHC_K("rowproj_full", c.st, launch_rowproj(X, (int64_t)d.N * d.C, d.N * d.C, c.T, wf,
-                                                       d.nfull, c.L.splits_full, c.W<float>(c.L.part),
+                                                       d.nfull, &nslots, c.W<float>(c.L.part),
                                                        c.W<float>(c.L.pstats), c.st));
+            sp = slots_of(nslots);
         } else {
         sp = slots_of(c.L.tc);
         XHC_K("pack_w", c.st, launch_pack_w(wf, d.nfull, c.L.tc.NB, d.N * d.C,
@@ -783,15 +786,11 @@ xhc_status xhc_post_fwd_decode(const xhc_handle* h, int slot, int64_t B, const x
     const bool last = (slot == d.G - 1);
     long long* ps = reinterpret_cast<long long*>(pos);
     uint16_t* rg = static_cast<uint16_t*>(ring);
-    if (conv && d.gs)
-        XHC_K("dec_gram", c.st, launch_dec_gram(d, slot, c.T, out, cw, rg, ps, c.W<float>(c.L.red), c.st));
-    XHC_K("wb_coef", c.st, launch_wb_coef(d, slot, c.T, c.W<float>(c.L.red), dec_nslice(d.C), c.S<float>(c.L.p),
-                                          c.S<float>(c.L.hpost[slot]),
-                                          (conv && d.gs) ? c.S<double>(c.L.gram[slot]) : nullptr,
-                                          c.W<float>(c.L.tokmat), c.st));
-    XHC_K("dec_fwd", c.st, launch_dec_fwd(d, slot, c.T, out, cw, rg, ps, c.W<float>(c.L.tokmat),
-                                          c.xact(slot), c.S<int>(c.L.I), c.S<float>(c.L.hres),
-                                          last ? nullptr : c.xact(slot + 1), X, c.st));
+    XHC_K("dec_post", c.st, launch_dec_post(d, slot, c.T, out, cw, rg, ps, c.S<float>(c.L.p),
+                                            c.S<float>(c.L.hpost[slot]),
+                                            (conv && d.gs) ? c.S<double>(c.L.gram[slot]) : nullptr,
+                                            c.xact(slot), c.S<int>(c.L.I), c.S<float>(c.L.hres),
+                                            last ? nullptr : c.xact(slot + 1), X, c.st));
     return XHC_OK;
 }
 

@@ -1,174 +1,313 @@
-// Decode: the write-back of a conv slot for one new token per sequence.
+// Decode: the write-back of a slot for one new token per sequence.
 //
 // In decoding, token t of the call is the next token of its own sequence b = t, at position
 // pos[t] of that sequence.  The causal conv of Eq. aug (Sec. 3.3.4: g_j[s] = sum_{i < kappa_j}
 // w_j[i] out[s - i], zero before the sequence start) needs the R = max(kappa) - 1 previous `out`
 // rows of the sequence, which no longer exist as a contiguous [T][C] buffer: they are kept in a
-// per-sequence ring [B][R][C] bf16 (row (s mod R) holds out[s]).  The kernels below are the
-// decode forms of the Gram reduction and of the write-back (Eq. gs, Eq. sparse_write_delta,
-// Eq. sparse_write): CTAs over (256-channel slice, 4 tokens), one channel pair per thread, the
-// conv read from the ring plus the token's own `out` row.  The write-back stores the token's
-// `out` into its ring row afterwards, and the group's last slot advances pos.
+// per-sequence ring [B][R][C] bf16 (row (s mod R) holds out[s]).
+//
+// One kernel does a slot's write-back (Eq. gs, Eq. sparse_write_delta, Eq. sparse_write): a cluster of
+// up to 8 CTAs takes DT tokens, its CTAs the channel slices.  Each CTA forms the conv components of
+// its channels once and keeps them in shared memory; the CTAs exchange their Gram partials through
+// distributed shared memory, CTA (token mod cluster size) turns a token's Gram matrix into the
+// coefficients E and hands them back, and every CTA applies them to its channels, stores the token's
+// `out` in its ring row, and on the group's last slot the cluster advances pos.  Bound by latency: the
+// loads of a token's 12 conv rows and 24 taps are issued together, and of the three launches before
+// (Gram reduction, coefficients, write-back with the conv over again) one is left.
 #include <algorithm>
+#include <utility>
+
+#include <cooperative_groups.h>
 
 #include "xhc_internal.cuh"
 
 namespace xhc {
 namespace {
 
+namespace cg = cooperative_groups;
+
+constexpr int DSL = 256;     // channels of a slice: 128 threads, a channel pair each
+constexpr int DMAXC = 8;     // CTAs of a cluster
+constexpr int DMAXT = 8;     // tokens of a cluster
+
 __device__ __forceinline__ float2 ldp(const uint16_t* p) {
     const uint32_t u = *reinterpret_cast<const uint32_t*>(p);
     return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
 }
 
-// the write-back components of channels (c, c + 1) of token t: u_0 = out, u_{1+j} = g_j
-__device__ __forceinline__ void dec_components(const Dims& d, int slot, int t, int c,
-                                               const uint16_t* __restrict__ out, ConvPtrs cw,
-                                               const uint16_t* __restrict__ ring, long long pos,
-                                               float2 (&u)[4]) {
+// the conv components of channels (c, c + 1): g_j = sum_i w_j[i] out[pos - i], i ascending.  KW: most
+// taps of a component; PAPER: the (4, 8, 12) taps, their loops folded.
+template <int KW, bool PAPER>
+__device__ __forceinline__ void dec_conv(const Dims& d, const ConvPtrs& cw, const uint16_t* __restrict__ rt, int c,
+                                         float2 o, long long pos, float2 (&g)[3]) {
     const int C = d.C, R = d.kapmax - 1;
-    const float2 o = ldp(out + (long long)t * C + c);
-    u[0] = o;
-    u[1] = u[2] = u[3] = make_float2(0.f, 0.f);
-    if (d.K[slot] <= 1) return;
-    const int r0 = (int)(pos % R);                             // ring row of position pos
-    const uint16_t* rt = ring + (long long)t * R * C + c;
-    // the component loop runs to its maximum of 3 with a guard, so that cw.w[j] and d.kap[j]
-    // are static indices (a dynamic index copies the parameter structs to local memory)
+    const int r0 = R > 0 ? (int)(pos % R) : 0;      // ring row of position pos
+    float2 v[KW];
+    v[0] = o;
+#pragma unroll
+    for (int i = 1; i < KW; ++i) {
+        int r = r0 - i;                              // row of position pos - i (i <= R)
+        if (r < 0) r += R;
+        v[i] = (i < d.kapmax && i <= pos) ? ldp(rt + (long long)r * C) : make_float2(0.f, 0.f);
+    }
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        if (j >= d.nconv) break;
-        float2 g = make_float2(0.f, 0.f);
-        for (int i = 0; i < d.kap[j]; ++i) {
-            if (pos - i < 0) break;                            // before the sequence start: zero
-            int r = r0 - i;                                    // row of position pos - i
-            if (r < 0) r += R;
-            const float2 v = (i == 0) ? o : ldp(rt + (long long)r * C);
-            const float2 w = make_float2(cw.w[j][(size_t)i * C + c], cw.w[j][(size_t)i * C + c + 1]);
-            g.x = fmaf(w.x, v.x, g.x);
-            g.y = fmaf(w.y, v.y, g.y);
+        g[j] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < KW; ++i) {
+            if (PAPER ? i >= 4 * (j + 1) : (j >= d.nconv || i >= d.kap[j])) break;
+            float2 w = make_float2(0.f, 0.f);        // no term before the sequence start
+            if (i <= pos) w = make_float2(cw.w[j][(size_t)i * C + c], cw.w[j][(size_t)i * C + c + 1]);
+            g[j].x = fmaf(w.x, v[i].x, g[j].x);
+            g[j].y = fmaf(w.y, v[i].y, g[j].y);
         }
-        u[1 + j] = g;
     }
 }
 
-// Both kernels: CTA (slice, block) takes the 256 channels of slice `slice` (one pair per
-// thread) for DT consecutive tokens, so the conv taps of its channels are read once per CTA and
-// reused from L1 for the following tokens.
-constexpr int DT = 4;
-constexpr int DTH = 128;
-
-// Gram matrix of the components of each token (lower triangle, the order of the prefill's
-// reduction), partial over the CTA's channel slice: red[t][slice][q]
-__global__ void __launch_bounds__(DTH) k_dec_gram(Dims d, int slot, int B, const uint16_t* __restrict__ out,
-                                                  ConvPtrs cw, const uint16_t* __restrict__ ring,
-                                                  const long long* __restrict__ pos, int nslice,
-                                                  float* __restrict__ red) {
-    __shared__ float sh[DTH / 32][NGRAM];
-    const int slice = blockIdx.x, K = d.K[slot];
-    const int c = slice * 2 * DTH + 2 * threadIdx.x;
-    const bool act = c < d.C;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int tt = 0; tt < DT; ++tt) {
-        const int t = blockIdx.y * DT + tt;
-        if (t >= B) break;
-        float v[NGRAM];
-#pragma unroll
-        for (int q = 0; q < NGRAM; ++q) v[q] = 0.f;
-        if (act) {
-            float2 u[4];
-            dec_components(d, slot, t, c, out, cw, ring, pos[t], u);
-            int q = 0;
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b <= a; ++b, ++q)
-                    if (a < K) v[q] = fmaf(u[a].x, u[b].x, u[a].y * u[b].y);
-        }
-#pragma unroll
-        for (int q = 0; q < NGRAM; ++q) {
-            float x = v[q];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-            if (lane == 0) sh[warp][q] = x;
-        }
-        __syncthreads();
-        if (threadIdx.x < NGRAM) {
-            float s2 = 0.f;
-#pragma unroll
-            for (int w = 0; w < DTH / 32; ++w) s2 += sh[w][threadIdx.x];
-            red[((long long)t * nslice + slice) * NRED + threadIdx.x] = s2;
-        }
-        __syncthreads();
+// shared memory of a CTA (dynamic), DT tokens and q slices of its own, ns slices in all
+struct DecSmem {
+    int u, wred, gpart, gs, bs, e, h, bytes;
+    __host__ __device__ DecSmem(int DT, int q, int ns, int k, bool conv) {
+        int o = 0;
+        gs = o; o += DT * 12 * 8;                            // f64 [DT][12]: Gram matrices (this rank's tokens)
+        u = o; o += conv ? DT * q * 3 * 128 * 8 : 0;         // float2 [DT][q][3][128]: conv components
+        wred = o; o += conv ? DT * q * 4 * 10 * 4 : 0;       // f32 [DT][q][4 warps][10]
+        gpart = o; o += conv ? DT * ns * 10 * 4 : 0;         // f32 [DT][ns][10]: Gram partials (this rank's tokens)
+        bs = o; o += DT * 16 * 4;                            // f32 [DT][4][4]: coefficients B
+        e = o; o += DT * k * 4 * 4;                          // f32 [DT][k][4]: E
+        h = o; o += DT * k * k * 4;                          // f32 [DT][k][k]: H_res (last slot)
+        bytes = o;
     }
+};
+
+// warp reduce-scatter of 16 values: every lane returns the total of value lane >> 1
+__device__ __forceinline__ float wred16(float (&v)[16], int lane) {
+#pragma unroll
+    for (int h = 8; h >= 1; h >>= 1) {
+        const bool up = (lane & (2 * h)) != 0;
+#pragma unroll
+        for (int q = 0; q < h; ++q) {
+            const float send = up ? v[q] : v[q + h], keep = up ? v[q + h] : v[q];
+            v[q] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * h);
+        }
+    }
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
-// X_act_new_j = (H_res x_act)_j (last slot) or x_act_j, + sum_a E[j][a] u_a; the last slot
-// scatters into the state rows I_j, the others write the next slot's active state.  Then the
-// token's out row goes into its ring row (each thread its own channels, after its last read of
-// them).
-__global__ void __launch_bounds__(DTH) k_dec_fwd(Dims d, int slot, int B, const uint16_t* __restrict__ out,
-                                                 ConvPtrs cw, uint16_t* __restrict__ ring,
-                                                 const long long* __restrict__ pos,
-                                                 const float* __restrict__ emat,
-                                                 const uint16_t* __restrict__ xact,
-                                                 const int* __restrict__ I,
-                                                 const float* __restrict__ hres,
-                                                 uint16_t* __restrict__ xact_next,
-                                                 uint16_t* __restrict__ X) {
-    const int C = d.C, k = d.k, R = d.kapmax - 1;
+// KM: most active slots; KW, PAPER: see dec_conv; KW = 0: a slot without conv (no exchange, so the
+// CTAs of a token need no cluster)
+template <int KM, int KW, bool PAPER>
+__global__ void __launch_bounds__(512) k_dec_post(Dims d, int slot, int B, int DT, int q, int ns,
+                                                  const uint16_t* __restrict__ out, ConvPtrs cw,
+                                                  uint16_t* __restrict__ ring, long long* __restrict__ pos,
+                                                  const float* __restrict__ p, const float* __restrict__ hpost,
+                                                  double* __restrict__ gram, const uint16_t* __restrict__ xact,
+                                                  const int* __restrict__ I, const float* __restrict__ hres,
+                                                  uint16_t* __restrict__ xact_next, uint16_t* __restrict__ X) {
+    constexpr bool CONV = KW > 0;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ long long ps[DMAXT];
+    const int C = d.C, k = d.k, K = d.K[slot], R = d.kapmax - 1;
     const bool last = (slot == d.G - 1);
-    const bool conv = d.K[slot] > 1;
-    const int c = blockIdx.x * 2 * DTH + 2 * threadIdx.x;
-    if (c >= C) return;
-    for (int tt = 0; tt < DT; ++tt) {
-        const int t = blockIdx.y * DT + tt;
-        if (t >= B) break;
-        const long long p = pos[t];
-        const float* E = emat + (long long)t * TOKMAT;
-        float2 u[4];
-        dec_components(d, slot, t, c, out, cw, ring, p, u);
-        float2 x[MAXK];
+    const DecSmem L(DT, q, ns, k, CONV);
+    double* Gs = reinterpret_cast<double*>(smem + L.gs);
+    float2* us = reinterpret_cast<float2*>(smem + L.u);
+    float* wr = reinterpret_cast<float*>(smem + L.wred);
+    float* gp = reinterpret_cast<float*>(smem + L.gpart);
+    float* Bs = reinterpret_cast<float*>(smem + L.bs);
+    float* Es = reinterpret_cast<float*>(smem + L.e);
+    float* Hs = reinterpret_cast<float*>(smem + L.h);
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+    const int sl = tid >> 7, st = tid & 127;         // slice of this thread in a step, its place there
+    const int nsl = nt >> 7;                         // slices at a time
+    const int t0 = blockIdx.x * DT, ntok = min(DT, B - t0);
+    const int rank = blockIdx.y, nr = gridDim.y;     // CTA of the cluster, and their number
+    const int s0 = rank * q, sn = min(q, ns - s0);   // this CTA's slices
+    if (tid < ntok) ps[tid] = pos[t0 + tid];
+    if (last)
+        for (int e = tid; e < ntok * k * k; e += nt) Hs[e] = hres[(long long)t0 * k * k + e];
+    __syncthreads();
+    if constexpr (CONV) {
+        cg::cluster_group cl = cg::this_cluster();
+        auto started = cl.barrier_arrive();   // waited for before the first access to another CTA
+        // the conv components, and the Gram partials of each slice (lower triangle, the order of the
+        // prefill's reduction)
+        for (int tt = 0; tt < ntok; ++tt) {
+            const long long t = t0 + tt;
+            for (int s = sl; s < sn; s += nsl) {
+                const int c = (s0 + s) * DSL + 2 * st;
+                float2 uu[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+                if (c < C) {
+                    uu[0] = ldp(out + t * C + c);
+                    float2 g[3];
+                    dec_conv<KW, PAPER>(d, cw, ring + t * R * C + c, c, uu[0], ps[tt], g);
 #pragma unroll
-        for (int j = 0; j < MAXK; ++j)
-            x[j] = (j < k) ? ldp(xact + ((long long)t * k + j) * C + c) : make_float2(0.f, 0.f);
-#pragma unroll
-        for (int j = 0; j < MAXK; ++j) {
-            if (j >= k) break;
-            float2 v;
-            if (last) {
-                v = make_float2(0.f, 0.f);
-#pragma unroll
-                for (int i = 0; i < MAXK; ++i) {
-                    if (i >= k) break;
-                    const float h = hres[((long long)t * k + j) * k + i];
-                    v.x = fmaf(h, x[i].x, v.x);
-                    v.y = fmaf(h, x[i].y, v.y);
+                    for (int j = 0; j < 3; ++j) {
+                        uu[1 + j] = g[j];
+                        us[((tt * q + s) * 3 + j) * 128 + st] = g[j];
+                    }
                 }
-            } else {
-                v = x[j];
+                if (d.gs) {
+                    float v[16];
+                    int e = 0;
+#pragma unroll
+                    for (int a = 0; a < 4; ++a)
+#pragma unroll
+                        for (int b = 0; b <= a; ++b, ++e) v[e] = fmaf(uu[a].x, uu[b].x, uu[a].y * uu[b].y);
+#pragma unroll
+                    for (; e < 16; ++e) v[e] = 0.f;
+                    const float tot = wred16(v, lane);
+                    if ((lane & 1) == 0 && lane < 20) wr[((tt * q + s) * 4 + (st >> 5)) * 10 + (lane >> 1)] = tot;
+                }
+            }
+        }
+        __syncthreads();
+        cl.barrier_wait(std::move(started));
+        if (d.gs) {
+            // each slice's partial to the CTA that owns the token
+            for (int e = tid; e < ntok * sn * 10; e += nt) {
+                const int tt = e / (sn * 10), r = e - tt * sn * 10, s = r / 10, x = r - s * 10;
+                const float* w = wr + (tt * q + s) * 40 + x;
+                float* dst = cl.map_shared_rank(gp, tt % nr);
+                dst[(tt * ns + s0 + s) * 10 + x] = ((w[0] + w[10]) + w[20]) + w[30];
+            }
+            cl.sync();
+            for (int e = tid; e < ntok * NGRAM; e += nt) {
+                const int tt = e / NGRAM, x = e - tt * NGRAM;
+                if (tt % nr != rank) continue;
+                double s = 0.0;
+                if (x < K * (K + 1) / 2) {
+                    for (int g = 0; g < ns; ++g) s += (double)gp[(tt * ns + g) * 10 + x];
+                    gram[(long long)(t0 + tt) * NGRAM + x] = s;
+                }
+                Gs[tt * 12 + x] = s;
+            }
+            __syncthreads();
+        }
+        if (tid < ntok && (tid % nr == rank)) {
+            float Bm[MAXCOMP][MAXCOMP];
+            if (d.gs) {
+                double Gm[NGRAM];
+#pragma unroll
+                for (int x = 0; x < NGRAM; ++x) Gm[x] = Gs[tid * 12 + x];
+                GramSchmidt G;
+                G.forward(Gm, (double)d.eps_gs);
+                G.coef(Bm);
             }
 #pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                const float e = E[j * 4 + a];
-                v.x = fmaf(e, u[a].x, v.x);
-                v.y = fmaf(e, u[a].y, v.y);
-            }
-            uint16_t* dst = last ? X + ((long long)t * d.N + I[(long long)t * k + j]) * C + c
-                                 : xact_next + ((long long)t * k + j) * C + c;
-            *reinterpret_cast<uint32_t*>(dst) = pack2(v.x, v.y);
+            for (int a = 0; a < MAXCOMP; ++a)
+#pragma unroll
+                for (int b = 0; b < MAXCOMP; ++b) Bs[tid * 16 + a * 4 + b] = d.gs ? Bm[a][b] : (a == b ? 1.f : 0.f);
         }
-        if (conv && R > 0)
-            *reinterpret_cast<uint32_t*>(ring + ((long long)t * R + (int)(p % R)) * C + c) =
-                *reinterpret_cast<const uint32_t*>(out + (long long)t * C + c);
+        __syncthreads();
+        // E[j][a] = p_j sum_b H_post[j][b] B[b][a] to every CTA of the cluster
+        for (int e = tid; e < ntok * k * 4 * nr; e += nt) {
+            const int to = e / (ntok * k * 4), r = e - to * ntok * k * 4;
+            const int tt = r / (k * 4), j = (r >> 2) % k, a = r & 3;
+            if (tt % nr != rank) continue;
+            const long long tj = (long long)(t0 + tt) * k + j;
+            float v = 0.f;
+            for (int b = a; b < K; ++b) v += hpost[tj * K + b] * Bs[tt * 16 + b * 4 + a];
+            cl.map_shared_rank(Es, to)[r] = p[tj] * v;
+        }
+        cl.sync();
+    } else {
+        for (int e = tid; e < ntok * k; e += nt) {
+            const long long tj = (long long)t0 * k + e;
+            Es[e * 4] = p[tj] * hpost[tj];
+        }
+        __syncthreads();
     }
+    // X_act_new_j = (H_res x_act)_j (last slot) or x_act_j, + sum_a E[j][a] u_a; the last slot scatters
+    // into the state rows I_j, the others write the next slot's active state
+    for (int tt = 0; tt < ntok; ++tt) {
+        const long long t = t0 + tt;
+        for (int s = sl; s < sn; s += nsl) {
+            const int c = (s0 + s) * DSL + 2 * st;
+            if (c >= C) continue;
+            float2 x[KM], uu[4];
+#pragma unroll
+            for (int j = 0; j < KM; ++j) x[j] = (j < k) ? ldp(xact + (t * k + j) * C + c) : make_float2(0.f, 0.f);
+            const uint32_t raw = *reinterpret_cast<const uint32_t*>(out + t * C + c);
+            uu[0] = make_float2(__uint_as_float(raw << 16), __uint_as_float(raw & 0xffff0000u));
+            if constexpr (CONV) {
+#pragma unroll
+                for (int j = 0; j < 3; ++j) uu[1 + j] = us[((tt * q + s) * 3 + j) * 128 + st];
+            }
+#pragma unroll
+            for (int j = 0; j < KM; ++j) {
+                if (j >= k) break;
+                float2 v = x[j];
+                if (last) {
+                    v = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int i = 0; i < KM; ++i) {
+                        if (i >= k) break;
+                        const float h = Hs[(tt * k + j) * k + i];
+                        v.x = fmaf(h, x[i].x, v.x);
+                        v.y = fmaf(h, x[i].y, v.y);
+                    }
+                }
+                const float* E = Es + (tt * k + j) * 4;
+#pragma unroll
+                for (int a = 0; a < (CONV ? 4 : 1); ++a) {
+                    v.x = fmaf(E[a], uu[a].x, v.x);
+                    v.y = fmaf(E[a], uu[a].y, v.y);
+                }
+                uint16_t* dst = last ? X + (t * d.N + I[t * k + j]) * C + c : xact_next + (t * k + j) * C + c;
+                *reinterpret_cast<uint32_t*>(dst) = pack2(v.x, v.y);
+            }
+            if (CONV && R > 0) *reinterpret_cast<uint32_t*>(ring + (t * R + (int)(ps[tt] % R)) * C + c) = raw;
+        }
+    }
+    // the conv's CTAs have all read pos (before their last cluster barrier); without conv none but this one does
+    if (last && rank == 0 && tid < ntok) pos[t0 + tid] = ps[tid] + 1;
 }
 
-// the last slot advances every token's position (after every CTA of the write-back is done:
-// a separate launch)
-__global__ void k_pos_advance(long long* __restrict__ pos, int B) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < B) pos[b] += 1;
+template <int KM, int KW, bool PAPER>
+cudaError_t dec_post_kw(const Dims& d, int slot, int B, const uint16_t* out, ConvPtrs cw, uint16_t* ring,
+                        long long* pos, const float* p, const float* hpost, double* gram, const uint16_t* xact,
+                        const int* I, const float* hres, uint16_t* xact_next, uint16_t* X, cudaStream_t st) {
+    constexpr bool CONV = KW > 0;
+    const int ns = (d.C + DSL - 1) / DSL;
+    const int q = (ns + DMAXC - 1) / DMAXC, nr = (ns + q - 1) / q;   // slices a CTA, CTAs a cluster
+    const int nt = std::min(q, 4) * 128;
+    // about two CTAs per SM, and the components within 64 KB
+    int DT = std::min(DMAXT, std::max(1, (int)(((long long)B * nr + 2 * device_sms() - 1) / (2 * device_sms()))));
+    while (DT > 1 && CONV && DT * q * 3 * 128 * 8 > 64 * 1024) --DT;
+    const DecSmem L(DT, q, ns, d.k, CONV);
+    cudaError_t e = cudaFuncSetAttribute((const void*)k_dec_post<KM, KW, PAPER>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, L.bytes);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((B + DT - 1) / DT), (unsigned)nr);
+    cfg.blockDim = dim3((unsigned)nt);
+    cfg.dynamicSmemBytes = (size_t)L.bytes;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 1;
+    at[0].val.clusterDim.y = CONV ? (unsigned)nr : 1u;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, k_dec_post<KM, KW, PAPER>, d, slot, B, DT, q, ns, out, cw, ring, pos, p, hpost, gram,
+                           xact, I, hres, xact_next, X);
+    note_launch();
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <int KM>
+cudaError_t dec_post_km(const Dims& d, int slot, int B, const uint16_t* out, ConvPtrs cw, uint16_t* ring,
+                        long long* pos, const float* p, const float* hpost, double* gram, const uint16_t* xact,
+                        const int* I, const float* hres, uint16_t* xact_next, uint16_t* X, cudaStream_t st) {
+#define XHC_DEC(KW_, PAPER_) \
+    dec_post_kw<KM, KW_, PAPER_>(d, slot, B, out, cw, ring, pos, p, hpost, gram, xact, I, hres, xact_next, X, st)
+    if (d.K[slot] <= 1) return XHC_DEC(0, false);
+    if (d.nconv == 3 && d.kap[0] == 4 && d.kap[1] == 8 && d.kap[2] == 12) return XHC_DEC(12, true);
+    if (d.kapmax <= 8) return XHC_DEC(8, false);
+    return XHC_DEC(16, false);
+#undef XHC_DEC
 }
 
 // ring rows from a prefill: sequence b of S tokens (rows b*S .. b*S + S - 1 of out) leaves its
@@ -227,30 +366,15 @@ __global__ void k_halo_add(uint16_t* __restrict__ d_out, int B, int S, int C, in
     }
 }
 
-int dec_slices(int C) { return (C + 2 * DTH - 1) / (2 * DTH); }
-
 }  // namespace
 
-cudaError_t launch_dec_gram(const Dims& d, int slot, int B, const uint16_t* out, ConvPtrs cw,
-                            const uint16_t* ring, const long long* pos, float* red, cudaStream_t st) {
-    const dim3 grid(dec_slices(d.C), (B + DT - 1) / DT);
-    k_dec_gram<<<grid, DTH, 0, st>>>(d, slot, B, out, cw, ring, pos, dec_slices(d.C), red); note_launch();
-    return cudaGetLastError();
-}
-
-int dec_nslice(int C) { return dec_slices(C); }
-
-cudaError_t launch_dec_fwd(const Dims& d, int slot, int B, const uint16_t* out, ConvPtrs cw,
-                           uint16_t* ring, long long* pos, const float* emat, const uint16_t* xact,
-                           const int* I, const float* hres, uint16_t* xact_next, uint16_t* X,
-                           cudaStream_t st) {
-    const dim3 grid(dec_slices(d.C), (B + DT - 1) / DT);
-    k_dec_fwd<<<grid, DTH, 0, st>>>(d, slot, B, out, cw, ring, pos, emat, xact, I, hres, xact_next,
-                                    X); note_launch();
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || slot != d.G - 1) return e;
-    k_pos_advance<<<(B + 255) / 256, 256, 0, st>>>(pos, B); note_launch();
-    return cudaGetLastError();
+cudaError_t launch_dec_post(const Dims& d, int slot, int B, const uint16_t* out, ConvPtrs cw,
+                            uint16_t* ring, long long* pos, const float* p, const float* hpost, double* gram,
+                            const uint16_t* xact, const int* I, const float* hres, uint16_t* xact_next,
+                            uint16_t* X, cudaStream_t st) {
+    if (d.k <= 4)
+        return dec_post_km<4>(d, slot, B, out, cw, ring, pos, p, hpost, gram, xact, I, hres, xact_next, X, st);
+    return dec_post_km<8>(d, slot, B, out, cw, ring, pos, p, hpost, gram, xact, I, hres, xact_next, X, st);
 }
 
 cudaError_t launch_ring_fill(const Dims& d, int B, int S, const uint16_t* out, uint16_t* ring,

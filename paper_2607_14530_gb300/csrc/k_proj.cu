@@ -1,10 +1,13 @@
 // Projection-shaped kernels of the connection op on the CUDA cores (fp32 FMA):
 //   rowproj   Z = A W over a row of the state (Eq. fused_normalized_projection, Eq. param_post /
-//             param_res), split over the reduction dimension, plus sum / sum of squares of A
+//             param_res), split over the reduction dimension, plus sum / sum of squares of A: fewer
+//             than 128 tokens, and the routing entry point without a workspace
 //   gemm_dzw  dX_act += dZ W^T (backward of the active projection)
 //   full_dx   dX = dX_base + dZ W^T + a + b x (backward of the full-state projection and norms)
 //   wgrad     dW += A^T dZ, reduced over tokens in a fixed order
 //   colsum    fixed-order partial column sums of W_r
+#include <algorithm>
+
 #include "xhc_internal.cuh"
 
 namespace xhc {
@@ -102,8 +105,158 @@ static cudaError_t rowproj_nt(const uint16_t* A, int64_t lda, int K, int T, cons
     return cudaGetLastError();
 }
 
+// The same for few tokens, where the weight is what is read: a block takes TT tokens and a range of
+// rows; each thread holds V neighbouring columns (V = 4 where every segment's width is a multiple of
+// 4) of one weight segment and walks the rows NT / (n / V) apart with one V-wide load a row, times the
+// rows' TT state values from shared memory (fp32 FMAs on token pairs).  The row lanes' sums are folded
+// in shared memory at the end.  The 64-token tile above spends its FMAs on padding here: at N = 16,
+// C = 4096 one token took it 52 us for the 21 MB of the full-state weight.
+constexpr int RS_NT = 512;
+constexpr int RS_ROWS = 256;   // rows of the state staged at a time
+
+template <int TT, int V>
+__global__ void __launch_bounds__(RS_NT) k_rowproj_small(const uint16_t* __restrict__ A, int64_t lda, int K, int T,
+                                                         WSegs W, int n, int kchunk, float* __restrict__ part,
+                                                         float* __restrict__ pstats) {
+    constexpr int TP = (TT + 1) / 2;                 // token pairs
+    extern __shared__ __align__(16) float sm[];      // [RS_ROWS][2 TP] state rows; then [row lanes][n][TT]
+    __shared__ float stat[TT][2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nv = n / V, nl = RS_NT / nv;           // column groups, row lanes
+    const int rl = tid / nv, o = (tid - rl * nv) * V;
+    const bool work = rl < nl;
+    const int k0 = blockIdx.x * kchunk, k1 = min(K, k0 + kchunk);
+    const int t0 = blockIdx.y * TT;
+    // this thread's weight segment, selected with static indices
+    const float* wp = W.ptr[0];
+    int width = W.width[0], off = W.off[0];
+#pragma unroll
+    for (int q = 1; q < MAXSEG; ++q)
+        if (q < W.n && o >= W.off[q]) {
+            wp = W.ptr[q];
+            width = W.width[q];
+            off = W.off[q];
+        }
+    wp += o - off;
+    float2 acc[V][TP];
+#pragma unroll
+    for (int c = 0; c < V; ++c)
+#pragma unroll
+        for (int u = 0; u < TP; ++u) acc[c][u] = make_float2(0.f, 0.f);
+    if (tid < 2 * TT) stat[tid >> 1][tid & 1] = 0.f;
+    for (int kb = k0; kb < k1; kb += RS_ROWS) {
+        const int rows = min(RS_ROWS, k1 - kb);      // a multiple of 8
+        __syncthreads();
+        // a warp stages 256 rows of one token and adds their sum and sum of squares
+        for (int tt = warp; tt < 2 * TP; tt += RS_NT / 32) {
+            float x[8], s1 = 0.f, s2 = 0.f;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) x[e] = 0.f;
+            if (tt < TT && t0 + tt < T && lane * 8 < rows)
+                unpack8(__ldg(reinterpret_cast<const uint4*>(A + (int64_t)(t0 + tt) * lda + kb + lane * 8)), x);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                sm[(lane * 8 + e) * (2 * TP) + tt] = x[e];
+                s1 += x[e];
+                s2 = fmaf(x[e], x[e], s2);
+            }
+            s1 = warp_sum(s1);
+            s2 = warp_sum(s2);
+            if (lane == 0 && tt < TT) {
+                stat[tt][0] += s1;
+                stat[tt][1] += s2;
+            }
+        }
+        __syncthreads();
+        if (work) {
+            constexpr int U = TT >= 8 ? 4 : 8;       // weight rows in flight
+            for (int r0 = rl; r0 < rows; r0 += U * nl) {
+                float w[U][V];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int r = r0 + u * nl;
+                    const float* p = wp + (int64_t)(kb + r) * width;
+                    if constexpr (V == 4) {
+                        const float4 f = r < rows ? __ldg(reinterpret_cast<const float4*>(p)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        w[u][0] = f.x; w[u][1] = f.y; w[u][2] = f.z; w[u][3] = f.w;
+                    } else {
+                        w[u][0] = r < rows ? __ldg(p) : 0.f;
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int r = r0 + u * nl;
+                    if (r >= rows) break;
+                    const float2* xr = reinterpret_cast<const float2*>(sm + r * (2 * TP));
+#pragma unroll
+                    for (int q = 0; q < TP; ++q) {
+                        const float2 x = xr[q];
+#pragma unroll
+                        for (int c = 0; c < V; ++c) acc[c][q] = __ffma2_rn(make_float2(w[u][c], w[u][c]), x, acc[c][q]);
+                    }
+                }
+            }
+        }
+    }
+    __syncthreads();
+    const int O = n * TT;
+    if (work) {
+#pragma unroll
+        for (int c = 0; c < V; ++c)
+#pragma unroll
+            for (int u = 0; u < TT; ++u) sm[rl * O + u * n + o + c] = (u & 1) ? acc[c][u / 2].y : acc[c][u / 2].x;
+    }
+    __syncthreads();
+    for (int m = nl; m > 1;) {
+        const int h = (m + 1) / 2;
+        for (int e = tid; e < (m - h) * O; e += RS_NT) sm[e] += sm[h * O + e];
+        __syncthreads();
+        m = h;
+    }
+    const int nt = min(TT, T - t0);
+    const int64_t row = (int64_t)blockIdx.x * T + t0;
+    for (int e = tid; e < nt * n; e += RS_NT) part[row * n + e] = sm[e];
+    if (tid < 2 * nt) pstats[row * 2 + tid] = stat[tid >> 1][tid & 1];
+}
+
+template <int TT, int V>
+static cudaError_t rowproj_small(const uint16_t* A, int64_t lda, int K, int T, const WSegs& W, int n, int* splits,
+                                 float* part, float* pstats, cudaStream_t st) {
+    const int nl = RS_NT / (n / V), ny = (T + TT - 1) / TT;
+    // a block per SM, with at least four rows a row lane
+    int s = std::min(*splits, std::max(1, device_sms() / ny));
+    s = std::max(1, std::min(s, K / (4 * nl)));
+    const int kchunk = ((K + s - 1) / s + 7) / 8 * 8;
+    s = (K + kchunk - 1) / kchunk;
+    *splits = s;
+    const size_t sm = sizeof(float) * std::max((size_t)RS_ROWS * ((TT + 1) / 2 * 2), (size_t)nl * n * TT);
+    const cudaError_t e = cudaFuncSetAttribute((const void*)k_rowproj_small<TT, V>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    k_rowproj_small<TT, V><<<dim3(s, ny), RS_NT, sm, st>>>(A, lda, K, T, W, n, kchunk, part, pstats); note_launch();
+    return cudaGetLastError();
+}
+
+template <int V>
+static cudaError_t rowproj_small_v(const uint16_t* A, int64_t lda, int K, int T, const WSegs& W, int n, int* splits,
+                                   float* part, float* pstats, cudaStream_t st) {
+    if (T <= 1) return rowproj_small<1, V>(A, lda, K, T, W, n, splits, part, pstats, st);
+    if (T <= 2) return rowproj_small<2, V>(A, lda, K, T, W, n, splits, part, pstats, st);
+    if (T <= 4) return rowproj_small<4, V>(A, lda, K, T, W, n, splits, part, pstats, st);
+    if (T <= 8) return rowproj_small<8, V>(A, lda, K, T, W, n, splits, part, pstats, st);
+    return rowproj_small<16, V>(A, lda, K, T, W, n, splits, part, pstats, st);
+}
+
 cudaError_t launch_rowproj(const uint16_t* A, int64_t lda, int K, int T, const WSegs& W, int n,
-                           int splits, float* part, float* pstats, cudaStream_t st) {
+                           int* nslots, float* part, float* pstats, cudaStream_t st) {
+    const int splits = *nslots;
+    if (T < ROWPROJ_SMALL) {
+        // four columns a load where the segments' rows allow 16-byte loads
+        bool v4 = true;
+        for (int q = 0; q < W.n; ++q) v4 = v4 && W.width[q] % 4 == 0 && ((uintptr_t)W.ptr[q] & 15u) == 0;
+        return v4 ? rowproj_small_v<4>(A, lda, K, T, W, n, nslots, part, pstats, st)
+                  : rowproj_small_v<1>(A, lda, K, T, W, n, nslots, part, pstats, st);
+    }
     const int nt = (n + 15) / 16;
     if (nt <= 1) return rowproj_nt<1>(A, lda, K, T, W, n, splits, part, pstats, st);
     if (nt <= 2) return rowproj_nt<2>(A, lda, K, T, W, n, splits, part, pstats, st);

@@ -45,7 +45,7 @@ extern "C" xhc_status xhc_route_noalloc(const xhc_handle* hh, int64_t T, const x
 
     // scratch layout, same split-K choice as xhc_pre_fwd
     const Layout L = make_layout(d, T);
-    const int splits = L.splits_full;
+    int splits = L.splits_full;
     const size_t t = (size_t)T;
     size_t o = 0;
     const size_t o_part = o;  o = al256(o + (size_t)splits * t * d.nfull * 4);
@@ -89,7 +89,7 @@ extern "C" xhc_status xhc_route_noalloc(const xhc_handle* hh, int64_t T, const x
         w.ptr[w.n] = P->W_pre[q]; w.width[w.n] = d.N; w.off[w.n] = off; off += d.N; ++w.n;
     }
     w.off[w.n] = off;
-    if (launch_rowproj(X, (int64_t)d.N * d.C, d.N * d.C, (int)T, w, d.nfull, splits, part, pst, st) !=
+    if (launch_rowproj(X, (int64_t)d.N * d.C, d.N * d.C, (int)T, w, d.nfull, &splits, part, pst, st) !=
         cudaSuccess)
         return XHC_ERR_CUDA;
     if (launch_coef_full(d, (int)T, part, pst, slots_of(splits), wsump, colsum_parts(d.N * d.C), P->alpha_pre, P->b_pre,

@@ -334,8 +334,10 @@ int debug_take_force_timeout();
 // ---------------------------------------------------------------------------------------------
 // launchers (each returns cudaGetLastError() after enqueueing)
 
+// fp32 CUDA-core projection into *nslots partial slots at most (on return: the number written)
+constexpr int ROWPROJ_SMALL = 128;   // fewer tokens than this: the kernel for few tokens
 cudaError_t launch_rowproj(const uint16_t* A, int64_t lda, int K, int T, const WSegs& W, int n,
-                           int splits, float* part, float* pstats, cudaStream_t st);
+                           int* nslots, float* part, float* pstats, cudaStream_t st);
 cudaError_t launch_pack_w(const WSegs& W, int nfull, int NB, int K, uint16_t* Wpack, cudaStream_t st);
 // pstats null: no row statistics (the caller has them from the kernel that wrote X)
 cudaError_t launch_proj_tc(const uint16_t* X, int T, int K, const uint16_t* Wpack, int nfull,
@@ -366,15 +368,12 @@ int wb_gram_slices(const Dims& d);  // partial-sum slices of wb_gram (and wb_coe
 int wb_conv_runs(const Dims& d, int64_t T);
 int wb_bred_slices(const Dims& d, int slot);  // partial-sum slices of wb_bred (and bwd_coef)  // runs (conv weight-gradient partials) of wb_bapp
 // decode (one token per sequence, conv history in a per-sequence ring of max(kappa) - 1 rows)
-cudaError_t launch_dec_gram(const Dims& d, int slot, int B, const uint16_t* out, ConvPtrs cw,
-                            const uint16_t* ring, const long long* pos, float* red, cudaStream_t st);
-cudaError_t launch_dec_fwd(const Dims& d, int slot, int B, const uint16_t* out, ConvPtrs cw,
-                           uint16_t* ring, long long* pos, const float* emat, const uint16_t* xact,
-                           const int* I, const float* hres, uint16_t* xact_next, uint16_t* X,
-                           cudaStream_t st);
+cudaError_t launch_dec_post(const Dims& d, int slot, int B, const uint16_t* out, ConvPtrs cw,
+                            uint16_t* ring, long long* pos, const float* p, const float* hpost, double* gram,
+                            const uint16_t* xact, const int* I, const float* hres, uint16_t* xact_next,
+                            uint16_t* X, cudaStream_t st);
 cudaError_t launch_ring_fill(const Dims& d, int B, int S, const uint16_t* out, uint16_t* ring,
                              cudaStream_t st);
-int dec_nslice(int C);  // channel slices (partial Gram slots) of the decode Gram reduction
 // model glue: N copies of a hidden vector per token, and the sum of the N streams
 cudaError_t launch_stream_bcast(int T, int N, int C, const uint16_t* h, uint16_t* X, cudaStream_t st);
 cudaError_t launch_stream_sum(int T, int N, int C, const uint16_t* X, uint16_t* y, cudaStream_t st);

@@ -1,10 +1,15 @@
 """GPU parity at the block and tile edges of the per-token and write-back kernels, whose block sizes
 and run lengths depend on the number of tokens: remainders on both sides of each switch, against the
 oracle with the bounds of the parity suite."""
+import dataclasses
+
 import pytest
+import torch
 
 import test_gpu_parity as parity
-from paper_2607_14530_gb300.xhc import Config
+import xhc_cases as cases
+from paper_2607_14530_gb300 import synth
+from paper_2607_14530_gb300.xhc import Config, Group
 
 pytestmark = pytest.mark.gpu
 
@@ -27,3 +32,69 @@ CASES = {
 def test_block_edges(name, monkeypatch):
     monkeypatch.setitem(parity.CASES, name, CASES[name])
     parity.test_forward_backward_parity(name)
+
+
+# decode: batches at the switches of the projection for few tokens (1, 2, 4, 8, 16 tokens a block, the
+# tensor cores from 128) and of the write-back's tokens per cluster; N and k with widths that are not a
+# multiple of 4 (one column a load); slices that fill no whole CTA; other tap sets; positions below R
+DECODE = {
+    "B1": (Config.flash(16, 4, 2, 520, 4), 1, 3, False),
+    "B3_N6": (Config.flash(6, 3, 1, 264, 2, conv_k=(2, 5)), 3, 40, False),
+    "B9_k8": (Config.full(12, 8, 3, 776, True), 9, 15, False),
+    "B17_no_gs": (Config.full(8, 4, 2, 64, True, gram_schmidt=False), 17, 11, False),
+    "B31_attn": (Config.full(8, 4, 2, 72, False), 31, 4, False),
+    "B127": (Config.flash(8, 4, 2, 2312, 2, conv_k=(16,)), 127, 20, True),
+    "B130": (Config.flash(8, 4, 2, 1024, 2), 130, 20, True),
+}
+
+
+@pytest.mark.parametrize("name", list(DECODE))
+def test_decode_sizes(name):
+    """One decoded token per sequence (positions S, S + 1, ...) against the forward of a sequence that
+    ends there: the ring holds the outputs before it."""
+    cfg, B, S, spread = DECODE[name]
+    dev = torch.device("cuda", 0)
+    R = max(cfg.conv_k) - 1
+    # the oracle's sequences: the R history rows (their own states do not matter) and the new token
+    seq = dataclasses.replace(cfg, seq_len=R + 1)
+    for seed in range(5, 50):
+        inp = synth.group_inputs(B * (R + 1), cfg.N, cfg.C, cfg.G, seed)
+        P = synth.params(cfg.param_shapes(), seed)
+        new = torch.arange(B) * (R + 1) + R
+        if not cfg.has_router or bool(cases.tie_free(cfg, inp["X"][new], P["W_r"]).all()):
+            break
+    pos = S + (torch.arange(B) if spread else torch.zeros(B, dtype=torch.int64))
+    for o in inp["outs"]:   # nothing before the start of a sequence shorter than the history
+        v = o.view(B, R + 1, cfg.C)
+        for b in range(B):
+            v[b, :max(0, R - int(pos[b]))] = 0
+    ref = cases.run_oracle(seq, inp, P)
+    g = Group(cfg)
+    saved, ws = g.alloc(B)
+    rings = g.alloc_rings(B)
+    for t, ring in enumerate(rings):
+        if ring is None:
+            continue
+        r = ring.view(torch.bfloat16).view(B, R, cfg.C)
+        r.fill_(float("nan"))   # rows that the conv must not read
+        for b in range(B):
+            for i in range(1, min(R, int(pos[b])) + 1):
+                r[b, (int(pos[b]) - i) % R] = inp["outs"][t].view(B, R + 1, cfg.C)[b, R - i].to(dev)
+    X = inp["X"][new].to(dev).contiguous()
+    outs = [o[new].to(dev).contiguous() for o in inp["outs"]]
+    dpos = pos.to(dev)
+    ins = g.forward_decode({n: v.to(dev) for n, v in P.items()}, X, outs, rings, dpos, saved, ws)
+    torch.cuda.synchronize()
+    co = g.coefficients(saved, B)
+    assert torch.equal(co["I"].cpu().long(), ref["aux"]["I"][new])
+    bases = cases.flash_bases(cfg, inp["X"], ref["aux"])
+    for t in range(cfg.G):
+        cases.assert_bf16_close(ins[t], ref["inputs"][t][new], f"input[{t}]",
+                                None if bases[t] is None else bases[t][new])
+        cases.assert_f32_close(co["hpost"][t], ref["aux"]["H_post"][t][new], f"H_post[{t}]")
+        if rings[t] is not None:
+            r = rings[t].view(torch.bfloat16).view(B, R, cfg.C)
+            assert torch.equal(r[torch.arange(B), (pos % R).to(dev)], outs[t])
+    cases.assert_bf16_close(X, ref["X"][new], "X")
+    assert torch.equal(dpos.cpu(), pos + 1)
+    assert g.device_error(ws) == 0
