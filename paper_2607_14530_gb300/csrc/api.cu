@@ -190,7 +190,8 @@ Layout make_layout(const Dims& d, int64_t T) {
     o = 0;
     L.err = o; o = al(o + 256);
     L.wpack = o;
-    o = al(o + std::max((size_t)L.tc.NB * d.N * d.C, (size_t)L.tca.NB * d.k * d.C) * 2);
+    o = al(o + (size_t)L.tc.NB * d.N * d.C * 2);
+    L.wpacka = o; o = al(o + (size_t)L.tca.NB * d.k * d.C * 2);
     L.dzpack = o; o = al(o + (size_t)std::max(L.twf.NB, L.twa.NB) * ((t + 7) / 8 * 8) * 2);
     {
         // bf16 operands of the tensor-core input gradients: full maps [T][nfull] and [N C][nfull],
@@ -587,6 +588,23 @@ ConvPtrs conv_of(const Dims& d, const xhc_params* P, int slot) {
     return c;
 }
 
+// the tensor-core projections take calls of at least one 128-token tile
+bool tc_full(const Ctx& c) { return c.T >= 128 && c.d.N * c.d.C >= 64; }
+bool tc_act(const Ctx& c) { return c.T >= 128 && c.d.k * c.d.C >= 64; }
+
+// the slot's active weight to be packed (nothing below a tile)
+PackJob act_pack(const Ctx& c, int slot, const xhc_params* P) {
+    PackJob j;
+    memset(&j, 0, sizeof(j));
+    if (!tc_act(c)) return j;
+    j.W = act_segs(c.d, P, slot);
+    j.n = c.d.nact[slot];
+    j.NB = plan_proj_tc(c.T, c.d.k * c.d.C, j.n, device_sms(), true).NB;
+    j.K = c.d.k * c.d.C;
+    j.dst = c.W<uint16_t>(c.L.wpacka);
+    return j;
+}
+
 // Active-state mapping generation of one slot (Eq. param_post, Eq. param_res).
 xhc_status active_maps(const Ctx& c, int slot, const xhc_params* P) {
     const Dims& d = c.d;
@@ -594,7 +612,7 @@ xhc_status active_maps(const Ctx& c, int slot, const xhc_params* P) {
     SlotPlan sp;
     int ssplits = c.L.splits_act;
     float* pstats = c.W<float>(c.L.pstats);
-    if (c.T < 128 || d.k * d.C < 64) {
+    if (!tc_act(c)) {
         XHC_K("rowproj_active", c.st, launch_rowproj(c.xact(slot), (int64_t)d.k * d.C, d.k * d.C, c.T, wa,
                                                      d.nact[slot], &ssplits, c.W<float>(c.L.part),
                                                      c.W<float>(c.L.pstats), c.st));
@@ -602,10 +620,8 @@ xhc_status active_maps(const Ctx& c, int slot, const xhc_params* P) {
     } else {
         ProjTcPlan pl = plan_proj_tc(c.T, d.k * d.C, d.nact[slot], device_sms(), true);
         sp = slots_of(pl);
-        XHC_K("pack_w", c.st, launch_pack_w(wa, d.nact[slot], pl.NB, d.k * d.C,
-                                            c.W<uint16_t>(c.L.wpack), c.st));
         // the norm statistics come from the read / input pass that produced x_act
-        XHC_K("proj_tc_active", c.st, launch_proj_tc(c.xact(slot), c.T, d.k * d.C, c.W<uint16_t>(c.L.wpack),
+        XHC_K("proj_tc_active", c.st, launch_proj_tc(c.xact(slot), c.T, d.k * d.C, c.W<uint16_t>(c.L.wpacka),
                                                      d.nact[slot], pl, c.W<float>(c.L.part), nullptr,
                                                      c.W<int>(c.L.err), c.st));
         pstats = c.W<float>(c.L.astat);
@@ -632,13 +648,13 @@ xhc_status xhc_pre_fwd(const xhc_handle* h, int slot, int64_t T, const xhc_param
     if (!aligned16(X) || !aligned16(input)) return XHC_ERR_ALIGNMENT;
     const Dims& d = c.d;
     if (slot == 0) {
-        if (d.hr)
-            XHC_K("colsum", c.st, launch_colsum(P->W_r, d.N * d.C, d.N, c.W<float>(c.L.wsump), c.st));
         const WSegs wf = full_segs(d, P);
         // partial slots written (and summed by coef_full): those of the path taken
         SlotPlan sp;
-        if (c.T < 128 || d.N * d.C < 64) {
+        if (!tc_full(c)) {
             // smaller than one tensor-core tile: fp32 CUDA-core projection
+            if (d.hr)
+                XHC_K("colsum", c.st, launch_colsum(P->W_r, d.N * d.C, d.N, c.W<float>(c.L.wsump), c.st));
             int nslots = c.L.splits_full;
             XHC_K("rowproj_full", c.st, launch_rowproj(X, (int64_t)d.N * d.C, d.N * d.C, c.T, wf,
                                                        d.nfull, &nslots, c.W<float>(c.L.part),
@@ -646,8 +662,14 @@ xhc_status xhc_pre_fwd(const xhc_handle* h, int slot, int64_t T, const xhc_param
             sp = slots_of(nslots);
         } else {
         sp = slots_of(c.L.tc);
-        XHC_K("pack_w", c.st, launch_pack_w(wf, d.nfull, c.L.tc.NB, d.N * d.C,
-                                            c.W<uint16_t>(c.L.wpack), c.st));
+        PackJob full;
+        full.W = wf;
+        full.n = d.nfull;
+        full.NB = c.L.tc.NB;
+        full.K = d.N * d.C;
+        full.dst = c.W<uint16_t>(c.L.wpack);
+        XHC_K("pack_w", c.st, launch_pack_full(full, d.hr ? P->W_r : nullptr, d.N, c.W<float>(c.L.wsump),
+                                               act_pack(c, slot, P), c.st));
         XHC_K("proj_tc", c.st, launch_proj_tc(X, c.T, d.N * d.C, c.W<uint16_t>(c.L.wpack), d.nfull,
                                               c.L.tc, c.W<float>(c.L.part), c.W<float>(c.L.pstats),
                                               c.W<int>(c.L.err), c.st));
@@ -660,7 +682,8 @@ xhc_status xhc_pre_fwd(const xhc_handle* h, int slot, int64_t T, const xhc_param
                              c.W<uint16_t>(c.L.base), c.xact(0), c.W<float>(c.L.astat), c.st));
     } else {
         XHC_K("input", c.st, launch_input(d, slot, c.T, c.W<uint16_t>(c.L.base), c.xact(slot),
-                              c.S<float>(c.L.hpre), c.S<int>(c.L.I), input, c.W<float>(c.L.astat), c.st));
+                              c.S<float>(c.L.hpre), c.S<int>(c.L.I), input, c.W<float>(c.L.astat),
+                              act_pack(c, slot, P), c.st));
     }
     return active_maps(c, slot, P);
 }

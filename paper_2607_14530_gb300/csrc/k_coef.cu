@@ -70,10 +70,13 @@ __device__ __forceinline__ float slot_sum(const float* __restrict__ p, long long
 // p1 + e * step1.  The slots of a stream-K plan are added in slot order (any number of tokens gives
 // the same bits for a token, and so the same routing); those of an even split, of which there are
 // many on few tokens, by groups of threads that take interleaved slots (scr: one float per thread).
-// Ends with a block barrier.
+// Few elements with many ordered slots pass through shared memory (stage: SS_STAGE floats), so that
+// the whole block loads them: 82 sums over 172 slots took 27 us with a thread each.  Ends with a
+// block barrier.
+constexpr int SS_STAGE = 4096;
 __device__ __forceinline__ void slot_sums(bool ordered, const float* __restrict__ p0, long long stride0, int cnt0,
                                           int n0, const float* __restrict__ p1, long long stride1, int cnt1, int n1,
-                                          int step1, float* dst, float* scr) {
+                                          int step1, float* dst, float* scr, float* stage) {
     const int n = n0 + n1, nt = blockDim.x, tid = threadIdx.x;
     const int ng = ordered ? 1 : nt / n;
     if (ng > 1) {
@@ -87,6 +90,27 @@ __device__ __forceinline__ void slot_sums(bool ordered, const float* __restrict_
             for (int q = 0; q < ng; ++q) s += scr[q * n + tid];
             dst[tid] = s;
         }
+    } else if (2 * n <= nt && cnt0 > 16) {
+        const int nl = nt / n, sc = SS_STAGE / n;    // slots loaded at a time, slots a chunk
+        const int g = tid / n, e = tid - g * n;
+        const int cnt = e < n0 ? cnt0 : cnt1;
+        const float* p = e < n0 ? p0 + e : p1 + (long long)(e - n0) * step1;
+        const long long stride = e < n0 ? stride0 : stride1;
+        float s = 0.f;
+        for (int q0 = 0; q0 < max(cnt0, cnt1); q0 += sc) {
+            const int m = min(sc, cnt - q0);
+            if (g < nl) {
+#pragma unroll 8
+                for (int q = g; q < m; q += nl) stage[q * n + e] = p[(q0 + q) * stride];
+            }
+            __syncthreads();
+            if (tid < n) {
+#pragma unroll 8
+                for (int q = 0; q < m; ++q) s += stage[q * n + tid];
+            }
+            __syncthreads();
+        }
+        if (tid < n) dst[tid] = s;
     } else {
         for (int e = tid; e < n; e += nt)
             dst[e] = (e < n0) ? slot_sum<16>(p0 + e, stride0, cnt0, 0, 1)
@@ -170,7 +194,7 @@ __global__ void __launch_bounds__(CF_NT) k_coef_full(Dims d, int T, int TB, cons
                                                      float* __restrict__ hpre, int* __restrict__ I,
                                                      float* __restrict__ p) {
     extern __shared__ float sm[];   // [TB][n] projections, [TB][2] statistics
-    __shared__ float scr[CF_NT], scw[8 * MAXN], ws[MAXN];
+    __shared__ float scr[CF_NT], scw[8 * MAXN], ws[MAXN], stage[SS_STAGE];
     const int tid = threadIdx.x, lane = tid & 31, N = d.N, n = d.nfull;
     const long long t0 = (long long)blockIdx.x * TB;
     const int ntok = (int)min((long long)TB, T - t0);
@@ -180,7 +204,7 @@ __global__ void __launch_bounds__(CF_NT) k_coef_full(Dims d, int T, int TB, cons
     float* zs = sm;
     float* st = sm + ntok * n;
     slot_sums(sp.n == 0, part + t0 * n, (long long)T * n, nsl, ntok * n, pstats + t0 * 2, (long long)T * 2, nsl,
-              ntok * 2, 1, zs, scr);
+              ntok * 2, 1, zs, scr, stage);
     if (d.hr && tid < N) {
         float s = 0.f;
 #pragma unroll
@@ -266,7 +290,7 @@ __global__ void __launch_bounds__(CF_NT) k_coef_act(Dims d, int slot, int T, int
                                                     float* __restrict__ rs, float* __restrict__ hpost,
                                                     float* __restrict__ hres) {
     extern __shared__ float sm[];   // [TB][n] projections, [TB] sums of squares
-    __shared__ float scr[CF_NT];
+    __shared__ float scr[CF_NT], stage[SS_STAGE];
     const int tid = threadIdx.x, k = d.k, kK = d.k * d.K[slot], n = d.nact[slot];
     const long long t0 = (long long)blockIdx.x * TB;
     const int ntok = (int)min((long long)TB, T - t0);
@@ -274,7 +298,7 @@ __global__ void __launch_bounds__(CF_NT) k_coef_act(Dims d, int slot, int T, int
     float* zs = sm;
     float* st = sm + ntok * n;
     slot_sums(sp.n == 0, part + t0 * n, (long long)T * n, nsl, ntok * n, pstats + t0 * 2 + 1, (long long)T * 2,
-              ssplits, ntok, 2, zs, scr);
+              ssplits, ntok, 2, zs, scr, stage);
     if (tid < ntok) {
         const float r = 1.0f / sqrtf(st[tid] / (float)(k * d.C) + d.eps);
         st[tid] = r;

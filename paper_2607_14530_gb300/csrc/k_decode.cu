@@ -36,12 +36,12 @@ __device__ __forceinline__ float2 ldp(const uint16_t* p) {
 }
 
 // the conv components of channels (c, c + 1): g_j = sum_i w_j[i] out[pos - i], i ascending.  KW: most
-// taps of a component; PAPER: the (4, 8, 12) taps, their loops folded.
+// taps of a component; PAPER: the (4, 8, 12) taps, their loops folded.  pos: the position, at most KW
+// of it; r0: its ring row.
 template <int KW, bool PAPER>
 __device__ __forceinline__ void dec_conv(const Dims& d, const ConvPtrs& cw, const uint16_t* __restrict__ rt, int c,
-                                         float2 o, long long pos, float2 (&g)[3]) {
+                                         float2 o, int pos, int r0, float2 (&g)[3]) {
     const int C = d.C, R = d.kapmax - 1;
-    const int r0 = R > 0 ? (int)(pos % R) : 0;      // ring row of position pos
     float2 v[KW];
     v[0] = o;
 #pragma unroll
@@ -97,7 +97,7 @@ __device__ __forceinline__ float wred16(float (&v)[16], int lane) {
 // KM: most active slots; KW, PAPER: see dec_conv; KW = 0: a slot without conv (no exchange, so the
 // CTAs of a token need no cluster)
 template <int KM, int KW, bool PAPER>
-__global__ void __launch_bounds__(512) k_dec_post(Dims d, int slot, int B, int DT, int q, int ns,
+__global__ void __launch_bounds__(512, 2) k_dec_post(Dims d, int slot, int B, int DT, int q, int ns,
                                                   const uint16_t* __restrict__ out, ConvPtrs cw,
                                                   uint16_t* __restrict__ ring, long long* __restrict__ pos,
                                                   const float* __restrict__ p, const float* __restrict__ hpost,
@@ -107,6 +107,7 @@ __global__ void __launch_bounds__(512) k_dec_post(Dims d, int slot, int B, int D
     constexpr bool CONV = KW > 0;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ long long ps[DMAXT];
+    __shared__ int rows[DMAXT];
     const int C = d.C, k = d.k, K = d.K[slot], R = d.kapmax - 1;
     const bool last = (slot == d.G - 1);
     const DecSmem L(DT, q, ns, k, CONV);
@@ -123,7 +124,11 @@ __global__ void __launch_bounds__(512) k_dec_post(Dims d, int slot, int B, int D
     const int t0 = blockIdx.x * DT, ntok = min(DT, B - t0);
     const int rank = blockIdx.y, nr = gridDim.y;     // CTA of the cluster, and their number
     const int s0 = rank * q, sn = min(q, ns - s0);   // this CTA's slices
-    if (tid < ntok) ps[tid] = pos[t0 + tid];
+    if (tid < ntok) {
+        const long long v = pos[t0 + tid];
+        ps[tid] = v;
+        rows[tid] = R > 0 ? (int)(v % R) : 0;        // ring row of the position
+    }
     if (last)
         for (int e = tid; e < ntok * k * k; e += nt) Hs[e] = hres[(long long)t0 * k * k + e];
     __syncthreads();
@@ -140,7 +145,7 @@ __global__ void __launch_bounds__(512) k_dec_post(Dims d, int slot, int B, int D
                 if (c < C) {
                     uu[0] = ldp(out + t * C + c);
                     float2 g[3];
-                    dec_conv<KW, PAPER>(d, cw, ring + t * R * C + c, c, uu[0], ps[tt], g);
+                    dec_conv<KW, PAPER>(d, cw, ring + t * R * C + c, c, uu[0], (int)min(ps[tt], (long long)KW), rows[tt], g);
 #pragma unroll
                     for (int j = 0; j < 3; ++j) {
                         uu[1 + j] = g[j];
@@ -257,7 +262,7 @@ __global__ void __launch_bounds__(512) k_dec_post(Dims d, int slot, int B, int D
                 uint16_t* dst = last ? X + (t * d.N + I[t * k + j]) * C + c : xact_next + (t * k + j) * C + c;
                 *reinterpret_cast<uint32_t*>(dst) = pack2(v.x, v.y);
             }
-            if (CONV && R > 0) *reinterpret_cast<uint32_t*>(ring + (t * R + (int)(ps[tt] % R)) * C + c) = raw;
+            if (CONV && R > 0) *reinterpret_cast<uint32_t*>(ring + (t * R + rows[tt]) * C + c) = raw;
         }
     }
     // the conv's CTAs have all read pos (before their last cluster barrier); without conv none but this one does
@@ -272,8 +277,11 @@ cudaError_t dec_post_kw(const Dims& d, int slot, int B, const uint16_t* out, Con
     const int ns = (d.C + DSL - 1) / DSL;
     const int q = (ns + DMAXC - 1) / DMAXC, nr = (ns + q - 1) / q;   // slices a CTA, CTAs a cluster
     const int nt = std::min(q, 4) * 128;
-    // about two CTAs per SM, and the components within 64 KB
-    int DT = std::min(DMAXT, std::max(1, (int)(((long long)B * nr + 2 * device_sms() - 1) / (2 * device_sms()))));
+    // as many tokens a cluster as fill the GPU once (1024 threads per SM: more clusters would wait for
+    // the 8 free CTA places of a GPC), and their components within 64 KB.  256 tokens of C = 4096: 4
+    // tokens a cluster; with 7 and half the threads resident it took 48 us, and three kernels 70.
+    const long long cap = (long long)(1024 / nt) * device_sms();
+    int DT = std::min(DMAXT, std::max(1, (int)(((long long)B * nr + cap - 1) / cap)));
     while (DT > 1 && CONV && DT * q * 3 * 128 * 8 > 64 * 1024) --DT;
     const DecSmem L(DT, q, ns, d.k, CONV);
     cudaError_t e = cudaFuncSetAttribute((const void*)k_dec_post<KM, KW, PAPER>,

@@ -268,46 +268,23 @@ cudaError_t launch_rowproj(const uint16_t* A, int64_t lda, int K, int T, const W
 }
 
 // ---------------------------------------------------------------------------------------------
-// colsum: partial column sums of in [rows][n] (n <= MAXN), a block per chunk of rows, eight threads a
-// column over interleaved rows (16 loads each in flight), then their sum in order
+// colsum: partial column sums of in [rows][n] (n <= MAXN), a block per chunk of rows
 
 __global__ void __launch_bounds__(8 * MAXN) k_colsum(const float* __restrict__ in, int rows, int n, int rchunk,
                                                      float* __restrict__ out) {
     __shared__ float sh[8 * MAXN];
-    const int o = threadIdx.x % n, ty = threadIdx.x / n;
-    const int r0 = blockIdx.x * rchunk, r1 = min(rows, r0 + rchunk);
-    float s = 0.f;
-    int r = r0 + ty;
-    for (; r + 120 < r1; r += 128) {
-        float v[16];
-#pragma unroll
-        for (int u = 0; u < 16; ++u) v[u] = in[(int64_t)(r + 8 * u) * n + o];
-#pragma unroll
-        for (int u = 0; u < 16; ++u) s += v[u];
-    }
-#pragma unroll 4
-    for (; r < r1; r += 8) s += in[(int64_t)r * n + o];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    if (ty == 0) {
-        float t = 0.f;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) t += sh[q * n + o];
-        out[blockIdx.x * n + o] = t;
-    }
+    colsum_chunk_of(in, rows, n, rchunk, blockIdx.x, sh, out);
 }
 
-// a single chunk up to 4096 rows; returns the number of partials
+// a single chunk up to 4096 rows
+int colsum_chunk(int rows) { return rows <= 4096 ? rows : (rows + COLSUM_PARTS - 1) / COLSUM_PARTS; }
 int colsum_parts(int rows) {
-    if (rows <= 4096) return 1;
-    const int rchunk = (rows + COLSUM_PARTS - 1) / COLSUM_PARTS;
+    const int rchunk = colsum_chunk(rows);
     return (rows + rchunk - 1) / rchunk;
 }
 
 cudaError_t launch_colsum(const float* in, int rows, int n, float* out, cudaStream_t st) {
-    const int parts = colsum_parts(rows);
-    const int rchunk = parts == 1 ? rows : (rows + COLSUM_PARTS - 1) / COLSUM_PARTS;
-    k_colsum<<<parts, 8 * n, 0, st>>>(in, rows, n, rchunk, out); note_launch();
+    k_colsum<<<colsum_parts(rows), 8 * n, 0, st>>>(in, rows, n, colsum_chunk(rows), out); note_launch();
     return cudaGetLastError();
 }
 

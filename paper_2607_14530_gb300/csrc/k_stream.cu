@@ -4,7 +4,7 @@
 //               paper's traffic model stores them), gather of the active streams (Alg. 1
 //               Gather), sum of squares of the gathered rows
 //   input       input_t = base_t + sum_j H_pre_t[I_j] x_act_j (Eq. app_active_state_correction),
-//               sum of squares of x_act
+//               sum of squares of x_act; the slot's active weight is packed by further blocks
 //   (the sums of squares are the norm statistics of the slot's active-state projection, which
 //   then reads its operand only through the tensor-core pipeline)
 //   restore     put the saved entry rows back into X before the backward
@@ -129,8 +129,12 @@ __global__ void __launch_bounds__(256) k_input(Dims d, int slot, int T,
                                                const float* __restrict__ hpre,
                                                const int* __restrict__ I,
                                                uint16_t* __restrict__ input,
-                                               float* __restrict__ astat) {
-    const int t = blockIdx.x, C = d.C, k = d.k;
+                                               float* __restrict__ astat, PackJob pack, int npack) {
+    if ((int)blockIdx.x < npack) {
+        pack_rows_of(pack, blockIdx.x);
+        return;
+    }
+    const int t = (int)blockIdx.x - npack, C = d.C, k = d.k;
     const int lane = threadIdx.x & 31;
     // the reads of this thread's first chunk (base row, k active rows) are issued before the
     // coefficients, which every warp fetches for itself (lanes j < k, then broadcast: no block
@@ -170,11 +174,13 @@ __global__ void __launch_bounds__(256) k_input(Dims d, int slot, int T,
 }
 
 cudaError_t launch_input(const Dims& d, int slot, int T, const uint16_t* base, const uint16_t* xact,
-                         const float* hpre, const int* I, uint16_t* input, float* astat, cudaStream_t st) {
+                         const float* hpre, const int* I, uint16_t* input, float* astat, const PackJob& pack,
+                         cudaStream_t st) {
+    const int np = pack_blocks(pack);
     if (d.k <= 4) {
-        k_input<4><<<T, chunk_threads(d.C), 0, st>>>(d, slot, T, base, xact, hpre, I, input, astat); note_launch();
+        k_input<4><<<T + np, chunk_threads(d.C), 0, st>>>(d, slot, T, base, xact, hpre, I, input, astat, pack, np); note_launch();
     } else {
-        k_input<8><<<T, chunk_threads(d.C), 0, st>>>(d, slot, T, base, xact, hpre, I, input, astat); note_launch();
+        k_input<8><<<T + np, chunk_threads(d.C), 0, st>>>(d, slot, T, base, xact, hpre, I, input, astat, pack, np); note_launch();
     }
     return cudaGetLastError();
 }

@@ -439,10 +439,19 @@ k_proj_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                 if (!last_sub) {
                     tmem_st16(tl + (uint32_t)(a.NB + o0), sum);
                 } else if (t < a.T) {
+                    // a row per lane: 16-byte stores where the rows allow them (4-byte ones touch a
+                    // sector per lane and value)
                     const int n = min(16, a.nfull - o0);
+                    if ((a.nfull & 3) == 0) {
 #pragma unroll
-                    for (int q = 0; q < 16; ++q)
-                        if (q < n) dst[o0 + q] = sum[q];
+                        for (int q = 0; q < 16; q += 4)
+                            if (q < n)
+                                *reinterpret_cast<float4*>(dst + o0 + q) = make_float4(sum[q], sum[q + 1], sum[q + 2], sum[q + 3]);
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < 16; ++q)
+                            if (q < n) dst[o0 + q] = sum[q];
+                    }
                 }
             }
             if (!last_sub) tmem_st_wait();
@@ -468,19 +477,77 @@ k_proj_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
 }
 
 // ---------------------------------------------------------------------------------------------
-// Wpack[r][e] = hi / lo bf16 parts of W[e][o] (r = o for hi, r = nfull + o for lo; 0 for pad)
+// The weight of the full-state projection packed (see PackJob), transposed through shared memory: a block
+// reads PF_E rows of every segment in memory order and writes the columns' hi and lo parts as 128-byte
+// runs.  (A thread per row, whose n columns it walked one after the other, took 17 us for the 65536 x 80
+// weight of N = 16, C = 4096; the bytes need 6.)  Further blocks take the column sums of W_r and the
+// slot's active weight, which nothing in this launch depends on.  (Every segment of the full-state weight
+// has N columns.)
 
-__global__ void k_pack_w(WSegs W, int nfull, int NB, int K, uint16_t* __restrict__ Wpack) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= K) return;
-    for (int o = 0; o < nfull; ++o) {
-        const float w = seg_elem(W, e, o);
-        const __nv_bfloat16 h = __float2bfloat16_rn(w);
-        const float rem = w - __bfloat162float(h);
-        Wpack[(int64_t)o * K + e] = __bfloat16_as_ushort(h);
-        Wpack[(int64_t)(nfull + o) * K + e] = __bfloat16_as_ushort(__float2bfloat16_rn(rem));
+constexpr int PF_E = 64;
+constexpr int PF_NT = 256;
+
+__global__ void __launch_bounds__(PF_NT) k_pack_full(PackJob j, int nblk, const float* __restrict__ Wr, int N,
+                                                     int rchunk, int nparts, float* __restrict__ wsump, PackJob act) {
+    extern __shared__ float sm[];   // [n][PF_E + 1]
+    const int tid = threadIdx.x;
+    int blk = blockIdx.x;
+    if (blk < nparts) {             // the longest chains first
+        colsum_chunk_of(Wr, j.K, N, rchunk, blk, sm, wsump);
+        return;
     }
-    for (int r = 2 * nfull; r < NB; ++r) Wpack[(int64_t)r * K + e] = 0;
+    blk -= nparts;
+    if (blk >= nblk) {
+        pack_rows_of(act, blk - nblk);
+        return;
+    }
+    const int e0 = blk * PF_E, ne = min(PF_E, j.K - e0);
+    // ne rows of N columns of every segment, each contiguous in memory; idx / N for idx < 64 * 32 by a
+    // product with the reciprocal (rounded up, exact there)
+    const int64_t at = (int64_t)e0 * N;
+    const uint32_t rec = (65536u + N - 1) / N;
+    bool v4 = (N & 3) == 0;
+#pragma unroll
+    for (int q = 0; q < MAXSEG; ++q) v4 = v4 && (q >= j.W.n || ((uintptr_t)j.W.ptr[q] & 15u) == 0);
+    if (v4) {
+        for (int i4 = tid; i4 < ne * N / 4; i4 += PF_NT) {
+            float4 v[MAXSEG];   // the segments' loads in flight together
+#pragma unroll
+            for (int q = 0; q < MAXSEG; ++q)
+                if (q < j.W.n) v[q] = __ldg(reinterpret_cast<const float4*>(j.W.ptr[q] + at) + i4);
+            const int e = (int)((uint32_t)(4 * i4) * rec >> 16), o = 4 * i4 - e * N;
+#pragma unroll
+            for (int q = 0; q < MAXSEG; ++q) {
+                if (q >= j.W.n) continue;
+                float* d = sm + (q * N + o) * (PF_E + 1) + e;
+                d[0] = v[q].x;
+                d[PF_E + 1] = v[q].y;
+                d[2 * (PF_E + 1)] = v[q].z;
+                d[3 * (PF_E + 1)] = v[q].w;
+            }
+        }
+    } else {
+        for (int idx = tid; idx < ne * N; idx += PF_NT) {
+            const int e = (int)((uint32_t)idx * rec >> 16), o = idx - e * N;
+#pragma unroll
+            for (int q = 0; q < MAXSEG; ++q)
+                if (q < j.W.n) sm[(q * N + o) * (PF_E + 1) + e] = __ldg(j.W.ptr[q] + at + idx);
+        }
+    }
+    __syncthreads();
+    // K is a multiple of 8, so pairs of rows stay whole
+    for (int idx = tid; idx < j.NB * (PF_E / 2); idx += PF_NT) {
+        const int r = idx / (PF_E / 2), e = 2 * (idx - r * (PF_E / 2));
+        if (e >= ne) continue;
+        uint32_t v = 0u;
+        if (r < 2 * j.n) {
+            const int o = r < j.n ? r : r - j.n;
+            const float a = sm[o * (PF_E + 1) + e], b = sm[o * (PF_E + 1) + e + 1];
+            v = pack2(a, b);
+            if (r >= j.n) v = pack2(a - __uint_as_float(v << 16), b - __uint_as_float(v & 0xffff0000u));
+        }
+        *reinterpret_cast<uint32_t*>(j.dst + (int64_t)r * j.K + e0 + e) = v;
+    }
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
@@ -572,8 +639,12 @@ size_t proj_tc_smem(const ProjTcPlan& p) {
     return (size_t)S * p.kps * (BM * BK * 2 + (size_t)p.NB * BK * 2) + (2 * S + 2) * 8 + 16 + 1024;
 }
 
-cudaError_t launch_pack_w(const WSegs& W, int nfull, int NB, int K, uint16_t* Wpack, cudaStream_t st) {
-    k_pack_w<<<(K + 255) / 256, 256, 0, st>>>(W, nfull, NB, K, Wpack); note_launch();
+cudaError_t launch_pack_full(const PackJob& full, const float* W_r, int N, float* wsump, const PackJob& act,
+                             cudaStream_t st) {
+    const int nblk = (full.K + PF_E - 1) / PF_E, nparts = W_r ? colsum_parts(full.K) : 0;
+    const size_t sm = sizeof(float) * std::max(full.n * (PF_E + 1), 8 * MAXN);
+    k_pack_full<<<nblk + nparts + pack_blocks(act), PF_NT, sm, st>>>(full, nblk, W_r, N, colsum_chunk(full.K), nparts,
+                                                                     wsump, act); note_launch();
     return cudaGetLastError();
 }
 

@@ -94,6 +94,7 @@ struct Layout {
     // workspace
     size_t err;             // int: device error word (first 256 bytes of the workspace)
     size_t wpack;           // bf16 [NB][N*C]: hi / lo rows of the full-state projection weight
+    size_t wpacka;          // bf16 [NB][k*C]: hi / lo rows of a slot's active-state projection weight
     size_t part;            // f32 [splits][T][nmax] projection split-K partials
     size_t pstats;          // f32 [splits][T][2]
     size_t astat;           // f32 [stream_warps(C)][T][2]: per-warp partial sums of squares (at 1;
@@ -338,7 +339,34 @@ int debug_take_force_timeout();
 constexpr int ROWPROJ_SMALL = 128;   // fewer tokens than this: the kernel for few tokens
 cudaError_t launch_rowproj(const uint16_t* A, int64_t lda, int K, int T, const WSegs& W, int n,
                            int* nslots, float* part, float* pstats, cudaStream_t st);
-cudaError_t launch_pack_w(const WSegs& W, int nfull, int NB, int K, uint16_t* Wpack, cudaStream_t st);
+// One weight packed for k_proj_tc: rows 0..n-1 of dst [NB][K] the bf16 hi parts of W[e][o], rows
+// n..2n-1 the lo parts, the rest zero.
+struct PackJob {
+    WSegs W;
+    int n, NB, K;
+    uint16_t* dst;   // null: nothing to pack
+};
+constexpr int PACK_E = 256;   // rows of the weight per block of pack_rows_of
+// A block's share of a pack job, a thread per weight row (its n columns are whole sectors, the stores are
+// contiguous over the threads): for the small weights of the active-state projections, which ride
+// along with a kernel that does not depend on them.
+__device__ __forceinline__ void pack_rows_of(const PackJob& j, int blk) {
+    for (int e = blk * PACK_E + threadIdx.x; e < min(j.K, (blk + 1) * PACK_E); e += blockDim.x) {
+#pragma unroll 4
+        for (int o = 0; o < j.n; ++o) {
+            const float w = seg_elem<true>(j.W, e, o);
+            const __nv_bfloat16 h = __float2bfloat16_rn(w);
+            j.dst[(int64_t)o * j.K + e] = __bfloat16_as_ushort(h);
+            j.dst[(int64_t)(j.n + o) * j.K + e] = __bfloat16_as_ushort(__float2bfloat16_rn(w - __bfloat162float(h)));
+        }
+        for (int r = 2 * j.n; r < j.NB; ++r) j.dst[(int64_t)r * j.K + e] = 0;
+    }
+}
+inline int pack_blocks(const PackJob& j) { return j.dst ? (j.K + PACK_E - 1) / PACK_E : 0; }
+// the full-state weight packed, the partial column sums of W_r (null: none) and the slot-0 active weight,
+// in one launch
+cudaError_t launch_pack_full(const PackJob& full, const float* W_r, int N, float* wsump, const PackJob& act,
+                             cudaStream_t st);
 // pstats null: no row statistics (the caller has them from the kernel that wrote X)
 cudaError_t launch_proj_tc(const uint16_t* X, int T, int K, const uint16_t* Wpack, int nfull,
                            const ProjTcPlan& p, float* part, float* pstats, int* err,
@@ -407,6 +435,36 @@ cudaError_t launch_wgrad_reduce(const float* wpart, const SlotPlan& sp, int E, i
 // partial column sums of in [rows][n]: out [colsum_parts(rows)][n], part q over the rows of chunk q
 constexpr int COLSUM_PARTS = 64;   // at most
 int colsum_parts(int rows);
+int colsum_chunk(int rows);        // rows of a chunk
+// chunk `part`, by the first 8 n threads of a block (n <= MAXN): eight threads a column over interleaved
+// rows (U loads each in flight), then their sum in order.  sh: 8 n floats.  Has block barriers.
+__device__ __forceinline__ void colsum_chunk_of(const float* __restrict__ in, int rows, int n, int rchunk, int part,
+                                                float* sh, float* __restrict__ out) {
+    constexpr int U = 32;
+    const int o = threadIdx.x % n, ty = threadIdx.x / n;
+    const int r0 = part * rchunk, r1 = min(rows, r0 + rchunk);
+    if (ty < 8) {
+        float s = 0.f;
+        int r = r0 + ty;
+        for (; r + 8 * (U - 1) < r1; r += 8 * U) {
+            float v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) v[u] = in[(int64_t)(r + 8 * u) * n + o];
+#pragma unroll
+            for (int u = 0; u < U; ++u) s += v[u];
+        }
+#pragma unroll 4
+        for (; r < r1; r += 8) s += in[(int64_t)r * n + o];
+        sh[threadIdx.x] = s;
+    }
+    __syncthreads();
+    if (ty == 0) {
+        float t = 0.f;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) t += sh[q * n + o];
+        out[part * n + o] = t;
+    }
+}
 cudaError_t launch_colsum(const float* in, int rows, int n, float* out, cudaStream_t st);
 // wsum: [nws][N] partial column sums of W_r; their sum is left in wsum_out [N]
 cudaError_t launch_coef_full(const Dims& d, int T, const float* part, const float* pstats,
@@ -420,8 +478,10 @@ cudaError_t launch_coef_act(const Dims& d, int slot, int T, const float* part,
 int stream_warps(int C);  // warps per block of the one-block-per-token stream kernels
 cudaError_t launch_read(const Dims& d, int T, const uint16_t* X, const float* hpre, const int* I,
                         uint16_t* input0, uint16_t* base, uint16_t* xact0, float* astat, cudaStream_t st);
+// pack: the slot's active weight, packed by further blocks of the same launch
 cudaError_t launch_input(const Dims& d, int slot, int T, const uint16_t* base, const uint16_t* xact,
-                         const float* hpre, const int* I, uint16_t* input, float* astat, cudaStream_t st);
+                         const float* hpre, const int* I, uint16_t* input, float* astat, const PackJob& pack,
+                         cudaStream_t st);
 cudaError_t launch_restore(const Dims& d, int T, const uint16_t* xact0, const int* I,
                            uint16_t* X, cudaStream_t st);
 cudaError_t launch_bwd_coef(const Dims& d, int slot, int T, const float* red, int nslice,
