@@ -16,6 +16,16 @@ namespace xhc {
 static std::atomic<unsigned long long> g_launches{0};
 void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
+// ---- programmatic launches ------------------------------------------------------------------
+static thread_local bool t_pdl = false;
+bool pdl_on() { return t_pdl; }
+void PdlScope::set(size_t state_bytes, cudaStream_t st) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    t_pdl = state_bytes <= ((size_t)256 << 20) && cudaStreamIsCapturing(st, &cap) == cudaSuccess &&
+            cap == cudaStreamCaptureStatusNone;
+}
+PdlScope::~PdlScope() { t_pdl = false; }
+
 // ---- test hooks -----------------------------------------------------------------------------
 static std::atomic<unsigned long long> g_wait_ns{0};   // 0: the default limit (~4 s)
 static std::atomic<int> g_force_timeout{0};
@@ -462,6 +472,7 @@ static xhc_status join_into(cudaStream_t main, cudaStream_t side) {
 }
 
 struct Ctx {
+    PdlScope pdl;
     Dims d;
     Layout L;
     int T;
@@ -492,6 +503,7 @@ xhc_status common_check(const xhc_handle* h, int slot, int64_t T, const void* sa
     cx.sv = (char*)saved;
     cx.ws = (char*)ws;
     cx.st = (cudaStream_t)stream;
+    cx.pdl.set((size_t)T * d0.N * d0.C * 2, cx.st);
     return XHC_OK;
 }
 

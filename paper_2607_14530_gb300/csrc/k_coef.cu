@@ -193,6 +193,7 @@ __global__ void __launch_bounds__(CF_NT) k_coef_full(Dims d, int T, int TB, cons
                                                      float* __restrict__ stats, float* __restrict__ wsum_out,
                                                      float* __restrict__ hpre, int* __restrict__ I,
                                                      float* __restrict__ p) {
+    pdl_entry();
     extern __shared__ float sm[];   // [TB][n] projections, [TB][2] statistics
     __shared__ float scr[CF_NT], scw[8 * MAXN], ws[MAXN], stage[SS_STAGE];
     const int tid = threadIdx.x, lane = tid & 31, N = d.N, n = d.nfull;
@@ -289,6 +290,7 @@ __global__ void __launch_bounds__(CF_NT) k_coef_act(Dims d, int slot, int T, int
                                                     const float* __restrict__ b_res, float* __restrict__ zact,
                                                     float* __restrict__ rs, float* __restrict__ hpost,
                                                     float* __restrict__ hres) {
+    pdl_entry();
     extern __shared__ float sm[];   // [TB][n] projections, [TB] sums of squares
     __shared__ float scr[CF_NT], stage[SS_STAGE];
     const int tid = threadIdx.x, k = d.k, kK = d.k * d.K[slot], n = d.nact[slot];
@@ -350,8 +352,7 @@ cudaError_t launch_coef_full(const Dims& d, int T, const float* part, const floa
                              int* I, float* p, cudaStream_t st) {
     const int TB = coef_tokens(T);
     const size_t sm = (size_t)TB * (d.nfull + 2) * 4;
-    k_coef_full<<<(T + TB - 1) / TB, CF_NT, sm, st>>>(d, T, TB, part, pstats, sp, wsum, nws, alpha_pre, b_pre,
-                                                      zfull, stats, wsum_out, hpre, I, p); note_launch();
+    XHC_LAUNCH(st, (T + TB - 1) / TB, CF_NT, sm, (k_coef_full), d, T, TB, part, pstats, sp, wsum, nws, alpha_pre, b_pre, zfull, stats, wsum_out, hpre, I, p);
     return cudaGetLastError();
 }
 
@@ -363,11 +364,9 @@ cudaError_t launch_coef_act(const Dims& d, int slot, int T, const float* part,
     const size_t sm = (size_t)TB * (d.nact[slot] + 1) * 4;
     const unsigned grid = (unsigned)((T + TB - 1) / TB);
     if (d.k <= 4) {
-        k_coef_act<4><<<grid, CF_NT, sm, st>>>(d, slot, T, TB, part, pstats, ssplits, sp, alpha_post, b_post,
-                                               alpha_res, b_res, zact, rs, hpost, hres); note_launch();
+        XHC_LAUNCH(st, grid, CF_NT, sm, (k_coef_act<4>), d, slot, T, TB, part, pstats, ssplits, sp, alpha_post, b_post, alpha_res, b_res, zact, rs, hpost, hres);
     } else {
-        k_coef_act<8><<<grid, CF_NT, sm, st>>>(d, slot, T, TB, part, pstats, ssplits, sp, alpha_post, b_post,
-                                               alpha_res, b_res, zact, rs, hpost, hres); note_launch();
+        XHC_LAUNCH(st, grid, CF_NT, sm, (k_coef_act<8>), d, slot, T, TB, part, pstats, ssplits, sp, alpha_post, b_post, alpha_res, b_res, zact, rs, hpost, hres);
     }
     return cudaGetLastError();
 }
@@ -466,6 +465,7 @@ __global__ void __launch_bounds__(160) k_bwd_coef(Dims d, int slot, int T, int T
                                                   const float* __restrict__ b_res, float* __restrict__ tokmat,
                                                   float* __restrict__ dzs, float* __restrict__ dp,
                                                   float* __restrict__ colp) {
+    pdl_entry();
     using L = BwdTok<KM>;
     extern __shared__ float sm[];   // [TB][ROW], then the Sinkhorn iterates
     const int tid = threadIdx.x, lane = tid & 31, nt = blockDim.x;
@@ -667,9 +667,7 @@ cudaError_t bwd_coef_km(const Dims& d, int slot, int T, const float* red, int ns
         cudaFuncSetAttribute((const void*)k_bwd_coef<KM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     *nblk = (T + TB - 1) / TB;
-    k_bwd_coef<KM><<<*nblk, 32 + TB * KM, sm, st>>>(d, slot, T, TB, red, nslice, zact, rs, p, hpost, gram,
-                                                   alpha_post, alpha_res, b_res, tokmat, dz, dp, colp);
-    note_launch();
+    XHC_LAUNCH(st, *nblk, 32 + TB * KM, sm, (k_bwd_coef<KM>), d, slot, T, TB, red, nslice, zact, rs, p, hpost, gram, alpha_post, alpha_res, b_res, tokmat, dz, dp, colp);
     return cudaGetLastError();
 }
 
@@ -707,6 +705,7 @@ __global__ void __launch_bounds__(FC_NT) k_full_coef(Dims d, int T, int TB, cons
                                                      const float* __restrict__ dp,
                                                      const float* __restrict__ alpha_pre, float* __restrict__ dz,
                                                      float* __restrict__ scal, float* __restrict__ colp) {
+    pdl_entry();
     __shared__ float sh[FC_NT / 32][NCOLP];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int N = d.N, GN = d.G * d.N, n = d.nfull, roff = d.hr ? N : 0;
@@ -831,8 +830,7 @@ cudaError_t launch_full_coef(const Dims& d, int T, const float* dhpre, const flo
     // 8 tokens a block (a token per warp) at few tokens, 32 at many
     const int TB = (T >= 32 * 2 * device_sms()) ? 32 : 8;
     *nblk = (T + TB - 1) / TB;
-    k_full_coef<<<*nblk, FC_NT, 0, st>>>(d, T, TB, dhpre, hpre, zfull, stats, wsum, I, dp, alpha_pre, dz, scal,
-                                         colp); note_launch();
+    XHC_LAUNCH(st, *nblk, FC_NT, 0, (k_full_coef), d, T, TB, dhpre, hpre, zfull, stats, wsum, I, dp, alpha_pre, dz, scal, colp);
     return cudaGetLastError();
 }
 
@@ -842,6 +840,7 @@ cudaError_t launch_full_coef(const Dims& d, int T, const float* dhpre, const flo
 namespace {
 
 __global__ void __launch_bounds__(128) k_colsum_out(const float* __restrict__ colp, int nblk, int ncol, ColOut out) {
+    pdl_entry();
     __shared__ float sh[4];
     int o = blockIdx.x;
     // the target of output o, selected with static indices
@@ -875,7 +874,7 @@ __global__ void __launch_bounds__(128) k_colsum_out(const float* __restrict__ co
 cudaError_t launch_colsum_out(const float* colp, int nblk, int ncol, const ColOut& out, cudaStream_t st) {
     int n = 0;
     for (int q = 0; q < 4; ++q) n += out.n[q];
-    k_colsum_out<<<n, 128, 0, st>>>(colp, nblk, ncol, out); note_launch();
+    XHC_LAUNCH(st, n, 128, 0, (k_colsum_out), colp, nblk, ncol, out);
     return cudaGetLastError();
 }
 
@@ -887,6 +886,7 @@ namespace {
 
 __global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ wpart, SlotPlan sp, int E, int n,
                                                       WSegsOut G, const float* __restrict__ sub) {
+    pdl_entry();
     const int e0 = blockIdx.y * 128, ne = min(128, E - e0) * n;
     const int nsl = slot_count(sp, blockIdx.y);
     for (int idx = blockIdx.x * 256 + threadIdx.x; idx < ne; idx += gridDim.x * 256) {
@@ -914,7 +914,7 @@ cudaError_t launch_wgrad_reduce(const float* wpart, const SlotPlan& sp, int E, i
     // a few elements a thread where there are many tiles (the slot count costs a division)
     const int tiles = (E + 127) / 128, per = (128 * n + 255) / 256;
     const dim3 grid((unsigned)std::max(1, tiles >= 256 ? per / 8 : per), (unsigned)tiles);
-    k_wgrad_reduce<<<grid, 256, 0, st>>>(wpart, sp, E, n, G, sub); note_launch();
+    XHC_LAUNCH(st, grid, 256, 0, (k_wgrad_reduce), wpart, sp, E, n, G, sub);
     return cudaGetLastError();
 }
 

@@ -104,6 +104,7 @@ __global__ void __launch_bounds__(512, 2) k_dec_post(Dims d, int slot, int B, in
                                                   double* __restrict__ gram, const uint16_t* __restrict__ xact,
                                                   const int* __restrict__ I, const float* __restrict__ hres,
                                                   uint16_t* __restrict__ xact_next, uint16_t* __restrict__ X) {
+    pdl_entry();
     constexpr bool CONV = KW > 0;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ long long ps[DMAXT];
@@ -292,13 +293,15 @@ cudaError_t dec_post_kw(const Dims& d, int slot, int B, const uint16_t* out, Con
     cfg.blockDim = dim3((unsigned)nt);
     cfg.dynamicSmemBytes = (size_t)L.bytes;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 1;
     at[0].val.clusterDim.y = CONV ? (unsigned)nr : 1u;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = pdl_on() ? 2 : 1;
     e = cudaLaunchKernelEx(&cfg, k_dec_post<KM, KW, PAPER>, d, slot, B, DT, q, ns, out, cw, ring, pos, p, hpost, gram,
                            xact, I, hres, xact_next, X);
     note_launch();
@@ -322,6 +325,7 @@ cudaError_t dec_post_km(const Dims& d, int slot, int B, const uint16_t* out, Con
 // last min(S, R) rows in ring rows (s mod R)
 __global__ void k_ring_fill(const uint16_t* __restrict__ out, int B, int S, int C, int R,
                             uint16_t* __restrict__ ring) {
+    pdl_entry();
     const long long n = (long long)B * R * (C / 8);
     for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -340,6 +344,7 @@ __global__ void k_ring_fill(const uint16_t* __restrict__ out, int B, int S, int 
 // S - R + r of sequence b (zero where that position is before the sequence start)
 __global__ void k_halo_fill(const uint16_t* __restrict__ out, int B, int S, int C, int R,
                             uint16_t* __restrict__ halo) {
+    pdl_entry();
     const long long n = (long long)B * R * (C / 8);
     for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -358,6 +363,7 @@ __global__ void k_halo_fill(const uint16_t* __restrict__ out, int B, int S, int 
 // position S - R + r of sequence b += d_halo[b][r] (in fp32, one bf16 rounding)
 __global__ void k_halo_add(uint16_t* __restrict__ d_out, int B, int S, int C, int R,
                            const float* __restrict__ dhalo) {
+    pdl_entry();
     const long long n = (long long)B * R * (C / 2);
     for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -391,7 +397,7 @@ cudaError_t launch_ring_fill(const Dims& d, int B, int S, const uint16_t* out, u
     if (R <= 0) return cudaSuccess;
     const long long n = (long long)B * R * (d.C / 8);
     const int blocks = (int)std::min<long long>((n + 255) / 256, 4096);
-    k_ring_fill<<<blocks, 256, 0, st>>>(out, B, S, d.C, R, ring); note_launch();
+    XHC_LAUNCH(st, blocks, 256, 0, (k_ring_fill), out, B, S, d.C, R, ring);
     return cudaGetLastError();
 }
 
@@ -401,7 +407,7 @@ cudaError_t launch_halo_fill(const Dims& d, int B, int S, const uint16_t* out, u
     if (R <= 0) return cudaSuccess;
     const long long n = (long long)B * R * (d.C / 8);
     const int blocks = (int)std::min<long long>((n + 255) / 256, 4096);
-    k_halo_fill<<<blocks, 256, 0, st>>>(out, B, S, d.C, R, halo); note_launch();
+    XHC_LAUNCH(st, blocks, 256, 0, (k_halo_fill), out, B, S, d.C, R, halo);
     return cudaGetLastError();
 }
 
@@ -411,7 +417,7 @@ cudaError_t launch_halo_add(const Dims& d, int B, int S, uint16_t* d_out, const 
     if (R <= 0) return cudaSuccess;
     const long long n = (long long)B * R * (d.C / 2);
     const int blocks = (int)std::min<long long>((n + 255) / 256, 4096);
-    k_halo_add<<<blocks, 256, 0, st>>>(d_out, B, S, d.C, R, dhalo); note_launch();
+    XHC_LAUNCH(st, blocks, 256, 0, (k_halo_add), d_out, B, S, d.C, R, dhalo);
     return cudaGetLastError();
 }
 

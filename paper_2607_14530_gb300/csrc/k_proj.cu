@@ -20,6 +20,7 @@ __global__ void __launch_bounds__(256) k_rowproj(const uint16_t* __restrict__ A,
                                                  int T, WSegs W, int n, int kchunk,
                                                  float* __restrict__ part,
                                                  float* __restrict__ pstats) {
+    pdl_entry();
     constexpr int BM = 64, BK = 32, NP = 16 * NT;
     __shared__ __align__(16) float As[BK][BM + 4];
     __shared__ __align__(16) float Ws[BK][NP];
@@ -101,7 +102,7 @@ static cudaError_t rowproj_nt(const uint16_t* A, int64_t lda, int K, int T, cons
                               int splits, float* part, float* pstats, cudaStream_t st) {
     const int kchunk = ((K + splits - 1) / splits + 31) / 32 * 32;
     dim3 grid((T + 63) / 64, splits);
-    k_rowproj<NT><<<grid, 256, 0, st>>>(A, lda, K, T, W, n, kchunk, part, pstats); note_launch();
+    XHC_LAUNCH(st, grid, 256, 0, (k_rowproj<NT>), A, lda, K, T, W, n, kchunk, part, pstats);
     return cudaGetLastError();
 }
 
@@ -118,6 +119,7 @@ template <int TT, int V>
 __global__ void __launch_bounds__(RS_NT) k_rowproj_small(const uint16_t* __restrict__ A, int64_t lda, int K, int T,
                                                          WSegs W, int n, int kchunk, float* __restrict__ part,
                                                          float* __restrict__ pstats) {
+    pdl_entry();
     constexpr int TP = (TT + 1) / 2;                 // token pairs
     extern __shared__ __align__(16) float sm[];      // [RS_ROWS][2 TP] state rows; then [row lanes][n][TT]
     __shared__ float stat[TT][2];
@@ -233,7 +235,7 @@ static cudaError_t rowproj_small(const uint16_t* A, int64_t lda, int K, int T, c
     const cudaError_t e = cudaFuncSetAttribute((const void*)k_rowproj_small<TT, V>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k_rowproj_small<TT, V><<<dim3(s, ny), RS_NT, sm, st>>>(A, lda, K, T, W, n, kchunk, part, pstats); note_launch();
+    XHC_LAUNCH(st, dim3(s, ny), RS_NT, sm, (k_rowproj_small<TT, V>), A, lda, K, T, W, n, kchunk, part, pstats);
     return cudaGetLastError();
 }
 
@@ -272,6 +274,7 @@ cudaError_t launch_rowproj(const uint16_t* A, int64_t lda, int K, int T, const W
 
 __global__ void __launch_bounds__(8 * MAXN) k_colsum(const float* __restrict__ in, int rows, int n, int rchunk,
                                                      float* __restrict__ out) {
+    pdl_entry();
     __shared__ float sh[8 * MAXN];
     colsum_chunk_of(in, rows, n, rchunk, blockIdx.x, sh, out);
 }
@@ -284,7 +287,7 @@ int colsum_parts(int rows) {
 }
 
 cudaError_t launch_colsum(const float* in, int rows, int n, float* out, cudaStream_t st) {
-    k_colsum<<<colsum_parts(rows), 8 * n, 0, st>>>(in, rows, n, colsum_chunk(rows), out); note_launch();
+    XHC_LAUNCH(st, colsum_parts(rows), 8 * n, 0, (k_colsum), in, rows, n, colsum_chunk(rows), out);
     return cudaGetLastError();
 }
 
@@ -294,6 +297,7 @@ cudaError_t launch_colsum(const float* in, int rows, int n, float* out, cudaStre
 __global__ void __launch_bounds__(256) k_gemm_dzw(const float* __restrict__ dz, int ldz, int n,
                                                   WSegs W, int E, int T,
                                                   float* __restrict__ out) {
+    pdl_entry();
     constexpr int BT = 64, BE = 64, BO = 32;
     __shared__ __align__(16) float Ds[BO][BT + 4];
     __shared__ __align__(16) float Wt[BO][BE + 4];
@@ -349,7 +353,7 @@ cudaError_t launch_gemm_dzw(const Dims& d, int T, const float* dz, int ldz, int 
                             const WSegs& W, int E, float* dxact, cudaStream_t st) {
     (void)d;
     dim3 grid((E + 63) / 64, (T + 63) / 64);
-    k_gemm_dzw<<<grid, 256, 0, st>>>(dz, ldz, n, W, E, T, dxact); note_launch();
+    XHC_LAUNCH(st, grid, 256, 0, (k_gemm_dzw), dz, ldz, n, W, E, T, dxact);
     return cudaGetLastError();
 }
 
@@ -367,6 +371,7 @@ __global__ void __launch_bounds__(256) k_full_dx(Dims d, int T, const float* __r
                                                  const float* __restrict__ dxact,
                                                  const float* __restrict__ scal,
                                                  uint16_t* __restrict__ dX) {
+    pdl_entry();
     constexpr int BT = 64, BE = 64, BO = 32;
     __shared__ __align__(16) float Ds[BO][BT + 4];
     __shared__ __align__(16) float Wt[BO][BE + 4];
@@ -449,7 +454,7 @@ cudaError_t launch_full_dx(const Dims& d, int T, const float* dz, const WSegs& W
                            cudaStream_t st) {
     const int E = d.N * d.C;
     dim3 grid((E + 63) / 64, (T + 63) / 64);
-    k_full_dx<<<grid, 256, 0, st>>>(d, T, dz, W, X, dinput, hpre, I, dxact, scal, dX); note_launch();
+    XHC_LAUNCH(st, grid, 256, 0, (k_full_dx), d, T, dz, W, X, dinput, hpre, I, dxact, scal, dX);
     return cudaGetLastError();
 }
 
@@ -460,6 +465,7 @@ template <int NT>
 __global__ void __launch_bounds__(256) k_wgrad(const uint16_t* __restrict__ A, int64_t lda, int E,
                                                int T, const float* __restrict__ dz, int ldz, int n,
                                                int tchunk, float* __restrict__ wpart) {
+    pdl_entry();
     constexpr int BE = 64, BT = 32, NP = 16 * NT;
     __shared__ __align__(16) float As[BT][BE + 4];
     __shared__ __align__(16) float Ds[BT][NP];
@@ -526,7 +532,7 @@ static cudaError_t wgrad_nt(const uint16_t* A, int64_t lda, int E, int T, const 
     const int tchunk = ((T + tsplits - 1) / tsplits + 31) / 32 * 32;
     const int splits = (T + tchunk - 1) / tchunk;
     dim3 grid((E + 63) / 64, splits);
-    k_wgrad<NT><<<grid, 256, 0, st>>>(A, lda, E, T, dz, ldz, n, tchunk, wpart); note_launch();
+    XHC_LAUNCH(st, grid, 256, 0, (k_wgrad<NT>), A, lda, E, T, dz, ldz, n, tchunk, wpart);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_wgrad_reduce(wpart, slots_of(splits), E, n, G, sub, st);

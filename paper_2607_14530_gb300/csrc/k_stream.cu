@@ -41,6 +41,7 @@ __global__ void __launch_bounds__(256, 3) k_read(Dims d, int T, const uint16_t* 
                                               uint16_t* __restrict__ base,
                                               uint16_t* __restrict__ xact0,
                                               float* __restrict__ astat) {
+    pdl_entry();
     __shared__ float sh[4 * MAXN];
     __shared__ int slotmap[MAXN];
     const int t = blockIdx.x;
@@ -115,7 +116,7 @@ __global__ void __launch_bounds__(256, 3) k_read(Dims d, int T, const uint16_t* 
 
 cudaError_t launch_read(const Dims& d, int T, const uint16_t* X, const float* hpre, const int* I,
                         uint16_t* input0, uint16_t* base, uint16_t* xact0, float* astat, cudaStream_t st) {
-    k_read<<<T, chunk_threads(d.C), 0, st>>>(d, T, X, hpre, I, input0, base, xact0, astat); note_launch();
+    XHC_LAUNCH(st, T, chunk_threads(d.C), 0, (k_read), d, T, X, hpre, I, input0, base, xact0, astat);
     return cudaGetLastError();
 }
 
@@ -130,6 +131,7 @@ __global__ void __launch_bounds__(256) k_input(Dims d, int slot, int T,
                                                const int* __restrict__ I,
                                                uint16_t* __restrict__ input,
                                                float* __restrict__ astat, PackJob pack, int npack) {
+    pdl_entry();
     if ((int)blockIdx.x < npack) {
         pack_rows_of(pack, blockIdx.x);
         return;
@@ -178,9 +180,9 @@ cudaError_t launch_input(const Dims& d, int slot, int T, const uint16_t* base, c
                          cudaStream_t st) {
     const int np = pack_blocks(pack);
     if (d.k <= 4) {
-        k_input<4><<<T + np, chunk_threads(d.C), 0, st>>>(d, slot, T, base, xact, hpre, I, input, astat, pack, np); note_launch();
+        XHC_LAUNCH(st, T + np, chunk_threads(d.C), 0, (k_input<4>), d, slot, T, base, xact, hpre, I, input, astat, pack, np);
     } else {
-        k_input<8><<<T + np, chunk_threads(d.C), 0, st>>>(d, slot, T, base, xact, hpre, I, input, astat, pack, np); note_launch();
+        XHC_LAUNCH(st, T + np, chunk_threads(d.C), 0, (k_input<8>), d, slot, T, base, xact, hpre, I, input, astat, pack, np);
     }
     return cudaGetLastError();
 }
@@ -191,6 +193,7 @@ cudaError_t launch_input(const Dims& d, int slot, int T, const uint16_t* base, c
 __global__ void __launch_bounds__(256) k_restore(Dims d, int T, const uint16_t* __restrict__ xact0,
                                                  const int* __restrict__ I,
                                                  uint16_t* __restrict__ X) {
+    pdl_entry();
     const int t = blockIdx.x, C = d.C;
     const int n8 = C / 8;
     for (int idx = threadIdx.x; idx < d.k * n8; idx += blockDim.x) {
@@ -203,7 +206,7 @@ __global__ void __launch_bounds__(256) k_restore(Dims d, int T, const uint16_t* 
 
 cudaError_t launch_restore(const Dims& d, int T, const uint16_t* xact0, const int* I,
                            uint16_t* X, cudaStream_t st) {
-    k_restore<<<T, 256, 0, st>>>(d, T, xact0, I, X); note_launch();
+    XHC_LAUNCH(st, T, 256, 0, (k_restore), d, T, xact0, I, X);
     return cudaGetLastError();
 }
 
@@ -212,6 +215,7 @@ cudaError_t launch_restore(const Dims& d, int T, const uint16_t* xact0, const in
 
 __global__ void k_conv_wgrad_reduce(Dims d, const float* __restrict__ cpart, int ntiles,
                                     ConvGradPtrs g) {
+    pdl_entry();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= d.kapsum * d.C) return;
     const int q = idx / d.C, c = idx - q * d.C;
@@ -240,7 +244,7 @@ cudaError_t launch_conv_wgrad_reduce(const Dims& d, int slot, const float* cpart
                                      ConvGradPtrs gconv, cudaStream_t st) {
     (void)slot;
     const int n = d.kapsum * d.C;
-    k_conv_wgrad_reduce<<<(n + 255) / 256, 256, 0, st>>>(d, cpart, ntiles, gconv); note_launch();
+    XHC_LAUNCH(st, (n + 255) / 256, 256, 0, (k_conv_wgrad_reduce), d, cpart, ntiles, gconv);
     return cudaGetLastError();
 }
 
@@ -258,6 +262,7 @@ __global__ void __launch_bounds__(256) k_dinput_act(Dims d, int slot, int T, int
                                                     float* __restrict__ dhpre,
                                                     uint16_t* __restrict__ dcopy,
                                                     const float* __restrict__ tokmat) {
+    pdl_entry();
     __shared__ float hj[KM];
     __shared__ float wsh[8][KM];
     const int t = blockIdx.x, C = d.C, k = d.k;
@@ -314,11 +319,9 @@ cudaError_t launch_dinput_act(const Dims& d, int slot, int T, int add_dx, const 
                               float* dhpre, uint16_t* dinput_copy, const float* tokmat,
                               cudaStream_t st) {
     if (d.k <= 4) {
-        k_dinput_act<4><<<T, chunk_threads(d.C), 0, st>>>(d, slot, T, add_dx, d_input, xact, hpre, I, dxact,
-                                                           dhpre, dinput_copy, tokmat); note_launch();
+        XHC_LAUNCH(st, T, chunk_threads(d.C), 0, (k_dinput_act<4>), d, slot, T, add_dx, d_input, xact, hpre, I, dxact, dhpre, dinput_copy, tokmat);
     } else {
-        k_dinput_act<8><<<T, chunk_threads(d.C), 0, st>>>(d, slot, T, add_dx, d_input, xact, hpre, I, dxact,
-                                                           dhpre, dinput_copy, tokmat); note_launch();
+        XHC_LAUNCH(st, T, chunk_threads(d.C), 0, (k_dinput_act<8>), d, slot, T, add_dx, d_input, xact, hpre, I, dxact, dhpre, dinput_copy, tokmat);
     }
     return cudaGetLastError();
 }
@@ -336,6 +339,7 @@ __global__ void __launch_bounds__(512) k_full_dots(Dims d, int T, const uint16_t
                                                    const uint16_t* __restrict__ dinput,
                                                    const int* __restrict__ I,
                                                    float* __restrict__ dhpre) {
+    pdl_entry();
     extern __shared__ __align__(16) uint16_t din[];   // [G][C]
     const int t = blockIdx.x, C = d.C, G = d.G;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -435,7 +439,7 @@ cudaError_t launch_full_dots(const Dims& d, int T, const uint16_t* X, const uint
                                              (int)sm);
         if (e != cudaSuccess) return e;
     }
-    k_full_dots<NS><<<T, 32 * nw, sm, st>>>(d, T, X, dinput, I, dhpre); note_launch();
+    XHC_LAUNCH(st, T, 32 * nw, sm, (k_full_dots<NS>), d, T, X, dinput, I, dhpre);
     return cudaGetLastError();
 }
 
@@ -445,6 +449,7 @@ cudaError_t launch_full_dots(const Dims& d, int T, const uint16_t* X, const uint
 // X[t][i] = h[t] for every stream i (N copies; also the backward of the stream sum)
 __global__ void __launch_bounds__(256) k_stream_bcast(int T, int N, int C, const uint16_t* __restrict__ h,
                                                       uint16_t* __restrict__ X) {
+    pdl_entry();
     const long long t = blockIdx.x;
     for (int c8 = threadIdx.x; c8 < C / 8; c8 += blockDim.x) {
         const uint4 v = *reinterpret_cast<const uint4*>(h + t * C + c8 * 8);
@@ -455,6 +460,7 @@ __global__ void __launch_bounds__(256) k_stream_bcast(int T, int N, int C, const
 // y[t] = sum_i X[t][i] in fp32, stored bf16 (also the backward of the expansion)
 __global__ void __launch_bounds__(256) k_stream_sum(int T, int N, int C, const uint16_t* __restrict__ X,
                                                     uint16_t* __restrict__ y) {
+    pdl_entry();
     const long long t = blockIdx.x;
     for (int c8 = threadIdx.x; c8 < C / 8; c8 += blockDim.x) {
         float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -469,12 +475,12 @@ __global__ void __launch_bounds__(256) k_stream_sum(int T, int N, int C, const u
 }
 
 cudaError_t launch_stream_bcast(int T, int N, int C, const uint16_t* h, uint16_t* X, cudaStream_t st) {
-    k_stream_bcast<<<T, chunk_threads(C), 0, st>>>(T, N, C, h, X); note_launch();
+    XHC_LAUNCH(st, T, chunk_threads(C), 0, (k_stream_bcast), T, N, C, h, X);
     return cudaGetLastError();
 }
 
 cudaError_t launch_stream_sum(int T, int N, int C, const uint16_t* X, uint16_t* y, cudaStream_t st) {
-    k_stream_sum<<<T, chunk_threads(C), 0, st>>>(T, N, C, X, y); note_launch();
+    XHC_LAUNCH(st, T, chunk_threads(C), 0, (k_stream_sum), T, N, C, X, y);
     return cudaGetLastError();
 }
 

@@ -254,6 +254,7 @@ k_proj_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    pdl_entry();   // barriers and TMEM are set up while the kernel before finishes
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------
@@ -489,6 +490,7 @@ constexpr int PF_NT = 256;
 
 __global__ void __launch_bounds__(PF_NT) k_pack_full(PackJob j, int nblk, const float* __restrict__ Wr, int N,
                                                      int rchunk, int nparts, float* __restrict__ wsump, PackJob act) {
+    pdl_entry();
     extern __shared__ float sm[];   // [n][PF_E + 1]
     const int tid = threadIdx.x;
     int blk = blockIdx.x;
@@ -643,8 +645,7 @@ cudaError_t launch_pack_full(const PackJob& full, const float* W_r, int N, float
                              cudaStream_t st) {
     const int nblk = (full.K + PF_E - 1) / PF_E, nparts = W_r ? colsum_parts(full.K) : 0;
     const size_t sm = sizeof(float) * std::max(full.n * (PF_E + 1), 8 * MAXN);
-    k_pack_full<<<nblk + nparts + pack_blocks(act), PF_NT, sm, st>>>(full, nblk, W_r, N, colsum_chunk(full.K), nparts,
-                                                                     wsump, act); note_launch();
+    XHC_LAUNCH(st, nblk + nparts + pack_blocks(act), PF_NT, sm, (k_pack_full), full, nblk, W_r, N, colsum_chunk(full.K), nparts, wsump, act);
     return cudaGetLastError();
 }
 
@@ -676,7 +677,7 @@ cudaError_t launch_proj_tc(const uint16_t* X, int T, int K, const uint16_t* Wpac
     a.err = err;
     a.wait_ns = debug_wait_ns();
     a.force_timeout = debug_take_force_timeout();
-    k_proj_tc<false><<<p.P, NTHREADS, sm, st>>>(ma, mb, a); note_launch();
+    XHC_LAUNCH(st, p.P, NTHREADS, sm, (k_proj_tc<false>), ma, mb, a);
     return cudaGetLastError();
 }
 
@@ -684,6 +685,7 @@ cudaError_t launch_proj_tc(const uint16_t* X, int T, int K, const uint16_t* Wpac
 // K-major B operand of the weight gradient.
 __global__ void k_pack_dz(const float* __restrict__ dz, int ldz, int n, int NB, int T, int Tp,
                           uint16_t* __restrict__ dzp) {
+    pdl_entry();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T) return;
     for (int o = 0; o < n; ++o) {
@@ -701,7 +703,7 @@ cudaError_t launch_wgrad_tc(const uint16_t* A, int T, int E, const float* dz, in
                             uint16_t* dzpack, const ProjTcPlan& p, float* part, int* err,
                             cudaStream_t st) {
     const int Tp = (T + 7) / 8 * 8;  // 16-byte row stride for the tensor map
-    k_pack_dz<<<(T + 255) / 256, 256, 0, st>>>(dz, ldz, n, p.NB, T, Tp, dzpack); note_launch();
+    XHC_LAUNCH(st, (T + 255) / 256, 256, 0, (k_pack_dz), dz, ldz, n, p.NB, T, Tp, dzpack);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     CUtensorMap ma, mb;
@@ -731,7 +733,7 @@ cudaError_t launch_wgrad_tc(const uint16_t* A, int T, int E, const float* dz, in
     a.err = err;
     a.wait_ns = debug_wait_ns();
     a.force_timeout = 0;
-    k_proj_tc<true><<<p.P, NTHREADS, sm, st>>>(ma, mb, a); note_launch();
+    XHC_LAUNCH(st, p.P, NTHREADS, sm, (k_proj_tc<true>), ma, mb, a);
     return cudaGetLastError();
 }
 
@@ -828,6 +830,7 @@ k_dx_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    pdl_entry();   // barriers and TMEM are set up while the kernel before finishes
     // 32-bit tile arithmetic (the host keeps ntiles below 2^31): the divisions run per tile
     const int nloc = (a.ntiles > blockIdx.x) ? (int)((a.ntiles - 1 - blockIdx.x) / a.P) + 1 : 0;
 
@@ -1146,6 +1149,7 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    pdl_entry();   // barriers and TMEM are set up while the kernel before finishes
     const int N = a.N;
     const int ndin = N - a.m;   // leading tiles of a block that may read d_input (streams m..N-1)
     const int nblk = (a.ntiles > blockIdx.x) ? (int)((a.ntiles - 1 - blockIdx.x) / a.P) + 1 : 0;
@@ -1400,6 +1404,7 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
 
 // bf16 copies with a padded row stride: dst[r][o] = src[r][o] (o < n), 0 for n <= o < ld
 __global__ void k_pack_rows(WSegs W, int n, int rows, int ld, uint16_t* __restrict__ dst) {
+    pdl_entry();
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (long long)rows * ld) return;
     const int r = (int)(idx / ld), o = (int)(idx - (long long)r * ld);
@@ -1411,6 +1416,7 @@ __global__ void k_pack_rows(WSegs W, int n, int rows, int ld, uint16_t* __restri
 // rows of three bf16 parts along K: A rows [hi | lo | hi] of dz, B rows [hi | hi | lo] of W, so
 // that sum_k A B = dz_hi W_hi + dz_lo W_hi + dz_hi W_lo (~2^-16 relative)
 __global__ void k_pack3(WSegs W, int n, int rows, int ld, int lo_part, uint16_t* __restrict__ dst) {
+    pdl_entry();
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (long long)rows * ld) return;
     const int r = (int)(idx / ld), col = (int)(idx - (long long)r * ld);
@@ -1443,9 +1449,9 @@ cudaError_t launch_dxa_tc(const Dims& d, int slot, int T, const float* dzs, int 
     memset(&dzsg, 0, sizeof(dzsg));
     dzsg.ptr[0] = dzs; dzsg.width[0] = nact; dzsg.off[0] = 0; dzsg.off[1] = nact; dzsg.n = 1;
     long long tot = (long long)T * ld;
-    k_pack3<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(dzsg, nact, T, ld, 1, dz3); note_launch();
+    XHC_LAUNCH(st, (unsigned)((tot + 255) / 256), 256, 0, (k_pack3), dzsg, nact, T, ld, 1, dz3);
     tot = (long long)KC * ld;
-    k_pack3<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(W, nact, KC, ld, 2, w3); note_launch();
+    XHC_LAUNCH(st, (unsigned)((tot + 255) / 256), 256, 0, (k_pack3), W, nact, KC, ld, 2, w3);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     CUtensorMap ma, mb;
@@ -1473,7 +1479,7 @@ cudaError_t launch_dxa_tc(const Dims& d, int slot, int T, const float* dzs, int 
                       (size_t)DX_EW * (32 * 33 + 32 * 8) * 4 + 1024;
     e = cudaFuncSetAttribute((const void*)k_dx_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k_dx_tc<true><<<a.P, DX_THREADS, sm, st>>>(ma, mb, a); note_launch();
+    XHC_LAUNCH(st, a.P, DX_THREADS, sm, (k_dx_tc<true>), ma, mb, a);
     return cudaGetLastError();
 }
 
@@ -1484,6 +1490,7 @@ namespace {
 __global__ void __launch_bounds__(256) k_dots_act(const float* __restrict__ dotp, int T, int k, int ncg,
                                                   int G, int N, int slot, const int* __restrict__ I,
                                                   float* __restrict__ dhpre) {
+    pdl_entry();
     __shared__ float part[8][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int j = blockIdx.y, t = blockIdx.x * 32 + lane;
@@ -1506,8 +1513,7 @@ __global__ void __launch_bounds__(256) k_dots_act(const float* __restrict__ dotp
 cudaError_t launch_dots_act(const Dims& d, int slot, int T, const float* dotp, const int* I, float* dhpre,
                             cudaStream_t st) {
     const dim3 grid((unsigned)((T + 31) / 32), (unsigned)d.k);
-    k_dots_act<<<grid, 256, 0, st>>>(dotp, T, d.k, d.C / 32, d.G, d.N, slot, I, dhpre);
-    note_launch();
+    XHC_LAUNCH(st, grid, 256, 0, (k_dots_act), dotp, T, d.k, d.C / 32, d.G, d.N, slot, I, dhpre);
     return cudaGetLastError();
 }
 
@@ -1536,9 +1542,9 @@ cudaError_t launch_dx_tc(const Dims& d, int T, const float* dz, const WSegs& W, 
     memset(&dzs, 0, sizeof(dzs));
     dzs.ptr[0] = dz; dzs.width[0] = n; dzs.off[0] = 0; dzs.off[1] = n; dzs.n = 1;
     long long tot = (long long)T * ld;
-    k_pack_rows<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(dzs, n, T, ld, dz16); note_launch();
+    XHC_LAUNCH(st, (unsigned)((tot + 255) / 256), 256, 0, (k_pack_rows), dzs, n, T, ld, dz16);
     tot = (long long)NC * ld;
-    k_pack_rows<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(W, n, NC, ld, w16); note_launch();
+    XHC_LAUNCH(st, (unsigned)((tot + 255) / 256), 256, 0, (k_pack_rows), W, n, NC, ld, w16);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     CUtensorMap ma, mb, mx, md, mg;
@@ -1564,7 +1570,7 @@ cudaError_t launch_dx_tc(const Dims& d, int T, const float* dz, const WSegs& W, 
     const size_t sm = dxf_smem(n, d.G);
     e = cudaFuncSetAttribute((const void*)k_dxf_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k_dxf_tc<<<a.P, DX_THREADS, sm, st>>>(ma, mb, mx, md, mg, a); note_launch();
+    XHC_LAUNCH(st, a.P, DX_THREADS, sm, (k_dxf_tc), ma, mb, mx, md, mg, a);
     return cudaGetLastError();
 }
 

@@ -249,6 +249,7 @@ template <int KW, int KS>
 __global__ void __launch_bounds__(WT) k_wb_gram(Dims d, int slot, int T, int TB,
                                                 const uint16_t* __restrict__ out, ConvPtrs cw,
                                                 int nslice, float* __restrict__ red) {
+    pdl_entry();
     extern __shared__ float wsh[];  // [TB][WT/32][16]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int slice = blockIdx.x, C = d.C;
@@ -319,6 +320,7 @@ constexpr int WSL2 = 4 * WT;
 __global__ void __launch_bounds__(WT, 2) k_wb_gram2(Dims d, int slot, int T, int TB,
                                                     const uint16_t* __restrict__ out, ConvPtrs cw,
                                                     int nslice, float* __restrict__ red) {
+    pdl_entry();
     constexpr int KW = 12, KS = 2;
     extern __shared__ float wsh[];  // [TB][WT/32][16]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -414,6 +416,7 @@ __global__ void __launch_bounds__(WT) k_wb_fwd(Dims d, int slot, int T, int TB,
                                                const float* __restrict__ hres,
                                                uint16_t* __restrict__ xact_next,
                                                uint16_t* __restrict__ X) {
+    pdl_entry();
     extern __shared__ __align__(16) unsigned char smu[];
     FRing<KM>& R = *reinterpret_cast<FRing<KM>*>(smu);
     const int k = (KS == 2) ? KM : d.k, C = d.C;
@@ -553,6 +556,7 @@ __global__ void __launch_bounds__(WT) k_wb_bred(Dims d, int slot, int T, int TB,
                                                 const float* __restrict__ dxact,
                                                 const uint16_t* __restrict__ xact, int nslice,
                                                 float* __restrict__ red) {
+    pdl_entry();
     static_assert(NV == 16 || NV % 32 == 0, "reduction width");
     constexpr int NVP = NV < 32 ? 16 : NV;      // values per token and warp in shared memory
     extern __shared__ __align__(16) unsigned char smu[];
@@ -720,6 +724,7 @@ __global__ void __launch_bounds__(WT, 2) k_wb_bred2(Dims d, int slot, int T, int
                                                     const float* __restrict__ dxact,
                                                     const uint16_t* __restrict__ xact, int nslice,
                                                     float* __restrict__ red) {
+    pdl_entry();
     constexpr int KW = 12, KS = 2;
     static_assert(NV == 16 || NV % 32 == 0, "reduction width");
     constexpr int NVP = NV < 32 ? 16 : NV;
@@ -889,6 +894,7 @@ __global__ void __launch_bounds__(WT, 2) k_wb_bapp(Dims d, int slot, int T, int 
                                                    float* dxact_out,
                                                    uint16_t* __restrict__ d_out,
                                                    float* __restrict__ cpart) {
+    pdl_entry();
     constexpr int HL = KW > 0 ? KW - 1 : 0;   // tokens after the run whose du the run needs
     constexpr int RU = UB;
     constexpr int NR = KW > 0 ? KW + UB - 1 : 1;   // block ring slots
@@ -1159,6 +1165,7 @@ __global__ void __launch_bounds__(WT) k_wb_fwd8(Dims d, int slot, int T, int TB,
                                                 const float* __restrict__ hres,
                                                 uint16_t* __restrict__ xact_next,
                                                 uint16_t* __restrict__ X) {
+    pdl_entry();
     extern __shared__ __align__(16) unsigned char smu[];
     float* Esh = reinterpret_cast<float*>(smu);        // [TB][KM]
     float* Hsh = Esh + TB * KM;                        // [TB][KM][KM]
@@ -1237,6 +1244,7 @@ __global__ void __launch_bounds__(WT, 3) k_wb_b8(Dims d, int slot, int T, int TB
                                               const uint16_t* __restrict__ xact, int nslice,
                                               float* __restrict__ red,
                                               uint16_t* __restrict__ d_out) {
+    pdl_entry();
     constexpr int NQ = KM + KM * KM;                  // P[j][0], then Q[j][i]
     constexpr int NV = NQ <= 32 ? 32 : 96;            // reduce-scatter width (blocks of 32)
     extern __shared__ __align__(16) unsigned char smu[];

@@ -14,8 +14,7 @@ cudaError_t bapp_kw(const Dims& d, int slot, int T, const uint16_t* out, ConvPtr
     cudaError_t e = smem_attr((const void*)k_wb_bapp<KM, KW, KS, HALO>, sm);
     if (e != cudaSuccess) return e;
     dim3 grid(nslice, (unsigned)n_runs(d, T, TB, KW > 0));
-    k_wb_bapp<KM, KW, KS, HALO><<<grid, WT, sm, st>>>(d, slot, T, TB, out, cw, dX, I, dn_in, tokmat,
-                                                      dxact_out, d_out, cpart); note_launch();
+    XHC_LAUNCH(st, grid, WT, sm, (k_wb_bapp<KM, KW, KS, HALO>), d, slot, T, TB, out, cw, dX, I, dn_in, tokmat, dxact_out, d_out, cpart);
     return cudaGetLastError();
 }
 

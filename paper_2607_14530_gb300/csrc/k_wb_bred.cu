@@ -16,7 +16,7 @@ cudaError_t bred_kw(const Dims& d, int slot, int T, const uint16_t* out, ConvPtr
     cudaError_t e = smem_attr((const void*)k_wb_bred<KM, KW, NV, KS>, sm);
     if (e != cudaSuccess) return e;
     dim3 grid(nslice, (unsigned)n_runs(d, T, TB, KW > 0));
-    k_wb_bred<KM, KW, NV, KS><<<grid, WT, sm, st>>>(d, slot, T, TB, out, cw, dX, I, dxact, xact, nslice, red); note_launch();
+    XHC_LAUNCH(st, grid, WT, sm, (k_wb_bred<KM, KW, NV, KS>), d, slot, T, TB, out, cw, dX, I, dxact, xact, nslice, red);
     return cudaGetLastError();
 }
 
@@ -30,7 +30,7 @@ cudaError_t bred2_kw(const Dims& d, int slot, int T, const uint16_t* out, ConvPt
     cudaError_t e = smem_attr((const void*)k_wb_bred2<KM, NV>, sm);
     if (e != cudaSuccess) return e;
     dim3 grid(d.C / WSL2, (unsigned)n_runs(d, T, TB, true));
-    k_wb_bred2<KM, NV><<<grid, WT, sm, st>>>(d, slot, T, TB, out, cw, dX, I, dxact, xact, nslice, red); note_launch();
+    XHC_LAUNCH(st, grid, WT, sm, (k_wb_bred2<KM, NV>), d, slot, T, TB, out, cw, dX, I, dxact, xact, nslice, red);
     return cudaGetLastError();
 }
 
@@ -49,8 +49,7 @@ cudaError_t b8_kw(const Dims& d, int slot, int T, const uint16_t* out, const uin
     cudaError_t e = smem_attr((const void*)k_wb_b8<KM>, sm);
     if (e != cudaSuccess) return e;
     dim3 grid((d.C + W8 - 1) / W8, (T + TB - 1) / TB);
-    k_wb_b8<KM><<<grid, WT, sm, st>>>(d, slot, T, TB, out, dX, I, p, hpost, hres, dxact, dxact_out, xact,
-                                      nslice, red, d_out); note_launch();
+    XHC_LAUNCH(st, grid, WT, sm, (k_wb_b8<KM>), d, slot, T, TB, out, dX, I, p, hpost, hres, dxact, dxact_out, xact, nslice, red, d_out);
     return cudaGetLastError();
 }
 

@@ -18,6 +18,7 @@ __global__ void __launch_bounds__(WC_NT) k_wb_coef(Dims d, int slot, int T, int 
                                                    int nslice, const float* __restrict__ p,
                                                    const float* __restrict__ hpost,
                                                    double* __restrict__ gram, float* __restrict__ emat) {
+    pdl_entry();
     __shared__ double Gs[32][NGRAM + 1];
     __shared__ float Bs[32][MAXCOMP * MAXCOMP + 1];
     const int tid = threadIdx.x, k = d.k, K = d.K[slot];
@@ -72,7 +73,7 @@ cudaError_t gram_kw(const Dims& d, int slot, int T, const uint16_t* out, ConvPtr
     cudaError_t e = smem_attr((const void*)k_wb_gram<KW, KS>, sm);
     if (e != cudaSuccess) return e;
     dim3 grid(nslice, (unsigned)n_runs(d, T, TB, true));
-    k_wb_gram<KW, KS><<<grid, WT, sm, st>>>(d, slot, T, TB, out, cw, nslice, red); note_launch();
+    XHC_LAUNCH(st, grid, WT, sm, (k_wb_gram<KW, KS>), d, slot, T, TB, out, cw, nslice, red);
     return cudaGetLastError();
 }
 
@@ -86,8 +87,7 @@ cudaError_t fwd_kw(const Dims& d, int slot, int T, const uint16_t* out, ConvPtrs
     cudaError_t e = smem_attr((const void*)k_wb_fwd<KM, KW, KS>, sm);
     if (e != cudaSuccess) return e;
     dim3 grid(nslice, (unsigned)n_runs(d, T, TB, KW > 0));
-    k_wb_fwd<KM, KW, KS><<<grid, WT, sm, st>>>(d, slot, T, TB, out, cw, emat, xact, I, hres, xact_next,
-                                               X); note_launch();
+    XHC_LAUNCH(st, grid, WT, sm, (k_wb_fwd<KM, KW, KS>), d, slot, T, TB, out, cw, emat, xact, I, hres, xact_next, X);
     return cudaGetLastError();
 }
 
@@ -98,7 +98,7 @@ cudaError_t fwd8_kw(const Dims& d, int slot, int T, const uint16_t* out, const f
     const int TB = pick_run(d, T, false, (d.C + W8 - 1) / W8, KM == 4 ? 6 : 3, 4, 32);
     const size_t sm = (size_t)TB * (KM + KM * KM + KM) * 4;
     dim3 grid((d.C + W8 - 1) / W8, (T + TB - 1) / TB);
-    k_wb_fwd8<KM><<<grid, WT, sm, st>>>(d, slot, T, TB, out, emat, xact, I, hres, xact_next, X); note_launch();
+    XHC_LAUNCH(st, grid, WT, sm, (k_wb_fwd8<KM>), d, slot, T, TB, out, emat, xact, I, hres, xact_next, X);
     return cudaGetLastError();
 }
 
@@ -121,7 +121,7 @@ cudaError_t launch_wb_gram(const Dims& d, int slot, int T, const uint16_t* out, 
         const int TB = pick_run(d, T, true, d.C / WSL2, 2, 12, 64);
         const size_t sm = (size_t)TB * (WT / 32) * 16 * sizeof(float);
         dim3 grid(d.C / WSL2, (unsigned)n_runs(d, T, TB, true));
-        k_wb_gram2<<<grid, WT, sm, st>>>(d, slot, T, TB, out, cw, nslice, red); note_launch();
+        XHC_LAUNCH(st, grid, WT, sm, (k_wb_gram2), d, slot, T, TB, out, cw, nslice, red);
         return cudaGetLastError();
     }
     XHC_KW_DISPATCH(d, d.C % WSL == 0, (gram_kw<KWC, KSC>(d, slot, T, out, cw, nslice, red, st)));
@@ -131,7 +131,7 @@ cudaError_t launch_wb_coef(const Dims& d, int slot, int T, const float* red, int
                            const float* hpost, double* gram, float* emat, cudaStream_t st) {
     // full fp64 warps at many tokens, more blocks at few
     const int TB = (T >= 32 * device_sms()) ? 32 : 8;
-    k_wb_coef<<<(T + TB - 1) / TB, WC_NT, 0, st>>>(d, slot, T, TB, red, nslice, p, hpost, gram, emat); note_launch();
+    XHC_LAUNCH(st, (T + TB - 1) / TB, WC_NT, 0, (k_wb_coef), d, slot, T, TB, red, nslice, p, hpost, gram, emat);
     return cudaGetLastError();
 }
 

@@ -98,3 +98,40 @@ def test_decode_sizes(name):
     cases.assert_bf16_close(X, ref["X"][new], "X")
     assert torch.equal(dpos.cpu(), pos + 1)
     assert g.device_error(ws) == 0
+
+
+def test_captured_step_equals_the_eager_one():
+    """A forward and backward captured as a CUDA graph (no programmatic launches, the side stream forked
+    and joined inside) gives the eager call's bits."""
+    cfg, T = Config.flash(8, 4, 2, 512, 4, seq_len=150), 300
+    inp, P, seed = cases.make_case(cfg, T, 1)
+    gin = synth.group_grads(T, cfg.N, cfg.C, cfg.G, seed)
+    g = Group(cfg)
+    Pd = {n: v.cuda() for n, v in P.items()}
+    X, X0 = inp["X"].cuda(), inp["X"].cuda()
+    outs, d_in = [o.cuda() for o in inp["outs"]], [d.cuda() for d in gin["d_inputs"]]
+    dX0 = gin["dX"].cuda()
+    dX = torch.empty_like(dX0)
+    gr = {n: torch.zeros_like(v) for n, v in Pd.items()}
+    rows = [torch.empty(T, cfg.C, dtype=torch.bfloat16, device="cuda") for _ in range(2 * cfg.G)]
+    saved, ws = g.alloc(T)
+
+    def step():
+        X.copy_(X0)
+        dX.copy_(dX0)
+        for v in gr.values():
+            v.zero_()
+        g.forward(Pd, X, outs, saved, ws, inputs=rows[:cfg.G])
+        g.backward(Pd, X, dX, outs, d_in, gr, saved, ws, d_outs=rows[cfg.G:])
+
+    step()
+    torch.cuda.synchronize()
+    want = [t.clone() for t in rows + [dX] + list(gr.values())]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        step()
+    graph.replay()
+    torch.cuda.synchronize()
+    for a, b in zip(want, rows + [dX] + list(gr.values())):
+        assert torch.equal(a, b)
+    assert g.device_error(ws) == 0
