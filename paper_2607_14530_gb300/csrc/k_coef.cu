@@ -664,7 +664,7 @@ cudaError_t bwd_coef_km(const Dims& d, int slot, int T, const float* red, int ns
     if (T < TB * 2 * device_sms() || smem(TB) > 200 * 1024) TB = 32 / KM;
     const size_t sm = smem(TB);
     const cudaError_t e =
-        cudaFuncSetAttribute((const void*)k_bwd_coef<KM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        smem_optin((const void*)k_bwd_coef<KM>, sm);
     if (e != cudaSuccess) return e;
     *nblk = (T + TB - 1) / TB;
     XHC_LAUNCH(st, *nblk, 32 + TB * KM, sm, (k_bwd_coef<KM>), d, slot, T, TB, red, nslice, zact, rs, p, hpost, gram, alpha_post, alpha_res, b_res, tokmat, dz, dp, colp);

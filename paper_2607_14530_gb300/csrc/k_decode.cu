@@ -285,8 +285,7 @@ cudaError_t dec_post_kw(const Dims& d, int slot, int B, const uint16_t* out, Con
     int DT = std::min(DMAXT, std::max(1, (int)(((long long)B * nr + cap - 1) / cap)));
     while (DT > 1 && CONV && DT * q * 3 * 128 * 8 > 64 * 1024) --DT;
     const DecSmem L(DT, q, ns, d.k, CONV);
-    cudaError_t e = cudaFuncSetAttribute((const void*)k_dec_post<KM, KW, PAPER>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, L.bytes);
+    cudaError_t e = smem_optin((const void*)k_dec_post<KM, KW, PAPER>, L.bytes);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((B + DT - 1) / DT), (unsigned)nr);

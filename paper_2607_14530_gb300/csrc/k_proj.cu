@@ -232,8 +232,7 @@ static cudaError_t rowproj_small(const uint16_t* A, int64_t lda, int K, int T, c
     s = (K + kchunk - 1) / kchunk;
     *splits = s;
     const size_t sm = sizeof(float) * std::max((size_t)RS_ROWS * ((TT + 1) / 2 * 2), (size_t)nl * n * TT);
-    const cudaError_t e = cudaFuncSetAttribute((const void*)k_rowproj_small<TT, V>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const cudaError_t e = smem_optin((const void*)k_rowproj_small<TT, V>, sm);
     if (e != cudaSuccess) return e;
     XHC_LAUNCH(st, dim3(s, ny), RS_NT, sm, (k_rowproj_small<TT, V>), A, lda, K, T, W, n, kchunk, part, pstats);
     return cudaGetLastError();

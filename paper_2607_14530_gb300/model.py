@@ -106,7 +106,9 @@ class _GroupFn(torch.autograd.Function):
         else:
             dX = dX_out.to(torch.bfloat16).contiguous().clone()
         P = mod.param_dict()
-        grads = {n: torch.zeros_like(v) for n, v in P.items()}
+        # one launch clears them all
+        grads = {n: torch.empty_like(v) for n, v in P.items()}
+        torch._foreach_zero_(list(grads.values()))
         pp, gg = g.params(P), g.params(grads)
         for t in reversed(range(cfg.G)):
             out, out_b = outs[t]
@@ -133,13 +135,18 @@ class XhcGroup(nn.Module):
         self.g = Group(cfg)
         self.sublayers = nn.ModuleList(sublayers)
         self.names = list(cfg.param_shapes())
+        self._attrs = [n.replace(".", "_") for n in self.names]
         init = synth.params(cfg.param_shapes(), seed, alpha=alpha, w_std=w_std)
         for n in self.names:
             self.register_parameter(n.replace(".", "_"), nn.Parameter(init[n].clone()))
         self._bufs = {}
 
     def param_dict(self) -> dict:
-        return {n: getattr(self, n.replace(".", "_")).detach().contiguous() for n in self.names}
+        out = {}
+        for n, a in zip(self.names, self._attrs):
+            v = getattr(self, a)
+            out[n] = v if v.is_contiguous() else v.detach().contiguous()
+        return out
 
     def buffers(self, T: int, device):
         """(saved, workspace) for one forward call: a fresh `saved` (it carries this call's
@@ -157,7 +164,7 @@ class XhcGroup(nn.Module):
     def forward(self, X):
         if not torch.is_grad_enabled():
             return self._forward_inference(X)
-        return _GroupFn.apply(X, self, *[getattr(self, n.replace(".", "_")) for n in self.names])
+        return _GroupFn.apply(X, self, *[getattr(self, a) for a in self._attrs])
 
     def _forward_inference(self, X):
         """The forward without autograd (grad mode off: prefill or evaluation): the same calls,

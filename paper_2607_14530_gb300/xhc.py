@@ -247,17 +247,23 @@ class Config:
         return c
 
 
+# Pointers and streams go to ctypes as plain integers (the argument types convert them): a call's own
+# Python time counts where a decode step or a small model is bound by the host.
+
+
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _fill(struct, d: dict, cfg: Config):
     """Fill a _Params/_Grads from a flat dict of fp32 CUDA tensors."""
+    f32 = torch.float32
+
     def get(n):
         v = d.get(n)
         if v is None:
             return None
-        if v.dtype != torch.float32 or not v.is_cuda or not v.is_contiguous():
+        if v.dtype is not f32 or not v.is_cuda or not v.is_contiguous():
             raise XhcError(f"parameter {n} must be a contiguous fp32 CUDA tensor")
         return v.data_ptr()
     struct.W_r = get("W_r")
@@ -277,14 +283,17 @@ def _fill(struct, d: dict, cfg: Config):
 
 
 def _bf16(t, name):
-    if t.dtype != torch.bfloat16 or not t.is_cuda or not t.is_contiguous():
+    if t.dtype is not torch.bfloat16 or not t.is_cuda or not t.is_contiguous():
         raise XhcError(f"{name} must be a contiguous bf16 CUDA tensor")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream(stream):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    """The stream's handle; None: the current stream of the current device (read directly: building the
+    Stream object took a third of a small call's host time)."""
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 class Group:
