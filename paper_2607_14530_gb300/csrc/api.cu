@@ -869,27 +869,32 @@ xhc_status post_bwd_impl(const xhc_handle* h, int slot, int64_t T, const xhc_par
         XHC_K("wb_bred", c.st, launch_wb_bred(d, slot, T32, out, cw, dX, c.S<int>(c.L.I), dxact, c.xact(slot),
                                               bslices, red, c.st));
     }
+    // the bf16 operands of the weight gradient and of pre_bwd(slot)'s input gradient, formed with dZ_act
+    const bool tcw = !(T32 < 64 || d.k * d.C < 128), tcx = dxa_tc_ok(T32, d.k, d.C, n);
+    const ProjTcPlan wpl = plan_proj_tc(d.k * d.C, T32, n, device_sms(), false);
+    const int Tp = (T32 + 7) / 8 * 8;   // 16-byte row stride for the tensor map
+    const DzPack pk = {tcw ? c.W<uint16_t>(c.L.dzpack) : nullptr, tcx ? c.W<uint16_t>(c.L.dz16) : nullptr, wpl.NB, Tp,
+                       dxa_ld(n), 3};
+    const WRows wr = {act_segs(d, P, slot), n, d.k * d.C, dxa_ld(n), 3, tcx ? c.W<uint16_t>(c.L.w16) : nullptr};
     int nblk = 0;
     XHC_K("bwd_coef", c.st, launch_bwd_coef(d, slot, T32, red, bslices, c.S<float>(c.L.zact[slot]),
                              c.S<float>(c.L.rs[slot]), c.S<float>(c.L.p),
                              c.S<float>(c.L.hpost[slot]),
                              (d.K[slot] > 1 && d.gs) ? c.S<double>(c.L.gram[slot]) : nullptr,
                              P->alpha_post, P->alpha_res, P->b_res, c.W<float>(c.L.tokmat),
-                             c.W<float>(c.L.dz), c.W<float>(c.L.dp), c.W<float>(c.L.colp), &nblk, c.st));
+                             c.W<float>(c.L.dz), c.W<float>(c.L.dp), c.W<float>(c.L.colp), &nblk, pk, wr, c.st));
     // weight gradient of the post/res projections and the alpha / b column sums need only dZ_act
     // and the per-token contributions: side stream, overlapping the apply kernel
     const cudaStream_t sd = fork_from(c.st);
-    if (T32 < 64 || d.k * d.C < 128) {
+    if (!tcw) {
         const int ts = std::min(c.L.tsplits, pick_tsplits(d.k * d.C, T32));
         XHC_K("wgrad_active", sd, launch_wgrad(c.xact(slot), (int64_t)d.k * d.C, d.k * d.C, T32,
                                                c.W<float>(c.L.dz), n, n, ts, c.W<float>(c.L.wpart),
                                                act_segs_g(d, g, slot), nullptr, sd));
     } else {
-        ProjTcPlan pl = plan_proj_tc(d.k * d.C, T32, n, device_sms(), false);
-        XHC_K("wgrad_tc_active", sd, launch_wgrad_tc(c.xact(slot), T32, d.k * d.C, c.W<float>(c.L.dz), n, n,
-                                                     c.W<uint16_t>(c.L.dzpack), pl, c.W<float>(c.L.wpart),
-                                                     c.W<int>(c.L.err), sd));
-        XHC_K("wgrad_reduce", sd, launch_wgrad_reduce(c.W<float>(c.L.wpart), slots_of(pl), d.k * d.C, n,
+        XHC_K("wgrad_tc_active", sd, launch_wgrad_tc(c.xact(slot), T32, d.k * d.C, n, pk.hilo, Tp, wpl,
+                                                     c.W<float>(c.L.wpart), c.W<int>(c.L.err), sd));
+        XHC_K("wgrad_reduce", sd, launch_wgrad_reduce(c.W<float>(c.L.wpart), slots_of(wpl), d.k * d.C, n,
                                                       act_segs_g(d, g, slot), nullptr, sd));
     }
     const int kK = d.k * K, kk = d.k * d.k;
@@ -906,7 +911,7 @@ xhc_status post_bwd_impl(const xhc_handle* h, int slot, int64_t T, const xhc_par
                                               c.W<float>(c.L.cpart), c.st));
     const WSegs wa = act_segs(d, P, slot);
     // dZ_act stays in the workspace: pre_bwd(slot) applies it to dX_act on the tensor cores
-    if (!dxa_tc_ok(T32, d.k, d.C, n))
+    if (!tcx)
         XHC_K("gemm_dzw", c.st, launch_gemm_dzw(d, T32, c.W<float>(c.L.dz), n, n, wa, d.k * d.C, dxact, c.st));
     if (K > 1) {
         ConvGradPtrs gc;
@@ -954,8 +959,7 @@ xhc_status xhc_pre_bwd(const xhc_handle* h, int slot, int64_t T, const xhc_param
     if (tc) {
         // post_bwd(slot) left dZ_act of this slot in the workspace; the update also forms the
         // dH_pre dots of the active streams (per 32 channels) and copies d_input
-        XHC_K("dxa_tc", c.st, launch_dxa_tc(d, slot, T32, c.W<float>(c.L.dz), n, act_segs(d, P, slot),
-                                            c.W<uint16_t>(c.L.dz16), c.W<uint16_t>(c.L.w16), d_input,
+        XHC_K("dxa_tc", c.st, launch_dxa_tc(d, slot, T32, n, c.W<uint16_t>(c.L.dz16), c.W<uint16_t>(c.L.w16), d_input,
                                             c.S<float>(c.L.hpre), c.S<int>(c.L.I), c.xact(slot),
                                             c.W<float>(c.L.tokmat), c.W<float>(c.L.dxact),
                                             c.W<float>(c.L.dotp), dinput, c.W<int>(c.L.err), c.st));
@@ -968,13 +972,23 @@ xhc_status xhc_pre_bwd(const xhc_handle* h, int slot, int64_t T, const xhc_param
     }
     if (slot != 0) return XHC_OK;
     XHC_K("full_dots", c.st, launch_full_dots(d, T32, X, dinput, c.S<int>(c.L.I), c.W<float>(c.L.dhpre), c.st));
+    const bool tcw = !(T32 < 64 || d.N * d.C < 128), tcx = dx_tc_ok(T32, d.N, d.C, d.nfull, d.G);
+    const ProjTcPlan& wpl = c.L.twf;
+    const int Tp = (T32 + 7) / 8 * 8;   // 16-byte row stride for the tensor map
+    const DzPack pk = {tcw ? c.W<uint16_t>(c.L.dzpack) : nullptr, tcx ? c.W<uint16_t>(c.L.dz16) : nullptr, wpl.NB, Tp,
+                       dx_ld(d.nfull), 1};
+    const WRows wr = {full_segs(d, P), d.nfull, d.N * d.C, dx_ld(d.nfull), 1, tcx ? c.W<uint16_t>(c.L.w16) : nullptr};
     int nblk = 0;
     XHC_K("full_coef", c.st, launch_full_coef(d, T32, c.W<float>(c.L.dhpre), c.S<float>(c.L.hpre),
                               c.S<float>(c.L.zfull), c.S<float>(c.L.stats), c.S<float>(c.L.wsum),
                               c.S<int>(c.L.I), c.W<float>(c.L.dp), P->alpha_pre,
-                              c.W<float>(c.L.dz), c.W<float>(c.L.scal), c.W<float>(c.L.colp), &nblk, c.st));
-    // the full-state weight gradient and the pre-map / router column sums need only dZ and the
-    // per-token contributions: side stream, overlapping the full-state dX
+                              c.W<float>(c.L.dz), c.W<float>(c.L.scal), c.W<float>(c.L.colp), &nblk, pk, wr,
+                              c.st));
+    // the full-state weight gradient and the pre-map / router column sums need only dZ and the per-token
+    // contributions.  On a small state the weight gradient runs on the side stream beside the full-state
+    // dX; on a large one each fills the GPU by itself, and a weight gradient that gets SMs first holds
+    // back the dX blocks that belong there (32768 tokens of N = 16, C = 4096: 22.2 or 23.0 ms a step,
+    // whichever came first), so it follows on the caller's stream.
     const cudaStream_t sd = fork_from(c.st);
     const int GN = d.G * d.N;
     float* rsum = d.hr ? c.W<float>(c.L.rsum) : nullptr;
@@ -983,31 +997,34 @@ xhc_status xhc_pre_bwd(const xhc_handle* h, int slot, int64_t T, const xhc_param
                        {GN, d.G, d.hr ? d.N : 0, 0},
                        {0, 0, 1, 0}};
     XHC_K("colsum_out", sd, launch_colsum_out(c.W<float>(c.L.colp), nblk, GN + d.G + (d.hr ? d.N : 0), co, sd));
-    if (T32 < 64 || d.N * d.C < 128) {
-        const int ts = std::min(c.L.tsplits, pick_tsplits(d.N * d.C, T32));
-        XHC_K("wgrad_full", sd, launch_wgrad(X, (int64_t)d.N * d.C, d.N * d.C, T32, c.W<float>(c.L.dz),
-                                               d.nfull, d.nfull, ts, c.W<float>(c.L.wpart),
-                                               full_segs_g(d, g), rsum, sd));
-    } else {
-        const ProjTcPlan& pl = c.L.twf;
-        XHC_K("wgrad_tc_full", sd, launch_wgrad_tc(X, T32, d.N * d.C, c.W<float>(c.L.dz), d.nfull, d.nfull,
-                                                     c.W<uint16_t>(c.L.dzpack), pl, c.W<float>(c.L.wpart),
-                                                     c.W<int>(c.L.err), sd));
-        XHC_K("wgrad_reduce", sd, launch_wgrad_reduce(c.W<float>(c.L.wpart), slots_of(pl), d.N * d.C, d.nfull,
-                                                        full_segs_g(d, g), rsum, sd));
-    }
-    const WSegs wf = full_segs(d, P);
-    if (dx_tc_ok(T32, d.N, d.C, d.nfull, d.G)) {
-        XHC_K("dx_tc", c.st, launch_dx_tc(d, T32, c.W<float>(c.L.dz), wf, c.W<uint16_t>(c.L.dz16),
-                                          c.W<uint16_t>(c.L.w16), X, dinput, c.S<float>(c.L.hpre),
+    auto wgrad = [&](cudaStream_t st) -> xhc_status {
+        if (!tcw) {
+            const int ts = std::min(c.L.tsplits, pick_tsplits(d.N * d.C, T32));
+            XHC_K("wgrad_full", st, launch_wgrad(X, (int64_t)d.N * d.C, d.N * d.C, T32, c.W<float>(c.L.dz),
+                                                 d.nfull, d.nfull, ts, c.W<float>(c.L.wpart),
+                                                 full_segs_g(d, g), rsum, st));
+        } else {
+            XHC_K("wgrad_tc_full", st, launch_wgrad_tc(X, T32, d.N * d.C, d.nfull, pk.hilo, Tp, wpl,
+                                                       c.W<float>(c.L.wpart), c.W<int>(c.L.err), st));
+            XHC_K("wgrad_reduce", st, launch_wgrad_reduce(c.W<float>(c.L.wpart), slots_of(wpl), d.N * d.C, d.nfull,
+                                                          full_segs_g(d, g), rsum, st));
+        }
+        return XHC_OK;
+    };
+    const bool follow = (size_t)T32 * d.N * d.C * 2 > ((size_t)256 << 20);
+    if (!follow && (s = wgrad(sd)) != XHC_OK) return s;
+    if (tcx) {
+        XHC_K("dx_tc", c.st, launch_dx_tc(d, T32, pk.rows, wr.dst, X, dinput, c.S<float>(c.L.hpre),
                                           c.S<int>(c.L.I), c.W<float>(c.L.dxact), c.W<float>(c.L.scal),
                                           2, dX, c.W<int>(c.L.err), c.st));
     } else {
+        const WSegs wf = full_segs(d, P);
         XHC_K("full_dx", c.st, launch_full_dx(d, T32, c.W<float>(c.L.dz), wf, X, dinput, c.S<float>(c.L.hpre),
                                               c.S<int>(c.L.I), c.W<float>(c.L.dxact),
                                               c.W<float>(c.L.scal), dX, c.st));
     }
-    return join_into(c.st, sd);
+    s = join_into(c.st, sd);
+    return s == XHC_OK && follow ? wgrad(c.st) : s;
 }
 
 }  // extern "C"

@@ -144,9 +144,10 @@ __device__ __forceinline__ void transpose(float (&A)[KM], int a) {
 #pragma unroll
         for (int b = 0; b < KM; ++b) {
             if (b & o) continue;
-            const float got = __shfl_xor_sync(0xffffffffu, up ? A[b] : A[b | o], o);
-            if (up) A[b] = got;
-            else A[b | o] = got;
+            const float lo = A[b], hi = A[b | o];
+            const float got = __shfl_xor_sync(0xffffffffu, up ? lo : hi, o);
+            A[b] = up ? got : lo;
+            A[b | o] = up ? hi : got;
         }
     }
 }
@@ -464,8 +465,12 @@ __global__ void __launch_bounds__(160) k_bwd_coef(Dims d, int slot, int T, int T
                                                   const float* __restrict__ alpha_res,
                                                   const float* __restrict__ b_res, float* __restrict__ tokmat,
                                                   float* __restrict__ dzs, float* __restrict__ dp,
-                                                  float* __restrict__ colp) {
+                                                  float* __restrict__ colp, DzPack pack, WRows wrows, int nblk) {
     pdl_entry();
+    if ((int)blockIdx.x >= nblk) {
+        pack_wrows_of(wrows, (int)blockIdx.x - nblk);
+        return;
+    }
     using L = BwdTok<KM>;
     extern __shared__ float sm[];   // [TB][ROW], then the Sinkhorn iterates
     const int tid = threadIdx.x, lane = tid & 31, nt = blockDim.x;
@@ -625,6 +630,7 @@ __global__ void __launch_bounds__(160) k_bwd_coef(Dims d, int slot, int T, int T
         const int tt = e / n, o = e - tt * n;
         dzs[t0 * n + e] = sm[tt * L::ROW + L::DZ + o];
     }
+    pack_dz_of(pack, sm + L::DZ, L::ROW, n, t0, ntok);
     if (tid < ntok) {
         // active RMS: z_o = r * zraw_o, r = (sum x^2 / kC + eps)^(-1/2)
         const float* row = sm + tid * L::ROW;
@@ -652,7 +658,8 @@ template <int KM>
 cudaError_t bwd_coef_km(const Dims& d, int slot, int T, const float* red, int nslice, const float* zact,
                         const float* rs, const float* p, const float* hpost, const double* gram,
                         const float* alpha_post, const float* alpha_res, const float* b_res, float* tokmat,
-                        float* dz, float* dp, float* colp, int* nblk, cudaStream_t st) {
+                        float* dz, float* dp, float* colp, int* nblk, const DzPack& pack, const WRows& wrows,
+                        cudaStream_t st) {
     // 32 tokens a block (k <= 4) fill the fp64 warp, which is what bounds the kernel at many tokens;
     // a quarter of that at few, for more blocks.  (k > 4: 16 and 4.)  The iterates of a long Sinkhorn
     // run (k > 4, more than 50 iterations) only fit with the small block.
@@ -667,7 +674,8 @@ cudaError_t bwd_coef_km(const Dims& d, int slot, int T, const float* red, int ns
         smem_optin((const void*)k_bwd_coef<KM>, sm);
     if (e != cudaSuccess) return e;
     *nblk = (T + TB - 1) / TB;
-    XHC_LAUNCH(st, *nblk, 32 + TB * KM, sm, (k_bwd_coef<KM>), d, slot, T, TB, red, nslice, zact, rs, p, hpost, gram, alpha_post, alpha_res, b_res, tokmat, dz, dp, colp);
+    XHC_LAUNCH(st, *nblk + wrows_blocks(wrows, 32 + TB * KM), 32 + TB * KM, sm, (k_bwd_coef<KM>), d, slot, T, TB, red, nslice, zact, rs, p,
+               hpost, gram, alpha_post, alpha_res, b_res, tokmat, dz, dp, colp, pack, wrows, *nblk);
     return cudaGetLastError();
 }
 
@@ -677,12 +685,13 @@ cudaError_t launch_bwd_coef(const Dims& d, int slot, int T, const float* red, in
                             const float* zact, const float* rs, const float* p,
                             const float* hpost, const double* gram, const float* alpha_post,
                             const float* alpha_res, const float* b_res,
-                            float* tokmat, float* dz, float* dp, float* colp, int* nblk, cudaStream_t st) {
+                            float* tokmat, float* dz, float* dp, float* colp, int* nblk, const DzPack& pack,
+                            const WRows& wrows, cudaStream_t st) {
     if (d.k <= 4)
         return bwd_coef_km<4>(d, slot, T, red, nslice, zact, rs, p, hpost, gram, alpha_post, alpha_res, b_res,
-                              tokmat, dz, dp, colp, nblk, st);
+                              tokmat, dz, dp, colp, nblk, pack, wrows, st);
     return bwd_coef_km<8>(d, slot, T, red, nslice, zact, rs, p, hpost, gram, alpha_post, alpha_res, b_res,
-                          tokmat, dz, dp, colp, nblk, st);
+                          tokmat, dz, dp, colp, nblk, pack, wrows, st);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -690,7 +699,9 @@ cudaError_t launch_bwd_coef(const Dims& d, int slot, int T, const float* red, in
 // at a time with a lane per column, and keeps the column sums of its tokens in registers:
 // [dy (G N) | dy * z * rstd (G N), summed over a slot's N columns: d alpha_pre (G) | mu dZ_r (N): the
 // router logit subtracts mu * colsum(W_r), so every row of dW_r also receives -sum_t mu_t dZ_r[t]].
-// scal: (d mu / NC, 2 d nu / NC), the per-token scalars of the full-state dX.
+// scal: (d mu / NC, 2 d nu / NC), the per-token scalars of the full-state dX.  Like bwd_coef it also leaves
+// dz as the bf16 operands of the tensor-core kernels, and further blocks pack their weight: five launches
+// a slot fewer.
 
 namespace {
 
@@ -704,8 +715,14 @@ __global__ void __launch_bounds__(FC_NT) k_full_coef(Dims d, int T, int TB, cons
                                                      const float* __restrict__ wsum, const int* __restrict__ I,
                                                      const float* __restrict__ dp,
                                                      const float* __restrict__ alpha_pre, float* __restrict__ dz,
-                                                     float* __restrict__ scal, float* __restrict__ colp) {
+                                                     float* __restrict__ scal, float* __restrict__ colp,
+                                                     DzPack pack, WRows wrows, int nblk) {
     pdl_entry();
+    extern __shared__ float dzs[];   // [TB][n] dz, for the packed operands
+    if ((int)blockIdx.x >= nblk) {
+        pack_wrows_of(wrows, (int)blockIdx.x - nblk);
+        return;
+    }
     __shared__ float sh[FC_NT / 32][NCOLP];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int N = d.N, GN = d.G * d.N, n = d.nfull, roff = d.hr ? N : 0;
@@ -733,7 +750,9 @@ __global__ void __launch_bounds__(FC_NT) k_full_coef(Dims d, int T, int TB, cons
             const float h = hpre[t * GN + e];
             const float dy = dhpre[t * GN + e] * h * (1.0f - h);
             const float z = zf[roff + e];
-            dz[t * n + roff + e] = al[q] * dy * rstd;
+            const float v = al[q] * dy * rstd;
+            dz[t * n + roff + e] = v;
+            dzs[tt * n + roff + e] = v;
             drstd += al[q] * dy * z;
             sdy[q] += dy;
             sda[q] += dy * (z * rstd);
@@ -776,7 +795,10 @@ __global__ void __launch_bounds__(FC_NT) k_full_coef(Dims d, int T, int TB, cons
                 const float s = ex / warp_sum(ex);
                 dzr = s * (g - warp_sum(g * s));
             }
-            if (lane < N) dz[t * n + lane] = dzr * lstd;
+            if (lane < N) {
+                dz[t * n + lane] = dzr * lstd;
+                dzs[tt * n + lane] = dzr * lstd;
+            }
             srt += mu * dzr * lstd;
             dmu = -warp_sum(dzr * lstd * ws);
             const float dlstd = warp_sum(dzr * zc);
@@ -799,6 +821,7 @@ __global__ void __launch_bounds__(FC_NT) k_full_coef(Dims d, int T, int TB, cons
     }
     if (d.hr && lane < N) sh[warp][2 * GN + lane] = srt;
     __syncthreads();
+    pack_dz_of(pack, dzs, n, n, t0, ntok);
     for (int c = tid; c < 2 * GN + roff; c += FC_NT) {
         float s = 0.f;
 #pragma unroll
@@ -826,11 +849,13 @@ __global__ void __launch_bounds__(FC_NT) k_full_coef(Dims d, int T, int TB, cons
 cudaError_t launch_full_coef(const Dims& d, int T, const float* dhpre, const float* hpre,
                              const float* zfull, const float* stats, const float* wsum,
                              const int* I, const float* dp, const float* alpha_pre, float* dz,
-                             float* scal, float* colp, int* nblk, cudaStream_t st) {
+                             float* scal, float* colp, int* nblk, const DzPack& pack, const WRows& wrows,
+                             cudaStream_t st) {
     // 8 tokens a block (a token per warp) at few tokens, 32 at many
     const int TB = (T >= 32 * 2 * device_sms()) ? 32 : 8;
     *nblk = (T + TB - 1) / TB;
-    XHC_LAUNCH(st, *nblk, FC_NT, 0, (k_full_coef), d, T, TB, dhpre, hpre, zfull, stats, wsum, I, dp, alpha_pre, dz, scal, colp);
+    XHC_LAUNCH(st, *nblk + wrows_blocks(wrows, FC_NT), FC_NT, (size_t)TB * d.nfull * 4, (k_full_coef), d, T, TB, dhpre, hpre, zfull,
+               stats, wsum, I, dp, alpha_pre, dz, scal, colp, pack, wrows, *nblk);
     return cudaGetLastError();
 }
 

@@ -681,31 +681,11 @@ cudaError_t launch_proj_tc(const uint16_t* X, int T, int K, const uint16_t* Wpac
     return cudaGetLastError();
 }
 
-// dZpack[r][t]: hi / lo bf16 parts of dz[t][o] (r = o for hi, r = n + o for lo, 0 for pad), the
-// K-major B operand of the weight gradient.
-__global__ void k_pack_dz(const float* __restrict__ dz, int ldz, int n, int NB, int T, int Tp,
-                          uint16_t* __restrict__ dzp) {
-    pdl_entry();
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= T) return;
-    for (int o = 0; o < n; ++o) {
-        const float w = dz[(int64_t)t * ldz + o];
-        const __nv_bfloat16 h = __float2bfloat16_rn(w);
-        dzp[(int64_t)o * Tp + t] = __bfloat16_as_ushort(h);
-        dzp[(int64_t)(n + o) * Tp + t] = __bfloat16_as_ushort(__float2bfloat16_rn(w - __bfloat162float(h)));
-    }
-    for (int r = 2 * n; r < NB; ++r) dzp[(int64_t)r * Tp + t] = 0;
-}
-
 // Weight gradient on the tensor cores: part[j][e][o] = sum over the segment's tokens of
 // A[t][e] dz[t][o] (A = X or the active state, [T, E] bf16), with dz split into bf16 hi/lo.
-cudaError_t launch_wgrad_tc(const uint16_t* A, int T, int E, const float* dz, int ldz, int n,
-                            uint16_t* dzpack, const ProjTcPlan& p, float* part, int* err,
-                            cudaStream_t st) {
-    const int Tp = (T + 7) / 8 * 8;  // 16-byte row stride for the tensor map
-    XHC_LAUNCH(st, (T + 255) / 256, 256, 0, (k_pack_dz), dz, ldz, n, p.NB, T, Tp, dzpack);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+cudaError_t launch_wgrad_tc(const uint16_t* A, int T, int E, int n, const uint16_t* dzpack, int Tp,
+                            const ProjTcPlan& p, float* part, int* err, cudaStream_t st) {
+    cudaError_t e;
     CUtensorMap ma, mb;
     // A: [T rows, E inner], box {64 e, 64 tokens}; B: [NB rows, T inner], box {64 tokens, NB}
     if (!make_map_box(&ma, A, (uint64_t)E, (uint64_t)T, 64, BK)) return cudaErrorInvalidValue;
@@ -788,6 +768,7 @@ struct DxArgs {
     float* dotp;          // active epilogue: [k][ncg][T] dot partials over 32-channel groups
     uint16_t* dcopy;      // active epilogue: [G][T][C] copies of d_input (written by slot-0 tiles)
     int ncg;              // active epilogue: C / 32
+    int nsplit;           // full-state dX: parts that a column block's streams are cut into (of two streams at least)
 };
 
 // ACT = true (the instantiated form): active-state epilogue, "streams" are the k active slots j:
@@ -1101,6 +1082,7 @@ constexpr int DG_PF = 4;                     // L2 prefetch distance of the X / 
 // once for all of them (the dense-read gradient of the non-active rows).  Streams m..N-1 come
 // first and the fixed (always active, no d_input) streams 0..m-1 last, so the d_input buffer is
 // released, and the next block's rows loaded, while the last tiles of a block are finished.
+// On calls with few blocks a block's streams are cut into nsplit parts, each a unit of its own.
 // Per tile: MMA 128 x 64 x nfull (A = the block's dZ rows, B = the stream's W rows), TMA-staged X
 // and dX tiles, the result written over the X tile and TMA-stored into dX.
 __global__ void __launch_bounds__(DX_THREADS, 1)
@@ -1150,38 +1132,58 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     pdl_entry();   // barriers and TMEM are set up while the kernel before finishes
-    const int N = a.N;
-    const int ndin = N - a.m;   // leading tiles of a block that may read d_input (streams m..N-1)
-    const int nblk = (a.ntiles > blockIdx.x) ? (int)((a.ntiles - 1 - blockIdx.x) / a.P) + 1 : 0;
-    const int nloc = nblk * N;   // < 2^31: the host checks ntiles * N
-    // local tile n: block n / N of this CTA, position p in the block, stream (p + m) mod N
-    // (32-bit arithmetic: the divisions run per tile in every role)
-    auto decode = [&](int n, int& p, int& tt, int& cb, int& i) {
-        const int b = n / N;
-        p = n - b * N;
-        const int block = (int)blockIdx.x + b * a.P;
-        tt = block / a.CT;
-        cb = block - tt * a.CT;
-        i = p + a.m;
-        if (i >= N) i -= N;
+    const int N = a.N, NU = a.N / a.nsplit;   // streams, streams of a unit (tiles of a "block" below)
+    const int nunits = (int)a.ntiles * a.nsplit;
+    const int nblk = (nunits > (int)blockIdx.x) ? (nunits - 1 - (int)blockIdx.x) / a.P + 1 : 0;
+    const int nloc = nblk * NU;   // < 2^31: the host checks ntiles * N
+    // local tile n: position p of unit `blk` of this CTA (column block unit / nsplit, streams [i0, i0 + NU)).
+    // A unit's leading ndin tiles are its streams from m on, which may read d_input, the fixed ones follow.
+    // Each role walks its tiles with a cursor: the divisions run once a unit.
+    struct Cursor {
+        int p, blk, tt, cb, i0, ndin;
+        __device__ int stream(int NU) const { return p < ndin ? i0 + NU - ndin + p : i0 + p - ndin; }
+    };
+    auto locate = [&](Cursor& c) {
+        const int unit = (int)blockIdx.x + c.blk * a.P;
+        const int block = unit / a.nsplit;
+        c.i0 = (unit - block * a.nsplit) * NU;
+        c.tt = block / a.CT;
+        c.cb = block - c.tt * a.CT;
+        c.ndin = min(NU, max(0, c.i0 + NU - a.m));
+    };
+    auto start = [&](Cursor& c, int n) {
+        c.blk = n / NU;
+        c.p = n - c.blk * NU;
+        locate(c);
+    };
+    auto advance = [&](Cursor& c, int by) {
+        c.p += by;
+        if (c.p >= NU) {
+            do {
+                c.p -= NU;
+                ++c.blk;
+            } while (c.p >= NU);
+            locate(c);
+        }
     };
 
     if (warp == 0) {
         if (lane == 0) {
-            for (int n = 0; n < nloc; ++n) {
+            Cursor cu, pf;   // the tile to load, and the one DG_PF tiles ahead
+            start(cu, 0);
+            start(pf, DG_PF);
+            for (int n = 0; n < nloc; ++n, advance(cu, 1), advance(pf, 1)) {
                 if (*s_abort) break;
-                int p, tt, cb, i;
                 if (DG_PF > 0 && n + DG_PF < nloc) {
                     // the tile DG_PF ahead into L2: its X / dX loads, issued once a stage frees,
                     // then wait for L2 rather than HBM
-                    decode(n + DG_PF, p, tt, cb, i);
-                    tma_prefetch_2d(&tmX, i * a.C + cb * DG_BN, tt * BM);
-                    if (p < ndin) tma_prefetch_2d(&tmD, i * a.C + cb * DG_BN, tt * BM);
-                    if (p == 0)
-                        for (int q = 0; q < a.G; ++q) tma_prefetch_2d(&tmG, cb * DG_BN, q * a.T + tt * BM);
+                    const int i = pf.stream(NU);
+                    tma_prefetch_2d(&tmX, i * a.C + pf.cb * DG_BN, pf.tt * BM);
+                    if (pf.p < pf.ndin) tma_prefetch_2d(&tmD, i * a.C + pf.cb * DG_BN, pf.tt * BM);
+                    if (pf.p == 0)
+                        for (int q = 0; q < a.G; ++q) tma_prefetch_2d(&tmG, pf.cb * DG_BN, q * a.T + pf.tt * BM);
                 }
-                decode(n, p, tt, cb, i);
-                const int blk = n / N;
+                const int p = cu.p, tt = cu.tt, cb = cu.cb, ndin = cu.ndin, blk = cu.blk, i = cu.stream(NU);
                 if (p == 0) {
                     if (blk >= 1 && !mbar_wait(smem_u32(&bars[1]), (uint32_t)((blk - 1) & 1), a.wait_ns)) {
                         atomicExch(a.err, 31);
@@ -1231,9 +1233,12 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
     } else if (warp == 1) {
         if (lane == 0) {
             const uint32_t idesc = idesc_bf16(BM, DG_BN);
+            int p = 0, blk = 0;
             for (int n = 0; n < nloc; ++n) {
-                const int blk = n / N;
-                const int p = n - blk * N;
+                if (n > 0 && ++p == NU) {
+                    p = 0;
+                    ++blk;
+                }
                 const int s = (int)(n & 1);
                 bool ok = (p != 0) || mbar_wait(smem_u32(&bars[0]), (uint32_t)(blk & 1), a.wait_ns);
                 ok = ok && mbar_wait(smem_u32(&bars[2 + s]), (uint32_t)((n >> 1) & 1), a.wait_ns);
@@ -1253,7 +1258,7 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
                 }
                 mma_commit(smem_u32(&bars[4 + s]));              // B stage consumed
                 mma_commit(smem_u32(&bars[8 + s]));              // accumulator ready
-                if (p == N - 1) mma_commit(smem_u32(&bars[1]));  // the block's A rows consumed
+                if (p == NU - 1) mma_commit(smem_u32(&bars[1]));  // the block's A rows consumed
             }
         }
     } else {
@@ -1276,10 +1281,10 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
         int cur_blk = -1;
         uint32_t ib[2] = {0xffffffffu, 0xffffffffu};
         float sa = 0.f, sb = 0.f;
-        for (int n = grp; n < nloc; n += 2) {
-            int p, tt, cb, i;
-            decode(n, p, tt, cb, i);
-            const int blk = n / N;
+        Cursor cu;
+        start(cu, grp);
+        for (int n = grp; n < nloc; n += 2, advance(cu, 2)) {
+            const int p = cu.p, tt = cu.tt, cb = cu.cb, ndin = cu.ndin, blk = cu.blk, i = cu.stream(NU);
             const bool usesg = p < ndin;
             const int t = tt * BM + r;
             // the dense-read weights of this tile's rows: loads issued first, used after the waits
@@ -1402,34 +1407,6 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
     }
 }
 
-// bf16 copies with a padded row stride: dst[r][o] = src[r][o] (o < n), 0 for n <= o < ld
-__global__ void k_pack_rows(WSegs W, int n, int rows, int ld, uint16_t* __restrict__ dst) {
-    pdl_entry();
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)rows * ld) return;
-    const int r = (int)(idx / ld), o = (int)(idx - (long long)r * ld);
-    float v = 0.f;
-    if (o < n) v = seg_elem(W, r, o);
-    dst[idx] = __bfloat16_as_ushort(__float2bfloat16_rn(v));
-}
-
-// rows of three bf16 parts along K: A rows [hi | lo | hi] of dz, B rows [hi | hi | lo] of W, so
-// that sum_k A B = dz_hi W_hi + dz_lo W_hi + dz_hi W_lo (~2^-16 relative)
-__global__ void k_pack3(WSegs W, int n, int rows, int ld, int lo_part, uint16_t* __restrict__ dst) {
-    pdl_entry();
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)rows * ld) return;
-    const int r = (int)(idx / ld), col = (int)(idx - (long long)r * ld);
-    float v = 0.f;
-    if (col < 3 * n) {
-        const int part = col / n, o = col - part * n;
-        const float w = seg_elem(W, r, o);
-        const float hi = __bfloat162float(__float2bfloat16_rn(w));
-        v = (part == lo_part) ? (w - hi) : hi;
-    }
-    dst[idx] = __bfloat16_as_ushort(__float2bfloat16_rn(v));
-}
-
 }  // namespace
 
 // two operand stages of up to two k-blocks each fit the 227 KB of shared memory
@@ -1438,22 +1415,14 @@ bool dxa_tc_ok(int T, int k, int C, int nact) {
            (long long)((T + BM - 1) / BM) * (C / DX_BN) * k < (1LL << 31);   // 32-bit tile indices
 }
 
-cudaError_t launch_dxa_tc(const Dims& d, int slot, int T, const float* dzs, int nact, const WSegs& W,
-                          uint16_t* dz3, uint16_t* w3, const uint16_t* d_input, const float* hpre,
+cudaError_t launch_dxa_tc(const Dims& d, int slot, int T, int nact,
+                          const uint16_t* dz3, const uint16_t* w3, const uint16_t* d_input, const float* hpre,
                           const int* I, const uint16_t* xact, const float* tokmat, float* dxact,
                           float* dotp, uint16_t* dcopy, int* err, cudaStream_t st) {
     const int KC = d.k * d.C;
     const int K3 = 3 * nact;
-    const int ld = (K3 + 7) / 8 * 8;
-    WSegs dzsg;
-    memset(&dzsg, 0, sizeof(dzsg));
-    dzsg.ptr[0] = dzs; dzsg.width[0] = nact; dzsg.off[0] = 0; dzsg.off[1] = nact; dzsg.n = 1;
-    long long tot = (long long)T * ld;
-    XHC_LAUNCH(st, (unsigned)((tot + 255) / 256), 256, 0, (k_pack3), dzsg, nact, T, ld, 1, dz3);
-    tot = (long long)KC * ld;
-    XHC_LAUNCH(st, (unsigned)((tot + 255) / 256), 256, 0, (k_pack3), W, nact, KC, ld, 2, w3);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    const int ld = dxa_ld(nact);
+    cudaError_t e;
     CUtensorMap ma, mb;
     if (!make_map_box(&ma, dz3, (uint64_t)K3, (uint64_t)T, BK, BM, (uint64_t)ld * 2)) return cudaErrorInvalidValue;
     if (!make_map_box(&mb, w3, (uint64_t)K3, (uint64_t)KC, BK, DX_BN, (uint64_t)ld * 2)) return cudaErrorInvalidValue;
@@ -1532,21 +1501,13 @@ bool dx_tc_ok(int T, int N, int C, int nfull, int G) {
            (long long)((T + BM - 1) / BM) * (C / DG_BN) * N < (1LL << 31);   // 32-bit tile indices
 }
 
-cudaError_t launch_dx_tc(const Dims& d, int T, const float* dz, const WSegs& W, uint16_t* dz16,
-                         uint16_t* w16, const uint16_t* X, const uint16_t* dinput, const float* hpre,
+cudaError_t launch_dx_tc(const Dims& d, int T, const uint16_t* dz16,
+                         const uint16_t* w16, const uint16_t* X, const uint16_t* dinput, const float* hpre,
                          const int* I, const float* dxact, const float* scal, int scal_ld,
                          uint16_t* dX, int* err, cudaStream_t st) {
     const int n = d.nfull, NC = d.N * d.C;
-    const int ld = (n + 7) / 8 * 8;
-    WSegs dzs;
-    memset(&dzs, 0, sizeof(dzs));
-    dzs.ptr[0] = dz; dzs.width[0] = n; dzs.off[0] = 0; dzs.off[1] = n; dzs.n = 1;
-    long long tot = (long long)T * ld;
-    XHC_LAUNCH(st, (unsigned)((tot + 255) / 256), 256, 0, (k_pack_rows), dzs, n, T, ld, dz16);
-    tot = (long long)NC * ld;
-    XHC_LAUNCH(st, (unsigned)((tot + 255) / 256), 256, 0, (k_pack_rows), W, n, NC, ld, w16);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    const int ld = dx_ld(n);
+    cudaError_t e;
     CUtensorMap ma, mb, mx, md, mg;
     if (!make_map_box(&ma, dz16, (uint64_t)n, (uint64_t)T, BK, BM, (uint64_t)ld * 2)) return cudaErrorInvalidValue;
     if (!make_map_box(&mb, w16, (uint64_t)n, (uint64_t)NC, BK, DG_BN, (uint64_t)ld * 2)) return cudaErrorInvalidValue;
@@ -1563,7 +1524,21 @@ cudaError_t launch_dx_tc(const Dims& d, int T, const float* dz, const WSegs& W, 
     a.TT = (T + BM - 1) / BM;
     a.CT = d.C / DG_BN;
     a.ntiles = (long long)a.TT * a.CT;   // column blocks, N tiles each
-    a.P = (int)std::min<long long>(num_sms(), a.ntiles);
+    // a block's streams are split over several CTAs where that shortens the longest CTA's work (few
+    // blocks): it takes its units x (their tiles + about 1.5 for the dZ rows and the token data).  512
+    // tokens of N = 16, C = 256 (16 blocks): 40 us unsplit, 16 in 8 parts.
+    const int sms = num_sms();
+    a.nsplit = 1;
+    double least = 1e30;
+    for (int sp = 1; 2 * sp <= d.N; ++sp) {
+        if (d.N % sp != 0) continue;
+        const double cost = (double)((a.ntiles * sp + sms - 1) / sms) * (d.N / sp + 1.5);
+        if (cost < 0.95 * least) {
+            least = cost;
+            a.nsplit = sp;
+        }
+    }
+    a.P = (int)std::min<long long>(sms, a.ntiles * a.nsplit);
     a.X = X; a.dX = dX; a.dinput = dinput; a.hpre = hpre; a.I = I; a.dxact = dxact;
     a.scal = scal; a.scal_ld = scal_ld; a.err = err;
     a.wait_ns = debug_wait_ns();

@@ -413,6 +413,77 @@ __device__ __forceinline__ void pack_rows_of(const PackJob& j, int blk) {
     }
 }
 inline int pack_blocks(const PackJob& j) { return j.dst ? (j.K + PACK_E - 1) / PACK_E : 0; }
+// bf16 operands that the tensor-core backward takes from a slot's (or the full-state) projection-output
+// gradient dz [T][n], written by the coefficient kernel that forms it:
+//   hilo [NB][Tp]  rows 0..n-1 the hi parts, n..2n-1 the lo parts, the rest zero (k_proj_tc's B operand of
+//                  the weight gradient)
+//   rows [T][ld]   the A operand of the input gradient, a token's columns `parts` times over: hi | lo | hi
+//                  (parts 3) or the value rounded once (parts 1), zero from parts * n on
+// null pointers: not wanted.
+struct DzPack {
+    uint16_t *hilo, *rows;
+    int NB, Tp, ld, parts;
+};
+// dz of a block's ntok tokens from t0 on, in shared memory (row stride rs), into the two operands
+__device__ __forceinline__ void pack_dz_of(const DzPack& p, const float* dz, int rs, int n, long long t0, int ntok) {
+    if (p.hilo != nullptr)
+        for (int idx = threadIdx.x; idx < p.NB * ntok; idx += blockDim.x) {
+            const int r = idx / ntok, tt = idx - r * ntok;
+            float v = 0.f;
+            if (r < 2 * n) {
+                v = dz[tt * rs + (r < n ? r : r - n)];
+                if (r >= n) v -= __bfloat162float(__float2bfloat16_rn(v));
+            }
+            p.hilo[(long long)r * p.Tp + t0 + tt] = f2bf(v);
+        }
+    if (p.rows != nullptr)
+        for (int idx = threadIdx.x; idx < ntok * p.ld; idx += blockDim.x) {
+            const int tt = idx / p.ld, c = idx - tt * p.ld;
+            float v = 0.f;
+            if (c < p.parts * n) {
+                const int part = c / n;
+                v = dz[tt * rs + c - part * n];
+                if (part == 1) v -= __bfloat162float(__float2bfloat16_rn(v));
+            }
+            p.rows[(t0 + tt) * p.ld + c] = f2bf(v);
+        }
+}
+// the weight side of the input gradient: dst [rows][ld] bf16, a weight row's n columns `parts` times over
+// (hi | hi | lo, or rounded once), zero from parts * n on; packed by further blocks of the same launch
+struct WRows {
+    WSegs W;
+    int n, rows, ld, parts;
+    uint16_t* dst;   // null: nothing to pack
+};
+constexpr int WROWS_U = 8;   // elements per thread
+__device__ __forceinline__ void pack_wrows_of(const WRows& j, int blk) {
+    const int at = blk * (int)blockDim.x * WROWS_U + threadIdx.x, tot = j.rows * j.ld;   // < 2^31
+    float v[WROWS_U];
+    int part[WROWS_U];
+#pragma unroll
+    for (int u = 0; u < WROWS_U; ++u) {
+        const int idx = at + u * (int)blockDim.x;
+        v[u] = 0.f;
+        part[u] = 0;
+        if (idx < tot) {
+            const int r = idx / j.ld, c = idx - r * j.ld;
+            if (c < j.parts * j.n) {
+                part[u] = c / j.n;
+                v[u] = seg_elem<true>(j.W, r, c - part[u] * j.n);
+            }
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < WROWS_U; ++u) {
+        const int idx = at + u * (int)blockDim.x;
+        if (part[u] == 2) v[u] -= __bfloat162float(__float2bfloat16_rn(v[u]));
+        if (idx < tot) j.dst[idx] = f2bf(v[u]);
+    }
+}
+inline int wrows_blocks(const WRows& j, int threads) {
+    return j.dst ? (int)(((long long)j.rows * j.ld + threads * WROWS_U - 1) / (threads * WROWS_U)) : 0;
+}
+
 // the full-state weight packed, the partial column sums of W_r (null: none) and the slot-0 active weight,
 // in one launch
 cudaError_t launch_pack_full(const PackJob& full, const float* W_r, int N, float* wsump, const PackJob& act,
@@ -421,24 +492,28 @@ cudaError_t launch_pack_full(const PackJob& full, const float* W_r, int N, float
 cudaError_t launch_proj_tc(const uint16_t* X, int T, int K, const uint16_t* Wpack, int nfull,
                            const ProjTcPlan& p, float* part, float* pstats, int* err,
                            cudaStream_t st);
-cudaError_t launch_wgrad_tc(const uint16_t* A, int T, int E, const float* dz, int ldz, int n,
-                            uint16_t* dzpack, const ProjTcPlan& p, float* part, int* err,
-                            cudaStream_t st);
+// dzpack: the hi / lo rows of dz (DzPack::hilo, Tp tokens a row)
+cudaError_t launch_wgrad_tc(const uint16_t* A, int T, int E, int n, const uint16_t* dzpack, int Tp,
+                            const ProjTcPlan& p, float* part, int* err, cudaStream_t st);
 bool dx_tc_ok(int T, int N, int C, int nfull, int G);
 bool dxa_tc_ok(int T, int k, int C, int nact);
 // dX_act += dZ_act W_act^T (three-term bf16 split on the tensor cores) + H_pre[slot][I_j] d_input
 //           - cx x_act (the write-back's own term, cx per token in tokmat);
 // in the same pass: dotp[j][g][t] = <x_act_j, d_input> over channels 32 g .. 32 g + 31, and the
 // copy dcopy[slot][t][:] = d_input[t][:]
-cudaError_t launch_dxa_tc(const Dims& d, int slot, int T, const float* dzs, int nact, const WSegs& W,
-                          uint16_t* dz3, uint16_t* w3, const uint16_t* d_input, const float* hpre,
+// (dz3, w3: the three-part operands, DzPack / WRows with parts 3)
+inline int dxa_ld(int nact) { return (3 * nact + 7) / 8 * 8; }
+cudaError_t launch_dxa_tc(const Dims& d, int slot, int T, int nact,
+                          const uint16_t* dz3, const uint16_t* w3, const uint16_t* d_input, const float* hpre,
                           const int* I, const uint16_t* xact, const float* tokmat, float* dxact,
                           float* dotp, uint16_t* dcopy, int* err, cudaStream_t st);
 // dH_pre[t][slot][I_j] = sum over the C/32 groups g of dotp[j][g][t] (g in order)
 cudaError_t launch_dots_act(const Dims& d, int slot, int T, const float* dotp, const int* I, float* dhpre,
                             cudaStream_t st);
-cudaError_t launch_dx_tc(const Dims& d, int T, const float* dz, const WSegs& W, uint16_t* dz16,
-                         uint16_t* w16, const uint16_t* X, const uint16_t* dinput, const float* hpre,
+// (dz16, w16: the operands rounded once, parts 1)
+inline int dx_ld(int nfull) { return (nfull + 7) / 8 * 8; }
+cudaError_t launch_dx_tc(const Dims& d, int T, const uint16_t* dz16,
+                         const uint16_t* w16, const uint16_t* X, const uint16_t* dinput, const float* hpre,
                          const int* I, const float* dxact, const float* scal, int scal_ld,
                          uint16_t* dX, int* err, cudaStream_t st);
 int wb_nslice(int C);
@@ -538,7 +613,8 @@ cudaError_t launch_bwd_coef(const Dims& d, int slot, int T, const float* red, in
                             const float* zact, const float* rs, const float* p,
                             const float* hpost, const double* gram, const float* alpha_post,
                             const float* alpha_res, const float* b_res,
-                            float* tokmat, float* dz, float* dp, float* colp, int* nblk, cudaStream_t st);
+                            float* tokmat, float* dz, float* dp, float* colp, int* nblk, const DzPack& pack,
+                            const WRows& wrows, cudaStream_t st);
 // adds the column sums over the blocks' partials colp [nblk][ncol] to up to four targets: target q
 // takes columns off[q] .. off[q] + n[q] - 1
 struct ColOut {
@@ -563,7 +639,8 @@ cudaError_t launch_full_dots(const Dims& d, int T, const uint16_t* X, const uint
 cudaError_t launch_full_coef(const Dims& d, int T, const float* dhpre, const float* hpre,
                              const float* zfull, const float* stats, const float* wsum,
                              const int* I, const float* dp, const float* alpha_pre, float* dz,
-                             float* scal, float* colp, int* nblk, cudaStream_t st);
+                             float* scal, float* colp, int* nblk, const DzPack& pack, const WRows& wrows,
+                             cudaStream_t st);
 cudaError_t launch_full_dx(const Dims& d, int T, const float* dz, const WSegs& W,
                            const uint16_t* X, const uint16_t* dinput, const float* hpre,
                            const int* I, const float* dxact, const float* scal,

@@ -24,6 +24,12 @@ CASES = {
     "coef_k8_iters64": (Config.full(8, 8, 8, 8, True, sinkhorn_iters=64, seq_len=4900), 4900, {}),
     "coef_k3_iters0": (Config.full(5, 3, 1, 32, True, sinkhorn_iters=0), 130, {}),
     # two conv components (a Gram-Schmidt basis smaller than its maximum), N with idle lanes
+    # full-state dX on few blocks: the streams of a block in parts (of 2, 3 or all streams; fixed ones in
+    # the first part, none, all), ragged token tiles
+    "dx_split_N16_m3": (Config.flash(16, 4, 3, 64, 2, seq_len=150), 300, {}),
+    "dx_split_N12_m0": (Config.full(12, 4, 0, 128, False), 131, {}),
+    "dx_split_N9": (Config.full(9, 4, 2, 128, False), 200, {}),
+    "dx_split_mhc": (Config.mhc(4, 128), 129, {}),
     "coef_N27_conv1": (Config.flash(27, 4, 2, 64, 2, conv_k=(4,), seq_len=131), 262, {}),
 }
 
