@@ -23,6 +23,7 @@
 //             the backward reductions and apply in one pass
 #pragma once
 #include <algorithm>
+#include <type_traits>
 
 #include "xhc_internal.cuh"
 
@@ -351,36 +352,42 @@ __global__ void __launch_bounds__(WT, 2) k_wb_gram2(Dims d, int slot, int T, int
             const int tn = tb + UB + u;
             on[u] = (tn < n1) ? *reinterpret_cast<const uint2*>(po + (long long)tn * C) : make_uint2(0u, 0u);
         }
-#pragma unroll
-        for (int u = 0; u < UB; ++u) {
+        auto token = [&](int u) {
             const int tt = tb + u;
-            if (tt < n1) {
-                float2 uu[2][4];
+            float2 uu[2][4];
 #pragma unroll
-                for (int p = 0; p < 2; ++p) {
-                    const float2 o = u2f2(p == 0 ? ob[u].x : ob[u].y);
-                    w[p][KW - 1 + u] = o;
-                    float2 g[3];
-                    conv_blk<KW, KS>(tw[p], w[p], u, g);
-                    uu[p][0] = o;
-                    uu[p][1] = g[0];
-                    uu[p][2] = g[1];
-                    uu[p][3] = g[2];
-                }
-                float v[16];
-                int q = 0;
-#pragma unroll
-                for (int a = 0; a < 4; ++a)
-#pragma unroll
-                    for (int b = 0; b <= a; ++b)
-                        v[q++] = (a < K) ? fmaf(uu[1][a].y, uu[1][b].y,
-                                                fmaf(uu[1][a].x, uu[1][b].x, dot2(uu[0][a], uu[0][b])))
-                                         : 0.f;
-#pragma unroll
-                for (int r = 10; r < 16; ++r) v[r] = 0.f;
-                const float tot = WRed<16, 16>::run(v, lane);
-                if ((lane & 1) == 0) wsh[(tt * (WT / 32) + warp) * 16 + (lane >> 1)] = tot;
+            for (int p = 0; p < 2; ++p) {
+                const float2 o = u2f2(p == 0 ? ob[u].x : ob[u].y);
+                w[p][KW - 1 + u] = o;
+                float2 g[3];
+                conv_blk<KW, KS>(tw[p], w[p], u, g);
+                uu[p][0] = o;
+                uu[p][1] = g[0];
+                uu[p][2] = g[1];
+                uu[p][3] = g[2];
             }
+            float v[16];
+            int q = 0;
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b <= a; ++b)
+                    v[q++] = (a < K) ? fmaf(uu[1][a].y, uu[1][b].y,
+                                            fmaf(uu[1][a].x, uu[1][b].x, dot2(uu[0][a], uu[0][b])))
+                                     : 0.f;
+#pragma unroll
+            for (int r = 10; r < 16; ++r) v[r] = 0.f;
+            const float tot = WRed<16, 16>::run(v, lane);
+            if ((lane & 1) == 0) wsh[(tt * (WT / 32) + warp) * 16 + (lane >> 1)] = tot;
+        };
+        // a whole block without a branch between its tokens: their reductions interleave
+        if (tb + UB <= n1) {
+#pragma unroll
+            for (int u = 0; u < UB; ++u) token(u);
+        } else {
+#pragma unroll
+            for (int u = 0; u < UB; ++u)
+                if (tb + u < n1) token(u);
         }
 #pragma unroll
         for (int p = 0; p < 2; ++p) ring_shift<KW>(w[p]);
@@ -402,9 +409,9 @@ __global__ void __launch_bounds__(WT, 2) k_wb_gram2(Dims d, int slot, int T, int
 // the out value and the k active values of its channel pair PD - 1 tokens ahead with cp.async.
 
 template <int KM>
-struct FRing {
-    uint32_t o[PD][WT];
-    uint32_t x[PD][KM][WT];
+struct FRing {   // two blocks of UB tokens
+    uint32_t o[2 * UB][WT];
+    uint32_t x[2 * UB][KM][WT];
 };
 
 template <int KM, int KW, int KS>
@@ -434,22 +441,26 @@ __global__ void __launch_bounds__(WT) k_wb_fwd(Dims d, int slot, int T, int TB,
     const uint16_t* po = out + t0 * C + c;
     const uint16_t* px = xact + t0 * k * C + c;
     const long long kC = (long long)k * C;
-    auto issue = [&](int sl, int tn) {
-        if (act && tn < ntok) {
-            cpa4(&R.o[sl][threadIdx.x], po);
-            const uint16_t* pj = px;
+    // the block of tokens from tn on into ring half `half`, one commit group
+    auto issue = [&](int half, int tn) {
 #pragma unroll
-            for (int j = 0; j < KM; ++j) {
-                if (j < k) cpa4(&R.x[sl][j][threadIdx.x], pj);
-                pj += C;
+        for (int u = 0; u < UB; ++u) {
+            const int sl = half * UB + u;
+            if (act && tn + u < ntok) {
+                cpa4(&R.o[sl][threadIdx.x], po);
+                const uint16_t* pj = px;
+#pragma unroll
+                for (int j = 0; j < KM; ++j) {
+                    if (j < k) cpa4(&R.x[sl][j][threadIdx.x], pj);
+                    pj += C;
+                }
             }
+            po += C;
+            px += kC;
         }
-        po += C;
-        px += kC;
         cpa_commit();
     };
-#pragma unroll
-    for (int q = 0; q < PD - 1; ++q) issue(q, q);
+    issue(0, 0);
     for (int idx = threadIdx.x; idx < ntok * KM * 4; idx += WT) {
         const int tt = idx / (KM * 4), q = idx - tt * (KM * 4);
         Esh[idx] = (q < k * 4) ? emat[(t0 + tt) * TOKMAT + q] : 0.f;
@@ -472,65 +483,74 @@ __global__ void __launch_bounds__(WT) k_wb_fwd(Dims d, int slot, int T, int TB,
     uint16_t* pn = last ? nullptr : xact_next + t0 * k * C + c;
     const long long NC = (long long)d.N * C;
     __syncthreads();
-    constexpr int RU = UB;
-    for (int tb = 0; tb < ntok; tb += RU) {
-#pragma unroll
-        for (int u = 0; u < RU; ++u) {
-            const int tt = tb + u;
-            if (tt < ntok) {
-                const int sl = u % PD;
-                issue((u + PD - 1) % PD, tt + PD - 1);
-                cpa_wait<PD - 1>();
-                if (act) {
-                    const float2 o = u2f2(R.o[sl][threadIdx.x]);
-                    float2 uu[4] = {o, f2z(), f2z(), f2z()};
-                    if constexpr (KW > 0) {
-                        w[KW - 1 + u] = o;
-                        float2 g[3];
-                        conv_blk<KW, KS>(tw, w, u, g);
-                        uu[1] = g[0];
-                        uu[2] = g[1];
-                        uu[3] = g[2];
-                    }
-                    float2 x[KM];
-#pragma unroll
-                    for (int j = 0; j < KM; ++j) x[j] = (j < k) ? u2f2(R.x[sl][j][threadIdx.x]) : f2z();
-                    const float4* E4 = reinterpret_cast<const float4*>(Esh + tt * KM * 4);
-                    const float4* H4 = reinterpret_cast<const float4*>(Hsh + tt * KM * KM);
-#pragma unroll
-                    for (int j = 0; j < KM; ++j) {
-                        if (j >= k) continue;
-                        float2 v;
-                        if (last) {
-                            v = f2z();
-#pragma unroll
-                            for (int q = 0; q < KM / 4; ++q) {
-                                const float4 h = H4[j * (KM / 4) + q];
-                                v = fma2(h.x, x[4 * q + 0], v);
-                                v = fma2(h.y, x[4 * q + 1], v);
-                                v = fma2(h.z, x[4 * q + 2], v);
-                                v = fma2(h.w, x[4 * q + 3], v);
-                            }
-                        } else {
-                            v = x[j];
-                        }
-                        const float4 e = E4[j];
-                        v = fma2(e.x, uu[0], v);
-                        if constexpr (KW > 0) {
-                            v = fma2(e.y, uu[1], v);
-                            v = fma2(e.z, uu[2], v);
-                            v = fma2(e.w, uu[3], v);
-                        }
-                        if (last)
-                            st2(pX + (long long)Ish[tt * KM + j] * C, v);
-                        else
-                            st2(pn + (long long)j * C, v);
-                    }
-                }
-                if (last) pX += NC;
-                else pn += kC;
+    for (int tb = 0, half = 0; tb < ntok; tb += UB, half ^= 1) {
+        issue(half ^ 1, tb + UB);
+        cpa_wait<1>();
+        auto token = [&](auto lastc, int u) {
+            constexpr bool LAST = decltype(lastc)::value;
+            const int tt = tb + u, sl = half * UB + u;
+            const float2 o = u2f2(R.o[sl][threadIdx.x]);
+            float2 uu[4] = {o, f2z(), f2z(), f2z()};
+            if constexpr (KW > 0) {
+                w[KW - 1 + u] = o;
+                float2 g[3];
+                conv_blk<KW, KS>(tw, w, u, g);
+                uu[1] = g[0];
+                uu[2] = g[1];
+                uu[3] = g[2];
             }
+            float2 x[KM];
+#pragma unroll
+            for (int j = 0; j < KM; ++j) x[j] = (j < k) ? u2f2(R.x[sl][j][threadIdx.x]) : f2z();
+            const float4* E4 = reinterpret_cast<const float4*>(Esh + tt * KM * 4);
+            const float4* H4 = reinterpret_cast<const float4*>(Hsh + tt * KM * KM);
+#pragma unroll
+            for (int j = 0; j < KM; ++j) {
+                if (j >= k) continue;
+                float2 v;
+                if constexpr (LAST) {
+                    v = f2z();
+#pragma unroll
+                    for (int q = 0; q < KM / 4; ++q) {
+                        const float4 h = H4[j * (KM / 4) + q];
+                        v = fma2(h.x, x[4 * q + 0], v);
+                        v = fma2(h.y, x[4 * q + 1], v);
+                        v = fma2(h.z, x[4 * q + 2], v);
+                        v = fma2(h.w, x[4 * q + 3], v);
+                    }
+                } else {
+                    v = x[j];
+                }
+                const float4 e = E4[j];
+                v = fma2(e.x, uu[0], v);
+                if constexpr (KW > 0) {
+                    v = fma2(e.y, uu[1], v);
+                    v = fma2(e.z, uu[2], v);
+                    v = fma2(e.w, uu[3], v);
+                }
+                if constexpr (LAST)
+                    st2(pX + u * NC + (long long)Ish[tt * KM + j] * C, v);
+                else
+                    st2(pn + u * kC + (long long)j * C, v);
+            }
+        };
+        // a whole block without a branch between its tokens: their chains interleave
+        auto block = [&](auto lastc) {
+            if (tb + UB <= ntok) {
+#pragma unroll
+                for (int u = 0; u < UB; ++u) token(lastc, u);
+            } else {
+#pragma unroll
+                for (int u = 0; u < UB; ++u)
+                    if (tb + u < ntok) token(lastc, u);
+            }
+        };
+        if (act) {
+            if (last) block(std::true_type{});
+            else block(std::false_type{});
         }
+        if (last) pX += UB * NC;
+        else pn += UB * kC;
         if constexpr (KW > 0) ring_shift<KW>(w);
     }
     cpa_wait<0>();
@@ -710,10 +730,9 @@ __global__ void __launch_bounds__(WT) k_wb_bred(Dims d, int slot, int T, int TB,
 // and C a multiple of WSL2 (every thread in range).
 
 template <int KM>
-struct BRing2 {
-    uint2 o[PD][WT];
-    uint2 x[PD][KM][WT];
-    uint4 dn[PD][KM][WT];
+struct BRing2 {   // two blocks of UB tokens
+    uint2 o[2 * UB][WT];
+    uint4 v[2 * UB][KM][WT];   // dn_j: four fp32, or at the last slot dX's four bf16 and x_j's four
 };
 
 template <int KM, int NV>
@@ -734,8 +753,8 @@ __global__ void __launch_bounds__(WT, 2) k_wb_bred2(Dims d, int slot, int T, int
     float* wsh = reinterpret_cast<float*>(Ish + TB * KM);                 // [TB][WT/32][NVP]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int slice = blockIdx.x, C = d.C, k = KM;
-    const bool last = (slot == d.G - 1);
-    const int nv = last ? KM * 4 + KM * KM : KM * 4;
+    constexpr bool LAST = NV >= KM * 4 + KM * KM;   // the last slot: bf16 rows of dX, and Q besides P
+    constexpr int nv = LAST ? KM * 4 + KM * KM : KM * 4;
     const int c = slice * WSL2 + 4 * threadIdx.x;
     long long t0, t1, send;
     int pos0;
@@ -751,104 +770,111 @@ __global__ void __launch_bounds__(WT, 2) k_wb_bred2(Dims d, int slot, int T, int
     const uint16_t* pX = dX + t0 * d.N * C + c;
     const float* pd = dxact + t0 * k * C + c;
     const long long kC = (long long)k * C, NC = (long long)d.N * C;
-    auto issue = [&](int sl, int tn) {
-        if (tn < ntok) {
-            cpa8(&R.o[sl][threadIdx.x], po);
+    // the block of tokens from tn on into ring half `half`, one commit group
+    auto issue = [&](int half, int tn) {
 #pragma unroll
-            for (int j = 0; j < KM; ++j) {
-                if (last) {
-                    cpa8(&R.x[sl][j][threadIdx.x], px + (long long)j * C);
-                    cpa8(&R.dn[sl][j][threadIdx.x], pX + (long long)Ish[tn * KM + j] * C);
-                } else {
-                    cpa16(&R.dn[sl][j][threadIdx.x], pd + (long long)j * C);
+        for (int u = 0; u < UB; ++u) {
+            const int sl = half * UB + u;
+            if (tn + u < ntok) {
+                cpa8(&R.o[sl][threadIdx.x], po);
+#pragma unroll
+                for (int j = 0; j < KM; ++j) {
+                    if (LAST) {
+                        cpa8(&R.v[sl][j][threadIdx.x].x, pX + (long long)Ish[(tn + u) * KM + j] * C);
+                        cpa8(&R.v[sl][j][threadIdx.x].z, px + (long long)j * C);
+                    } else {
+                        cpa16(&R.v[sl][j][threadIdx.x], pd + (long long)j * C);
+                    }
                 }
             }
-        }
-        po += C;
-        if (last) {
-            px += kC;
-            pX += NC;
-        } else {
-            pd += kC;
+            po += C;
+            if (LAST) {
+                px += kC;
+                pX += NC;
+            } else {
+                pd += kC;
+            }
         }
         cpa_commit();
     };
-#pragma unroll
-    for (int q = 0; q < PD - 1; ++q) issue(q, q);
+    issue(0, 0);
     float2 tw[2][3][KW], w[2][KW + UB - 1];
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
         taps_reg<KW, KS>(d, cw, c + 2 * p, true, tw[p]);
         ring_init_b<KW>(d, cw, out, c + 2 * p, true, t0, pos0, w[p]);
     }
-    for (int tb = 0; tb < ntok; tb += UB) {
+    for (int tb = 0, half = 0; tb < ntok; tb += UB, half ^= 1) {
+        issue(half ^ 1, tb + UB);
+        cpa_wait<1>();
+        auto token = [&](int u) {
+            const int tt = tb + u, sl = half * UB + u;
+            float2 uu[2][4], dn[2][KM], x[2][KM];
+            const uint2 orow = R.o[sl][threadIdx.x];
 #pragma unroll
-        for (int u = 0; u < UB; ++u) {
-            const int tt = tb + u;
-            if (tt < ntok) {
-                const int sl = u % PD;
-                issue((u + PD - 1) % PD, tt + PD - 1);
-                cpa_wait<PD - 1>();
-                float2 uu[2][4], dn[2][KM], x[2][KM];
-                const uint2 orow = R.o[sl][threadIdx.x];
+            for (int p = 0; p < 2; ++p) {
+                const float2 o = u2f2(p == 0 ? orow.x : orow.y);
+                w[p][KW - 1 + u] = o;
+                float2 g[3];
+                conv_blk<KW, KS>(tw[p], w[p], u, g);
+                uu[p][0] = o;
+                uu[p][1] = g[0];
+                uu[p][2] = g[1];
+                uu[p][3] = g[2];
+            }
 #pragma unroll
-                for (int p = 0; p < 2; ++p) {
-                    const float2 o = u2f2(p == 0 ? orow.x : orow.y);
-                    w[p][KW - 1 + u] = o;
-                    float2 g[3];
-                    conv_blk<KW, KS>(tw[p], w[p], u, g);
-                    uu[p][0] = o;
-                    uu[p][1] = g[0];
-                    uu[p][2] = g[1];
-                    uu[p][3] = g[2];
-                }
-#pragma unroll
-                for (int j = 0; j < KM; ++j) {
-                    const uint4 r = R.dn[sl][j][threadIdx.x];
-                    if (last) {
-                        const uint2 rb = *reinterpret_cast<const uint2*>(&r);
-                        dn[0][j] = u2f2(rb.x);
-                        dn[1][j] = u2f2(rb.y);
-                        const uint2 xr = R.x[sl][j][threadIdx.x];
-                        x[0][j] = u2f2(xr.x);
-                        x[1][j] = u2f2(xr.y);
-                    } else {
-                        dn[0][j] = make_float2(__uint_as_float(r.x), __uint_as_float(r.y));
-                        dn[1][j] = make_float2(__uint_as_float(r.z), __uint_as_float(r.w));
-                        x[0][j] = x[1][j] = f2z();
-                    }
-                }
-                float v[NVP];
-#pragma unroll
-                for (int q = 0; q < NVP; ++q) v[q] = 0.f;
-#pragma unroll
-                for (int j = 0; j < KM; ++j)
-#pragma unroll
-                    for (int a = 0; a < 4; ++a)
-                        if (j * 4 + a < NVP)
-                            v[j * 4 + a] = fmaf(dn[1][j].y, uu[1][a].y,
-                                                fmaf(dn[1][j].x, uu[1][a].x, dot2(dn[0][j], uu[0][a])));
-                if constexpr (NVP >= KM * 4 + KM * KM) {
-                    if (last) {
-#pragma unroll
-                        for (int j = 0; j < KM; ++j)
-#pragma unroll
-                            for (int i = 0; i < KM; ++i)
-                                v[KM * 4 + j * KM + i] = fmaf(dn[1][j].y, x[1][i].y,
-                                                              fmaf(dn[1][j].x, x[1][i].x, dot2(dn[0][j], x[0][i])));
-                    }
-                }
-                float* dst = wsh + ((size_t)tt * (WT / 32) + warp) * NVP;
-                if constexpr (NV == 16) {
-                    const float tot = WRed<16, 16>::run(v, lane);
-                    if ((lane & 1) == 0) dst[lane >> 1] = tot;
+            for (int j = 0; j < KM; ++j) {
+                const uint4 r = R.v[sl][j][threadIdx.x];
+                if constexpr (LAST) {
+                    dn[0][j] = u2f2(r.x);
+                    dn[1][j] = u2f2(r.y);
+                    x[0][j] = u2f2(r.z);
+                    x[1][j] = u2f2(r.w);
                 } else {
-                    float tot[NV / 32];
-                    wred32<NV / 32>(v, lane, tot);
-#pragma unroll
-                    for (int bb = 0; bb < NV / 32; ++bb) dst[bb * 32 + lane] = tot[bb];
+                    dn[0][j] = make_float2(__uint_as_float(r.x), __uint_as_float(r.y));
+                    dn[1][j] = make_float2(__uint_as_float(r.z), __uint_as_float(r.w));
+                    x[0][j] = x[1][j] = f2z();
                 }
             }
+            float v[NVP];
+#pragma unroll
+            for (int q = 0; q < NVP; ++q) v[q] = 0.f;
+#pragma unroll
+            for (int j = 0; j < KM; ++j)
+#pragma unroll
+                for (int a = 0; a < 4; ++a)
+                    if (j * 4 + a < NVP)
+                        v[j * 4 + a] = fmaf(dn[1][j].y, uu[1][a].y,
+                                            fmaf(dn[1][j].x, uu[1][a].x, dot2(dn[0][j], uu[0][a])));
+            if constexpr (NVP >= KM * 4 + KM * KM) {
+                if constexpr (LAST) {
+#pragma unroll
+                    for (int j = 0; j < KM; ++j)
+#pragma unroll
+                        for (int i = 0; i < KM; ++i)
+                            v[KM * 4 + j * KM + i] = fmaf(dn[1][j].y, x[1][i].y,
+                                                          fmaf(dn[1][j].x, x[1][i].x, dot2(dn[0][j], x[0][i])));
+                }
+            }
+            float* dst = wsh + ((size_t)tt * (WT / 32) + warp) * NVP;
+            if constexpr (NV == 16) {
+                const float tot = WRed<16, 16>::run(v, lane);
+                if ((lane & 1) == 0) dst[lane >> 1] = tot;
+            } else {
+                float tot[NV / 32];
+                wred32<NV / 32>(v, lane, tot);
+#pragma unroll
+                for (int bb = 0; bb < NV / 32; ++bb) dst[bb * 32 + lane] = tot[bb];
+            }
+        };
+        // a whole block without a branch between its tokens: their reductions interleave
+        if (tb + UB <= ntok) {
+#pragma unroll
+            for (int u = 0; u < UB; ++u) token(u);
+        } else {
+#pragma unroll
+            for (int u = 0; u < UB; ++u)
+                if (tb + u < ntok) token(u);
         }
 #pragma unroll
         for (int p = 0; p < 2; ++p) ring_shift<KW>(w[p]);
@@ -876,9 +902,9 @@ __global__ void __launch_bounds__(WT, 2) k_wb_bred2(Dims d, int slot, int T, int
 // the backward of the slot's pre-map.
 
 template <int KM>
-struct ARing {
-    uint32_t o[PD][WT];
-    uint2 dn[PD][KM][WT];
+struct ARing {   // two blocks of UB tokens
+    uint32_t o[2 * UB][WT];
+    uint2 dn[2 * UB][KM][WT];
 };
 
 // HALO: the variant for a call on a later chunk of its sequences, which also returns the
@@ -944,25 +970,29 @@ __global__ void __launch_bounds__(WT, 2) k_wb_bapp(Dims d, int slot, int T, int 
     float* pxo = dxact_out + t0 * k * C + c;
     uint16_t* pdo = d_out + t0 * C + c;
     const long long kC = (long long)k * C, NC = (long long)d.N * C;
-    auto issue = [&](int sl, int tn) {
-        if (act && tn < ntok) {
-            cpa4(&R.o[sl][threadIdx.x], po);
+    // the block of tokens from tn on into ring half `half`, one commit group
+    auto issue = [&](int half, int tn) {
 #pragma unroll
-            for (int j = 0; j < KM; ++j) {
-                if (j >= k) continue;
-                if (last)
-                    cpa4(&R.dn[sl][j][threadIdx.x], pX + (long long)Ish[tn * KM + j] * C);
-                else
-                    cpa8(&R.dn[sl][j][threadIdx.x], pd + (long long)j * C);
+        for (int u = 0; u < UB; ++u) {
+            const int sl = half * UB + u;
+            if (act && tn + u < ntok) {
+                cpa4(&R.o[sl][threadIdx.x], po);
+#pragma unroll
+                for (int j = 0; j < KM; ++j) {
+                    if (j >= k) continue;
+                    if (last)
+                        cpa4(&R.dn[sl][j][threadIdx.x], pX + (long long)Ish[(tn + u) * KM + j] * C);
+                    else
+                        cpa8(&R.dn[sl][j][threadIdx.x], pd + (long long)j * C);
+                }
             }
+            po += C;
+            if (last) pX += NC;
+            else pd += kC;
         }
-        po += C;
-        if (last) pX += NC;
-        else pd += kC;
         cpa_commit();
     };
-#pragma unroll
-    for (int q = 0; q < PD - 1; ++q) issue(q, q);
+    issue(0, 0);
     // pend: the block ring of pending outputs, slot KW - 1 + u - i <-> output tb + u - i
     float2 tw[3][KW > 0 ? KW : 1], w[NR], pend[NR];
     float2 acc[3][KW > 0 ? KW : 1];
@@ -979,110 +1009,121 @@ __global__ void __launch_bounds__(WT, 2) k_wb_bapp(Dims d, int slot, int T, int 
     // the halo gradient (a call on a later chunk): rows of this sequence, this channel pair
     float* dhalo_row = (HALO && KW > 0 && cw.dhalo != nullptr && pos0 == 0)
                            ? cw.dhalo + (t0 / d.S) * (d.kapmax - 1) * C + c : nullptr;
-    for (int tb = 0; tb < nloop; tb += RU) {
+    // the work of token tt (position u of its block, ring slot sl); FULL: a token of the run itself, as the
+    // whole block is, so that no branch parts its tokens and their chains interleave
+    auto token = [&](auto full, auto lastc, int u, int tt, int sl) {
+        constexpr bool FULL = decltype(full)::value, LAST = decltype(lastc)::value;
+        float2 du[4] = {f2z(), f2z(), f2z(), f2z()};
+        if (FULL || tt < ntok) {
+            const float2 o = u2f2(R.o[sl][threadIdx.x]);
+            float2 dn[KM];
 #pragma unroll
-        for (int u = 0; u < RU; ++u) {
-            const int tt = tb + u;
-            if (tt < nloop) {
-                const int sl = u % PD;
-                issue((u + PD - 1) % PD, tt + PD - 1);
-                cpa_wait<PD - 1>();
-                if (act) {
-                    float2 du[4] = {f2z(), f2z(), f2z(), f2z()};
-                    if (tt < ntok) {
-                        const float2 o = u2f2(R.o[sl][threadIdx.x]);
-                        float2 dn[KM];
-#pragma unroll
-                        for (int j = 0; j < KM; ++j) {
-                            dn[j] = f2z();
-                            if (j < k) {
-                                const uint2 r = R.dn[sl][j][threadIdx.x];
-                                dn[j] = last ? u2f2(r.x) : make_float2(__uint_as_float(r.x), __uint_as_float(r.y));
-                            }
-                        }
-                        const float4* E4 = reinterpret_cast<const float4*>(Esh + tt * KM * 4);
-#pragma unroll
-                        for (int j = 0; j < KM; ++j) {
-                            if (j >= k) continue;
-                            const float4 e = E4[j];
-                            du[0] = fma2s(e.x, dn[j], du[0]);
-                            if constexpr (KW > 0) {
-                                du[1] = fma2s(e.y, dn[j], du[1]);
-                                du[2] = fma2s(e.z, dn[j], du[2]);
-                                du[3] = fma2s(e.w, dn[j], du[3]);
-                            }
-                        }
-                        if constexpr (KW > 0) {
-                            w[KW - 1 + u] = o;
-                            float2 g[3];
-                            conv_blk<KW, KS>(tw, w, u, g);
-                            const float2 uu[4] = {o, g[0], g[1], g[2]};
-                            const float4* D4 = reinterpret_cast<const float4*>(Dsh + tt * 16);
-#pragma unroll
-                            for (int a = 0; a < 4; ++a) {
-                                const float4 m = D4[a];
-                                du[a] = fma2s(m.x, uu[0], du[a]);
-                                du[a] = fma2s(m.y, uu[1], du[a]);
-                                du[a] = fma2s(m.z, uu[2], du[a]);
-                                du[a] = fma2s(m.w, uu[3], du[a]);
-                            }
-                        }
-                        if (last && tt < n1) {
-                            const float4* H4 = reinterpret_cast<const float4*>(Hsh + tt * KM * KM);
-                            float2 v[KM];
-#pragma unroll
-                            for (int i = 0; i < KM; ++i) v[i] = f2z();
-#pragma unroll
-                            for (int j = 0; j < KM; ++j) {
-                                if (j >= k) continue;
-#pragma unroll
-                                for (int q = 0; q < KM / 4; ++q) {
-                                    const float4 h = H4[j * (KM / 4) + q];
-                                    v[4 * q + 0] = fma2s(h.x, dn[j], v[4 * q + 0]);
-                                    v[4 * q + 1] = fma2s(h.y, dn[j], v[4 * q + 1]);
-                                    v[4 * q + 2] = fma2s(h.z, dn[j], v[4 * q + 2]);
-                                    v[4 * q + 3] = fma2s(h.w, dn[j], v[4 * q + 3]);
-                                }
-                            }
-#pragma unroll
-                            for (int i = 0; i < KM; ++i)
-                                if (i < k) *reinterpret_cast<float2*>(pxo + (long long)i * C) = v[i];
-                            pxo += kC;
-                        }
-                    } else if constexpr (KW > 0) {
-                        w[KW - 1 + u] = f2z();   // past the sequence end
-                    }
-                    if constexpr (KW == 0) {
-                        if (tt < n1) {
-                            st2(pdo, du[0]);
-                            pdo += C;
-                        }
-                    } else {
-                        // conv weight gradient of the run's tokens
-                        if (tt < n1) {
-#pragma unroll
-                            for (int j = 0; j < 3; ++j)
-#pragma unroll
-                                for (int i = 0; i < KW; ++i) {
-                                    if (i >= ntap<KW, KS>(j)) continue;
-                                    const float2 o = w[KW - 1 + u - i];
-                                    acc[j][i] = ffma2(du[1 + j], o, acc[j][i]);
-                                }
-                        }
-                        // d_out[t - i] += w_j[i] du_{1+j}[t]
-                        pend[KW - 1 + u] = du[0];
-#pragma unroll
-                        for (int i = 0; i < KW; ++i) {
-#pragma unroll
-                            for (int j = 0; j < 3; ++j) {
-                                if (i >= ntap<KW, KS>(j)) continue;
-                                float2& q = pend[KW - 1 + u - i];
-                                q = ffma2(tw[j][i], du[1 + j], q);
-                            }
-                        }
-                    }
+            for (int j = 0; j < KM; ++j) {
+                dn[j] = f2z();
+                if (j < k) {
+                    const uint2 r = R.dn[sl][j][threadIdx.x];
+                    dn[j] = LAST ? u2f2(r.x) : make_float2(__uint_as_float(r.x), __uint_as_float(r.y));
                 }
             }
+            const float4* E4 = reinterpret_cast<const float4*>(Esh + tt * KM * 4);
+#pragma unroll
+            for (int j = 0; j < KM; ++j) {
+                if (j >= k) continue;
+                const float4 e = E4[j];
+                du[0] = fma2s(e.x, dn[j], du[0]);
+                if constexpr (KW > 0) {
+                    du[1] = fma2s(e.y, dn[j], du[1]);
+                    du[2] = fma2s(e.z, dn[j], du[2]);
+                    du[3] = fma2s(e.w, dn[j], du[3]);
+                }
+            }
+            if constexpr (KW > 0) {
+                w[KW - 1 + u] = o;
+                float2 g[3];
+                conv_blk<KW, KS>(tw, w, u, g);
+                const float2 uu[4] = {o, g[0], g[1], g[2]};
+                const float4* D4 = reinterpret_cast<const float4*>(Dsh + tt * 16);
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    const float4 m = D4[a];
+                    du[a] = fma2s(m.x, uu[0], du[a]);
+                    du[a] = fma2s(m.y, uu[1], du[a]);
+                    du[a] = fma2s(m.z, uu[2], du[a]);
+                    du[a] = fma2s(m.w, uu[3], du[a]);
+                }
+            }
+            if (LAST && (FULL || tt < n1)) {
+                const float4* H4 = reinterpret_cast<const float4*>(Hsh + tt * KM * KM);
+                float2 v[KM];
+#pragma unroll
+                for (int i = 0; i < KM; ++i) v[i] = f2z();
+#pragma unroll
+                for (int j = 0; j < KM; ++j) {
+                    if (j >= k) continue;
+#pragma unroll
+                    for (int q = 0; q < KM / 4; ++q) {
+                        const float4 h = H4[j * (KM / 4) + q];
+                        v[4 * q + 0] = fma2s(h.x, dn[j], v[4 * q + 0]);
+                        v[4 * q + 1] = fma2s(h.y, dn[j], v[4 * q + 1]);
+                        v[4 * q + 2] = fma2s(h.z, dn[j], v[4 * q + 2]);
+                        v[4 * q + 3] = fma2s(h.w, dn[j], v[4 * q + 3]);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < KM; ++i)
+                    if (i < k) *reinterpret_cast<float2*>(pxo + (long long)i * C) = v[i];
+                pxo += kC;
+            }
+        } else if constexpr (KW > 0) {
+            w[KW - 1 + u] = f2z();   // past the sequence end
+        }
+        if constexpr (KW == 0) {
+            if (FULL || tt < n1) {
+                st2(pdo, du[0]);
+                pdo += C;
+            }
+        } else {
+            // conv weight gradient of the run's tokens
+            if (FULL || tt < n1) {
+#pragma unroll
+                for (int j = 0; j < 3; ++j)
+#pragma unroll
+                    for (int i = 0; i < KW; ++i) {
+                        if (i >= ntap<KW, KS>(j)) continue;
+                        const float2 o = w[KW - 1 + u - i];
+                        acc[j][i] = ffma2(du[1 + j], o, acc[j][i]);
+                    }
+            }
+            // d_out[t - i] += w_j[i] du_{1+j}[t]
+            pend[KW - 1 + u] = du[0];
+#pragma unroll
+            for (int i = 0; i < KW; ++i) {
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    if (i >= ntap<KW, KS>(j)) continue;
+                    float2& q = pend[KW - 1 + u - i];
+                    q = ffma2(tw[j][i], du[1 + j], q);
+                }
+            }
+        }
+    };
+    // a block of tokens from tb on
+    auto block = [&](auto lastc, int tb, int half) {
+        if (tb + RU <= n1) {
+#pragma unroll
+            for (int u = 0; u < RU; ++u) token(std::true_type{}, lastc, u, tb + u, half * UB + u);
+        } else {
+#pragma unroll
+            for (int u = 0; u < RU; ++u)
+                if (tb + u < nloop) token(std::false_type{}, lastc, u, tb + u, half * UB + u);
+        }
+    };
+    for (int tb = 0, half = 0; tb < nloop; tb += RU, half ^= 1) {
+        issue(half ^ 1, tb + RU);
+        cpa_wait<1>();
+        if (act) {
+            if (last) block(std::true_type{}, tb, half);
+            else block(std::false_type{}, tb, half);
         }
         if constexpr (KW > 0) {
             // outputs tb + q - (KW - 1), q < UB, have all their terms (du is zero past the
