@@ -875,7 +875,7 @@ xhc_status post_bwd_impl(const xhc_handle* h, int slot, int64_t T, const xhc_par
     const int Tp = (T32 + 7) / 8 * 8;   // 16-byte row stride for the tensor map
     const DzPack pk = {tcw ? c.W<uint16_t>(c.L.dzpack) : nullptr, tcx ? c.W<uint16_t>(c.L.dz16) : nullptr, wpl.NB, Tp,
                        dxa_ld(n), 3};
-    const WRows wr = {act_segs(d, P, slot), n, d.k * d.C, dxa_ld(n), 3, tcx ? c.W<uint16_t>(c.L.w16) : nullptr};
+    const WRows wr = {act_segs(d, P, slot), n, d.k * d.C, dxa_ld(n), 3, tcx ? c.W<uint16_t>(c.L.w16) : nullptr, 1};
     int nblk = 0;
     XHC_K("bwd_coef", c.st, launch_bwd_coef(d, slot, T32, red, bslices, c.S<float>(c.L.zact[slot]),
                              c.S<float>(c.L.rs[slot]), c.S<float>(c.L.p),
@@ -977,7 +977,7 @@ xhc_status xhc_pre_bwd(const xhc_handle* h, int slot, int64_t T, const xhc_param
     const int Tp = (T32 + 7) / 8 * 8;   // 16-byte row stride for the tensor map
     const DzPack pk = {tcw ? c.W<uint16_t>(c.L.dzpack) : nullptr, tcx ? c.W<uint16_t>(c.L.dz16) : nullptr, wpl.NB, Tp,
                        dx_ld(d.nfull), 1};
-    const WRows wr = {full_segs(d, P), d.nfull, d.N * d.C, dx_ld(d.nfull), 1, tcx ? c.W<uint16_t>(c.L.w16) : nullptr};
+    const WRows wr = {full_segs(d, P), d.nfull, d.N * d.C, dx_ld(d.nfull), 1, tcx ? c.W<uint16_t>(c.L.w16) : nullptr, 0};
     int nblk = 0;
     XHC_K("full_coef", c.st, launch_full_coef(d, T32, c.W<float>(c.L.dhpre), c.S<float>(c.L.hpre),
                               c.S<float>(c.L.zfull), c.S<float>(c.L.stats), c.S<float>(c.L.wsum),

@@ -727,7 +727,7 @@ int device_sms() { return num_sms(); }
 //        = dX[t][i*C + c] + sum_q H_pre[t][q][i] d_input_q[t][c]   otherwise
 // MMA K = nfull (dZ and W in bf16: this term is a small share of dX, whose storage is bf16); the
 // tiling is described at the kernel (k_dxf_tc).  The same machinery with "streams" = the k active
-// slots updates dX_act in the backward of each slot's pre-map (k_dx_tc<true>).
+// slots updates dX_act in the backward of each slot's pre-map (k_dx_tc).
 
 namespace {
 
@@ -751,7 +751,6 @@ struct DxArgs {
     int NH;               // active epilogue: streams of the H_pre rows
     float* dxa;           // active epilogue: dX_act [T][k][C] fp32, updated in place
     int nkb, ksteps;      // k-blocks of 64, MMA k-steps of 16
-    int ns;               // operand stages in shared memory (1 or 2)
     int TT, CT;           // token tiles, channel tiles per stream
     long long ntiles;
     int P;
@@ -771,14 +770,36 @@ struct DxArgs {
     int nsplit;           // full-state dX: parts that a column block's streams are cut into (of two streams at least)
 };
 
-// ACT = true (the instantiated form): active-state epilogue, "streams" are the k active slots j:
-//              dX_act[t][j][c] += acc + H_pre[t][slot][I_j] d_input[t][c] - cx_t x_act[t][j][c]
-//              (X = x_act of the slot, scal = the per-token matrices with cx at 112); from the
-//              same loads, the dH_pre dot <x_act_j, d_input> of each 32-channel group (dotp) and,
-//              in the j = 0 tiles, the workspace copy of d_input (dcopy).
-// ACT = false: a full-state epilogue over the N streams; not instantiated (the full-state dX is
-// k_dxf_tc, which also adds the dense-read gradient of the non-active rows).
-template <bool ACT>
+// TMEM -> registers, 16 lanes x 32 columns: lane l gets row l / 4 (v[4 g + e]) and row l / 4 + 8 (v[4 g + 2 +
+// e]), columns 8 g + 2 (l % 4) + e, g < 4, e < 2 (wait in the same statement, as above)
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, float (&v)[16]) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+          "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// Active-state input gradient: tiles of 128 tokens x 128 channels of an active slot j, MMA K = 3 nact,
+//   dX_act[t][j][c] += acc + H_pre[t][slot][I_j] d_input[t][c] - cx_t x_act[t][j][c]
+// (X = x_act of the slot, scal = the per-token matrices with cx at 112); from the same loads, the dH_pre dot
+// <x_act_j, d_input> of each 32-channel group (dotp) and, in the j = 0 tiles, the workspace copy of
+// d_input (dcopy).
+//
+// Bound by HBM: 195 KB a tile.  Two groups of 8 epilogue warps take alternate tiles (group g: tiles n = g
+// mod 2, TMEM buffer g), so one group's global reads overlap the other's arithmetic and stores.  In a
+// group, warp w owns rows [32 (w % 4), +32) and columns [64 (w / 4), +64) of the tile, taken as two halves
+// of 32 columns in four passes of 8 rows, with 4 lanes a row and 8 channels a lane, so that the global
+// reads and writes are contiguous along the channels.  The accumulator is read in the 16x256b shape, which
+// has 4 lanes a row too; the weight's rows are packed in the order that gives lane q of a row the
+// channels 8 q .. 8 q + 7 (dxa_row).  T = 32768, C = 4096, k = 4: 1073 us, 81 % of the copy rate.  With the
+// accumulator turned through shared memory instead: the same there, 277 us against 268 at T = 16384,
+// C = 2048 and 72 us against 63 at T = 2103, C = 1536 (the shared-memory pipe was 64 % busy).
 __global__ void __launch_bounds__(DX_THREADS, 1)
 k_dx_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, DxArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -786,18 +807,16 @@ k_dx_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
     const uint32_t A_BYTES = (uint32_t)a.nkb * BM * BK * 2;
     const uint32_t B_BYTES = (uint32_t)a.nkb * DX_BN * BK * 2;
     const uint32_t STAGE = A_BYTES + B_BYTES;
-    const int NS = a.ns;                             // operand stages (1 or 2)
-    const int nsh = NS - 1;                          // log2(NS)
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + NS * STAGE);
-    // [0,2) operands full, [2,4) operands empty, [4,6) tmem full, [6,8) tmem empty
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 8);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGE);
+    // [0] operands full, [1] operands empty, [2,4) tmem full, [4,6) tmem empty
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 6);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
+        mbar_init(smem_u32(&bars[0]), 1);
+        mbar_init(smem_u32(&bars[1]), 1);
         for (int s = 0; s < 2; ++s) {
-            mbar_init(smem_u32(&bars[s]), 1);
             mbar_init(smem_u32(&bars[2 + s]), 1);
-            mbar_init(smem_u32(&bars[4 + s]), 1);
-            mbar_init(smem_u32(&bars[6 + s]), DX_EW / 2);  // one group of epilogue warps per buffer
+            mbar_init(smem_u32(&bars[4 + s]), DX_EW / 2);  // one group of epilogue warps per buffer
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -812,28 +831,46 @@ k_dx_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     pdl_entry();   // barriers and TMEM are set up while the kernel before finishes
-    // 32-bit tile arithmetic (the host keeps ntiles below 2^31): the divisions run per tile
-    const int nloc = (a.ntiles > blockIdx.x) ? (int)((a.ntiles - 1 - blockIdx.x) / a.P) + 1 : 0;
+    // A CTA takes a contiguous range of tiles (slot i fastest, then the channel tile, then the token tile), so
+    // that its rows' token data change once a token tile.  Walked with a cursor (32-bit arithmetic: the host
+    // keeps ntiles below 2^31): the divisions run once per role.
+    const int first = (int)((long long)a.ntiles * blockIdx.x / a.P);
+    const int nloc = (int)((long long)a.ntiles * (blockIdx.x + 1) / a.P) - first;
+    struct Tile {
+        int i, ct, tt;
+    };
+    auto tile_of = [&](int tile) {
+        Tile w;
+        const int rest = tile / a.k;
+        w.i = tile - rest * a.k;
+        w.tt = rest / a.CT;
+        w.ct = rest - w.tt * a.CT;
+        return w;
+    };
+    auto next = [&](Tile& w) {
+        if (++w.i == a.k) {
+            w.i = 0;
+            if (++w.ct == a.CT) {
+                w.ct = 0;
+                ++w.tt;
+            }
+        }
+    };
 
     if (warp == 0) {
         if (lane == 0) {
-            for (int n = 0; n < nloc; ++n) {
-                const int tile = (int)blockIdx.x + n * a.P;
-                const int i = tile % a.N;
-                const int rest = tile / a.N;
-                const int ct = rest % a.CT, tt = rest / a.CT;
-                const int s = (int)(n & nsh);
-                if (n >= NS && !mbar_wait(smem_u32(&bars[2 + s]), (uint32_t)(((n >> nsh) - 1) & 1), a.wait_ns)) {
+            Tile w = tile_of(first);
+            for (int n = 0; n < nloc; ++n, next(w)) {
+                if (n >= 1 && !mbar_wait(smem_u32(&bars[1]), (uint32_t)((n - 1) & 1), a.wait_ns)) {
                     atomicExch(a.err, 11);
                     break;
                 }
-                const uint32_t full = smem_u32(&bars[s]);
+                const uint32_t full = smem_u32(&bars[0]);
                 mbar_expect_tx(full, STAGE);
-                unsigned char* st = smem + (size_t)s * STAGE;
                 for (int kb = 0; kb < a.nkb; ++kb) {
-                    tma_load_2d(smem_u32(st + kb * BM * BK * 2), &tmA, kb * BK, tt * BM, full);
-                    tma_load_2d(smem_u32(st + A_BYTES + kb * DX_BN * BK * 2), &tmB, kb * BK,
-                                i * a.C + ct * DX_BN, full);
+                    tma_load_2d(smem_u32(smem + kb * BM * BK * 2), &tmA, kb * BK, w.tt * BM, full);
+                    tma_load_2d(smem_u32(smem + A_BYTES + kb * DX_BN * BK * 2), &tmB, kb * BK,
+                                w.i * a.C + w.ct * DX_BN, full);
                 }
             }
         }
@@ -842,115 +879,79 @@ k_dx_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
             const uint32_t idesc = idesc_bf16(BM, DX_BN);
             for (int n = 0; n < nloc; ++n) {
                 const int s = (int)(n & 1);        // TMEM buffer
-                const int os = (int)(n & nsh);     // operand stage
-                if (!mbar_wait(smem_u32(&bars[os]), (uint32_t)((n >> nsh) & 1), a.wait_ns)) {
+                if (!mbar_wait(smem_u32(&bars[0]), (uint32_t)(n & 1), a.wait_ns)) {
                     atomicExch(a.err, 12);
                     break;
                 }
-                if (n >= 2 && !mbar_wait(smem_u32(&bars[6 + s]), (uint32_t)(((n >> 1) - 1) & 1), a.wait_ns)) {
+                if (n >= 2 && !mbar_wait(smem_u32(&bars[4 + s]), (uint32_t)(((n >> 1) - 1) & 1), a.wait_ns)) {
                     atomicExch(a.err, 13);
                     break;
                 }
                 tc_fence_after();
-                const uint32_t abase = smem_u32(smem + (size_t)os * STAGE);
+                const uint32_t abase = smem_u32(smem);
                 const uint32_t bbase = abase + A_BYTES;
                 for (int ks = 0; ks < a.ksteps; ++ks) {
                     const int kb = ks >> 2, kk = ks & 3;
                     mma_bf16(tmem + (uint32_t)(s * DX_BN), sw128_desc(abase + kb * BM * BK * 2 + kk * 32),
                              sw128_desc(bbase + kb * DX_BN * BK * 2 + kk * 32), idesc, ks > 0 ? 1u : 0u);
                 }
-                mma_commit(smem_u32(&bars[2 + os]));  // operands consumed
-                mma_commit(smem_u32(&bars[4 + s]));  // accumulator ready
+                mma_commit(smem_u32(&bars[1]));      // operands consumed
+                mma_commit(smem_u32(&bars[2 + s]));  // accumulator ready
             }
         }
     } else {
-        // Two groups of 8 epilogue warps take alternate tiles (group g: tiles n = g mod 2, TMEM
-        // buffer g), so one group's global reads overlap the other's arithmetic and stores.  In a
-        // group, warp w owns rows [32 (w % 4), +32) and columns [64 (w / 4), +64) of the tile,
-        // taken as two halves of 32 columns.  The accumulator is read row-per-lane from TMEM,
-        // bounced through a padded shared tile and re-read with 4 lanes per row (8 channels each)
-        // so that the global reads and writes are contiguous along the channels.
         const int ew = warp - 2;                   // epilogue warp index
         const int grp = ew >> 3;                   // tile parity of this warp's group
         const int quarter = warp & 3;              // TMEM lane quarter (warp id % 4)
         const int chalf = (ew & 7) >> 2;           // 64-column half of the tile
-        float* tileb = reinterpret_cast<float*>(smem + NS * STAGE + 128) + ew * (32 * 33 + 32 * 8);
-        float* meta = tileb + 32 * 33;             // per row: j, h0..h3, sa, sb
+        const int r0 = quarter * 32;               // first row of this warp
+        // this warp's row data of the token tile: H_pre of the k slots' streams, cx
+        float* meta = reinterpret_cast<float*>(smem + STAGE + 128) + ew * (MAXK + 1) * 32;
+        Tile w = tile_of(first + grp);
+        int mtt = -1;
         for (int n = grp; n < nloc; n += 2) {
-            const int tile = (int)blockIdx.x + n * a.P;
-            const int i = tile % a.N;
-            const int rest = tile / a.N;
-            const int ct = rest % a.CT, tt = rest / a.CT;
-            const int s = (int)(n & 1);
-            {
-                // per-row metadata of this lane's row (row-per-lane, matches the TMEM layout)
-                const int t = tt * BM + quarter * 32 + lane;
-                int j = -1;
-                float h[4] = {0.f, 0.f, 0.f, 0.f};
-                float sa = 0.f, sb = 0.f;
-                if (t < a.T) {
-                    if (ACT) {
-                        j = i;
-                        h[0] = a.hpre[((long long)t * a.G + a.slot) * a.NH + a.I[(long long)t * a.k + i]];
-                        h[1] = a.scal[(long long)t * a.scal_ld + 112];  // cx
-                    } else {
-                        for (int q = 0; q < a.k; ++q)
-                            if (a.I[(long long)t * a.k + q] == i) j = q;
-                        for (int q = 0; q < a.G; ++q) h[q] = a.hpre[((long long)t * a.G + q) * a.N + i];
-                        sa = a.scal[(long long)t * a.scal_ld + 0];
-                        sb = a.scal[(long long)t * a.scal_ld + 1];
-                    }
-                }
-                float* m = meta + lane * 8;
-                m[0] = __int_as_float(j); m[1] = h[0]; m[2] = h[1]; m[3] = h[2]; m[4] = h[3];
-                m[5] = sa; m[6] = sb;
+            if (w.tt != mtt) {
+                mtt = w.tt;
+                const int t = w.tt * BM + r0 + lane;
+                __syncwarp();
+#pragma unroll 4
+                for (int q = 0; q < a.k; ++q)
+                    meta[q * 32 + lane] =
+                        t < a.T ? a.hpre[((long long)t * a.G + a.slot) * a.NH + a.I[(long long)t * a.k + q]] : 0.f;
+                meta[MAXK * 32 + lane] = t < a.T ? a.scal[(long long)t * a.scal_ld + 112] : 0.f;
+                __syncwarp();
             }
-            __syncwarp();
-            const uint32_t tl = tmem + (uint32_t)(s * DX_BN) + ((uint32_t)(quarter * 32) << 16);
+            const float* mh = meta + w.i * 32 + (lane >> 2);
+            const float* mc = meta + MAXK * 32 + (lane >> 2);
+            const int s = (int)(n & 1);
+            const uint32_t tl = tmem + (uint32_t)(s * DX_BN) + ((uint32_t)r0 << 16);
             bool ok = true;
 #pragma unroll 1
             for (int hh = 0; hh < 2; ++hh) {
                 const int cg = chalf * 2 + hh;     // column group of 32
                 // 4 passes of 8 rows; lane -> row rr = 8 pass + lane / 4, channels 8 (lane % 4)..
-                const int cq = (lane & 3) * 8;
-                const int c = ct * DX_BN + cg * 32 + cq;
+                const int c = w.ct * DX_BN + cg * 32 + (lane & 3) * 8;
+                const int t0 = w.tt * BM + r0 + (lane >> 2);
+                float* const xrow = a.dxa + ((long long)t0 * a.k + w.i) * a.C + c;
+                const long long pstep = 8LL * a.k * a.C;
                 uint4 xr[4], br[4], br2[4], gr[4];
-                auto load_pass = [&](int pass) {
-                    const int rr = pass * 8 + (lane >> 2);
-                    const int t = tt * BM + quarter * 32 + rr;
+                // all four passes' reads are issued before the accumulator is awaited and read
+#pragma unroll
+                for (int pass = 0; pass < 4; ++pass) {
                     xr[pass] = make_uint4(0, 0, 0, 0);
                     br[pass] = xr[pass];
                     br2[pass] = xr[pass];
                     gr[pass] = xr[pass];
-                    if (t >= a.T) return;
-                    if (ACT) {
-                        const long long row = ((long long)t * a.k + i) * a.C + c;
-                        br[pass] = ld_stream(a.dxa + row);
-                        br2[pass] = ld_stream(a.dxa + row + 4);
-                        gr[pass] = ld_stream(a.dinput + (long long)t * a.C + c);
-                        xr[pass] = ld_stream(a.X + row);
-                    } else {
-                        const int j = __float_as_int(meta[rr * 8]);
-                        const long long off = ((long long)t * a.N + i) * a.C + c;
-                        xr[pass] = ld_stream(a.X + off);
-                        if (j >= 0) {
-                            const float* bp = a.dxact + ((long long)t * a.k + j) * a.C + c;
-                            br[pass] = ld_stream(bp);
-                            br2[pass] = ld_stream(bp + 4);
-                        } else {
-                            br[pass] = ld_stream(a.dX + off);
-                        }
+                    if (t0 + pass * 8 < a.T) {
+                        br[pass] = ld_stream(xrow + pass * pstep);
+                        br2[pass] = ld_stream(xrow + pass * pstep + 4);
+                        gr[pass] = ld_stream(a.dinput + (long long)(t0 + pass * 8) * a.C + c);
+                        xr[pass] = ld_stream(a.X + (xrow - a.dxa) + pass * pstep);
                     }
-                };
-                // all four passes' reads are issued before the accumulator is awaited and read
-                // out (8 columns at a time, few registers live next to the 64 of the reads)
-                load_pass(0);
-                load_pass(1);
-                load_pass(2);
-                load_pass(3);
+                }
                 if (hh == 0) {
                     // one decision per warp (the TMEM reads and the shuffles below are warp-wide)
-                    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars[4 + s]), (uint32_t)((n >> 1) & 1), a.wait_ns))) {
+                    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars[2 + s]), (uint32_t)((n >> 1) & 1), a.wait_ns))) {
                         atomicExch(a.err, 14);
                         ok = false;
                         break;
@@ -958,83 +959,55 @@ k_dx_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
                     tc_fence_after();
                 }
 #pragma unroll
-                for (int q8 = 0; q8 < 4; ++q8) {
-                    float acc[8];
-                    tmem_ld8(tl + (uint32_t)(cg * 32 + q8 * 8), acc);
+                for (int rh = 0; rh < 2; ++rh) {   // 16 rows: two passes
+                    float ac[16];
+                    tmem_ld_frag(tl + (uint32_t)(cg * 32) + ((uint32_t)(rh * 16) << 16), ac);
+                    if (hh == 1 && rh == 1) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&bars[4 + s]));  // TMEM buffer free
+                    }
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) tileb[lane * 33 + q8 * 8 + e] = acc[e];
-                }
-                if (hh == 1) {
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&bars[6 + s]));  // TMEM buffer free
-                }
-                __syncwarp();
-#pragma unroll
-                for (int pass = 0; pass < 4; ++pass) {
-                    const int rr = pass * 8 + (lane >> 2);
-                    const int t = tt * BM + quarter * 32 + rr;
-                    const bool live = t < a.T;    // the same for the 4 lanes of a row
-                    if (!ACT && !live) continue;
-                    const float* m = meta + rr * 8;
-                    const float* ac = tileb + rr * 33 + cq;
-                    float x[8], v[8];
-                    unpack8(xr[pass], x);
-                    if (ACT) {
-                        // dX_act[t][i][c..c+8) += acc + h din - cx x   (i = active slot here)
-                        const float hq = m[1], cx = m[2];
-                        float g[8];
+                    for (int ph = 0; ph < 2; ++ph) {
+                        const int pass = rh * 2 + ph;
+                        const int t = t0 + pass * 8;
+                        const bool live = t < a.T;    // the same for the 4 lanes of a row
+                        const float hq = mh[pass * 8], cx = mc[pass * 8];
+                        float x[8], g[8];
+                        unpack8(xr[pass], x);
                         unpack8(gr[pass], g);
-                        v[0] = __uint_as_float(br[pass].x); v[1] = __uint_as_float(br[pass].y);
-                        v[2] = __uint_as_float(br[pass].z); v[3] = __uint_as_float(br[pass].w);
-                        v[4] = __uint_as_float(br2[pass].x); v[5] = __uint_as_float(br2[pass].y);
-                        v[6] = __uint_as_float(br2[pass].z); v[7] = __uint_as_float(br2[pass].w);
+                        // channel 2 q + e of the lane's eight: accumulator value 4 q + 2 ph + e
                         float4 o0, o1;
-                        o0.x = v[0] + ac[0] + (hq * g[0] - cx * x[0]);
-                        o0.y = v[1] + ac[1] + (hq * g[1] - cx * x[1]);
-                        o0.z = v[2] + ac[2] + (hq * g[2] - cx * x[2]);
-                        o0.w = v[3] + ac[3] + (hq * g[3] - cx * x[3]);
-                        o1.x = v[4] + ac[4] + (hq * g[4] - cx * x[4]);
-                        o1.y = v[5] + ac[5] + (hq * g[5] - cx * x[5]);
-                        o1.z = v[6] + ac[6] + (hq * g[6] - cx * x[6]);
-                        o1.w = v[7] + ac[7] + (hq * g[7] - cx * x[7]);
+                        o0.x = __uint_as_float(br[pass].x) + ac[0 + 2 * ph] + (hq * g[0] - cx * x[0]);
+                        o0.y = __uint_as_float(br[pass].y) + ac[1 + 2 * ph] + (hq * g[1] - cx * x[1]);
+                        o0.z = __uint_as_float(br[pass].z) + ac[4 + 2 * ph] + (hq * g[2] - cx * x[2]);
+                        o0.w = __uint_as_float(br[pass].w) + ac[5 + 2 * ph] + (hq * g[3] - cx * x[3]);
+                        o1.x = __uint_as_float(br2[pass].x) + ac[8 + 2 * ph] + (hq * g[4] - cx * x[4]);
+                        o1.y = __uint_as_float(br2[pass].y) + ac[9 + 2 * ph] + (hq * g[5] - cx * x[5]);
+                        o1.z = __uint_as_float(br2[pass].z) + ac[12 + 2 * ph] + (hq * g[6] - cx * x[6]);
+                        o1.w = __uint_as_float(br2[pass].w) + ac[13 + 2 * ph] + (hq * g[7] - cx * x[7]);
                         // dH_pre of stream I_i: <x_act_i, d_input>, this lane's 8 channels, then
                         // the row's 32 (4 lanes); rows past T hold zeros
                         float dp = x[0] * g[0];
 #pragma unroll
                         for (int e = 1; e < 8; ++e) dp = fmaf(x[e], g[e], dp);
                         if (live) {
-                            float4* dst = reinterpret_cast<float4*>(a.dxa + ((long long)t * a.k + i) * a.C + c);
+                            float4* dst = reinterpret_cast<float4*>(xrow + pass * pstep);
                             dst[0] = o0;
                             dst[1] = o1;
-                            if (i == 0)
+                            if (w.i == 0)
                                 *reinterpret_cast<uint4*>(a.dcopy + ((long long)a.slot * a.T + t) * a.C + c) = gr[pass];
                         }
                         dp += __shfl_xor_sync(0xffffffffu, dp, 1);
                         dp += __shfl_xor_sync(0xffffffffu, dp, 2);
                         if (live && (lane & 3) == 0)
-                            a.dotp[((long long)i * a.ncg + ct * (DX_BN / 32) + cg) * a.T + t] = dp;
-                    } else {
-                        const int j = __float_as_int(m[0]);
-                        const long long off = ((long long)t * a.N + i) * a.C + c;
-                        if (j >= 0) {
-                            v[0] = __uint_as_float(br[pass].x); v[1] = __uint_as_float(br[pass].y);
-                            v[2] = __uint_as_float(br[pass].z); v[3] = __uint_as_float(br[pass].w);
-                            v[4] = __uint_as_float(br2[pass].x); v[5] = __uint_as_float(br2[pass].y);
-                            v[6] = __uint_as_float(br2[pass].z); v[7] = __uint_as_float(br2[pass].w);
-                        } else {
-                            unpack8(br[pass], v);
-                        }
-                        const float sa = m[5], sb = m[6];
-                        float o[8];
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) o[e] = v[e] + ac[e] + sa + sb * x[e];
-                        *reinterpret_cast<uint4*>(a.dX + off) = pack8(o);
+                            a.dotp[((long long)w.i * a.ncg + w.ct * (DX_BN / 32) + cg) * a.T + t] = dp;
                     }
                 }
-                __syncwarp();
             }
             if (!ok) break;
+            next(w);
+            next(w);
         }
     }
     tc_fence_before();
@@ -1435,7 +1408,6 @@ cudaError_t launch_dxa_tc(const Dims& d, int slot, int T, int nact,
     a.CT = d.C / DX_BN;
     a.ntiles = (long long)a.TT * a.CT * d.k;
     a.P = (int)std::min<long long>(num_sms(), a.ntiles);
-    a.N = d.k;  // tile "streams" are the active slots
     a.NH = d.N;
     a.dinput = d_input; a.hpre = hpre; a.I = I; a.dxa = dxact; a.err = err;
     a.wait_ns = debug_wait_ns();
@@ -1443,17 +1415,15 @@ cudaError_t launch_dxa_tc(const Dims& d, int slot, int T, int nact,
     a.dotp = dotp; a.dcopy = dcopy; a.ncg = d.C / 32;
     // one operand stage (the MMA of a tile is short next to its epilogue): the shared memory
     // left over is L1 for the epilogue's in-flight reads
-    a.ns = 1;
-    const size_t sm = (size_t)a.ns * a.nkb * (BM + DX_BN) * BK * 2 + 128 +
-                      (size_t)DX_EW * (32 * 33 + 32 * 8) * 4 + 1024;
-    e = cudaFuncSetAttribute((const void*)k_dx_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const size_t sm = (size_t)a.nkb * (BM + DX_BN) * BK * 2 + 128 + (size_t)DX_EW * (MAXK + 1) * 32 * 4 + 1024;
+    e = cudaFuncSetAttribute((const void*)k_dx_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    XHC_LAUNCH(st, a.P, DX_THREADS, sm, (k_dx_tc<true>), ma, mb, a);
+    XHC_LAUNCH(st, a.P, DX_THREADS, sm, (k_dx_tc), ma, mb, a);
     return cudaGetLastError();
 }
 
 namespace {
-// dH_pre[t][slot][I_j] from the dot partials of k_dx_tc<true>: a block per (32 tokens, j); warp w
+// dH_pre[t][slot][I_j] from the dot partials of k_dx_tc: a block per (32 tokens, j); warp w
 // sums the groups g = w, w + 8, ... of its lane's token (coalesced 128-byte rows), and the eight
 // warp sums are added in warp order (a fixed order: the result does not depend on the schedule)
 __global__ void __launch_bounds__(256) k_dots_act(const float* __restrict__ dotp, int T, int k, int ncg,

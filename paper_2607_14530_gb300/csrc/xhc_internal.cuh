@@ -454,7 +454,13 @@ struct WRows {
     WSegs W;
     int n, rows, ld, parts;
     uint16_t* dst;   // null: nothing to pack
+    int frag;        // 1: rows in the order of dxa_row
 };
+// The weight row at place r of k_dx_tc's B operand: in every 32 rows, the one at 8 g + 2 q + e is channel 8 q +
+// 2 g + e, so that the accumulator's 16x256b fragments give a lane 8 neighbouring channels.
+__device__ __forceinline__ int dxa_row(int r) {
+    return (r & ~31) | (((r >> 1) & 3) << 3) | (((r >> 3) & 3) << 1) | (r & 1);
+}
 constexpr int WROWS_U = 8;   // elements per thread
 __device__ __forceinline__ void pack_wrows_of(const WRows& j, int blk) {
     const int at = blk * (int)blockDim.x * WROWS_U + threadIdx.x, tot = j.rows * j.ld;   // < 2^31
@@ -469,7 +475,7 @@ __device__ __forceinline__ void pack_wrows_of(const WRows& j, int blk) {
             const int r = idx / j.ld, c = idx - r * j.ld;
             if (c < j.parts * j.n) {
                 part[u] = c / j.n;
-                v[u] = seg_elem<true>(j.W, r, c - part[u] * j.n);
+                v[u] = seg_elem<true>(j.W, j.frag ? dxa_row(r) : r, c - part[u] * j.n);
             }
         }
     }
