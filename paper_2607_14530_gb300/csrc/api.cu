@@ -204,12 +204,13 @@ Layout make_layout(const Dims& d, int64_t T) {
     L.wpacka = o; o = al(o + (size_t)L.tca.NB * d.k * d.C * 2);
     L.dzpack = o; o = al(o + (size_t)std::max(L.twf.NB, L.twa.NB) * ((t + 7) / 8 * 8) * 2);
     {
-        // bf16 operands of the tensor-core input gradients: full maps [T][nfull] and [N C][nfull],
-        // active maps in three parts [T][3 nact] and [k C][3 nact] (rows padded to 8)
-        const size_t ld = (size_t)(d.nfull + 7) / 8 * 8;
-        const size_t ld3 = (size_t)(3 * nact_max + 7) / 8 * 8;
+        // bf16 operands of the tensor-core input gradients: full maps [T][nfull] and [N C][nfull] (three
+        // times the columns at some widths), active maps in three parts [T][3 nact] and [k][C][3 nact]
+        // (rows padded to 8, the C rows to 32)
+        const size_t ld = dx_ld(std::max(1, dx_tc_parts((int)T, d.N, d.C, d.nfull, d.G)) * d.nfull);
+        const size_t ld3 = dxa_ld(nact_max);
         L.dz16 = o; o = al(o + t * std::max(ld, ld3) * 2);
-        L.w16 = o; o = al(o + std::max((size_t)d.N * d.C * ld, (size_t)d.k * d.C * ld3) * 2);
+        L.w16 = o; o = al(o + std::max((size_t)d.N * d.C * ld, (size_t)d.k * dxa_width(d.C) * ld3) * 2);
     }
     L.part = o;
     o = al(o + std::max((size_t)L.splits_full * d.nfull, (size_t)L.splits_act * nact_max) * t * 4);
@@ -221,7 +222,7 @@ Layout make_layout(const Dims& d, int64_t T) {
     L.red = o; o = al(o + t * L.nslice * NRED * 4);
     L.dxact = o; o = al(o + t * d.k * d.C * 4);
     L.dinput = o; o = al(o + (size_t)d.G * t * d.C * 2);
-    L.dotp = o; o = al(o + (size_t)d.k * (d.C / 32) * t * 4);
+    L.dotp = o; o = al(o + (size_t)d.k * ((d.C + 31) / 32) * t * 4);
     L.dp = o; o = al(o + t * d.k * 4);
     L.dhpre = o; o = al(o + t * d.G * d.N * 4);
     L.tokmat = o; o = al(o + t * TOKMAT * 4);
@@ -875,7 +876,8 @@ xhc_status post_bwd_impl(const xhc_handle* h, int slot, int64_t T, const xhc_par
     const int Tp = (T32 + 7) / 8 * 8;   // 16-byte row stride for the tensor map
     const DzPack pk = {tcw ? c.W<uint16_t>(c.L.dzpack) : nullptr, tcx ? c.W<uint16_t>(c.L.dz16) : nullptr, wpl.NB, Tp,
                        dxa_ld(n), 3};
-    const WRows wr = {act_segs(d, P, slot), n, d.k * d.C, dxa_ld(n), 3, tcx ? c.W<uint16_t>(c.L.w16) : nullptr, 1};
+    const WRows wr = {act_segs(d, P, slot), n, d.k * dxa_width(d.C), dxa_ld(n), 3,
+                      tcx ? c.W<uint16_t>(c.L.w16) : nullptr, d.C};
     int nblk = 0;
     XHC_K("bwd_coef", c.st, launch_bwd_coef(d, slot, T32, red, bslices, c.S<float>(c.L.zact[slot]),
                              c.S<float>(c.L.rs[slot]), c.S<float>(c.L.p),
@@ -972,12 +974,13 @@ xhc_status xhc_pre_bwd(const xhc_handle* h, int slot, int64_t T, const xhc_param
     }
     if (slot != 0) return XHC_OK;
     XHC_K("full_dots", c.st, launch_full_dots(d, T32, X, dinput, c.S<int>(c.L.I), c.W<float>(c.L.dhpre), c.st));
-    const bool tcw = !(T32 < 64 || d.N * d.C < 128), tcx = dx_tc_ok(T32, d.N, d.C, d.nfull, d.G);
+    const int parts = dx_tc_parts(T32, d.N, d.C, d.nfull, d.G);
+    const bool tcw = !(T32 < 64 || d.N * d.C < 128), tcx = parts > 0;
     const ProjTcPlan& wpl = c.L.twf;
     const int Tp = (T32 + 7) / 8 * 8;   // 16-byte row stride for the tensor map
     const DzPack pk = {tcw ? c.W<uint16_t>(c.L.dzpack) : nullptr, tcx ? c.W<uint16_t>(c.L.dz16) : nullptr, wpl.NB, Tp,
-                       dx_ld(d.nfull), 1};
-    const WRows wr = {full_segs(d, P), d.nfull, d.N * d.C, dx_ld(d.nfull), 1, tcx ? c.W<uint16_t>(c.L.w16) : nullptr, 0};
+                       dx_ld(parts * d.nfull), parts};
+    const WRows wr = {full_segs(d, P), d.nfull, d.N * d.C, dx_ld(parts * d.nfull), parts, tcx ? c.W<uint16_t>(c.L.w16) : nullptr, 0};
     int nblk = 0;
     XHC_K("full_coef", c.st, launch_full_coef(d, T32, c.W<float>(c.L.dhpre), c.S<float>(c.L.hpre),
                               c.S<float>(c.L.zfull), c.S<float>(c.L.stats), c.S<float>(c.L.wsum),

@@ -74,6 +74,20 @@ __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, i
                  : "memory");
 }
 
+// the same for a box of one row group of a 3D map
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z,
+                                            uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst), "l"((uint64_t)map), "r"(x), "r"(y), "r"(z), "r"(bar)
+        : "memory");
+}
+__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int x, int y, int z) {
+    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global [%0, {%1, %2, %3}];" ::"l"((uint64_t)map), "r"(x),
+                 "r"(y), "r"(z)
+                 : "memory");
+}
+
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, 8-row groups 1024 B apart.
 __device__ __forceinline__ uint64_t sw128_desc(uint32_t addr) {
     uint64_t d = 0;
@@ -579,6 +593,22 @@ bool make_map_box(CUtensorMap* m, const void* base, uint64_t inner, uint64_t row
     return r == CUDA_SUCCESS;
 }
 
+// a state [T][N][C] in boxes of box_c channels of one stream and box_t tokens: what a box has past C or T
+// reads as zero and is not stored
+bool make_map_state(CUtensorMap* m, const void* base, uint64_t C, uint64_t N, uint64_t T, uint32_t box_c,
+                    uint32_t box_t) {
+    auto enc = get_encode();
+    if (!enc) return false;
+    cuuint64_t gdim[3] = {C, N, T};
+    cuuint64_t gstride[2] = {C * 2, N * C * 2};
+    cuuint32_t box[3] = {box_c, 1, box_t};
+    cuuint32_t es[3] = {1, 1, 1};
+    CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), gdim, gstride,
+                     box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS;
+}
+
 bool make_map(CUtensorMap* m, const void* base, uint64_t inner, uint64_t rows, uint32_t box_rows) {
     return make_map_box(m, base, inner, rows, (uint32_t)BK, box_rows);
 }
@@ -766,7 +796,9 @@ struct DxArgs {
     uint64_t wait_ns;     // limit of every bounded wait
     float* dotp;          // active epilogue: [k][ncg][T] dot partials over 32-channel groups
     uint16_t* dcopy;      // active epilogue: [G][T][C] copies of d_input (written by slot-0 tiles)
-    int ncg;              // active epilogue: C / 32
+    int ncg;              // active epilogue: groups of 32 channels, the last one may be part full
+    int Cp;               // active epilogue: weight rows packed per slot
+    int nbs;              // full-state dX: stages of W rows
     int nsplit;           // full-state dX: parts that a column block's streams are cut into (of two streams at least)
 };
 
@@ -797,9 +829,12 @@ __device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, float (&v)[16]) {
 // of 32 columns in four passes of 8 rows, with 4 lanes a row and 8 channels a lane, so that the global
 // reads and writes are contiguous along the channels.  The accumulator is read in the 16x256b shape, which
 // has 4 lanes a row too; the weight's rows are packed in the order that gives lane q of a row the
-// channels 8 q .. 8 q + 7 (dxa_row).  T = 32768, C = 4096, k = 4: 1073 us, 81 % of the copy rate.  With the
+// channels 8 q .. 8 q + 7 (dxa_row).  CUT: DX_BN does not divide C, and the lanes
+// past it move nothing (two forms: the test costs registers, and the kernel sits at its 96: T = 8192,
+// C = 2048: 131 -> 135 us with it).  T = 32768, C = 4096, k = 4: 1073 us, 81 % of the copy rate.  With the
 // accumulator turned through shared memory instead: the same there, 277 us against 268 at T = 16384,
 // C = 2048 and 72 us against 63 at T = 2103, C = 1536 (the shared-memory pipe was 64 % busy).
+template <bool CUT>
 __global__ void __launch_bounds__(DX_THREADS, 1)
 k_dx_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, DxArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -870,7 +905,7 @@ k_dx_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
                 for (int kb = 0; kb < a.nkb; ++kb) {
                     tma_load_2d(smem_u32(smem + kb * BM * BK * 2), &tmA, kb * BK, w.tt * BM, full);
                     tma_load_2d(smem_u32(smem + A_BYTES + kb * DX_BN * BK * 2), &tmB, kb * BK,
-                                w.i * a.C + w.ct * DX_BN, full);
+                                w.i * a.Cp + w.ct * DX_BN, full);
                 }
             }
         }
@@ -931,6 +966,7 @@ k_dx_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
                 const int cg = chalf * 2 + hh;     // column group of 32
                 // 4 passes of 8 rows; lane -> row rr = 8 pass + lane / 4, channels 8 (lane % 4)..
                 const int c = w.ct * DX_BN + cg * 32 + (lane & 3) * 8;
+                const bool cin = !CUT || c < a.C;   // C is a multiple of a lane's 8 channels
                 const int t0 = w.tt * BM + r0 + (lane >> 2);
                 float* const xrow = a.dxa + ((long long)t0 * a.k + w.i) * a.C + c;
                 const long long pstep = 8LL * a.k * a.C;
@@ -942,7 +978,7 @@ k_dx_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
                     br[pass] = xr[pass];
                     br2[pass] = xr[pass];
                     gr[pass] = xr[pass];
-                    if (t0 + pass * 8 < a.T) {
+                    if (cin && t0 + pass * 8 < a.T) {
                         br[pass] = ld_stream(xrow + pass * pstep);
                         br2[pass] = ld_stream(xrow + pass * pstep + 4);
                         gr[pass] = ld_stream(a.dinput + (long long)(t0 + pass * 8) * a.C + c);
@@ -971,7 +1007,7 @@ k_dx_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
                     for (int ph = 0; ph < 2; ++ph) {
                         const int pass = rh * 2 + ph;
                         const int t = t0 + pass * 8;
-                        const bool live = t < a.T;    // the same for the 4 lanes of a row
+                        const bool live = cin && t < a.T;
                         const float hq = mh[pass * 8], cx = mc[pass * 8];
                         float x[8], g[8];
                         unpack8(xr[pass], x);
@@ -987,7 +1023,7 @@ k_dx_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
                         o1.z = __uint_as_float(br2[pass].z) + ac[12 + 2 * ph] + (hq * g[6] - cx * x[6]);
                         o1.w = __uint_as_float(br2[pass].w) + ac[13 + 2 * ph] + (hq * g[7] - cx * x[7]);
                         // dH_pre of stream I_i: <x_act_i, d_input>, this lane's 8 channels, then
-                        // the row's 32 (4 lanes); rows past T hold zeros
+                        // the row's 32 (4 lanes); lanes past T or C hold zeros
                         float dp = x[0] * g[0];
 #pragma unroll
                         for (int e = 1; e < 8; ++e) dp = fmaf(x[e], g[e], dp);
@@ -1023,9 +1059,9 @@ k_dx_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
 // TMA store, bulk-group and proxy-fence helpers of the full-state dX kernel below, and a named
 // barrier that also ORs a flag over the participating threads.
 
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t src, int x, int y) {
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
-                     (uint64_t)map), "r"(src), "r"(x), "r"(y)
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, uint32_t src, int x, int y, int z) {
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(
+                     (uint64_t)map), "r"(src), "r"(x), "r"(y), "r"(z)
                  : "memory");
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
@@ -1057,7 +1093,9 @@ constexpr int DG_PF = 4;                     // L2 prefetch distance of the X / 
 // released, and the next block's rows loaded, while the last tiles of a block are finished.
 // On calls with few blocks a block's streams are cut into nsplit parts, each a unit of its own.
 // Per tile: MMA 128 x 64 x nfull (A = the block's dZ rows, B = the stream's W rows), TMA-staged X
-// and dX tiles, the result written over the X tile and TMA-stored into dX.
+// and dX tiles, the result written over the X tile and TMA-stored into dX.  The state's map has the streams
+// as a dimension, so that the last block of a width that 64 does not divide (CUT) is cut at C.
+template <bool CUT>
 __global__ void __launch_bounds__(DX_THREADS, 1)
 k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
          const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmD,
@@ -1069,8 +1107,9 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
     const uint32_t A_BYTES = (uint32_t)a.nkb * BM * BK * 2;      // dZ rows of the token tile
     const uint32_t B_BYTES = (uint32_t)a.nkb * DG_BN * BK * 2;   // W rows of one stream's block
     unsigned char* sA = smem;
-    unsigned char* sB = sA + A_BYTES;                // [2 stages]
-    unsigned char* sG = sB + 2 * B_BYTES;            // [G][128 tokens][64 channels]
+    unsigned char* sB = sA + A_BYTES;                // [2 stages, or 1]
+    const int bsh = CUT ? a.nbs - 1 : 1;                       // tile n has B stage n & bsh, in its use n >> bsh
+    unsigned char* sG = sB + (bsh + 1) * B_BYTES;    // [G][128 tokens][64 channels]
     unsigned char* sE = sG + (size_t)a.G * DG_TILE;  // [2 groups][X tile | dX tile]
     uint64_t* bars = reinterpret_cast<uint64_t*>(sE + 2 * 2 * DG_TILE);
     // [0] A full [1] A empty [2,4) B full [4,6) B empty [6] G full [7] G empty
@@ -1151,8 +1190,8 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
                     // the tile DG_PF ahead into L2: its X / dX loads, issued once a stage frees,
                     // then wait for L2 rather than HBM
                     const int i = pf.stream(NU);
-                    tma_prefetch_2d(&tmX, i * a.C + pf.cb * DG_BN, pf.tt * BM);
-                    if (pf.p < pf.ndin) tma_prefetch_2d(&tmD, i * a.C + pf.cb * DG_BN, pf.tt * BM);
+                    tma_prefetch_3d(&tmX, pf.cb * DG_BN, i, pf.tt * BM);
+                    if (pf.p < pf.ndin) tma_prefetch_3d(&tmD, pf.cb * DG_BN, i, pf.tt * BM);
                     if (pf.p == 0)
                         for (int q = 0; q < a.G; ++q) tma_prefetch_2d(&tmG, pf.cb * DG_BN, q * a.T + pf.tt * BM);
                 }
@@ -1169,15 +1208,16 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
                         tma_load_2d(smem_u32(sA + kb * BM * BK * 2), &tmA, kb * BK, tt * BM, fa);
                 }
                 const int s = (int)(n & 1);
-                if (n >= 2 && !mbar_wait(smem_u32(&bars[4 + s]), (uint32_t)(((n >> 1) - 1) & 1), a.wait_ns)) {
+                const int b = n & bsh;
+                if (n > bsh && !mbar_wait(smem_u32(&bars[4 + b]), (uint32_t)(((n >> bsh) - 1) & 1), a.wait_ns)) {
                     atomicExch(a.err, 32);
                     *s_abort = 1;
                     break;
                 }
-                const uint32_t fb = smem_u32(&bars[2 + s]);
+                const uint32_t fb = smem_u32(&bars[2 + b]);
                 mbar_expect_tx(fb, B_BYTES);
                 for (int kb = 0; kb < a.nkb; ++kb)
-                    tma_load_2d(smem_u32(sB + s * B_BYTES + kb * DG_BN * BK * 2), &tmB, kb * BK,
+                    tma_load_2d(smem_u32(sB + b * B_BYTES + kb * DG_BN * BK * 2), &tmB, kb * BK,
                                 i * a.C + cb * DG_BN, fb);
                 if (n >= 2 && !mbar_wait(smem_u32(&bars[14 + s]), (uint32_t)(((n >> 1) - 1) & 1), a.wait_ns)) {
                     atomicExch(a.err, 33);
@@ -1188,8 +1228,8 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
                 const uint32_t fe = smem_u32(&bars[12 + s]);
                 mbar_expect_tx(fe, need_dx ? 2 * DG_TILE : DG_TILE);
                 unsigned char* xt = sE + (size_t)s * 2 * DG_TILE;
-                tma_load_2d(smem_u32(xt), &tmX, i * a.C + cb * DG_BN, tt * BM, fe);
-                if (need_dx) tma_load_2d(smem_u32(xt + DG_TILE), &tmD, i * a.C + cb * DG_BN, tt * BM, fe);
+                tma_load_3d(smem_u32(xt), &tmX, cb * DG_BN, i, tt * BM, fe);
+                if (need_dx) tma_load_3d(smem_u32(xt + DG_TILE), &tmD, cb * DG_BN, i, tt * BM, fe);
                 if (p == 0) {
                     if (blk >= 1 && !mbar_wait(smem_u32(&bars[7]), (uint32_t)((blk - 1) & 1), a.wait_ns)) {
                         atomicExch(a.err, 34);
@@ -1214,7 +1254,8 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
                 }
                 const int s = (int)(n & 1);
                 bool ok = (p != 0) || mbar_wait(smem_u32(&bars[0]), (uint32_t)(blk & 1), a.wait_ns);
-                ok = ok && mbar_wait(smem_u32(&bars[2 + s]), (uint32_t)((n >> 1) & 1), a.wait_ns);
+                const int b = n & bsh;
+                ok = ok && mbar_wait(smem_u32(&bars[2 + b]), (uint32_t)((n >> bsh) & 1), a.wait_ns);
                 ok = ok && (n < 2 || mbar_wait(smem_u32(&bars[10 + s]), (uint32_t)(((n >> 1) - 1) & 1), a.wait_ns));
                 if (!ok) {
                     atomicExch(a.err, 35);
@@ -1223,13 +1264,13 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
                 }
                 tc_fence_after();
                 const uint32_t abase = smem_u32(sA);
-                const uint32_t bbase = smem_u32(sB + s * B_BYTES);
+                const uint32_t bbase = smem_u32(sB + b * B_BYTES);
                 for (int ks = 0; ks < a.ksteps; ++ks) {
                     const int kb = ks >> 2, kk = ks & 3;
                     mma_bf16(tmem + (uint32_t)(s * DG_BN), sw128_desc(abase + kb * BM * BK * 2 + kk * 32),
                              sw128_desc(bbase + kb * DG_BN * BK * 2 + kk * 32), idesc, ks > 0 ? 1u : 0u);
                 }
-                mma_commit(smem_u32(&bars[4 + s]));              // B stage consumed
+                mma_commit(smem_u32(&bars[4 + b]));              // B stage consumed
                 mma_commit(smem_u32(&bars[8 + s]));              // accumulator ready
                 if (p == NU - 1) mma_commit(smem_u32(&bars[1]));  // the block's A rows consumed
             }
@@ -1285,12 +1326,13 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
             for (int q = 0; q < MAXK; ++q)
                 if (q < a.k && ((ib[q >> 2] >> (8 * (q & 3))) & 0xffu) == (uint32_t)i) j = q;
             const bool arow = (j >= 0) && (t < a.T);
+            const int cleft = a.C - cb * DG_BN - half * 32;   // channels of this row from the half on
             // an active row's fp32 base, 8 channels per chunk, read one chunk ahead (the first
             // before the waits)
             const float* brow = a.dxact + ((long long)t * a.k + (j < 0 ? 0 : j)) * a.C + cb * DG_BN + half * 32;
             uint4 pfa[2], pfb[2];
             auto prefetch = [&](int c4, uint4 (&dst)[2]) {
-                if (arow) {
+                if (arow && (!CUT || c4 * 8 < cleft)) {
                     dst[0] = ld_stream(brow + c4 * 8);
                     dst[1] = ld_stream(brow + c4 * 8 + 4);
                 }
@@ -1362,7 +1404,7 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
                 // block's d_input tiles, its first tile of the block) releases them: one arrival
                 // per group and block
                 if ((usesg && p + 2 >= ndin) || (!usesg && p < 2)) mbar_arrive(smem_u32(&bars[7]));
-                tma_store_2d(&tmD, smem_u32(xt), i * a.C + cb * DG_BN, tt * BM);
+                tma_store_3d(&tmD, smem_u32(xt), cb * DG_BN, i, tt * BM);
                 bulk_commit();
                 bulk_wait_read0();                                   // the stage may be reloaded
                 mbar_arrive(smem_u32(&bars[14 + grp]));
@@ -1382,43 +1424,46 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
 
 }  // namespace
 
-// two operand stages of up to two k-blocks each fit the 227 KB of shared memory
+// Any width (a multiple of 8), and up to five k-blocks of the three parts (k = 8 with a conv: nact = 96): 160
+// of the 227 KB of shared memory.  Below a tile of tokens the CUDA-core pair gemm_dzw + dinput_act stays.
+// T = 1000, C = 1160, k = 8, nact = 96: gemm_dzw + dinput_act 92 + 29 us, here 38.
 bool dxa_tc_ok(int T, int k, int C, int nact) {
-    return T >= BM && C % DX_BN == 0 && 3 * nact <= 2 * BK &&
-           (long long)((T + BM - 1) / BM) * (C / DX_BN) * k < (1LL << 31);   // 32-bit tile indices
+    return T >= BM && 3 * nact <= 5 * BK &&
+           (long long)((T + BM - 1) / BM) * ((C + DX_BN - 1) / DX_BN) * k < (1LL << 31);   // 32-bit tile indices
 }
 
 cudaError_t launch_dxa_tc(const Dims& d, int slot, int T, int nact,
                           const uint16_t* dz3, const uint16_t* w3, const uint16_t* d_input, const float* hpre,
                           const int* I, const uint16_t* xact, const float* tokmat, float* dxact,
                           float* dotp, uint16_t* dcopy, int* err, cudaStream_t st) {
-    const int KC = d.k * d.C;
     const int K3 = 3 * nact;
     const int ld = dxa_ld(nact);
     cudaError_t e;
     CUtensorMap ma, mb;
     if (!make_map_box(&ma, dz3, (uint64_t)K3, (uint64_t)T, BK, BM, (uint64_t)ld * 2)) return cudaErrorInvalidValue;
-    if (!make_map_box(&mb, w3, (uint64_t)K3, (uint64_t)KC, BK, DX_BN, (uint64_t)ld * 2)) return cudaErrorInvalidValue;
+    if (!make_map_box(&mb, w3, (uint64_t)K3, (uint64_t)d.k * dxa_width(d.C), BK, DX_BN, (uint64_t)ld * 2)) return cudaErrorInvalidValue;
     DxArgs a;
     memset(&a, 0, sizeof(a));
     a.T = T; a.C = d.C; a.N = d.N; a.k = d.k; a.G = d.G; a.slot = slot;
     a.nkb = (K3 + BK - 1) / BK;
     a.ksteps = (K3 + 15) / 16;
     a.TT = (T + BM - 1) / BM;
-    a.CT = d.C / DX_BN;
+    a.CT = (d.C + DX_BN - 1) / DX_BN;
+    a.Cp = dxa_width(d.C);
     a.ntiles = (long long)a.TT * a.CT * d.k;
     a.P = (int)std::min<long long>(num_sms(), a.ntiles);
     a.NH = d.N;
     a.dinput = d_input; a.hpre = hpre; a.I = I; a.dxa = dxact; a.err = err;
     a.wait_ns = debug_wait_ns();
     a.X = xact; a.scal = tokmat; a.scal_ld = TOKMAT;
-    a.dotp = dotp; a.dcopy = dcopy; a.ncg = d.C / 32;
+    a.dotp = dotp; a.dcopy = dcopy; a.ncg = (d.C + 31) / 32;
     // one operand stage (the MMA of a tile is short next to its epilogue): the shared memory
     // left over is L1 for the epilogue's in-flight reads
     const size_t sm = (size_t)a.nkb * (BM + DX_BN) * BK * 2 + 128 + (size_t)DX_EW * (MAXK + 1) * 32 * 4 + 1024;
-    e = cudaFuncSetAttribute((const void*)k_dx_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    auto* const kern = d.C % DX_BN == 0 ? &k_dx_tc<false> : &k_dx_tc<true>;
+    e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    XHC_LAUNCH(st, a.P, DX_THREADS, sm, (k_dx_tc), ma, mb, a);
+    XHC_LAUNCH(st, a.P, DX_THREADS, sm, (kern), ma, mb, a);
     return cudaGetLastError();
 }
 
@@ -1452,37 +1497,46 @@ __global__ void __launch_bounds__(256) k_dots_act(const float* __restrict__ dotp
 cudaError_t launch_dots_act(const Dims& d, int slot, int T, const float* dotp, const int* I, float* dhpre,
                             cudaStream_t st) {
     const dim3 grid((unsigned)((T + 31) / 32), (unsigned)d.k);
-    XHC_LAUNCH(st, grid, 256, 0, (k_dots_act), dotp, T, d.k, d.C / 32, d.G, d.N, slot, I, dhpre);
+    XHC_LAUNCH(st, grid, 256, 0, (k_dots_act), dotp, T, d.k, (d.C + 31) / 32, d.G, d.N, slot, I, dhpre);
     return cudaGetLastError();
 }
 
-// shared memory of k_dxf_tc: the token tile's dZ rows and two stages of W rows (nkb k-blocks
+// shared memory of k_dxf_tc: the token tile's dZ rows and nbs stages of W rows (nkb k-blocks
 // each), the G d_input tiles and two X | dX tile pairs, barriers, alignment slack
-static size_t dxf_smem(int nfull, int G) {
-    const int nkb = (nfull + BK - 1) / BK;
-    return (size_t)nkb * (BM + 2 * DG_BN) * BK * 2 + (size_t)(G + 4) * DG_TILE + 256 + 1024;
+static size_t dxf_smem(int K, int G, int nbs) {
+    const int nkb = (K + BK - 1) / BK;
+    return (size_t)nkb * (BM + nbs * DG_BN) * BK * 2 + (size_t)(G + 4) * DG_TILE + 256 + 1024;
 }
+// two stages of W rows where they fit the 227 KB a block may use, else one, or none
+static int dxf_stages(int K, int G) { return dxf_smem(K, G, 2) <= 232448 ? 2 : dxf_smem(K, G, 1) <= 232448 ? 1 : 0; }
 
-// up to three k-blocks (nfull <= 192: N = 32 with a router and four pre-maps) fit the 227 KB a
-// block may use
-bool dx_tc_ok(int T, int N, int C, int nfull, int G) {
-    return T >= BM && C % DG_BN == 0 && nfull <= 3 * BK && N >= 2 && G >= 1 && G <= 4 &&
-           dxf_smem(nfull, G) <= 232448 &&
-           (long long)((T + BM - 1) / BM) * (C / DG_BN) * N < (1LL << 31);   // 32-bit tile indices
+// How the full-state dX takes dZ and W: 1 rounded to bf16, where 64 divides the width (up to three k-blocks:
+// nfull <= 192, N = 32 with a router and four pre-maps); 3 in three bf16 parts, hi | lo | hi times hi | hi |
+// lo, at other widths: the CUDA-core full_dx that they went to takes both in fp32, and the products keep 16
+// bits.  0: full_dx (less than a tile of tokens, or too many columns for the shared memory).
+// T = 1000, N = 12, C = 1160: full_dx 79 us, here 37; T = 4944, N = 16, C = 2840, four
+// slots (G N + N = 80 columns, one stage of weight rows): the step 5.99 -> 3.40 ms with both gradients here.
+int dx_tc_parts(int T, int N, int C, int nfull, int G) {
+    if (T < BM || N < 2 || G < 1 || G > 4 ||
+        (long long)((T + BM - 1) / BM) * ((C + DG_BN - 1) / DG_BN) * N >= (1LL << 31))   // 32-bit tile indices
+        return 0;
+    if (C % DG_BN == 0) return nfull <= 3 * BK && dxf_smem(nfull, G, 2) <= 232448 ? 1 : 0;
+    return dxf_stages(3 * nfull, G) > 0 ? 3 : 0;
 }
 
 cudaError_t launch_dx_tc(const Dims& d, int T, const uint16_t* dz16,
                          const uint16_t* w16, const uint16_t* X, const uint16_t* dinput, const float* hpre,
                          const int* I, const float* dxact, const float* scal, int scal_ld,
                          uint16_t* dX, int* err, cudaStream_t st) {
-    const int n = d.nfull, NC = d.N * d.C;
+    const int parts = dx_tc_parts(T, d.N, d.C, d.nfull, d.G);
+    const int n = parts * d.nfull, NC = d.N * d.C;
     const int ld = dx_ld(n);
     cudaError_t e;
     CUtensorMap ma, mb, mx, md, mg;
     if (!make_map_box(&ma, dz16, (uint64_t)n, (uint64_t)T, BK, BM, (uint64_t)ld * 2)) return cudaErrorInvalidValue;
     if (!make_map_box(&mb, w16, (uint64_t)n, (uint64_t)NC, BK, DG_BN, (uint64_t)ld * 2)) return cudaErrorInvalidValue;
-    if (!make_map_box(&mx, X, (uint64_t)NC, (uint64_t)T, DG_BN, BM)) return cudaErrorInvalidValue;
-    if (!make_map_box(&md, dX, (uint64_t)NC, (uint64_t)T, DG_BN, BM)) return cudaErrorInvalidValue;
+    if (!make_map_state(&mx, X, d.C, d.N, T, DG_BN, BM)) return cudaErrorInvalidValue;
+    if (!make_map_state(&md, dX, d.C, d.N, T, DG_BN, BM)) return cudaErrorInvalidValue;
     // the G d_input copies [G][T][C] as one [G T][C] matrix (rows of a token tile past T read the
     // next copy's rows or zeros; those rows are never stored)
     if (!make_map_box(&mg, dinput, (uint64_t)d.C, (uint64_t)d.G * T, DG_BN, BM)) return cudaErrorInvalidValue;
@@ -1492,7 +1546,8 @@ cudaError_t launch_dx_tc(const Dims& d, int T, const uint16_t* dz16,
     a.nkb = (n + BK - 1) / BK;
     a.ksteps = (n + 15) / 16;
     a.TT = (T + BM - 1) / BM;
-    a.CT = d.C / DG_BN;
+    a.CT = (d.C + DG_BN - 1) / DG_BN;
+    a.nbs = dxf_stages(n, d.G);
     a.ntiles = (long long)a.TT * a.CT;   // column blocks, N tiles each
     // a block's streams are split over several CTAs where that shortens the longest CTA's work (few
     // blocks): it takes its units x (their tiles + about 1.5 for the dZ rows and the token data).  512
@@ -1512,10 +1567,11 @@ cudaError_t launch_dx_tc(const Dims& d, int T, const uint16_t* dz16,
     a.X = X; a.dX = dX; a.dinput = dinput; a.hpre = hpre; a.I = I; a.dxact = dxact;
     a.scal = scal; a.scal_ld = scal_ld; a.err = err;
     a.wait_ns = debug_wait_ns();
-    const size_t sm = dxf_smem(n, d.G);
-    e = cudaFuncSetAttribute((const void*)k_dxf_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const size_t sm = dxf_smem(n, d.G, a.nbs);
+    auto* const kern = d.C % DG_BN == 0 ? &k_dxf_tc<false> : &k_dxf_tc<true>;
+    e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    XHC_LAUNCH(st, a.P, DX_THREADS, sm, (k_dxf_tc), ma, mb, mx, md, mg, a);
+    XHC_LAUNCH(st, a.P, DX_THREADS, sm, (kern), ma, mb, mx, md, mg, a);
     return cudaGetLastError();
 }
 

@@ -454,13 +454,14 @@ struct WRows {
     WSegs W;
     int n, rows, ld, parts;
     uint16_t* dst;   // null: nothing to pack
-    int frag;        // 1: rows in the order of dxa_row
+    int C;           // > 0: slots of C rows, each padded to dxa_width(C), in the order of dxa_row
 };
 // The weight row at place r of k_dx_tc's B operand: in every 32 rows, the one at 8 g + 2 q + e is channel 8 q +
 // 2 g + e, so that the accumulator's 16x256b fragments give a lane 8 neighbouring channels.
 __device__ __forceinline__ int dxa_row(int r) {
     return (r & ~31) | (((r >> 1) & 3) << 3) | (((r >> 3) & 3) << 1) | (r & 1);
 }
+inline int __host__ __device__ dxa_width(int C) { return (C + 31) / 32 * 32; }
 constexpr int WROWS_U = 8;   // elements per thread
 __device__ __forceinline__ void pack_wrows_of(const WRows& j, int blk) {
     const int at = blk * (int)blockDim.x * WROWS_U + threadIdx.x, tot = j.rows * j.ld;   // < 2^31
@@ -472,10 +473,17 @@ __device__ __forceinline__ void pack_wrows_of(const WRows& j, int blk) {
         v[u] = 0.f;
         part[u] = 0;
         if (idx < tot) {
-            const int r = idx / j.ld, c = idx - r * j.ld;
-            if (c < j.parts * j.n) {
+            int r = idx / j.ld;
+            const int c = idx - r * j.ld;
+            bool in = c < j.parts * j.n;
+            if (j.C > 0) {
+                const int slot = r / dxa_width(j.C), ch = dxa_row(r - slot * dxa_width(j.C));
+                in = in && ch < j.C;
+                r = slot * j.C + ch;
+            }
+            if (in) {
                 part[u] = c / j.n;
-                v[u] = seg_elem<true>(j.W, j.frag ? dxa_row(r) : r, c - part[u] * j.n);
+                v[u] = seg_elem<true>(j.W, r, c - part[u] * j.n);
             }
         }
     }
@@ -501,7 +509,7 @@ cudaError_t launch_proj_tc(const uint16_t* X, int T, int K, const uint16_t* Wpac
 // dzpack: the hi / lo rows of dz (DzPack::hilo, Tp tokens a row)
 cudaError_t launch_wgrad_tc(const uint16_t* A, int T, int E, int n, const uint16_t* dzpack, int Tp,
                             const ProjTcPlan& p, float* part, int* err, cudaStream_t st);
-bool dx_tc_ok(int T, int N, int C, int nfull, int G);
+int dx_tc_parts(int T, int N, int C, int nfull, int G);   // parts of the operands, 0: not on the tensor cores
 bool dxa_tc_ok(int T, int k, int C, int nact);
 // dX_act += dZ_act W_act^T (three-term bf16 split on the tensor cores) + H_pre[slot][I_j] d_input
 //           - cx x_act (the write-back's own term, cx per token in tokmat);
@@ -513,11 +521,11 @@ cudaError_t launch_dxa_tc(const Dims& d, int slot, int T, int nact,
                           const uint16_t* dz3, const uint16_t* w3, const uint16_t* d_input, const float* hpre,
                           const int* I, const uint16_t* xact, const float* tokmat, float* dxact,
                           float* dotp, uint16_t* dcopy, int* err, cudaStream_t st);
-// dH_pre[t][slot][I_j] = sum over the C/32 groups g of dotp[j][g][t] (g in order)
+// dH_pre[t][slot][I_j] = sum over the groups g of 32 channels of dotp[j][g][t] (g in order)
 cudaError_t launch_dots_act(const Dims& d, int slot, int T, const float* dotp, const int* I, float* dhpre,
                             cudaStream_t st);
-// (dz16, w16: the operands rounded once, parts 1)
-inline int dx_ld(int nfull) { return (nfull + 7) / 8 * 8; }
+// (dz16, w16: the operands in dx_tc_parts parts, K columns altogether)
+inline int dx_ld(int K) { return (K + 7) / 8 * 8; }
 cudaError_t launch_dx_tc(const Dims& d, int T, const uint16_t* dz16,
                          const uint16_t* w16, const uint16_t* X, const uint16_t* dinput, const float* hpre,
                          const int* I, const float* dxact, const float* scal, int scal_ld,

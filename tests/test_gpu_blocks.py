@@ -30,6 +30,13 @@ CASES = {
     "dx_split_N12_m0": (Config.full(12, 4, 0, 128, False), 131, {}),
     "dx_split_N9": (Config.full(9, 4, 2, 128, False), 200, {}),
     "dx_split_mhc": (Config.mhc(4, 128), 129, {}),
+    # input gradients on widths that their channel tiles do not divide: last tiles of 8, 40, 72, 8 and 72 channels,
+    # one or two stages of weight rows, eight active streams, no conv
+    "dx_width_C72_N20": (Config.flash(20, 4, 4, 72, 4, seq_len=100), 200, {}),
+    "dx_width_C40_mhc": (Config.mhc(4, 40), 131, {}),
+    "dx_width_C200_k6": (Config.flash(8, 6, 6, 200, 2, seq_len=128), 128, {}),
+    "dx_width_C1160_k8": (Config.full(12, 8, 3, 1160, True), 129, {}),
+    "dx_width_C584_N16": (Config.flash(16, 4, 2, 584, 4, seq_len=257), 257, {}),
     "coef_N27_conv1": (Config.flash(27, 4, 2, 64, 2, conv_k=(4,), seq_len=131), 262, {}),
 }
 
