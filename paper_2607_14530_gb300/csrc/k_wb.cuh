@@ -1178,15 +1178,16 @@ __device__ __forceinline__ uint4 ld16(const void* p) { return __ldg(reinterpret_
 __device__ __forceinline__ void l2_prefetch(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 constexpr int B8_PF = 2;   // L2 prefetch distance of the one-pass attention backward, in tokens
 
-// per-token tables shared by the CTA: E[j][0] (write-back coefficient of out), H_res, I
+// per-token tables shared by the CTA: E[j][0] = p_j H_post[j] (write-back coefficient of out), H_res, I
 template <int KM>
-__device__ __forceinline__ void k1_tables(int ntok, long long t0, int k, bool last, const float* emat,
-                                          int estride, const float* hres, const int* I, float* Esh,
+__device__ __forceinline__ void k1_tables(int ntok, long long t0, int k, bool last, const float* p,
+                                          const float* hpost, const float* hres, const int* I, float* Esh,
                                           float* Hsh, int* Ish) {
     for (int idx = threadIdx.x; idx < ntok * KM; idx += WT) {
         const int tt = idx / KM, j = idx - tt * KM;
-        Esh[idx] = (j < k) ? emat[(t0 + tt) * estride + j * 4] : 0.f;
-        Ish[idx] = (j < k) ? I[(t0 + tt) * k + j] : 0;
+        const long long tj = (t0 + tt) * k + j;
+        Ish[idx] = (j < k) ? I[tj] : 0;
+        Esh[idx] = (j < k) ? p[tj] * hpost[tj] : 0.f;
     }
     if (last)
         for (int idx = threadIdx.x; idx < ntok * KM * KM; idx += WT) {
@@ -1200,7 +1201,8 @@ __device__ __forceinline__ void k1_tables(int ntok, long long t0, int k, bool la
 template <int KM>
 __global__ void __launch_bounds__(WT) k_wb_fwd8(Dims d, int slot, int T, int TB,
                                                 const uint16_t* __restrict__ out,
-                                                const float* __restrict__ emat,
+                                                const float* __restrict__ p,
+                                                const float* __restrict__ hpost,
                                                 const uint16_t* __restrict__ xact,
                                                 const int* __restrict__ I,
                                                 const float* __restrict__ hres,
@@ -1215,7 +1217,7 @@ __global__ void __launch_bounds__(WT) k_wb_fwd8(Dims d, int slot, int T, int TB,
     const bool last = (slot == d.G - 1);
     const long long t0 = (long long)blockIdx.y * TB;
     const int ntok = (int)(min((long long)T, t0 + TB) - t0);
-    k1_tables<KM>(ntok, t0, k, last, emat, TOKMAT, hres, I, Esh, Hsh, Ish);
+    k1_tables<KM>(ntok, t0, k, last, p, hpost, hres, I, Esh, Hsh, Ish);
     __syncthreads();
     const int c = blockIdx.x * W8 + threadIdx.x * 8;
     if (c >= C) return;
@@ -1298,18 +1300,7 @@ __global__ void __launch_bounds__(WT, 3) k_wb_b8(Dims d, int slot, int T, int TB
     const bool last = (slot == d.G - 1);
     const long long t0 = (long long)blockIdx.y * TB;
     const int ntok = (int)(min((long long)T, t0 + TB) - t0);
-    for (int idx = threadIdx.x; idx < ntok * KM; idx += WT) {
-        const int tt = idx / KM, j = idx - tt * KM;
-        const long long tj = (t0 + tt) * k + j;
-        Ish[idx] = (j < k) ? I[tj] : 0;
-        Esh[idx] = (j < k) ? p[tj] * hpost[tj] : 0.f;
-    }
-    if (last)
-        for (int idx = threadIdx.x; idx < ntok * KM * KM; idx += WT) {
-            const int tt = idx / (KM * KM), q = idx - tt * (KM * KM);
-            const int j = q / KM, i = q - j * KM;
-            Hsh[idx] = (j < k && i < k) ? hres[(t0 + tt) * k * k + j * k + i] : 0.f;
-        }
+    k1_tables<KM>(ntok, t0, k, last, p, hpost, hres, I, Esh, Hsh, Ish);
     __syncthreads();
     const int c = blockIdx.x * W8 + threadIdx.x * 8;
     const bool act = c < C;

@@ -9,7 +9,8 @@ namespace {
 // for the backward and turned into the coefficients B of Eq. gs (orthogonalised component q = sum_a
 // B[q][a] u_a), so that the write-back of active slot j is sum_a E[j][a] u_a with E[j][a] = p_j sum_q
 // H_post[j][q] B[q][a]; without it B is the identity.  E goes to the per-token matrix buffer (rows
-// j < k, four entries each).  A block takes TB <= 32 tokens: a thread per (token, Gram entry) for the
+// j < k, four entries each).  Slots without a conv (K = 1, E[j][0] = p_j H_post[j]) form it in wb_fwd8
+// instead, a launch less: T = 8192, N = 4, one slot: 6 us of 762; T = 1536, four slots: 3.4 of 293.  A block takes TB <= 32 tokens: a thread per (token, Gram entry) for the
 // sums, a lane per token for the coefficients, a thread per (token, entry of E).
 
 constexpr int WC_NT = 128;
@@ -92,13 +93,13 @@ cudaError_t fwd_kw(const Dims& d, int slot, int T, const uint16_t* out, ConvPtrs
 }
 
 template <int KM>
-cudaError_t fwd8_kw(const Dims& d, int slot, int T, const uint16_t* out, const float* emat,
+cudaError_t fwd8_kw(const Dims& d, int slot, int T, const uint16_t* out, const float* p, const float* hpost,
                     const uint16_t* xact, const int* I, const float* hres, uint16_t* xact_next,
                     uint16_t* X, cudaStream_t st) {
     const int TB = pick_run(d, T, false, (d.C + W8 - 1) / W8, KM == 4 ? 6 : 3, 4, 32);
     const size_t sm = (size_t)TB * (KM + KM * KM + KM) * 4;
     dim3 grid((d.C + W8 - 1) / W8, (T + TB - 1) / TB);
-    XHC_LAUNCH(st, grid, WT, sm, (k_wb_fwd8<KM>), d, slot, T, TB, out, emat, xact, I, hres, xact_next, X);
+    XHC_LAUNCH(st, grid, WT, sm, (k_wb_fwd8<KM>), d, slot, T, TB, out, p, hpost, xact, I, hres, xact_next, X);
     return cudaGetLastError();
 }
 
@@ -136,14 +137,15 @@ cudaError_t launch_wb_coef(const Dims& d, int slot, int T, const float* red, int
 }
 
 cudaError_t launch_wb_fwd(const Dims& d, int slot, int T, const uint16_t* out, ConvPtrs cw,
-                          const float* emat, int nslice, const uint16_t* xact, const int* I,
-                          const float* hres, uint16_t* xact_next, uint16_t* X, cudaStream_t st) {
+                          const float* emat, const float* p, const float* hpost, int nslice,
+                          const uint16_t* xact, const int* I, const float* hres, uint16_t* xact_next, uint16_t* X,
+                          cudaStream_t st) {
     const bool conv = d.K[slot] > 1;
     if (d.k <= 4) {
-        if (!conv) return fwd8_kw<4>(d, slot, T, out, emat, xact, I, hres, xact_next, X, st);
+        if (!conv) return fwd8_kw<4>(d, slot, T, out, p, hpost, xact, I, hres, xact_next, X, st);
         XHC_KW_DISPATCH(d, wb_fast(d), (fwd_kw<4, KWC, KSC>(d, slot, T, out, cw, emat, nslice, xact, I, hres, xact_next, X, st)));
     }
-    if (!conv) return fwd8_kw<8>(d, slot, T, out, emat, xact, I, hres, xact_next, X, st);
+    if (!conv) return fwd8_kw<8>(d, slot, T, out, p, hpost, xact, I, hres, xact_next, X, st);
     XHC_KW_DISPATCH(d, false, (fwd_kw<8, KWC, KSC>(d, slot, T, out, cw, emat, nslice, xact, I, hres, xact_next, X, st)));
 }
 

@@ -554,8 +554,9 @@ cudaError_t launch_wb_gram(const Dims& d, int slot, int T, const uint16_t* out, 
 cudaError_t launch_wb_coef(const Dims& d, int slot, int T, const float* red, int nslice, const float* p,
                            const float* hpost, double* gram, float* emat, cudaStream_t st);
 cudaError_t launch_wb_fwd(const Dims& d, int slot, int T, const uint16_t* out, ConvPtrs cw,
-                          const float* emat, int nslice, const uint16_t* xact, const int* I,
-                          const float* hres, uint16_t* xact_next, uint16_t* X, cudaStream_t st);
+                          const float* emat, const float* p, const float* hpost, int nslice,
+                          const uint16_t* xact, const int* I, const float* hres, uint16_t* xact_next, uint16_t* X,
+                          cudaStream_t st);
 cudaError_t launch_wb_bred(const Dims& d, int slot, int T, const uint16_t* out, ConvPtrs cw,
                            const uint16_t* dX, const int* I, const float* dxact,
                            const uint16_t* xact, int nslice, float* red, cudaStream_t st);
