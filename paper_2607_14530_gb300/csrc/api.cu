@@ -628,7 +628,7 @@ xhc_status active_maps(const Ctx& c, int slot, const xhc_params* P) {
     if (!tc_act(c)) {
         XHC_K("rowproj_active", c.st, launch_rowproj(c.xact(slot), (int64_t)d.k * d.C, d.k * d.C, c.T, wa,
                                                      d.nact[slot], &ssplits, c.W<float>(c.L.part),
-                                                     c.W<float>(c.L.pstats), c.st));
+                                                     c.W<float>(c.L.pstats), ColJob{}, c.st));
         sp = slots_of(ssplits);
     } else {
         ProjTcPlan pl = plan_proj_tc(c.T, d.k * d.C, d.nact[slot], device_sms(), true);
@@ -666,12 +666,11 @@ xhc_status xhc_pre_fwd(const xhc_handle* h, int slot, int64_t T, const xhc_param
         SlotPlan sp;
         if (!tc_full(c)) {
             // smaller than one tensor-core tile: fp32 CUDA-core projection
-            if (d.hr)
-                XHC_K("colsum", c.st, launch_colsum(P->W_r, d.N * d.C, d.N, c.W<float>(c.L.wsump), c.st));
+            const ColJob cj = d.hr ? colsum_of(P->W_r, d.N * d.C, d.N, c.W<float>(c.L.wsump)) : ColJob{};
             int nslots = c.L.splits_full;
             XHC_K("rowproj_full", c.st, launch_rowproj(X, (int64_t)d.N * d.C, d.N * d.C, c.T, wf,
                                                        d.nfull, &nslots, c.W<float>(c.L.part),
-                                                       c.W<float>(c.L.pstats), c.st));
+                                                       c.W<float>(c.L.pstats), cj, c.st));
             sp = slots_of(nslots);
         } else {
         sp = slots_of(c.L.tc);

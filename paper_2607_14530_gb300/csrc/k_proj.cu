@@ -111,23 +111,29 @@ static cudaError_t rowproj_nt(const uint16_t* A, int64_t lda, int K, int T, cons
 // 4) of one weight segment and walks the rows NT / (n / V) apart with one V-wide load a row, times the
 // rows' TT state values from shared memory (fp32 FMAs on token pairs).  The row lanes' sums are folded
 // in shared memory at the end.  The 64-token tile above spends its FMAs on padding here: at N = 16,
-// C = 4096 one token took it 52 us for the 21 MB of the full-state weight.
+// C = 4096 one token took it 52 us for the 21 MB of the full-state weight.  The first blocks add up W_r's
+// columns (ColJob): as a kernel of its own before this one it cost a decoded token 6 us of 118.
 constexpr int RS_NT = 512;
 constexpr int RS_ROWS = 256;   // rows of the state staged at a time
 
 template <int TT, int V>
 __global__ void __launch_bounds__(RS_NT) k_rowproj_small(const uint16_t* __restrict__ A, int64_t lda, int K, int T,
                                                          WSegs W, int n, int kchunk, float* __restrict__ part,
-                                                         float* __restrict__ pstats) {
+                                                         float* __restrict__ pstats, ColJob cj) {
     pdl_entry();
     constexpr int TP = (TT + 1) / 2;                 // token pairs
     extern __shared__ __align__(16) float sm[];      // [RS_ROWS][2 TP] state rows; then [row lanes][n][TT]
     __shared__ float stat[TT][2];
+    if ((int)blockIdx.x < cj.parts) {
+        if (blockIdx.y == 0) colsum_chunk_of(cj.W, K, cj.N, cj.rchunk, blockIdx.x, sm, cj.out);
+        return;
+    }
+    const int split = blockIdx.x - cj.parts;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nv = n / V, nl = RS_NT / nv;           // column groups, row lanes
     const int rl = tid / nv, o = (tid - rl * nv) * V;
     const bool work = rl < nl;
-    const int k0 = blockIdx.x * kchunk, k1 = min(K, k0 + kchunk);
+    const int k0 = split * kchunk, k1 = min(K, k0 + kchunk);
     const int t0 = blockIdx.y * TT;
     // this thread's weight segment, selected with static indices
     const float* wp = W.ptr[0];
@@ -216,14 +222,14 @@ __global__ void __launch_bounds__(RS_NT) k_rowproj_small(const uint16_t* __restr
         m = h;
     }
     const int nt = min(TT, T - t0);
-    const int64_t row = (int64_t)blockIdx.x * T + t0;
+    const int64_t row = (int64_t)split * T + t0;
     for (int e = tid; e < nt * n; e += RS_NT) part[row * n + e] = sm[e];
     if (tid < 2 * nt) pstats[row * 2 + tid] = stat[tid >> 1][tid & 1];
 }
 
 template <int TT, int V>
 static cudaError_t rowproj_small(const uint16_t* A, int64_t lda, int K, int T, const WSegs& W, int n, int* splits,
-                                 float* part, float* pstats, cudaStream_t st) {
+                                 float* part, float* pstats, const ColJob& cj, cudaStream_t st) {
     const int nl = RS_NT / (n / V), ny = (T + TT - 1) / TT;
     // a block per SM, with at least four rows a row lane
     int s = std::min(*splits, std::max(1, device_sms() / ny));
@@ -234,41 +240,20 @@ static cudaError_t rowproj_small(const uint16_t* A, int64_t lda, int K, int T, c
     const size_t sm = sizeof(float) * std::max((size_t)RS_ROWS * ((TT + 1) / 2 * 2), (size_t)nl * n * TT);
     const cudaError_t e = smem_optin((const void*)k_rowproj_small<TT, V>, sm);
     if (e != cudaSuccess) return e;
-    XHC_LAUNCH(st, dim3(s, ny), RS_NT, sm, (k_rowproj_small<TT, V>), A, lda, K, T, W, n, kchunk, part, pstats);
+    XHC_LAUNCH(st, dim3(cj.parts + s, ny), RS_NT, sm, (k_rowproj_small<TT, V>), A, lda, K, T, W, n, kchunk, part, pstats, cj);
     return cudaGetLastError();
 }
 
 template <int V>
 static cudaError_t rowproj_small_v(const uint16_t* A, int64_t lda, int K, int T, const WSegs& W, int n, int* splits,
-                                   float* part, float* pstats, cudaStream_t st) {
-    if (T <= 1) return rowproj_small<1, V>(A, lda, K, T, W, n, splits, part, pstats, st);
-    if (T <= 2) return rowproj_small<2, V>(A, lda, K, T, W, n, splits, part, pstats, st);
-    if (T <= 4) return rowproj_small<4, V>(A, lda, K, T, W, n, splits, part, pstats, st);
-    if (T <= 8) return rowproj_small<8, V>(A, lda, K, T, W, n, splits, part, pstats, st);
-    return rowproj_small<16, V>(A, lda, K, T, W, n, splits, part, pstats, st);
+                                   float* part, float* pstats, const ColJob& cj, cudaStream_t st) {
+    if (T <= 1) return rowproj_small<1, V>(A, lda, K, T, W, n, splits, part, pstats, cj, st);
+    if (T <= 2) return rowproj_small<2, V>(A, lda, K, T, W, n, splits, part, pstats, cj, st);
+    if (T <= 4) return rowproj_small<4, V>(A, lda, K, T, W, n, splits, part, pstats, cj, st);
+    if (T <= 8) return rowproj_small<8, V>(A, lda, K, T, W, n, splits, part, pstats, cj, st);
+    return rowproj_small<16, V>(A, lda, K, T, W, n, splits, part, pstats, cj, st);
 }
 
-cudaError_t launch_rowproj(const uint16_t* A, int64_t lda, int K, int T, const WSegs& W, int n,
-                           int* nslots, float* part, float* pstats, cudaStream_t st) {
-    const int splits = *nslots;
-    if (T < ROWPROJ_SMALL) {
-        // four columns a load where the segments' rows allow 16-byte loads
-        bool v4 = true;
-        for (int q = 0; q < W.n; ++q) v4 = v4 && W.width[q] % 4 == 0 && ((uintptr_t)W.ptr[q] & 15u) == 0;
-        return v4 ? rowproj_small_v<4>(A, lda, K, T, W, n, nslots, part, pstats, st)
-                  : rowproj_small_v<1>(A, lda, K, T, W, n, nslots, part, pstats, st);
-    }
-    const int nt = (n + 15) / 16;
-    if (nt <= 1) return rowproj_nt<1>(A, lda, K, T, W, n, splits, part, pstats, st);
-    if (nt <= 2) return rowproj_nt<2>(A, lda, K, T, W, n, splits, part, pstats, st);
-    if (nt <= 4) return rowproj_nt<4>(A, lda, K, T, W, n, splits, part, pstats, st);
-    if (nt <= 6) return rowproj_nt<6>(A, lda, K, T, W, n, splits, part, pstats, st);
-    if (nt <= 8) return rowproj_nt<8>(A, lda, K, T, W, n, splits, part, pstats, st);
-    if (nt <= 10) return rowproj_nt<10>(A, lda, K, T, W, n, splits, part, pstats, st);
-    return cudaErrorInvalidValue;
-}
-
-// ---------------------------------------------------------------------------------------------
 // colsum: partial column sums of in [rows][n] (n <= MAXN), a block per chunk of rows
 
 __global__ void __launch_bounds__(8 * MAXN) k_colsum(const float* __restrict__ in, int rows, int n, int rchunk,
@@ -284,10 +269,34 @@ int colsum_parts(int rows) {
     const int rchunk = colsum_chunk(rows);
     return (rows + rchunk - 1) / rchunk;
 }
+ColJob colsum_of(const float* W_r, int rows, int N, float* out) {
+    const ColJob j = {W_r, N, colsum_parts(rows), colsum_chunk(rows), out};
+    return j;
+}
 
-cudaError_t launch_colsum(const float* in, int rows, int n, float* out, cudaStream_t st) {
-    XHC_LAUNCH(st, colsum_parts(rows), 8 * n, 0, (k_colsum), in, rows, n, colsum_chunk(rows), out);
-    return cudaGetLastError();
+cudaError_t launch_rowproj(const uint16_t* A, int64_t lda, int K, int T, const WSegs& W, int n,
+                           int* nslots, float* part, float* pstats, const ColJob& cj, cudaStream_t st) {
+    const int splits = *nslots;
+    if (T < ROWPROJ_SMALL) {
+        // four columns a load where the segments' rows allow 16-byte loads
+        bool v4 = true;
+        for (int q = 0; q < W.n; ++q) v4 = v4 && W.width[q] % 4 == 0 && ((uintptr_t)W.ptr[q] & 15u) == 0;
+        return v4 ? rowproj_small_v<4>(A, lda, K, T, W, n, nslots, part, pstats, cj, st)
+                  : rowproj_small_v<1>(A, lda, K, T, W, n, nslots, part, pstats, cj, st);
+    }
+    if (cj.parts > 0) {   // 128 tokens of a state narrower than 64: a launch of its own
+        XHC_LAUNCH(st, cj.parts, 8 * cj.N, 0, (k_colsum), cj.W, K, cj.N, cj.rchunk, cj.out);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    const int nt = (n + 15) / 16;
+    if (nt <= 1) return rowproj_nt<1>(A, lda, K, T, W, n, splits, part, pstats, st);
+    if (nt <= 2) return rowproj_nt<2>(A, lda, K, T, W, n, splits, part, pstats, st);
+    if (nt <= 4) return rowproj_nt<4>(A, lda, K, T, W, n, splits, part, pstats, st);
+    if (nt <= 6) return rowproj_nt<6>(A, lda, K, T, W, n, splits, part, pstats, st);
+    if (nt <= 8) return rowproj_nt<8>(A, lda, K, T, W, n, splits, part, pstats, st);
+    if (nt <= 10) return rowproj_nt<10>(A, lda, K, T, W, n, splits, part, pstats, st);
+    return cudaErrorInvalidValue;
 }
 
 // ---------------------------------------------------------------------------------------------

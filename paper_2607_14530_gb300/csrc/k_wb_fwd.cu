@@ -10,8 +10,9 @@ namespace {
 // B[q][a] u_a), so that the write-back of active slot j is sum_a E[j][a] u_a with E[j][a] = p_j sum_q
 // H_post[j][q] B[q][a]; without it B is the identity.  E goes to the per-token matrix buffer (rows
 // j < k, four entries each).  Slots without a conv (K = 1, E[j][0] = p_j H_post[j]) form it in wb_fwd8
-// instead, a launch less: T = 8192, N = 4, one slot: 6 us of 762; T = 1536, four slots: 3.4 of 293.  A block takes TB <= 32 tokens: a thread per (token, Gram entry) for the
-// sums, a lane per token for the coefficients, a thread per (token, entry of E).
+// instead, a launch less: T = 8192, N = 4, one slot: 6 us of 762; T = 1536, four slots: 3.4 of 293.
+// A block takes TB <= 32 tokens: a thread per (token, Gram entry) for the sums, a lane per token for the
+// coefficients, a thread per (token, entry of E).
 
 constexpr int WC_NT = 128;
 

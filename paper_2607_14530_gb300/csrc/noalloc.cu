@@ -77,8 +77,7 @@ extern "C" xhc_status xhc_route_noalloc(const xhc_handle* hh, int64_t T, const x
     float* wsump = (float*)(base + o_wsump);
     // every scratch word read below is first written by this call (split-K partials, column
     // sums, statistics), so no clearing is needed
-    if (d.hr && launch_colsum(P->W_r, d.N * d.C, d.N, wsump, st) != cudaSuccess)
-        return XHC_ERR_CUDA;
+    const ColJob cj = d.hr ? colsum_of(P->W_r, d.N * d.C, d.N, wsump) : ColJob{};
     WSegs w;
     memset(&w, 0, sizeof(w));
     int off = 0;
@@ -89,7 +88,7 @@ extern "C" xhc_status xhc_route_noalloc(const xhc_handle* hh, int64_t T, const x
         w.ptr[w.n] = P->W_pre[q]; w.width[w.n] = d.N; w.off[w.n] = off; off += d.N; ++w.n;
     }
     w.off[w.n] = off;
-    if (launch_rowproj(X, (int64_t)d.N * d.C, d.N * d.C, (int)T, w, d.nfull, &splits, part, pst, st) !=
+    if (launch_rowproj(X, (int64_t)d.N * d.C, d.N * d.C, (int)T, w, d.nfull, &splits, part, pst, cj, st) !=
         cudaSuccess)
         return XHC_ERR_CUDA;
     if (launch_coef_full(d, (int)T, part, pst, slots_of(splits), wsump, colsum_parts(d.N * d.C), P->alpha_pre, P->b_pre,

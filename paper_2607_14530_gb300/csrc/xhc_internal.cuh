@@ -385,10 +385,17 @@ int debug_take_force_timeout();
 // ---------------------------------------------------------------------------------------------
 // launchers (each returns cudaGetLastError() after enqueueing)
 
+// Partial column sums of W_r [rows][N], formed in the launch of the projection: parts 0, none wanted.
+struct ColJob {
+    const float* W;
+    int N, parts, rchunk;
+    float* out;   // [parts][N]
+};
+ColJob colsum_of(const float* W_r, int rows, int N, float* out);
 // fp32 CUDA-core projection into *nslots partial slots at most (on return: the number written)
 constexpr int ROWPROJ_SMALL = 128;   // fewer tokens than this: the kernel for few tokens
 cudaError_t launch_rowproj(const uint16_t* A, int64_t lda, int K, int T, const WSegs& W, int n,
-                           int* nslots, float* part, float* pstats, cudaStream_t st);
+                           int* nslots, float* part, float* pstats, const ColJob& cj, cudaStream_t st);
 // One weight packed for k_proj_tc: rows 0..n-1 of dst [NB][K] the bf16 hi parts of W[e][o], rows
 // n..2n-1 the lo parts, the rest zero.
 struct PackJob {
@@ -605,7 +612,6 @@ __device__ __forceinline__ void colsum_chunk_of(const float* __restrict__ in, in
         out[part * n + o] = t;
     }
 }
-cudaError_t launch_colsum(const float* in, int rows, int n, float* out, cudaStream_t st);
 // wsum: [nws][N] partial column sums of W_r; their sum is left in wsum_out [N]
 cudaError_t launch_coef_full(const Dims& d, int T, const float* part, const float* pstats,
                              const SlotPlan& sp, const float* wsum, int nws, const float* alpha_pre,
