@@ -859,17 +859,19 @@ xhc_status post_bwd_impl(const xhc_handle* h, int slot, int64_t T, const xhc_par
     const int K = d.K[slot], n = d.nact[slot];
     float* red = c.W<float>(c.L.red);
     float* dxact = c.W<float>(c.L.dxact);
-    if (last)
+    // the entry rows go back into X, in groups of one slot mostly by the reductions below
+    uint16_t* const Xr = wb_puts_back(d) ? X : nullptr;
+    if (last && !Xr)
         XHC_K("restore", c.st, launch_restore(d, T32, c.xact(0), c.S<int>(c.L.I), X, c.st));
     const int bslices = wb_bred_slices(d, slot);
     if (K == 1) {
         // no conv: reductions and apply in one pass (the apply coefficients are forward values)
         XHC_K("wb_b8", c.st, launch_wb_b8(d, slot, T32, out, dX, c.S<int>(c.L.I), c.S<float>(c.L.p),
                                           c.S<float>(c.L.hpost[slot]), c.S<float>(c.L.hres), dxact, dxact,
-                                          c.xact(slot), bslices, red, d_out, c.st));
+                                          c.xact(slot), bslices, red, d_out, Xr, c.st));
     } else {
         XHC_K("wb_bred", c.st, launch_wb_bred(d, slot, T32, out, cw, dX, c.S<int>(c.L.I), dxact, c.xact(slot),
-                                              bslices, red, c.st));
+                                              bslices, red, Xr, c.st));
     }
     // the bf16 operands of the weight gradient and of pre_bwd(slot)'s input gradient, formed with dZ_act
     const bool tcw = !(T32 < 64 || d.k * d.C < 128), tcx = dxa_tc_ok(T32, d.k, d.C, n);

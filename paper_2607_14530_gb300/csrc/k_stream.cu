@@ -7,7 +7,8 @@
 //               sum of squares of x_act; the slot's active weight is packed by further blocks
 //   (the sums of squares are the norm statistics of the slot's active-state projection, which
 //   then reads its operand only through the tensor-core pipeline)
-//   restore     put the saved entry rows back into X before the backward
+//   restore     put the saved entry rows back into X before the backward (groups of one slot with k <= 4: the
+//               write-back's reductions do)
 //   conv_wgrad_reduce  sum of the per-run conv weight-gradient partials
 //   dinput_act  dense-read backward on the active streams (and dH_pre of the active streams)
 //   full_dots   dH_pre of the non-active streams: <x_i, d_input_t>

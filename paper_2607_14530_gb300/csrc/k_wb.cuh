@@ -2,10 +2,10 @@
 //
 // Every kernel here walks a run of consecutive tokens for one pair of channels per thread.  The
 // conv taps of the pair and a ring of the recent values of `out` stay in registers, indexed by
-// compile-time positions: wb_gram unrolls the token loop by KW over a KW-slot ring; the forward
-// apply and the backward kernels unroll it by 4-token blocks over a ring of KW + 3 slots that
-// moves by 4 after each block (a shorter loop body: the 12-token one overflowed the instruction
-// cache).  Each out value is loaded once per run instead of once per tap.  Runs never cross a sequence boundary (Sec.
+// compile-time positions: the general wb_gram unrolls the token loop by KW over a KW-slot ring; the
+// others unroll it by 4-token blocks over a ring of KW + 3 slots that moves by 4 after each block (a
+// shorter loop body: the 12-token one overflowed the instruction cache).  Each out value is loaded once
+// per run instead of once per tap.  Runs never cross a sequence boundary (Sec.
 // 3.3.4: the conv restarts with every sequence), so the conv needs no per-tap test.  KS = 1
 // specialises the tap counts to the (4, 8, 12) kernels of the MLP sublayers, so no FMA is spent
 // on zero taps.  Per-token reductions over the channels use a reduce-scatter butterfly inside
@@ -567,15 +567,15 @@ struct BRing {
 
 // Per token, NV partial sums over this CTA's channel slice: P[j][a] = <dXn_j, u_a> at j*4 + a
 // and, on the last slot, Q[j][i] = <dXn_j, x_i> at KM*4 + j*KM + i.  NV = 16 is reduced to
-// lane pairs, larger NV in blocks of 32.
-template <int KM, int KW, int NV, int KS>
+// lane pairs, larger NV in blocks of 32.  PUT (last slot): the x_j rows also go back into Xr.
+template <int KM, int KW, int NV, int KS, bool PUT>
 __global__ void __launch_bounds__(WT) k_wb_bred(Dims d, int slot, int T, int TB,
                                                 const uint16_t* __restrict__ out, ConvPtrs cw,
                                                 const uint16_t* __restrict__ dX,
                                                 const int* __restrict__ I,
                                                 const float* __restrict__ dxact,
                                                 const uint16_t* __restrict__ xact, int nslice,
-                                                float* __restrict__ red) {
+                                                float* __restrict__ red, uint16_t* __restrict__ Xr) {
     pdl_entry();
     static_assert(NV == 16 || NV % 32 == 0, "reduction width");
     constexpr int NVP = NV < 32 ? 16 : NV;      // values per token and warp in shared memory
@@ -666,8 +666,11 @@ __global__ void __launch_bounds__(WT) k_wb_bred(Dims d, int slot, int T, int TB,
                         if (j >= k) continue;
                         const uint2 r = R.dn[sl][j][threadIdx.x];
                         if (last) {
+                            const uint32_t xv = R.x[sl][j][threadIdx.x];
                             dn[j] = u2f2(r.x);
-                            x[j] = u2f2(R.x[sl][j][threadIdx.x]);
+                            x[j] = u2f2(xv);
+                            if constexpr (PUT)
+                                *reinterpret_cast<uint32_t*>(Xr + (t0 + tt) * NC + (long long)Ish[tt * KM + j] * C + c) = xv;
                         } else {
                             dn[j] = make_float2(__uint_as_float(r.x), __uint_as_float(r.y));
                         }
@@ -727,7 +730,8 @@ __global__ void __launch_bounds__(WT) k_wb_bred(Dims d, int slot, int T, int TB,
 // The same reductions with two channel pairs per thread (4 consecutive channels, WSL2 channels
 // per CTA): a token's warp reduction then covers 128 channels instead of 64, halving its cost
 // per channel, and the loads are 8 / 16 bytes wide.  For the (4, 8, 12) tap set with k = KM
-// and C a multiple of WSL2 (every thread in range).
+// and C a multiple of WSL2 (every thread in range).  PUT: the x_j rows also go back into Xr (a branch in its
+// place broke up the interleaved tokens below: T = 2103, C = 1536, where nothing is put: 514 -> 521 us a step).
 
 template <int KM>
 struct BRing2 {   // two blocks of UB tokens
@@ -735,14 +739,14 @@ struct BRing2 {   // two blocks of UB tokens
     uint4 v[2 * UB][KM][WT];   // dn_j: four fp32, or at the last slot dX's four bf16 and x_j's four
 };
 
-template <int KM, int NV>
+template <int KM, int NV, bool PUT>
 __global__ void __launch_bounds__(WT, 2) k_wb_bred2(Dims d, int slot, int T, int TB,
                                                     const uint16_t* __restrict__ out, ConvPtrs cw,
                                                     const uint16_t* __restrict__ dX,
                                                     const int* __restrict__ I,
                                                     const float* __restrict__ dxact,
                                                     const uint16_t* __restrict__ xact, int nslice,
-                                                    float* __restrict__ red) {
+                                                    float* __restrict__ red, uint16_t* __restrict__ Xr) {
     pdl_entry();
     constexpr int KW = 12, KS = 2;
     static_assert(NV == 16 || NV % 32 == 0, "reduction width");
@@ -830,6 +834,9 @@ __global__ void __launch_bounds__(WT, 2) k_wb_bred2(Dims d, int slot, int T, int
                     dn[1][j] = u2f2(r.y);
                     x[0][j] = u2f2(r.z);
                     x[1][j] = u2f2(r.w);
+                    if constexpr (PUT)
+                        *reinterpret_cast<uint2*>(Xr + (t0 + tt) * NC + (long long)Ish[tt * KM + j] * C + c) =
+                            make_uint2(r.z, r.w);
                 } else {
                     dn[0][j] = make_float2(__uint_as_float(r.x), __uint_as_float(r.y));
                     dn[1][j] = make_float2(__uint_as_float(r.z), __uint_as_float(r.w));
@@ -1274,7 +1281,8 @@ __global__ void __launch_bounds__(WT) k_wb_fwd8(Dims d, int slot, int T, int TB,
 // d_out = sum_j E[j][0] dXn_j (last slot: dX_act_i = sum_j H_res[j][i] dXn_j) read dXn once.
 // Partial sums per W8-channel slice: P[j][0] at j*4, Q[j][i] at KM*4 + j*KM + i (the layout
 // bwd_coef reads).
-template <int KM>
+// PUT: the x_j rows also go back into Xr.
+template <int KM, bool PUT>
 __global__ void __launch_bounds__(WT, 3) k_wb_b8(Dims d, int slot, int T, int TB,
                                               const uint16_t* __restrict__ out,
                                               const uint16_t* __restrict__ dX,
@@ -1286,7 +1294,7 @@ __global__ void __launch_bounds__(WT, 3) k_wb_b8(Dims d, int slot, int T, int TB
                                               float* dxact_out,     // written (last slot)
                                               const uint16_t* __restrict__ xact, int nslice,
                                               float* __restrict__ red,
-                                              uint16_t* __restrict__ d_out) {
+                                              uint16_t* __restrict__ d_out, uint16_t* __restrict__ Xr) {
     pdl_entry();
     constexpr int NQ = KM + KM * KM;                  // P[j][0], then Q[j][i]
     constexpr int NV = NQ <= 32 ? 32 : 96;            // reduce-scatter width (blocks of 32)
@@ -1430,6 +1438,8 @@ __global__ void __launch_bounds__(WT, 3) k_wb_b8(Dims d, int slot, int T, int TB
                     float4* dst = reinterpret_cast<float4*>(dxact_out + t * kC + (long long)i * C + c);
                     dst[0] = make_float4(w[0], w[1], w[2], w[3]);
                     dst[1] = make_float4(w[4], w[5], w[6], w[7]);
+                    if constexpr (PUT)
+                        *reinterpret_cast<uint4*>(Xr + t * NC + (long long)Ish[tt * KM + i] * C + c) = xc[i];
                 }
             }
         }

@@ -564,13 +564,16 @@ cudaError_t launch_wb_fwd(const Dims& d, int slot, int T, const uint16_t* out, C
                           const float* emat, const float* p, const float* hpost, int nslice,
                           const uint16_t* xact, const int* I, const float* hres, uint16_t* xact_next, uint16_t* X,
                           cudaStream_t st);
+// Xr (both): the last slot's x_j rows are also put back into this state; null: not, as it has to be unless
+// wb_puts_back
+bool wb_puts_back(const Dims& d);
 cudaError_t launch_wb_bred(const Dims& d, int slot, int T, const uint16_t* out, ConvPtrs cw,
                            const uint16_t* dX, const int* I, const float* dxact,
-                           const uint16_t* xact, int nslice, float* red, cudaStream_t st);
+                           const uint16_t* xact, int nslice, float* red, uint16_t* Xr, cudaStream_t st);
 cudaError_t launch_wb_b8(const Dims& d, int slot, int T, const uint16_t* out, const uint16_t* dX,
                          const int* I, const float* p, const float* hpost, const float* hres,
                          const float* dxact, float* dxact_out, const uint16_t* xact, int nslice,
-                         float* red, uint16_t* d_out, cudaStream_t st);
+                         float* red, uint16_t* d_out, uint16_t* Xr, cudaStream_t st);
 cudaError_t launch_wb_bapp(const Dims& d, int slot, int T, const uint16_t* out, ConvPtrs cw,
                            const uint16_t* dX, const int* I, const float* dn_in,
                            const float* tokmat, float* dxact_out, uint16_t* d_out, float* cpart,
