@@ -86,45 +86,50 @@ def kernel_model(cfg, T):
     tb = 296 if kw else 0  # tokens per run of the backward apply (bapp_run)
     runs = (T // S) * -(-S // tb) + -(-(T % S) // tb) if kw else 0
     cpart = runs * sum(cfg.conv_k) * C * f32
-    # forward
-    if hr:
-        add("colsum", N * C * N * f32)
+    # forward; the active weights are packed ahead of their projections: slot 0's with the full-state one,
+    # later slots' in blocks of the input kernel
+    def pack_act(t):
+        return k * C * nact[t] * f32 + 2 * nact[t] * k * C * b16
+
     nb = 2 * nfull  # hi + lo bf16 rows of the packed weight
-    add("pack_w", N * C * nfull * f32 + nb * N * C * b16)
+    # with the column sums of W_r
+    add("pack_w", N * C * nfull * f32 + nb * N * C * b16 + (N * C * N * f32 if hr else 0) + pack_act(0))
     # tensor-core projection: X read once; the packed weight streams from L2
     add("proj_tc", X + T * nfull * f32, 2.0 * T * N * C * nb, "hbm")
     add("coef_full", T * nfull * f32 + T * (G * N + 2 * k) * f32)
     add("read", X + row + (G - 1) * row + xa)
     for t in range(G):
         if t > 0:
-            add("input", row + xa + row)
-        add("pack_w", k * C * nact[t] * f32 + 2 * nact[t] * k * C * b16)
+            add("input", row + xa + row + pack_act(t))
         add("proj_tc_active", xa + T * nact[t] * f32, 2.0 * T * k * C * 2 * nact[t], "hbm")
         add("coef_act", T * nact[t] * f32 * 2)
         if Ks[t] > 1 and gs:
             add("wb_gram", row)
+        if Ks[t] > 1:
+            add("wb_coef", T * (k * Ks[t] + k + 4 * k) * f32)
         add("wb_fwd", row + xa + xa)
     # backward
     for t in reversed(range(G)):
         last = t == G - 1
         dxn = xa if last else xa32
-        if last:
+        put = G == 1 and k <= 4   # the reductions put the entry rows back, else a copy does
+        if last and not put:
             add("restore", 2 * xa)
         if Ks[t] == 1:
             # one pass: out, dXn (and x_act on the last slot) read; d_out and, on the last slot,
             # the mixed active gradient written
-            add("wb_b8", row + dxn + (xa if last else 0) + row + (xa32 if last else 0))
+            add("wb_b8", row + dxn + (xa if last else 0) + row + (xa32 if last else 0) + (xa if put else 0))
         else:
-            add("wb_bred", row + dxn + (xa if last else 0))
-        add("bwd_coef", T * nact[t] * f32 * 2)
+            add("wb_bred", row + dxn + (xa if last else 0) + (xa if put else 0))
+        # also dZ and the weight as the bf16 operands of the gradient products
+        add("bwd_coef", T * nact[t] * (2 * f32 + 5 * b16) + k * C * nact[t] * (f32 + 3 * b16))
         if Ks[t] > 1:
             # out, dXn read; d_out written; last slot writes the mixed active gradient; conv partials
             add("wb_bapp", row + dxn + row + (xa32 if last else 0) + cpart)
         add("wgrad_tc_active", xa + T * nact[t] * f32 + 2 * T * nact[t] * b16 + k * C * nact[t] * f32,
             2.0 * T * k * C * 2 * nact[t], "hbm")
         add("wgrad_reduce", 2 * k * C * nact[t] * f32)
-        for _ in range(4 if last else 2):
-            add("colsum", T * 16 * f32)
+        add("colsum_out", T / 32 * (k * Ks[t] + 1 + (k * k + 1 if last else 0)) * f32)
         if Ks[t] > 1:
             add("conv_wgrad_reduce", cpart)
         # pre-map backward of the slot on the tensor cores: dX_act += dZ W^T + H_pre d_input
@@ -134,22 +139,16 @@ def kernel_model(cfg, T):
         add("dxa_tc", 2 * xa32 + xa + row + row + dotp + 3 * T * nact[t] * b16,
             2.0 * T * k * C * 3 * nact[t], "hbm")
         add("dots_act", dotp + T * k * 4 + T * k * f32)
-    if hr:
-        add("colsum", N * C * N * f32)
     # dH_pre of the inactive streams: their X rows and the G d_input rows read
     add("full_dots", T * (N - k) * C * b16 + G * row)
-    add("full_coef", T * (nfull + G * N) * f32)
+    add("full_coef", T * ((nfull + G * N) * f32 + 3 * nfull * b16) + N * C * nfull * (f32 + b16))
     # tensor-core dX: X read, inactive dX rows read, active-row gradient read, the G d_input rows
     # read once per column block (dense-read gradient of the inactive rows), dX written
     add("dx_tc", X + T * (N - k) * C * b16 + xa32 + G * row + X, 2.0 * T * N * C * nfull, "hbm")
     add("wgrad_tc_full", X + T * nfull * f32 + 2 * T * nfull * b16 + N * C * nfull * f32,
         2.0 * T * N * C * 2 * nfull, "hbm")
     add("wgrad_reduce", 2 * N * C * nfull * f32)
-    add("colsum", T * G * N * f32)
-    add("colsum", T * G * f32)
-    if hr:
-        add("colsum", T * N * f32)
-        add("sub_rows", 2 * N * C * N * f32)
+    add("colsum_out", T / 32 * (G * N + G + (N if hr else 0)) * f32)
     return m
 
 

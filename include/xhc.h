@@ -27,7 +27,8 @@
  * unless stated).  The library allocates no device memory, never synchronises, and enqueues
  * all work asynchronously on the caller's stream (a cudaStream_t passed as void*; NULL = the
  * legacy default stream).  post_bwd and pre_bwd(0) run their weight-gradient and column-sum
- * kernels on an internal stream of the device (created on first use, one per device), forked
+ * kernels (on states above 256 MB not the full-state weight gradient, which follows the rest of
+ * pre_bwd(0)) on an internal stream of the device (created on first use, one per device), forked
  * from the caller's stream with an event after the work they depend on and joined back into
  * it with an event before the call returns: to the caller every call stays ordered on its
  * stream.  `saved` (xhc_saved_bytes) carries the group's forward state to its
@@ -227,8 +228,8 @@ xhc_status xhc_post_fwd_decode(const xhc_handle* h, int slot, int64_t B, const x
                                void* saved, void* workspace, void* stream);
 
 /* Backward of post_fwd(slot).  Reads dX (slot G-1: the gradient w.r.t. the group output) or the
- * workspace-held active gradient, leaves the post/res map-logit gradient in the workspace for
- * pre_bwd(slot), writes d_out [T, C] (= dL/d out, including the paths through
+ * workspace-held active gradient, leaves the post/res map-logit gradient and its projection
+ * weight (both as pre_bwd(slot) multiplies them) in the workspace, writes d_out [T, C] (= dL/d out, including the paths through
  * later sublayer inputs), accumulates the post/res/conv parameter gradients.  slot G-1 also
  * restores the active rows of X to the group-entry state. */
 xhc_status xhc_post_bwd(const xhc_handle* h, int slot, int64_t T, const xhc_params* P,
@@ -236,8 +237,8 @@ xhc_status xhc_post_bwd(const xhc_handle* h, int slot, int64_t T, const xhc_para
                         const xhc_grads* grads, void* saved, void* workspace, void* stream);
 
 /* Backward of pre_fwd(slot).  Adds the dense-read gradient of d_input and the gradient through
- * the post/res map projections of this slot to the active gradient (the map-logit gradient is
- * left in the workspace by post_bwd(slot), so the calls of one slot run back to back on the same
+ * the post/res map projections of this slot to the active gradient (the map-logit gradient and
+ * the weight are left in the workspace by post_bwd(slot), so the calls of one slot run back to back on the same
  * workspace; P needs W_post[slot], and W_res at the last slot, on every slot); slot 0 finishes
  * the group: dX becomes the gradient w.r.t. the entry state (dense reads,
  * norm statistics, router through the selected routed scores only) and the W_r / W_pre /
@@ -350,7 +351,7 @@ xhc_status xhc_workspace_error(const void* workspace, int* code, int clear);
  *   nothing triggers, so that every wait of that launch runs out: it sets the workspace's error
  *   word and returns without touching its outputs.  One-shot.
  * XHC_DEBUG_ONE_STREAM: value != 0 runs the work that later calls put on the library's side
- *   stream (weight gradients, column sums, dH_pre dots) on the caller's stream instead, in the
+ *   stream (weight gradients, column sums) on the caller's stream instead, in the
  *   same order; the results are the same.  0 restores the side stream.
  * Returns XHC_ERR_INVALID_ARG for an unknown `what` or a negative limit. */
 #define XHC_DEBUG_WAIT_LIMIT_NS 1

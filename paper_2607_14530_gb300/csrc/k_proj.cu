@@ -3,9 +3,10 @@
 //             param_res), split over the reduction dimension, plus sum / sum of squares of A: fewer
 //             than 128 tokens, and the routing entry point without a workspace
 //   gemm_dzw  dX_act += dZ W^T (backward of the active projection)
-//   full_dx   dX = dX_base + dZ W^T + a + b x (backward of the full-state projection and norms)
+//   full_dx   dX = dX_base + dZ W^T + a + b x (backward of the full-state projection and norms); both
+//             where the tensor-core kernels do not apply (fewer than 128 tokens, very many columns)
 //   wgrad     dW += A^T dZ, reduced over tokens in a fixed order
-//   colsum    fixed-order partial column sums of W_r
+//   colsum    fixed-order partial column sums of W_r (within rowproj below 128 tokens)
 #include <algorithm>
 
 #include "xhc_internal.cuh"

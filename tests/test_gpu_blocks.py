@@ -37,6 +37,8 @@ CASES = {
     "dx_width_C200_k6": (Config.flash(8, 6, 6, 200, 2, seq_len=128), 128, {}),
     "dx_width_C1160_k8": (Config.full(12, 8, 3, 1160, True), 129, {}),
     "dx_width_C584_N16": (Config.flash(16, 4, 2, 584, 4, seq_len=257), 257, {}),
+    # entry rows put back by the two-pair reductions (512-channel slices): a run that ends inside a block of 4
+    "put_back_C1024": (Config.full(16, 4, 4, 1024, True, seq_len=67), 134, {}),
     "coef_N27_conv1": (Config.flash(27, 4, 2, 64, 2, conv_k=(4,), seq_len=131), 262, {}),
 }
 
