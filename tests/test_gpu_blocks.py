@@ -23,13 +23,17 @@ CASES = {
     # Sinkhorn iterates that fit only the small block, and none at all
     "coef_k8_iters64": (Config.full(8, 8, 8, 8, True, sinkhorn_iters=64, seq_len=4900), 4900, {}),
     "coef_k3_iters0": (Config.full(5, 3, 1, 32, True, sinkhorn_iters=0), 130, {}),
-    # two conv components (a Gram-Schmidt basis smaller than its maximum), N with idle lanes
     # full-state dX on few blocks: the streams of a block in parts (of 2, 3 or all streams; fixed ones in
     # the first part, none, all), ragged token tiles
     "dx_split_N16_m3": (Config.flash(16, 4, 3, 64, 2, seq_len=150), 300, {}),
     "dx_split_N12_m0": (Config.full(12, 4, 0, 128, False), 131, {}),
     "dx_split_N9": (Config.full(9, 4, 2, 128, False), 200, {}),
     "dx_split_mhc": (Config.mhc(4, 128), 129, {}),
+    # three and four units a CTA, those of the fixed streams alone (no d_input rows) before, between and after
+    # the others; fixed streams only; a unit with one d_input tile
+    "dx_split_N9_m3_units": (Config.full(9, 3, 3, 768, False), 1659, {}),
+    "dx_units_mhc": (Config.mhc(4, 768), 1659, {}),
+    "dx_split_N9_m2_units": (Config.full(9, 2, 2, 768, False), 1659, {}),
     # input gradients on widths that their channel tiles do not divide: last tiles of 8, 40, 72, 8 and 72 channels,
     # one or two stages of weight rows, eight active streams, no conv
     "dx_width_C72_N20": (Config.flash(20, 4, 4, 72, 4, seq_len=100), 200, {}),
@@ -39,6 +43,7 @@ CASES = {
     "dx_width_C584_N16": (Config.flash(16, 4, 2, 584, 4, seq_len=257), 257, {}),
     # entry rows put back by the two-pair reductions (512-channel slices): a run that ends inside a block of 4
     "put_back_C1024": (Config.full(16, 4, 4, 1024, True, seq_len=67), 134, {}),
+    # two components (a Gram-Schmidt basis smaller than its maximum), N with idle lanes
     "coef_N27_conv1": (Config.flash(27, 4, 2, 64, 2, conv_k=(4,), seq_len=131), 262, {}),
 }
 
