@@ -26,6 +26,44 @@ void PdlScope::set(size_t state_bytes, cudaStream_t st) {
 }
 PdlScope::~PdlScope() { t_pdl = false; }
 
+// ---- shared memory of the kernels -----------------------------------------------------------
+// the limits raised so far, per kernel and device; past the table's end the driver is asked
+static std::mutex g_smem_mu;
+static struct {
+    const void* fn;
+    int dev, bytes;
+} g_smem[1024];
+static int g_nsmem = 0;
+cudaError_t smem_optin(const void* fn, size_t bytes) {
+    if (bytes <= 40 * 1024) return cudaSuccess;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lk(g_smem_mu);
+    int q = 0;
+    while (q < g_nsmem && (g_smem[q].fn != fn || g_smem[q].dev != dev)) ++q;
+    int have = 0;
+    if (q < g_nsmem) {
+        have = g_smem[q].bytes;
+    } else {
+        cudaFuncAttributes at;
+        if ((e = cudaFuncGetAttributes(&at, fn)) != cudaSuccess) return e;
+        have = at.maxDynamicSharedSizeBytes;
+    }
+    if (have < (int)bytes) {
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e != cudaSuccess) return e;
+        have = (int)bytes;
+    }
+    if (q < 1024) {
+        g_smem[q].fn = fn;
+        g_smem[q].dev = dev;
+        g_smem[q].bytes = have;
+        if (q == g_nsmem) ++g_nsmem;
+    }
+    return cudaSuccess;
+}
+
 // ---- test hooks -----------------------------------------------------------------------------
 static std::atomic<unsigned long long> g_wait_ns{0};   // 0: the default limit (~4 s)
 static std::atomic<int> g_force_timeout{0};

@@ -446,11 +446,8 @@ cudaError_t launch_full_dots(const Dims& d, int T, const uint16_t* X, const uint
     const int nw = (d.N - d.k + NS - 1) / NS;   // warps per token
     if (nw <= 0) return cudaSuccess;
     const size_t sm = (size_t)d.G * d.C * 2;
-    if (sm > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute((const void*)k_full_dots<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)sm);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = smem_optin((const void*)k_full_dots<NS>, sm);
+    if (e != cudaSuccess) return e;
     XHC_LAUNCH(st, T, 32 * nw, sm, (k_full_dots<NS>), d, T, X, dinput, I, dhpre);
     return cudaGetLastError();
 }

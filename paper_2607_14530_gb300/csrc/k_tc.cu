@@ -687,7 +687,7 @@ cudaError_t launch_proj_tc(const uint16_t* X, int T, int K, const uint16_t* Wpac
     if (!make_map(&mb, Wpack, (uint64_t)K, (uint64_t)p.NB, (uint32_t)(p.NB / p.nchunk)))
         return cudaErrorInvalidValue;
     const size_t sm = proj_tc_smem(p);
-    cudaError_t e = cudaFuncSetAttribute((const void*)k_proj_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = smem_optin((const void*)k_proj_tc<false>, sm);
     if (e != cudaSuccess) return e;
     ProjTcArgs a;
     a.T = T;
@@ -723,7 +723,7 @@ cudaError_t launch_wgrad_tc(const uint16_t* A, int T, int E, int n, const uint16
                       (uint64_t)Tp * 2))
         return cudaErrorInvalidValue;
     const size_t sm = proj_tc_smem(p);
-    e = cudaFuncSetAttribute((const void*)k_proj_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    e = smem_optin((const void*)k_proj_tc<true>, sm);
     if (e != cudaSuccess) return e;
     ProjTcArgs a;
     a.T = E;  // rows of the output
@@ -1463,7 +1463,7 @@ cudaError_t launch_dxa_tc(const Dims& d, int slot, int T, int nact,
     // left over is L1 for the epilogue's in-flight reads
     const size_t sm = (size_t)a.nkb * (BM + DX_BN) * BK * 2 + 128 + (size_t)DX_EW * (MAXK + 1) * 32 * 4 + 1024;
     auto* const kern = d.C % DX_BN == 0 ? &k_dx_tc<false> : &k_dx_tc<true>;
-    e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    e = smem_optin((const void*)kern, sm);
     if (e != cudaSuccess) return e;
     XHC_LAUNCH(st, a.P, DX_THREADS, sm, (kern), ma, mb, a);
     return cudaGetLastError();
@@ -1571,7 +1571,7 @@ cudaError_t launch_dx_tc(const Dims& d, int T, const uint16_t* dz16,
     a.wait_ns = debug_wait_ns();
     const size_t sm = dxf_smem(n, d.G, a.nbs);
     auto* const kern = d.C % DG_BN == 0 ? &k_dxf_tc<false> : &k_dxf_tc<true>;
-    e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    e = smem_optin((const void*)kern, sm);
     if (e != cudaSuccess) return e;
     XHC_LAUNCH(st, a.P, DX_THREADS, sm, (kern), ma, mb, mx, md, mg, a);
     return cudaGetLastError();

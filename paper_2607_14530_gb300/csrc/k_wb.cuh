@@ -1511,11 +1511,6 @@ inline int bapp_run(const Dims& d, int64_t T) {
     return pick_run(d, T, true, wb_nslice(d.C), 2, kw_of(d) + 5, 296);
 }
 
-inline cudaError_t smem_attr(const void* fn, size_t bytes) {
-    if (bytes <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 // KWC: conv taps held per component (0: no conv); KSC: the kernel variant (see ntap)
 #define XHC_KW_DISPATCH(D, FAST, CALL)                                        \
     switch (kw_of(D)) {                                                       \

@@ -11,7 +11,7 @@ cudaError_t bapp_kw(const Dims& d, int slot, int T, const uint16_t* out, ConvPtr
     const int TB = bapp_run(d, T);
     const int TH = TB + (KW > 0 ? KW - 1 : 0);
     const size_t sm = sizeof(ARing<KM>) + (size_t)TH * (KM * 4 + 16 + KM * KM + KM) * 4;
-    cudaError_t e = smem_attr((const void*)k_wb_bapp<KM, KW, KS, HALO>, sm);
+    cudaError_t e = smem_optin((const void*)k_wb_bapp<KM, KW, KS, HALO>, sm);
     if (e != cudaSuccess) return e;
     dim3 grid(nslice, (unsigned)n_runs(d, T, TB, KW > 0));
     XHC_LAUNCH(st, grid, WT, sm, (k_wb_bapp<KM, KW, KS, HALO>), d, slot, T, TB, out, cw, dX, I, dn_in, tokmat, dxact_out, d_out, cpart);

@@ -13,7 +13,7 @@ cudaError_t bred_kw(const Dims& d, int slot, int T, const uint16_t* out, ConvPtr
     int TB = pick_run(d, T, true, nslice, KM == 4 ? 3 : 2, 12, 64);
     while (TB > 4 && (size_t)TB * (WT / 32) * NVP * 4 > 96 * 1024) TB -= 4;
     const size_t sm = sizeof(BRing<KM>) + (size_t)TB * KM * 4 + (size_t)TB * (WT / 32) * NVP * sizeof(float);
-    cudaError_t e = smem_attr((const void*)k_wb_bred<KM, KW, NV, KS, PUT>, sm);
+    cudaError_t e = smem_optin((const void*)k_wb_bred<KM, KW, NV, KS, PUT>, sm);
     if (e != cudaSuccess) return e;
     dim3 grid(nslice, (unsigned)n_runs(d, T, TB, KW > 0));
     XHC_LAUNCH(st, grid, WT, sm, (k_wb_bred<KM, KW, NV, KS, PUT>), d, slot, T, TB, out, cw, dX, I, dxact, xact, nslice, red, Xr);
@@ -27,7 +27,7 @@ cudaError_t bred2_kw(const Dims& d, int slot, int T, const uint16_t* out, ConvPt
     constexpr int NVP = NV < 32 ? 16 : NV;
     const int TB = pick_run(d, T, true, d.C / WSL2, 2, 12, 64);
     const size_t sm = sizeof(BRing2<KM>) + (size_t)TB * KM * 4 + (size_t)TB * (WT / 32) * NVP * sizeof(float);
-    cudaError_t e = smem_attr((const void*)k_wb_bred2<KM, NV, PUT>, sm);
+    cudaError_t e = smem_optin((const void*)k_wb_bred2<KM, NV, PUT>, sm);
     if (e != cudaSuccess) return e;
     dim3 grid(d.C / WSL2, (unsigned)n_runs(d, T, TB, true));
     XHC_LAUNCH(st, grid, WT, sm, (k_wb_bred2<KM, NV, PUT>), d, slot, T, TB, out, cw, dX, I, dxact, xact, nslice, red, Xr);
@@ -46,7 +46,7 @@ cudaError_t b8_kw(const Dims& d, int slot, int T, const uint16_t* out, const uin
     constexpr int NV = NQ <= 32 ? 32 : 96;
     const int TB = pick_run(d, T, false, (d.C + W8 - 1) / W8, KM == 4 ? 3 : 2, 4, 32);
     const size_t sm = (size_t)TB * (2 * KM + KM * KM) * 4 + (size_t)TB * (WT / 32) * NV * 4;
-    cudaError_t e = smem_attr((const void*)k_wb_b8<KM, PUT>, sm);
+    cudaError_t e = smem_optin((const void*)k_wb_b8<KM, PUT>, sm);
     if (e != cudaSuccess) return e;
     dim3 grid((d.C + W8 - 1) / W8, (T + TB - 1) / TB);
     XHC_LAUNCH(st, grid, WT, sm, (k_wb_b8<KM, PUT>), d, slot, T, TB, out, dX, I, p, hpost, hres, dxact, dxact_out, xact, nslice, red, d_out, Xr);

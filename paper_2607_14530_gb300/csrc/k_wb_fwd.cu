@@ -72,7 +72,7 @@ cudaError_t gram_kw(const Dims& d, int slot, int T, const uint16_t* out, ConvPtr
                     float* red, cudaStream_t st) {
     const int TB = pick_run(d, T, true, nslice, 4, 12, 64);
     const size_t sm = (size_t)TB * (WT / 32) * 16 * sizeof(float);
-    cudaError_t e = smem_attr((const void*)k_wb_gram<KW, KS>, sm);
+    cudaError_t e = smem_optin((const void*)k_wb_gram<KW, KS>, sm);
     if (e != cudaSuccess) return e;
     dim3 grid(nslice, (unsigned)n_runs(d, T, TB, true));
     XHC_LAUNCH(st, grid, WT, sm, (k_wb_gram<KW, KS>), d, slot, T, TB, out, cw, nslice, red);
@@ -86,7 +86,7 @@ cudaError_t fwd_kw(const Dims& d, int slot, int T, const uint16_t* out, ConvPtrs
     // 128 measured faster than 96 with the block ring
     const int TB = pick_run(d, T, true, nslice, KM == 4 ? 4 : 3, 12, 128);
     const size_t sm = sizeof(FRing<KM>) + (size_t)TB * (KM * 4 + KM * KM + KM) * 4;
-    cudaError_t e = smem_attr((const void*)k_wb_fwd<KM, KW, KS>, sm);
+    cudaError_t e = smem_optin((const void*)k_wb_fwd<KM, KW, KS>, sm);
     if (e != cudaSuccess) return e;
     dim3 grid(nslice, (unsigned)n_runs(d, T, TB, KW > 0));
     XHC_LAUNCH(st, grid, WT, sm, (k_wb_fwd<KM, KW, KS>), d, slot, T, TB, out, cw, emat, xact, I, hres, xact_next, X);

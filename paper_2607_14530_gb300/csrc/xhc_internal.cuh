@@ -365,11 +365,10 @@ inline cudaError_t launch_pdl(cudaStream_t st, dim3 grid, dim3 block, size_t sme
     note_launch();
     return e;
 }
-// more dynamic shared memory than a launch has without asking (48 KB with the static part)
-inline cudaError_t smem_optin(const void* fn, size_t bytes) {
-    if (bytes <= 40 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
+// More dynamic shared memory than a launch has without asking (48 KB with the static part).  The limit of
+// a kernel is only ever raised: a call's size depends on its tokens and widths, and a smaller one set from another
+// host thread, between this call and its launch, would make the launch fail.
+cudaError_t smem_optin(const void* fn, size_t bytes);
 // launch of kernel `k` (in parentheses), counted; returns from the launcher on failure
 #define XHC_LAUNCH(st, grid, block, smem, k, ...)                                        \
     do {                                                                                  \
