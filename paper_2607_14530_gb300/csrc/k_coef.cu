@@ -51,7 +51,7 @@ __device__ __forceinline__ int slot_count(const SlotPlan& s, int m) {
 // sum over `cnt` slots of p, `stride` apart, starting at slot q0 in steps of dq, added in slot order with
 // U loads in flight
 template <int U>
-__device__ __forceinline__ float slot_sum(const float* __restrict__ p, long long stride, int cnt, int q0, int dq) {
+__device__ __forceinline__ float slot_sum(const float* p, long long stride, int cnt, int q0, int dq) {
     float s = 0.f;
     int q = q0;
     for (; q + (U - 1) * dq < cnt; q += U * dq) {
@@ -74,8 +74,8 @@ __device__ __forceinline__ float slot_sum(const float* __restrict__ p, long long
 // the whole block loads them: 82 sums over 172 slots took 27 us with a thread each.  Ends with a
 // block barrier.
 constexpr int SS_STAGE = 4096;
-__device__ __forceinline__ void slot_sums(bool ordered, const float* __restrict__ p0, long long stride0, int cnt0,
-                                          int n0, const float* __restrict__ p1, long long stride1, int cnt1, int n1,
+__device__ __forceinline__ void slot_sums(bool ordered, const float* p0, long long stride0, int cnt0,
+                                          int n0, const float* p1, long long stride1, int cnt1, int n1,
                                           int step1, float* dst, float* scr, float* stage) {
     const int n = n0 + n1, nt = blockDim.x, tid = threadIdx.x;
     const int ng = ordered ? 1 : nt / n;
@@ -186,11 +186,11 @@ __device__ __forceinline__ float row_total(const float (&A)[KM]) {
 
 constexpr int CF_NT = 512;
 
-__global__ void __launch_bounds__(CF_NT) k_coef_full(Dims d, int T, int TB, const float* __restrict__ part,
-                                                     const float* __restrict__ pstats, SlotPlan sp,
-                                                     const float* __restrict__ wsum, int nws,
-                                                     const float* __restrict__ alpha_pre,
-                                                     const float* __restrict__ b_pre, float* __restrict__ zfull,
+__global__ void __launch_bounds__(CF_NT) k_coef_full(Dims d, int T, int TB, const float* part,
+                                                     const float* pstats, SlotPlan sp,
+                                                     const float* wsum, int nws,
+                                                     const float* alpha_pre,
+                                                     const float* b_pre, float* __restrict__ zfull,
                                                      float* __restrict__ stats, float* __restrict__ wsum_out,
                                                      float* __restrict__ hpre, int* __restrict__ I,
                                                      float* __restrict__ p) {
@@ -283,12 +283,12 @@ __global__ void __launch_bounds__(CF_NT) k_coef_full(Dims d, int T, int TB, cons
 // coef_act
 
 template <int KM>
-__global__ void __launch_bounds__(CF_NT) k_coef_act(Dims d, int slot, int T, int TB, const float* __restrict__ part,
-                                                    const float* __restrict__ pstats, int ssplits, SlotPlan sp,
-                                                    const float* __restrict__ alpha_post,
-                                                    const float* __restrict__ b_post,
-                                                    const float* __restrict__ alpha_res,
-                                                    const float* __restrict__ b_res, float* __restrict__ zact,
+__global__ void __launch_bounds__(CF_NT) k_coef_act(Dims d, int slot, int T, int TB, const float* part,
+                                                    const float* pstats, int ssplits, SlotPlan sp,
+                                                    const float* alpha_post,
+                                                    const float* b_post,
+                                                    const float* alpha_res,
+                                                    const float* b_res, float* __restrict__ zact,
                                                     float* __restrict__ rs, float* __restrict__ hpost,
                                                     float* __restrict__ hres) {
     pdl_entry();
@@ -457,14 +457,14 @@ struct BwdTok {
 };
 
 template <int KM>
-__global__ void __launch_bounds__(160) k_bwd_coef(Dims d, int slot, int T, int TB, const float* __restrict__ red,
-                                                  int nslice, const float* __restrict__ zact,
-                                                  const float* __restrict__ rs, const float* __restrict__ p,
-                                                  const float* __restrict__ hpost, const double* __restrict__ gram,
-                                                  const float* __restrict__ alpha_post,
-                                                  const float* __restrict__ alpha_res,
-                                                  const float* __restrict__ b_res, float* __restrict__ tokmat,
-                                                  float* __restrict__ dzs, float* __restrict__ dp,
+__global__ void __launch_bounds__(160) k_bwd_coef(Dims d, int slot, int T, int TB, const float* red,
+                                                  int nslice, const float* zact,
+                                                  const float* rs, const float* p,
+                                                  const float* hpost, const double* gram,
+                                                  const float* alpha_post,
+                                                  const float* alpha_res,
+                                                  const float* b_res, float* __restrict__ tokmat,
+                                                  float* __restrict__ dzs, float* dp,
                                                   float* __restrict__ colp, DzPack pack, WRows wrows, int nblk) {
     pdl_entry();
     if ((int)blockIdx.x >= nblk) {
@@ -708,13 +708,13 @@ namespace {
 constexpr int FC_NT = 256;
 constexpr int FC_R = 4;   // pre-map columns per lane: G N <= 128
 
-__global__ void __launch_bounds__(FC_NT) k_full_coef(Dims d, int T, int TB, const float* __restrict__ dhpre,
-                                                     const float* __restrict__ hpre,
-                                                     const float* __restrict__ zfull,
-                                                     const float* __restrict__ stats,
-                                                     const float* __restrict__ wsum, const int* __restrict__ I,
-                                                     const float* __restrict__ dp,
-                                                     const float* __restrict__ alpha_pre, float* __restrict__ dz,
+__global__ void __launch_bounds__(FC_NT) k_full_coef(Dims d, int T, int TB, const float* dhpre,
+                                                     const float* hpre,
+                                                     const float* zfull,
+                                                     const float* stats,
+                                                     const float* wsum, const int* I,
+                                                     const float* dp,
+                                                     const float* alpha_pre, float* __restrict__ dz,
                                                      float* __restrict__ scal, float* __restrict__ colp,
                                                      DzPack pack, WRows wrows, int nblk) {
     pdl_entry();
@@ -864,7 +864,7 @@ cudaError_t launch_full_coef(const Dims& d, int T, const float* dhpre, const flo
 
 namespace {
 
-__global__ void __launch_bounds__(128) k_colsum_out(const float* __restrict__ colp, int nblk, int ncol, ColOut out) {
+__global__ void __launch_bounds__(128) k_colsum_out(const float* colp, int nblk, int ncol, ColOut out) {
     pdl_entry();
     __shared__ float sh[4];
     int o = blockIdx.x;
@@ -909,8 +909,8 @@ cudaError_t launch_colsum_out(const float* colp, int nblk, int ncol, const ColOu
 
 namespace {
 
-__global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ wpart, SlotPlan sp, int E, int n,
-                                                      WSegsOut G, const float* __restrict__ sub) {
+__global__ void __launch_bounds__(256) k_wgrad_reduce(const float* wpart, SlotPlan sp, int E, int n,
+                                                      WSegsOut G, const float* sub) {
     pdl_entry();
     const int e0 = blockIdx.y * 128, ne = min(128, E - e0) * n;
     const int nsl = slot_count(sp, blockIdx.y);

@@ -39,7 +39,7 @@ __device__ __forceinline__ float2 ldp(const uint16_t* p) {
 // taps of a component; PAPER: the (4, 8, 12) taps, their loops folded.  pos: the position, at most KW
 // of it; r0: its ring row.
 template <int KW, bool PAPER>
-__device__ __forceinline__ void dec_conv(const Dims& d, const ConvPtrs& cw, const uint16_t* __restrict__ rt, int c,
+__device__ __forceinline__ void dec_conv(const Dims& d, const ConvPtrs& cw, const uint16_t* rt, int c,
                                          float2 o, int pos, int r0, float2 (&g)[3]) {
     const int C = d.C, R = d.kapmax - 1;
     float2 v[KW];
@@ -98,11 +98,11 @@ __device__ __forceinline__ float wred16(float (&v)[16], int lane) {
 // CTAs of a token need no cluster)
 template <int KM, int KW, bool PAPER>
 __global__ void __launch_bounds__(512, 2) k_dec_post(Dims d, int slot, int B, int DT, int q, int ns,
-                                                  const uint16_t* __restrict__ out, ConvPtrs cw,
-                                                  uint16_t* __restrict__ ring, long long* __restrict__ pos,
-                                                  const float* __restrict__ p, const float* __restrict__ hpost,
-                                                  double* __restrict__ gram, const uint16_t* __restrict__ xact,
-                                                  const int* __restrict__ I, const float* __restrict__ hres,
+                                                  const uint16_t* out, ConvPtrs cw,
+                                                  uint16_t* ring, long long* pos,
+                                                  const float* p, const float* hpost,
+                                                  double* __restrict__ gram, const uint16_t* xact,
+                                                  const int* I, const float* hres,
                                                   uint16_t* __restrict__ xact_next, uint16_t* __restrict__ X) {
     pdl_entry();
     constexpr bool CONV = KW > 0;
@@ -322,7 +322,7 @@ cudaError_t dec_post_km(const Dims& d, int slot, int B, const uint16_t* out, Con
 
 // ring rows from a prefill: sequence b of S tokens (rows b*S .. b*S + S - 1 of out) leaves its
 // last min(S, R) rows in ring rows (s mod R)
-__global__ void k_ring_fill(const uint16_t* __restrict__ out, int B, int S, int C, int R,
+__global__ void k_ring_fill(const uint16_t* out, int B, int S, int C, int R,
                             uint16_t* __restrict__ ring) {
     pdl_entry();
     const long long n = (long long)B * R * (C / 8);
@@ -341,7 +341,7 @@ __global__ void k_ring_fill(const uint16_t* __restrict__ out, int B, int S, int 
 
 // halo rows for the next chunk of B sequences of S tokens: halo[b][r] = out of position
 // S - R + r of sequence b (zero where that position is before the sequence start)
-__global__ void k_halo_fill(const uint16_t* __restrict__ out, int B, int S, int C, int R,
+__global__ void k_halo_fill(const uint16_t* out, int B, int S, int C, int R,
                             uint16_t* __restrict__ halo) {
     pdl_entry();
     const long long n = (long long)B * R * (C / 8);
@@ -360,8 +360,8 @@ __global__ void k_halo_fill(const uint16_t* __restrict__ out, int B, int S, int 
 
 // the gradient of a chunk's halo rows, returned to the chunk that produced them: d_out of
 // position S - R + r of sequence b += d_halo[b][r] (in fp32, one bf16 rounding)
-__global__ void k_halo_add(uint16_t* __restrict__ d_out, int B, int S, int C, int R,
-                           const float* __restrict__ dhalo) {
+__global__ void k_halo_add(uint16_t* d_out, int B, int S, int C, int R,
+                           const float* dhalo) {
     pdl_entry();
     const long long n = (long long)B * R * (C / 2);
     for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < n;

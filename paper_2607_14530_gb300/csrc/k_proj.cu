@@ -17,7 +17,7 @@ namespace xhc {
 // rowproj: part[split][t][o] = sum_{e in split} A[t][e] * W[e][o];  pstats[split][t] = (sum a, sum a^2)
 
 template <int NT>
-__global__ void __launch_bounds__(256) k_rowproj(const uint16_t* __restrict__ A, int64_t lda, int K,
+__global__ void __launch_bounds__(256) k_rowproj(const uint16_t* A, int64_t lda, int K,
                                                  int T, WSegs W, int n, int kchunk,
                                                  float* __restrict__ part,
                                                  float* __restrict__ pstats) {
@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(256) k_rowproj(const uint16_t* __restrict__ A,
         float av[8];
         const int kc = k0 + lseg * 8;
         if (grow < T && kc < kend) {
-            const uint4 u = __ldg(reinterpret_cast<const uint4*>(A + (int64_t)grow * lda + kc));
+            const uint4 u = *reinterpret_cast<const uint4*>(A + (int64_t)grow * lda + kc);
             unpack8(u, av);
         } else {
 #pragma unroll
@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(256) k_rowproj(const uint16_t* __restrict__ A,
             const int kr = k0 + kk;
             float v = 0.f;
             if (o < n && kr < kend) {
-                v = seg_elem<true>(W, kr, o);
+                v = seg_elem(W, kr, o);
             }
             Ws[kk][o] = v;
         }
@@ -118,7 +118,7 @@ constexpr int RS_NT = 512;
 constexpr int RS_ROWS = 256;   // rows of the state staged at a time
 
 template <int TT, int V>
-__global__ void __launch_bounds__(RS_NT) k_rowproj_small(const uint16_t* __restrict__ A, int64_t lda, int K, int T,
+__global__ void __launch_bounds__(RS_NT) k_rowproj_small(const uint16_t* A, int64_t lda, int K, int T,
                                                          WSegs W, int n, int kchunk, float* __restrict__ part,
                                                          float* __restrict__ pstats, ColJob cj) {
     pdl_entry();
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(RS_NT) k_rowproj_small(const uint16_t* __restr
 #pragma unroll
             for (int e = 0; e < 8; ++e) x[e] = 0.f;
             if (tt < TT && t0 + tt < T && lane * 8 < rows)
-                unpack8(__ldg(reinterpret_cast<const uint4*>(A + (int64_t)(t0 + tt) * lda + kb + lane * 8)), x);
+                unpack8(*reinterpret_cast<const uint4*>(A + (int64_t)(t0 + tt) * lda + kb + lane * 8), x);
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
                 sm[(lane * 8 + e) * (2 * TP) + tt] = x[e];
@@ -186,10 +186,10 @@ __global__ void __launch_bounds__(RS_NT) k_rowproj_small(const uint16_t* __restr
                     const int r = r0 + u * nl;
                     const float* p = wp + (int64_t)(kb + r) * width;
                     if constexpr (V == 4) {
-                        const float4 f = r < rows ? __ldg(reinterpret_cast<const float4*>(p)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        const float4 f = r < rows ? *reinterpret_cast<const float4*>(p) : make_float4(0.f, 0.f, 0.f, 0.f);
                         w[u][0] = f.x; w[u][1] = f.y; w[u][2] = f.z; w[u][3] = f.w;
                     } else {
-                        w[u][0] = r < rows ? __ldg(p) : 0.f;
+                        w[u][0] = r < rows ? *p : 0.f;
                     }
                 }
 #pragma unroll
@@ -257,7 +257,7 @@ static cudaError_t rowproj_small_v(const uint16_t* A, int64_t lda, int K, int T,
 
 // colsum: partial column sums of in [rows][n] (n <= MAXN), a block per chunk of rows
 
-__global__ void __launch_bounds__(8 * MAXN) k_colsum(const float* __restrict__ in, int rows, int n, int rchunk,
+__global__ void __launch_bounds__(8 * MAXN) k_colsum(const float* in, int rows, int n, int rchunk,
                                                      float* __restrict__ out) {
     pdl_entry();
     __shared__ float sh[8 * MAXN];
@@ -303,9 +303,9 @@ cudaError_t launch_rowproj(const uint16_t* A, int64_t lda, int K, int T, const W
 // ---------------------------------------------------------------------------------------------
 // gemm_dzw: out[t][e] += sum_o dz[t][o] * W[e][o]   (t < T, e < E, o < n)
 
-__global__ void __launch_bounds__(256) k_gemm_dzw(const float* __restrict__ dz, int ldz, int n,
+__global__ void __launch_bounds__(256) k_gemm_dzw(const float* dz, int ldz, int n,
                                                   WSegs W, int E, int T,
-                                                  float* __restrict__ out) {
+                                                  float* out) {
     pdl_entry();
     constexpr int BT = 64, BE = 64, BO = 32;
     __shared__ __align__(16) float Ds[BO][BT + 4];
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(256) k_gemm_dzw(const float* __restrict__ dz, 
             const int e = e0 + ee, o = o0 + oo;
             float v = 0.f;
             if (e < E && o < n) {
-                v = seg_elem<true>(W, e, o);
+                v = seg_elem(W, e, o);
             }
             Wt[oo][ee] = v;
         }
@@ -372,14 +372,14 @@ cudaError_t launch_gemm_dzw(const Dims& d, int T, const float* dz, int ldz, int 
 // gradient sum_q H_pre[t][q][i] d_input_q[t][c] (Eq. dense_read reversed; din holds the G
 // d_input copies [G][T][C])
 
-__global__ void __launch_bounds__(256) k_full_dx(Dims d, int T, const float* __restrict__ dz,
-                                                 WSegs W, const uint16_t* __restrict__ X,
-                                                 const uint16_t* __restrict__ din,
-                                                 const float* __restrict__ hpre,
-                                                 const int* __restrict__ I,
-                                                 const float* __restrict__ dxact,
-                                                 const float* __restrict__ scal,
-                                                 uint16_t* __restrict__ dX) {
+__global__ void __launch_bounds__(256) k_full_dx(Dims d, int T, const float* dz,
+                                                 WSegs W, const uint16_t* X,
+                                                 const uint16_t* din,
+                                                 const float* hpre,
+                                                 const int* I,
+                                                 const float* dxact,
+                                                 const float* scal,
+                                                 uint16_t* dX) {
     pdl_entry();
     constexpr int BT = 64, BE = 64, BO = 32;
     __shared__ __align__(16) float Ds[BO][BT + 4];
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(256) k_full_dx(Dims d, int T, const float* __r
             const int e = e0 + ee, o = o0 + oo;
             float v = 0.f;
             if (e < E && o < n) {
-                v = seg_elem<true>(W, e, o);
+                v = seg_elem(W, e, o);
             }
             Wt[oo][ee] = v;
         }
@@ -471,8 +471,8 @@ cudaError_t launch_full_dx(const Dims& d, int T, const float* dz, const WSegs& W
 // wgrad: wpart[split][e][o] = sum_{t in split} A[t][e] dz[t][o]; then G[e][o] += sum_split
 
 template <int NT>
-__global__ void __launch_bounds__(256) k_wgrad(const uint16_t* __restrict__ A, int64_t lda, int E,
-                                               int T, const float* __restrict__ dz, int ldz, int n,
+__global__ void __launch_bounds__(256) k_wgrad(const uint16_t* A, int64_t lda, int E,
+                                               int T, const float* dz, int ldz, int n,
                                                int tchunk, float* __restrict__ wpart) {
     pdl_entry();
     constexpr int BE = 64, BT = 32, NP = 16 * NT;
@@ -493,7 +493,7 @@ __global__ void __launch_bounds__(256) k_wgrad(const uint16_t* __restrict__ A, i
             const int t = tk + lt, e = e0 + lseg * 8;
             float av[8];
             if (t < tend && e < E) {
-                const uint4 u = __ldg(reinterpret_cast<const uint4*>(A + (int64_t)t * lda + e));
+                const uint4 u = *reinterpret_cast<const uint4*>(A + (int64_t)t * lda + e);
                 unpack8(u, av);
             } else {
 #pragma unroll

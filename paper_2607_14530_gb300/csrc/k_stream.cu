@@ -35,9 +35,9 @@ int stream_warps(int C) { return chunk_threads(C) / 32; }
 // ---------------------------------------------------------------------------------------------
 // read: one block per token, threads over 8-channel chunks.
 
-__global__ void __launch_bounds__(256, 3) k_read(Dims d, int T, const uint16_t* __restrict__ X,
-                                              const float* __restrict__ hpre,
-                                              const int* __restrict__ I,
+__global__ void __launch_bounds__(256, 3) k_read(Dims d, int T, const uint16_t* X,
+                                              const float* hpre,
+                                              const int* I,
                                               uint16_t* __restrict__ input0,
                                               uint16_t* __restrict__ base,
                                               uint16_t* __restrict__ xact0,
@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(256, 3) k_read(Dims d, int T, const uint16_t* 
     if (threadIdx.x < C / 8) {
 #pragma unroll
         for (int ii = 0; ii < 8; ++ii)
-            if (ii < N) ub[ii] = __ldg(reinterpret_cast<const uint4*>(xt + (int64_t)ii * C + threadIdx.x * 8));
+            if (ii < N) ub[ii] = *reinterpret_cast<const uint4*>(xt + (int64_t)ii * C + threadIdx.x * 8);
     }
     for (int q = threadIdx.x; q < G * N; q += blockDim.x) sh[q] = hpre[(int64_t)t * G * N + q];
     for (int i = threadIdx.x; i < N; i += blockDim.x) {
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(256, 3) k_read(Dims d, int T, const uint16_t* 
             if (i0 != 0 || c8 != (int)threadIdx.x) {
 #pragma unroll
                 for (int ii = 0; ii < 8; ++ii)
-                    if (i0 + ii < N) ub[ii] = __ldg(reinterpret_cast<const uint4*>(xt + (int64_t)(i0 + ii) * C + c8 * 8));
+                    if (i0 + ii < N) ub[ii] = *reinterpret_cast<const uint4*>(xt + (int64_t)(i0 + ii) * C + c8 * 8);
             }
 #pragma unroll
             for (int ii = 0; ii < 8; ++ii) {
@@ -126,10 +126,10 @@ cudaError_t launch_read(const Dims& d, int T, const uint16_t* X, const float* hp
 
 template <int KM>
 __global__ void __launch_bounds__(256) k_input(Dims d, int slot, int T,
-                                               const uint16_t* __restrict__ base,
-                                               const uint16_t* __restrict__ xact,
-                                               const float* __restrict__ hpre,
-                                               const int* __restrict__ I,
+                                               const uint16_t* base,
+                                               const uint16_t* xact,
+                                               const float* hpre,
+                                               const int* I,
                                                uint16_t* __restrict__ input,
                                                float* __restrict__ astat, PackJob pack, int npack) {
     pdl_entry();
@@ -191,8 +191,8 @@ cudaError_t launch_input(const Dims& d, int slot, int T, const uint16_t* base, c
 // ---------------------------------------------------------------------------------------------
 // restore: X[t][I_j] = X_act^(0)[t][j]
 
-__global__ void __launch_bounds__(256) k_restore(Dims d, int T, const uint16_t* __restrict__ xact0,
-                                                 const int* __restrict__ I,
+__global__ void __launch_bounds__(256) k_restore(Dims d, int T, const uint16_t* xact0,
+                                                 const int* I,
                                                  uint16_t* __restrict__ X) {
     pdl_entry();
     const int t = blockIdx.x, C = d.C;
@@ -219,7 +219,7 @@ cudaError_t launch_restore(const Dims& d, int T, const uint16_t* xact0, const in
 // runs, 16 us with a thread per sum).
 constexpr int CW_G = 4;
 
-__global__ void __launch_bounds__(64 * CW_G) k_conv_wgrad_reduce(Dims d, const float* __restrict__ cpart, int ntiles,
+__global__ void __launch_bounds__(64 * CW_G) k_conv_wgrad_reduce(Dims d, const float* cpart, int ntiles,
                                                                  ConvGradPtrs g) {
     pdl_entry();
     __shared__ float sh[CW_G][64];
@@ -266,14 +266,14 @@ cudaError_t launch_conv_wgrad_reduce(const Dims& d, int slot, const float* cpart
 
 template <int KM>
 __global__ void __launch_bounds__(256) k_dinput_act(Dims d, int slot, int T, int add_dx,
-                                                    const uint16_t* __restrict__ din,
-                                                    const uint16_t* __restrict__ xact,
-                                                    const float* __restrict__ hpre,
-                                                    const int* __restrict__ I,
-                                                    float* __restrict__ dxact,
+                                                    const uint16_t* din,
+                                                    const uint16_t* xact,
+                                                    const float* hpre,
+                                                    const int* I,
+                                                    float* dxact,
                                                     float* __restrict__ dhpre,
                                                     uint16_t* __restrict__ dcopy,
-                                                    const float* __restrict__ tokmat) {
+                                                    const float* tokmat) {
     pdl_entry();
     __shared__ float hj[KM];
     __shared__ float wsh[8][KM];
@@ -347,9 +347,9 @@ cudaError_t launch_dinput_act(const Dims& d, int slot, int T, int add_dx, const 
 // each chunk read back from shared memory serves the warp's two X rows.
 
 template <int NS>
-__global__ void __launch_bounds__(512) k_full_dots(Dims d, int T, const uint16_t* __restrict__ X,
-                                                   const uint16_t* __restrict__ dinput,
-                                                   const int* __restrict__ I,
+__global__ void __launch_bounds__(512) k_full_dots(Dims d, int T, const uint16_t* X,
+                                                   const uint16_t* dinput,
+                                                   const int* I,
                                                    float* __restrict__ dhpre) {
     pdl_entry();
     extern __shared__ __align__(16) uint16_t din[];   // [G][C]
@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(512) k_full_dots(Dims d, int T, const uint16_t
         for (int u = 0; u < 4; ++u) {
             const int c8 = lane + 32 * u;
             xr[h][u] = make_uint4(0u, 0u, 0u, 0u);
-            if (is[h] >= 0 && c8 < C / 8) xr[h][u] = __ldg(reinterpret_cast<const uint4*>(X + row[h] + c8 * 8));
+            if (is[h] >= 0 && c8 < C / 8) xr[h][u] = *reinterpret_cast<const uint4*>(X + row[h] + c8 * 8);
         }
     for (int idx = threadIdx.x; idx < G * C / 8; idx += blockDim.x) {
         const int q = idx / (C / 8), c8 = idx - q * (C / 8);
@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(512) k_full_dots(Dims d, int T, const uint16_t
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const int c8 = c0 + 32 * u;
-                    if (is[h] >= 0 && c8 < C / 8) xr[h][u] = __ldg(reinterpret_cast<const uint4*>(X + row[h] + c8 * 8));
+                    if (is[h] >= 0 && c8 < C / 8) xr[h][u] = *reinterpret_cast<const uint4*>(X + row[h] + c8 * 8);
                 }
         }
 #pragma unroll
@@ -456,7 +456,7 @@ cudaError_t launch_full_dots(const Dims& d, int T, const uint16_t* X, const uint
 // model glue: stream expansion and the final stream sum, one CTA per token, 16-byte accesses
 
 // X[t][i] = h[t] for every stream i (N copies; also the backward of the stream sum)
-__global__ void __launch_bounds__(256) k_stream_bcast(int T, int N, int C, const uint16_t* __restrict__ h,
+__global__ void __launch_bounds__(256) k_stream_bcast(int T, int N, int C, const uint16_t* h,
                                                       uint16_t* __restrict__ X) {
     pdl_entry();
     const long long t = blockIdx.x;
@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(256) k_stream_bcast(int T, int N, int C, const
 }
 
 // y[t] = sum_i X[t][i] in fp32, stored bf16 (also the backward of the expansion)
-__global__ void __launch_bounds__(256) k_stream_sum(int T, int N, int C, const uint16_t* __restrict__ X,
+__global__ void __launch_bounds__(256) k_stream_sum(int T, int N, int C, const uint16_t* X,
                                                     uint16_t* __restrict__ y) {
     pdl_entry();
     const long long t = blockIdx.x;

@@ -502,7 +502,7 @@ k_proj_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
 constexpr int PF_E = 64;
 constexpr int PF_NT = 256;
 
-__global__ void __launch_bounds__(PF_NT) k_pack_full(PackJob j, int nblk, const float* __restrict__ Wr, int N,
+__global__ void __launch_bounds__(PF_NT) k_pack_full(PackJob j, int nblk, const float* Wr, int N,
                                                      int rchunk, int nparts, float* __restrict__ wsump, PackJob act) {
     pdl_entry();
     extern __shared__ float sm[];   // [n][PF_E + 1]
@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(PF_NT) k_pack_full(PackJob j, int nblk, const 
             float4 v[MAXSEG];   // the segments' loads in flight together
 #pragma unroll
             for (int q = 0; q < MAXSEG; ++q)
-                if (q < j.W.n) v[q] = __ldg(reinterpret_cast<const float4*>(j.W.ptr[q] + at) + i4);
+                if (q < j.W.n) v[q] = reinterpret_cast<const float4*>(j.W.ptr[q] + at)[i4];
             const int e = (int)((uint32_t)(4 * i4) * rec >> 16), o = 4 * i4 - e * N;
 #pragma unroll
             for (int q = 0; q < MAXSEG; ++q) {
@@ -547,7 +547,7 @@ __global__ void __launch_bounds__(PF_NT) k_pack_full(PackJob j, int nblk, const 
             const int e = (int)((uint32_t)idx * rec >> 16), o = idx - e * N;
 #pragma unroll
             for (int q = 0; q < MAXSEG; ++q)
-                if (q < j.W.n) sm[(q * N + o) * (PF_E + 1) + e] = __ldg(j.W.ptr[q] + at + idx);
+                if (q < j.W.n) sm[(q * N + o) * (PF_E + 1) + e] = j.W.ptr[q][at + idx];
         }
     }
     __syncthreads();
@@ -1473,8 +1473,8 @@ namespace {
 // dH_pre[t][slot][I_j] from the dot partials of k_dx_tc: a block per (32 tokens, j); warp w
 // sums the groups g = w, w + 8, ... of its lane's token (coalesced 128-byte rows), and the eight
 // warp sums are added in warp order (a fixed order: the result does not depend on the schedule)
-__global__ void __launch_bounds__(256) k_dots_act(const float* __restrict__ dotp, int T, int k, int ncg,
-                                                  int G, int N, int slot, const int* __restrict__ I,
+__global__ void __launch_bounds__(256) k_dots_act(const float* dotp, int T, int k, int ncg,
+                                                  int G, int N, int slot, const int* I,
                                                   float* __restrict__ dhpre) {
     pdl_entry();
     __shared__ float part[8][32];

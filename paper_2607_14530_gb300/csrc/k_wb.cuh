@@ -248,7 +248,7 @@ __device__ __forceinline__ void wred32(float (&v)[NB * 32], int lane, float (&to
 
 template <int KW, int KS>
 __global__ void __launch_bounds__(WT) k_wb_gram(Dims d, int slot, int T, int TB,
-                                                const uint16_t* __restrict__ out, ConvPtrs cw,
+                                                const uint16_t* out, ConvPtrs cw,
                                                 int nslice, float* __restrict__ red) {
     pdl_entry();
     extern __shared__ float wsh[];  // [TB][WT/32][16]
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(WT) k_wb_gram(Dims d, int slot, int T, int TB,
 constexpr int WSL2 = 4 * WT;
 
 __global__ void __launch_bounds__(WT, 2) k_wb_gram2(Dims d, int slot, int T, int TB,
-                                                    const uint16_t* __restrict__ out, ConvPtrs cw,
+                                                    const uint16_t* out, ConvPtrs cw,
                                                     int nslice, float* __restrict__ red) {
     pdl_entry();
     constexpr int KW = 12, KS = 2;
@@ -416,11 +416,11 @@ struct FRing {   // two blocks of UB tokens
 
 template <int KM, int KW, int KS>
 __global__ void __launch_bounds__(WT) k_wb_fwd(Dims d, int slot, int T, int TB,
-                                               const uint16_t* __restrict__ out, ConvPtrs cw,
-                                               const float* __restrict__ emat,
-                                               const uint16_t* __restrict__ xact,
-                                               const int* __restrict__ I,
-                                               const float* __restrict__ hres,
+                                               const uint16_t* out, ConvPtrs cw,
+                                               const float* emat,
+                                               const uint16_t* xact,
+                                               const int* I,
+                                               const float* hres,
                                                uint16_t* __restrict__ xact_next,
                                                uint16_t* __restrict__ X) {
     pdl_entry();
@@ -570,11 +570,11 @@ struct BRing {
 // lane pairs, larger NV in blocks of 32.  PUT (last slot): the x_j rows also go back into Xr.
 template <int KM, int KW, int NV, int KS, bool PUT>
 __global__ void __launch_bounds__(WT) k_wb_bred(Dims d, int slot, int T, int TB,
-                                                const uint16_t* __restrict__ out, ConvPtrs cw,
-                                                const uint16_t* __restrict__ dX,
-                                                const int* __restrict__ I,
-                                                const float* __restrict__ dxact,
-                                                const uint16_t* __restrict__ xact, int nslice,
+                                                const uint16_t* out, ConvPtrs cw,
+                                                const uint16_t* dX,
+                                                const int* I,
+                                                const float* dxact,
+                                                const uint16_t* xact, int nslice,
                                                 float* __restrict__ red, uint16_t* __restrict__ Xr) {
     pdl_entry();
     static_assert(NV == 16 || NV % 32 == 0, "reduction width");
@@ -741,11 +741,11 @@ struct BRing2 {   // two blocks of UB tokens
 
 template <int KM, int NV, bool PUT>
 __global__ void __launch_bounds__(WT, 2) k_wb_bred2(Dims d, int slot, int T, int TB,
-                                                    const uint16_t* __restrict__ out, ConvPtrs cw,
-                                                    const uint16_t* __restrict__ dX,
-                                                    const int* __restrict__ I,
-                                                    const float* __restrict__ dxact,
-                                                    const uint16_t* __restrict__ xact, int nslice,
+                                                    const uint16_t* out, ConvPtrs cw,
+                                                    const uint16_t* dX,
+                                                    const int* I,
+                                                    const float* dxact,
+                                                    const uint16_t* xact, int nslice,
                                                     float* __restrict__ red, uint16_t* __restrict__ Xr) {
     pdl_entry();
     constexpr int KW = 12, KS = 2;
@@ -919,11 +919,11 @@ struct ARing {   // two blocks of UB tokens
 // common variants carry none of its registers
 template <int KM, int KW, int KS, bool HALO = false>
 __global__ void __launch_bounds__(WT, 2) k_wb_bapp(Dims d, int slot, int T, int TB,
-                                                   const uint16_t* __restrict__ out, ConvPtrs cw,
-                                                   const uint16_t* __restrict__ dX,
-                                                   const int* __restrict__ I,
+                                                   const uint16_t* out, ConvPtrs cw,
+                                                   const uint16_t* dX,
+                                                   const int* I,
                                                    const float* dn_in,  // may alias dxact_out
-                                                   const float* __restrict__ tokmat,
+                                                   const float* tokmat,
                                                    float* dxact_out,
                                                    uint16_t* __restrict__ d_out,
                                                    float* __restrict__ cpart) {
@@ -1181,7 +1181,7 @@ __global__ void __launch_bounds__(WT, 2) k_wb_bapp(Dims d, int slot, int T, int 
 
 constexpr int W8 = WT * 8;   // channels per CTA
 
-__device__ __forceinline__ uint4 ld16(const void* p) { return __ldg(reinterpret_cast<const uint4*>(p)); }
+__device__ __forceinline__ uint4 ld16(const void* p) { return *reinterpret_cast<const uint4*>(p); }
 __device__ __forceinline__ void l2_prefetch(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 constexpr int B8_PF = 2;   // L2 prefetch distance of the one-pass attention backward, in tokens
 
@@ -1207,12 +1207,12 @@ __device__ __forceinline__ void k1_tables(int ntok, long long t0, int k, bool la
 // forward: X_act_new_j = (sum_i H_res[j][i] x_i  |  x_j) + E[j][0] out
 template <int KM>
 __global__ void __launch_bounds__(WT) k_wb_fwd8(Dims d, int slot, int T, int TB,
-                                                const uint16_t* __restrict__ out,
-                                                const float* __restrict__ p,
-                                                const float* __restrict__ hpost,
-                                                const uint16_t* __restrict__ xact,
-                                                const int* __restrict__ I,
-                                                const float* __restrict__ hres,
+                                                const uint16_t* out,
+                                                const float* p,
+                                                const float* hpost,
+                                                const uint16_t* xact,
+                                                const int* I,
+                                                const float* hres,
                                                 uint16_t* __restrict__ xact_next,
                                                 uint16_t* __restrict__ X) {
     pdl_entry();
@@ -1284,15 +1284,15 @@ __global__ void __launch_bounds__(WT) k_wb_fwd8(Dims d, int slot, int T, int TB,
 // PUT: the x_j rows also go back into Xr.
 template <int KM, bool PUT>
 __global__ void __launch_bounds__(WT, 3) k_wb_b8(Dims d, int slot, int T, int TB,
-                                              const uint16_t* __restrict__ out,
-                                              const uint16_t* __restrict__ dX,
-                                              const int* __restrict__ I,
-                                              const float* __restrict__ p,
-                                              const float* __restrict__ hpost,
-                                              const float* __restrict__ hres,
+                                              const uint16_t* out,
+                                              const uint16_t* dX,
+                                              const int* I,
+                                              const float* p,
+                                              const float* hpost,
+                                              const float* hres,
                                               const float* dxact,   // read (earlier slots)
                                               float* dxact_out,     // written (last slot)
-                                              const uint16_t* __restrict__ xact, int nslice,
+                                              const uint16_t* xact, int nslice,
                                               float* __restrict__ red,
                                               uint16_t* __restrict__ d_out, uint16_t* __restrict__ Xr) {
     pdl_entry();

@@ -16,9 +16,9 @@ namespace {
 
 constexpr int WC_NT = 128;
 
-__global__ void __launch_bounds__(WC_NT) k_wb_coef(Dims d, int slot, int T, int TB, const float* __restrict__ red,
-                                                   int nslice, const float* __restrict__ p,
-                                                   const float* __restrict__ hpost,
+__global__ void __launch_bounds__(WC_NT) k_wb_coef(Dims d, int slot, int T, int TB, const float* red,
+                                                   int nslice, const float* p,
+                                                   const float* hpost,
                                                    double* __restrict__ gram, float* __restrict__ emat) {
     pdl_entry();
     __shared__ double Gs[32][NGRAM + 1];

@@ -209,7 +209,6 @@ __device__ __forceinline__ int seg_of(const WSegs& w, int o) {
 }
 // W[r][o] of the segmented weight (the segment of column o): the segment's fields are selected
 // with static indices, so the kernel parameter is not copied to local memory for a dynamic index
-template <bool RO = false>
 __device__ __forceinline__ float seg_elem(const WSegs& w, long long r, int o) {
     const float* p = w.ptr[0];
     int width = w.width[0], off = w.off[0];
@@ -220,7 +219,7 @@ __device__ __forceinline__ float seg_elem(const WSegs& w, long long r, int o) {
             width = w.width[q];
             off = w.off[q];
         }
-    return RO ? __ldg(p + r * width + (o - off)) : p[r * width + (o - off)];
+    return p[r * width + (o - off)];
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -332,6 +331,9 @@ void note_launch();  // counts every kernel launch of the library
 // placed while the last blocks of the kernel before run out, and wait there until that kernel's
 // writes are visible; launched without, both instructions do nothing.  No kernel touches global memory
 // before, so one whose wait has ended follows all that came before it in its stream.
+// The buffers it reads may be written while its blocks already wait, so they are not read-only for the life
+// of the kernel: they are read with plain loads, never with __ldg, and pointers to const are not
+// __restrict__, which would let the compiler take the read-only path or lift a load over the wait.
 __device__ __forceinline__ void pdl_entry() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -410,7 +412,7 @@ __device__ __forceinline__ void pack_rows_of(const PackJob& j, int blk) {
     for (int e = blk * PACK_E + threadIdx.x; e < min(j.K, (blk + 1) * PACK_E); e += blockDim.x) {
 #pragma unroll 4
         for (int o = 0; o < j.n; ++o) {
-            const float w = seg_elem<true>(j.W, e, o);
+            const float w = seg_elem(j.W, e, o);
             const __nv_bfloat16 h = __float2bfloat16_rn(w);
             j.dst[(int64_t)o * j.K + e] = __bfloat16_as_ushort(h);
             j.dst[(int64_t)(j.n + o) * j.K + e] = __bfloat16_as_ushort(__float2bfloat16_rn(w - __bfloat162float(h)));
@@ -489,7 +491,7 @@ __device__ __forceinline__ void pack_wrows_of(const WRows& j, int blk) {
             }
             if (in) {
                 part[u] = c / j.n;
-                v[u] = seg_elem<true>(j.W, r, c - part[u] * j.n);
+                v[u] = seg_elem(j.W, r, c - part[u] * j.n);
             }
         }
     }
@@ -587,7 +589,7 @@ int colsum_parts(int rows);
 int colsum_chunk(int rows);        // rows of a chunk
 // chunk `part`, by the first 8 n threads of a block (n <= MAXN): eight threads a column over interleaved
 // rows (U loads each in flight), then their sum in order.  sh: 8 n floats.  Has block barriers.
-__device__ __forceinline__ void colsum_chunk_of(const float* __restrict__ in, int rows, int n, int rchunk, int part,
+__device__ __forceinline__ void colsum_chunk_of(const float* in, int rows, int n, int rchunk, int part,
                                                 float* sh, float* __restrict__ out) {
     constexpr int U = 32;
     const int o = threadIdx.x % n, ty = threadIdx.x / n;
