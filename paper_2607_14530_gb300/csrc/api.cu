@@ -242,13 +242,14 @@ Layout make_layout(const Dims& d, int64_t T) {
     L.wpacka = o; o = al(o + (size_t)L.tca.NB * d.k * d.C * 2);
     L.dzpack = o; o = al(o + (size_t)std::max(L.twf.NB, L.twa.NB) * ((t + 7) / 8 * 8) * 2);
     {
-        // bf16 operands of the tensor-core input gradients: full maps [T][nfull] and [N C][nfull] (three
-        // times the columns at some widths), active maps in three parts [T][3 nact] and [k][C][3 nact]
-        // (rows padded to 8, the C rows to 32)
-        const size_t ld = dx_ld(std::max(1, dx_tc_parts((int)T, d.N, d.C, d.nfull, d.G)) * d.nfull);
-        const size_t ld3 = dxa_ld(nact_max);
-        L.dz16 = o; o = al(o + t * std::max(ld, ld3) * 2);
-        L.w16 = o; o = al(o + std::max((size_t)d.N * d.C * ld, (size_t)d.k * dxa_width(d.C) * ld3) * 2);
+        // bf16 operands of the tensor-core input gradients, in the columns of their terms: full maps [T] and
+        // [N C] rows, active maps [T] and [k][C] rows (the C rows padded to 32)
+        const size_t ld = split_ld(d.nfull, std::max(1, dx_tc_terms((int)T, d.N, d.C, d.nfull, d.G)));
+        size_t lda = 0;
+        for (int q = 0; q < d.G; ++q)
+            lda = std::max(lda, (size_t)split_ld(d.nact[q], std::max(1, dxa_tc_terms((int)T, d.k, d.C, d.nact[q]))));
+        L.dz16 = o; o = al(o + t * std::max(ld, lda) * 2);
+        L.w16 = o; o = al(o + std::max((size_t)d.N * d.C * ld, (size_t)d.k * dxa_width(d.C) * lda) * 2);
     }
     L.part = o;
     o = al(o + std::max((size_t)L.splits_full * d.nfull, (size_t)L.splits_act * nact_max) * t * 4);
@@ -912,12 +913,13 @@ xhc_status post_bwd_impl(const xhc_handle* h, int slot, int64_t T, const xhc_par
                                               bslices, red, Xr, c.st));
     }
     // the bf16 operands of the weight gradient and of pre_bwd(slot)'s input gradient, formed with dZ_act
-    const bool tcw = !(T32 < 64 || d.k * d.C < 128), tcx = dxa_tc_ok(T32, d.k, d.C, n);
+    const bool tcw = !(T32 < 64 || d.k * d.C < 128), tcx = dxa_tc_terms(T32, d.k, d.C, n) > 0;
+    const int terms = dxa_tc_terms(T32, d.k, d.C, n);
     const ProjTcPlan wpl = plan_proj_tc(d.k * d.C, T32, n, device_sms(), false);
     const int Tp = (T32 + 7) / 8 * 8;   // 16-byte row stride for the tensor map
     const DzPack pk = {tcw ? c.W<uint16_t>(c.L.dzpack) : nullptr, tcx ? c.W<uint16_t>(c.L.dz16) : nullptr, wpl.NB, Tp,
-                       dxa_ld(n), 3};
-    const WRows wr = {act_segs(d, P, slot), n, d.k * dxa_width(d.C), dxa_ld(n), 3,
+                       split_ld(n, terms), terms};
+    const WRows wr = {act_segs(d, P, slot), n, d.k * dxa_width(d.C), split_ld(n, terms), terms,
                       tcx ? c.W<uint16_t>(c.L.w16) : nullptr, d.C};
     int nblk = 0;
     XHC_K("bwd_coef", c.st, launch_bwd_coef(d, slot, T32, red, bslices, c.S<float>(c.L.zact[slot]),
@@ -998,7 +1000,7 @@ xhc_status xhc_pre_bwd(const xhc_handle* h, int slot, int64_t T, const xhc_param
     const int T32 = c.T;
     uint16_t* dinput = c.W<uint16_t>(c.L.dinput);
     const int n = d.nact[slot];
-    const bool tc = dxa_tc_ok(T32, d.k, d.C, n);
+    const bool tc = dxa_tc_terms(T32, d.k, d.C, n) > 0;
     if (tc) {
         // post_bwd(slot) left dZ_act of this slot in the workspace; the update also forms the
         // dH_pre dots of the active streams (per 32 channels) and copies d_input
@@ -1015,13 +1017,13 @@ xhc_status xhc_pre_bwd(const xhc_handle* h, int slot, int64_t T, const xhc_param
     }
     if (slot != 0) return XHC_OK;
     XHC_K("full_dots", c.st, launch_full_dots(d, T32, X, dinput, c.S<int>(c.L.I), c.W<float>(c.L.dhpre), c.st));
-    const int parts = dx_tc_parts(T32, d.N, d.C, d.nfull, d.G);
-    const bool tcw = !(T32 < 64 || d.N * d.C < 128), tcx = parts > 0;
+    const int terms = dx_tc_terms(T32, d.N, d.C, d.nfull, d.G);
+    const bool tcw = !(T32 < 64 || d.N * d.C < 128), tcx = terms > 0;
     const ProjTcPlan& wpl = c.L.twf;
     const int Tp = (T32 + 7) / 8 * 8;   // 16-byte row stride for the tensor map
     const DzPack pk = {tcw ? c.W<uint16_t>(c.L.dzpack) : nullptr, tcx ? c.W<uint16_t>(c.L.dz16) : nullptr, wpl.NB, Tp,
-                       dx_ld(parts * d.nfull), parts};
-    const WRows wr = {full_segs(d, P), d.nfull, d.N * d.C, dx_ld(parts * d.nfull), parts, tcx ? c.W<uint16_t>(c.L.w16) : nullptr, 0};
+                       split_ld(d.nfull, terms), terms};
+    const WRows wr = {full_segs(d, P), d.nfull, d.N * d.C, split_ld(d.nfull, terms), terms, tcx ? c.W<uint16_t>(c.L.w16) : nullptr, 0};
     int nblk = 0;
     XHC_K("full_coef", c.st, launch_full_coef(d, T32, c.W<float>(c.L.dhpre), c.S<float>(c.L.hpre),
                               c.S<float>(c.L.zfull), c.S<float>(c.L.stats), c.S<float>(c.L.wsum),

@@ -780,7 +780,8 @@ struct DxArgs {
     int slot;             // active epilogue: slot of the pre-map
     int NH;               // active epilogue: streams of the H_pre rows
     float* dxa;           // active epilogue: dX_act [T][k][C] fp32, updated in place
-    int nkb, ksteps;      // k-blocks of 64, MMA k-steps of 16
+    int nkb, ksteps;      // k-blocks of 64, MMA k-steps of 16 of a pair of parts
+    int pr0;              // first pair of parts (6 terms: 0), or 5 for one pass over all columns
     int TT, CT;           // token tiles, channel tiles per stream
     long long ntiles;
     int P;
@@ -801,6 +802,27 @@ struct DxArgs {
     int nbs;              // full-state dX: stages of W rows
     int nsplit;           // full-state dX: parts that a column block's streams are cut into (of two streams at least)
 };
+
+// the MMAs of one tile: the k-steps of every pair of parts (see split_cols), from operands in k-blocks of 64 columns
+template <int BN>
+__device__ __forceinline__ void dx_mma(const DxArgs& a, uint32_t d, uint32_t abase, uint32_t bbase, uint32_t idesc) {
+    uint32_t accum = 0;
+    for (int pr = a.pr0; pr < 6; ++pr) {
+        const int a0 = split_pair_a(pr) * a.ksteps, b0 = split_pair_b(pr) * a.ksteps;
+        for (int ks = 0; ks < a.ksteps; ++ks) {
+            const uint32_t ka = (uint32_t)(a0 + ks), kb = (uint32_t)(b0 + ks);
+            mma_bf16(d, sw128_desc(abase + (ka >> 2) * (BM * BK * 2) + (ka & 3) * 32),
+                     sw128_desc(bbase + (kb >> 2) * (BN * BK * 2) + (kb & 3) * 32), idesc, accum);
+            accum = 1;
+        }
+    }
+}
+// k-blocks, k-steps and pairs of a product of n columns in `terms` terms
+void dx_ksteps(DxArgs& a, int n, int terms) {
+    a.nkb = (split_cols(n, terms) + BK - 1) / BK;
+    a.ksteps = ((terms == 6 ? n : split_cols(n, terms)) + 15) / 16;
+    a.pr0 = terms == 6 ? 0 : 5;
+}
 
 // TMEM -> registers, 16 lanes x 32 columns: lane l gets row l / 4 (v[4 g + e]) and row l / 4 + 8 (v[4 g + 2 +
 // e]), columns 8 g + 2 (l % 4) + e, g < 4, e < 2 (wait in the same statement, as above)
@@ -925,11 +947,7 @@ k_dx_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
                 tc_fence_after();
                 const uint32_t abase = smem_u32(smem);
                 const uint32_t bbase = abase + A_BYTES;
-                for (int ks = 0; ks < a.ksteps; ++ks) {
-                    const int kb = ks >> 2, kk = ks & 3;
-                    mma_bf16(tmem + (uint32_t)(s * DX_BN), sw128_desc(abase + kb * BM * BK * 2 + kk * 32),
-                             sw128_desc(bbase + kb * DX_BN * BK * 2 + kk * 32), idesc, ks > 0 ? 1u : 0u);
-                }
+                dx_mma<DX_BN>(a, tmem + (uint32_t)(s * DX_BN), abase, bbase, idesc);
                 mma_commit(smem_u32(&bars[1]));      // operands consumed
                 mma_commit(smem_u32(&bars[2 + s]));  // accumulator ready
             }
@@ -1267,11 +1285,7 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
                 tc_fence_after();
                 const uint32_t abase = smem_u32(sA);
                 const uint32_t bbase = smem_u32(sB + b * B_BYTES);
-                for (int ks = 0; ks < a.ksteps; ++ks) {
-                    const int kb = ks >> 2, kk = ks & 3;
-                    mma_bf16(tmem + (uint32_t)(s * DG_BN), sw128_desc(abase + kb * BM * BK * 2 + kk * 32),
-                             sw128_desc(bbase + kb * DG_BN * BK * 2 + kk * 32), idesc, ks > 0 ? 1u : 0u);
-                }
+                dx_mma<DG_BN>(a, tmem + (uint32_t)(s * DG_BN), abase, bbase, idesc);
                 mma_commit(smem_u32(&bars[4 + b]));              // B stage consumed
                 mma_commit(smem_u32(&bars[8 + s]));              // accumulator ready
                 if (p == NU - 1) mma_commit(smem_u32(&bars[1]));  // the block's A rows consumed
@@ -1426,29 +1440,32 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
 
 }  // namespace
 
-// Any width (a multiple of 8), and up to five k-blocks of the three parts (k = 8 with a conv: nact = 96): 160
-// of the 227 KB of shared memory.  Below a tile of tokens the CUDA-core pair gemm_dzw + dinput_act stays.
+// Any width (a multiple of 8) and number of columns (nact <= 96: five k-blocks of the three parts, 160 of the 227
+// KB of shared memory).  Below a tile of tokens the CUDA-core pair gemm_dzw + dinput_act stays.  Three terms where
+// DX_BN divides the width and two k-blocks hold them; six elsewhere, where gemm_dzw would take the operands in
+// fp32 and dX_act, which is fp32 and feeds the earlier slots' parameter gradients, shows it.
 // T = 1000, C = 1160, k = 8, nact = 96: gemm_dzw + dinput_act 92 + 29 us, here 38.
-bool dxa_tc_ok(int T, int k, int C, int nact) {
-    return T >= BM && 3 * nact <= 5 * BK &&
-           (long long)((T + BM - 1) / BM) * ((C + DX_BN - 1) / DX_BN) * k < (1LL << 31);   // 32-bit tile indices
+int dxa_tc_terms(int T, int k, int C, int nact) {
+    if (T < BM || split_cols(nact, 6) > 5 * BK ||
+        (long long)((T + BM - 1) / BM) * ((C + DX_BN - 1) / DX_BN) * k >= (1LL << 31))   // 32-bit tile indices
+        return 0;
+    return C % DX_BN == 0 && 3 * nact <= 2 * BK ? 3 : 6;
 }
 
 cudaError_t launch_dxa_tc(const Dims& d, int slot, int T, int nact,
-                          const uint16_t* dz3, const uint16_t* w3, const uint16_t* d_input, const float* hpre,
+                          const uint16_t* dzr, const uint16_t* wr, const uint16_t* d_input, const float* hpre,
                           const int* I, const uint16_t* xact, const float* tokmat, float* dxact,
                           float* dotp, uint16_t* dcopy, int* err, cudaStream_t st) {
-    const int K3 = 3 * nact;
-    const int ld = dxa_ld(nact);
+    const int terms = dxa_tc_terms(T, d.k, d.C, nact);
+    const int cols = split_cols(nact, terms), ld = split_ld(nact, terms);
     cudaError_t e;
     CUtensorMap ma, mb;
-    if (!make_map_box(&ma, dz3, (uint64_t)K3, (uint64_t)T, BK, BM, (uint64_t)ld * 2)) return cudaErrorInvalidValue;
-    if (!make_map_box(&mb, w3, (uint64_t)K3, (uint64_t)d.k * dxa_width(d.C), BK, DX_BN, (uint64_t)ld * 2)) return cudaErrorInvalidValue;
+    if (!make_map_box(&ma, dzr, (uint64_t)cols, (uint64_t)T, BK, BM, (uint64_t)ld * 2)) return cudaErrorInvalidValue;
+    if (!make_map_box(&mb, wr, (uint64_t)cols, (uint64_t)d.k * dxa_width(d.C), BK, DX_BN, (uint64_t)ld * 2)) return cudaErrorInvalidValue;
     DxArgs a;
     memset(&a, 0, sizeof(a));
     a.T = T; a.C = d.C; a.N = d.N; a.k = d.k; a.G = d.G; a.slot = slot;
-    a.nkb = (K3 + BK - 1) / BK;
-    a.ksteps = (K3 + 15) / 16;
+    dx_ksteps(a, nact, terms);
     a.TT = (T + BM - 1) / BM;
     a.CT = (d.C + DX_BN - 1) / DX_BN;
     a.Cp = dxa_width(d.C);
@@ -1512,27 +1529,26 @@ static size_t dxf_smem(int K, int G, int nbs) {
 // two stages of W rows where they fit the 227 KB a block may use, else one, or none
 static int dxf_stages(int K, int G) { return dxf_smem(K, G, 2) <= 232448 ? 2 : dxf_smem(K, G, 1) <= 232448 ? 1 : 0; }
 
-// How the full-state dX takes dZ and W: 1 rounded to bf16, where 64 divides the width (up to three k-blocks:
-// nfull <= 192, N = 32 with a router and four pre-maps); 3 in three bf16 parts, hi | lo | hi times hi | hi |
-// lo, at other widths: the CUDA-core full_dx that they went to takes both in fp32, and the products keep 16
-// bits.  0: full_dx (less than a tile of tokens, or too many columns for the shared memory).
+// How the full-state dX takes dZ and W: in one term where 64 divides the width (up to three k-blocks: nfull <=
+// 192, N = 32 with a router and four pre-maps); in six at other widths, where the CUDA-core full_dx would take
+// both in fp32.  0: full_dx (less than a tile of tokens, or too many columns for the shared memory).
 // T = 1000, N = 12, C = 1160: full_dx 79 us, here 37; T = 4944, N = 16, C = 2840, four
 // slots (G N + N = 80 columns, one stage of weight rows): the step 5.99 -> 3.40 ms with both gradients here.
-int dx_tc_parts(int T, int N, int C, int nfull, int G) {
+int dx_tc_terms(int T, int N, int C, int nfull, int G) {
     if (T < BM || N < 2 || G < 1 || G > 4 ||
         (long long)((T + BM - 1) / BM) * ((C + DG_BN - 1) / DG_BN) * N >= (1LL << 31))   // 32-bit tile indices
         return 0;
     if (C % DG_BN == 0) return nfull <= 3 * BK && dxf_smem(nfull, G, 2) <= 232448 ? 1 : 0;
-    return dxf_stages(3 * nfull, G) > 0 ? 3 : 0;
+    return dxf_stages(split_cols(nfull, 6), G) > 0 ? 6 : 0;
 }
 
 cudaError_t launch_dx_tc(const Dims& d, int T, const uint16_t* dz16,
                          const uint16_t* w16, const uint16_t* X, const uint16_t* dinput, const float* hpre,
                          const int* I, const float* dxact, const float* scal, int scal_ld,
                          uint16_t* dX, int* err, cudaStream_t st) {
-    const int parts = dx_tc_parts(T, d.N, d.C, d.nfull, d.G);
-    const int n = parts * d.nfull, NC = d.N * d.C;
-    const int ld = dx_ld(n);
+    const int terms = dx_tc_terms(T, d.N, d.C, d.nfull, d.G);
+    const int n = split_cols(d.nfull, terms), NC = d.N * d.C;
+    const int ld = split_ld(d.nfull, terms);
     cudaError_t e;
     CUtensorMap ma, mb, mx, md, mg;
     if (!make_map_box(&ma, dz16, (uint64_t)n, (uint64_t)T, BK, BM, (uint64_t)ld * 2)) return cudaErrorInvalidValue;
@@ -1545,8 +1561,7 @@ cudaError_t launch_dx_tc(const Dims& d, int T, const uint16_t* dz16,
     DxArgs a;
     memset(&a, 0, sizeof(a));
     a.T = T; a.C = d.C; a.N = d.N; a.k = d.k; a.G = d.G; a.m = d.m; a.dense = d.dense;
-    a.nkb = (n + BK - 1) / BK;
-    a.ksteps = (n + 15) / 16;
+    dx_ksteps(a, d.nfull, terms);
     a.TT = (T + BM - 1) / BM;
     a.CT = (d.C + DG_BN - 1) / DG_BN;
     a.nbs = dxf_stages(n, d.G);

@@ -420,17 +420,38 @@ __device__ __forceinline__ void pack_rows_of(const PackJob& j, int blk) {
         for (int r = 2 * j.n; r < j.NB; ++r) j.dst[(int64_t)r * j.K + e] = 0;
     }
 }
+// How a bf16 product takes two fp32 operands of n columns each:
+//   1 term   both rounded once
+//   3 terms  two parts each, hi and lo: columns hi | lo | hi of one operand times hi | hi | lo of the other (the
+//            products keep 16 bits)
+//   6 terms  three parts each, hi | mid | lo with every part padded to whole MMA k-steps of 16 columns; the
+//            product's k-steps take the pairs of parts lo hi, mid mid, hi lo, mid hi, hi mid, hi hi, the smallest
+//            first (a part has 8 bits, so that what is left out is 2^-24 of the product, as fp32 leaves)
+__host__ __device__ inline int split_step(int n) { return (n + 15) / 16 * 16; }
+__host__ __device__ inline int split_cols(int n, int terms) { return terms == 6 ? 3 * split_step(n) : terms * n; }
+inline int split_ld(int n, int terms) { return (split_cols(n, terms) + 7) / 8 * 8; }   // 16-byte rows
+// the parts of a pair of the six terms, at its place in their order
+__device__ __forceinline__ int split_pair_a(int pr) { return (0x046 >> (2 * pr)) & 3; }   // 2 1 0 1 0 0
+__device__ __forceinline__ int split_pair_b(int pr) { return (0x124 >> (2 * pr)) & 3; }   // 0 1 2 0 1 0
+// part q of v (6 terms).  A value that bf16 cannot round to a finite one is its lo part alone, which only one
+// product takes: an infinity stays one (inf - inf, and infinity times another part, would be NaN).
+__device__ __forceinline__ float split_part(float v, int q) {
+    const float hi = __bfloat162float(__float2bfloat16_rn(v));
+    if (!(fabsf(hi) <= 3.4e38f)) return q < 2 ? 0.f : __bfloat162float(__float2bfloat16_rz(v));
+    if (q == 0) return hi;
+    const float mid = __bfloat162float(__float2bfloat16_rn(v - hi));
+    return q == 1 ? mid : (v - hi) - mid;
+}
 inline int pack_blocks(const PackJob& j) { return j.dst ? (j.K + PACK_E - 1) / PACK_E : 0; }
 // bf16 operands that the tensor-core backward takes from a slot's (or the full-state) projection-output
 // gradient dz [T][n], written by the coefficient kernel that forms it:
 //   hilo [NB][Tp]  rows 0..n-1 the hi parts, n..2n-1 the lo parts, the rest zero (k_proj_tc's B operand of
 //                  the weight gradient)
-//   rows [T][ld]   the A operand of the input gradient, a token's columns `parts` times over: hi | lo | hi
-//                  (parts 3) or the value rounded once (parts 1), zero from parts * n on
+//   rows [T][ld]   the A operand of the input gradient, in the columns of `terms`, zero past them
 // null pointers: not wanted.
 struct DzPack {
     uint16_t *hilo, *rows;
-    int NB, Tp, ld, parts;
+    int NB, Tp, ld, terms;
 };
 // dz of a block's ntok tokens from t0 on, in shared memory (row stride rs), into the two operands
 __device__ __forceinline__ void pack_dz_of(const DzPack& p, const float* dz, int rs, int n, long long t0, int ntok) {
@@ -448,7 +469,10 @@ __device__ __forceinline__ void pack_dz_of(const DzPack& p, const float* dz, int
         for (int idx = threadIdx.x; idx < ntok * p.ld; idx += blockDim.x) {
             const int tt = idx / p.ld, c = idx - tt * p.ld;
             float v = 0.f;
-            if (c < p.parts * n) {
+            if (p.terms == 6) {
+                const int np = split_step(n), part = c / np, o = c - part * np;
+                if (o < n && part < 3) v = split_part(dz[tt * rs + o], part);
+            } else if (c < p.terms * n) {
                 const int part = c / n;
                 v = dz[tt * rs + c - part * n];
                 if (part == 1) v -= __bfloat162float(__float2bfloat16_rn(v));
@@ -456,11 +480,11 @@ __device__ __forceinline__ void pack_dz_of(const DzPack& p, const float* dz, int
             p.rows[(t0 + tt) * p.ld + c] = f2bf(v);
         }
 }
-// the weight side of the input gradient: dst [rows][ld] bf16, a weight row's n columns `parts` times over
-// (hi | hi | lo, or rounded once), zero from parts * n on; packed by further blocks of the same launch
+// the weight side of the input gradient: dst [rows][ld] bf16, a weight row in the columns of `terms`, zero past
+// them; packed by further blocks of the same launch
 struct WRows {
     WSegs W;
-    int n, rows, ld, parts;
+    int n, rows, ld, terms;
     uint16_t* dst;   // null: nothing to pack
     int C;           // > 0: slots of C rows, each padded to dxa_width(C), in the order of dxa_row
 };
@@ -483,22 +507,25 @@ __device__ __forceinline__ void pack_wrows_of(const WRows& j, int blk) {
         if (idx < tot) {
             int r = idx / j.ld;
             const int c = idx - r * j.ld;
-            bool in = c < j.parts * j.n;
+            const int np = j.terms == 6 ? split_step(j.n) : j.n;
+            const int q = c / np, o = c - q * np;
+            bool in = q < (j.terms == 6 ? 3 : j.terms) && o < j.n;
             if (j.C > 0) {
                 const int slot = r / dxa_width(j.C), ch = dxa_row(r - slot * dxa_width(j.C));
                 in = in && ch < j.C;
                 r = slot * j.C + ch;
             }
             if (in) {
-                part[u] = c / j.n;
-                v[u] = seg_elem(j.W, r, c - part[u] * j.n);
+                part[u] = q;
+                v[u] = seg_elem(j.W, r, o);
             }
         }
     }
 #pragma unroll
     for (int u = 0; u < WROWS_U; ++u) {
         const int idx = at + u * (int)blockDim.x;
-        if (part[u] == 2) v[u] -= __bfloat162float(__float2bfloat16_rn(v[u]));
+        if (j.terms == 6) v[u] = split_part(v[u], part[u]);
+        else if (part[u] == 2) v[u] -= __bfloat162float(__float2bfloat16_rn(v[u]));
         if (idx < tot) j.dst[idx] = f2bf(v[u]);
     }
 }
@@ -517,23 +544,22 @@ cudaError_t launch_proj_tc(const uint16_t* X, int T, int K, const uint16_t* Wpac
 // dzpack: the hi / lo rows of dz (DzPack::hilo, Tp tokens a row)
 cudaError_t launch_wgrad_tc(const uint16_t* A, int T, int E, int n, const uint16_t* dzpack, int Tp,
                             const ProjTcPlan& p, float* part, int* err, cudaStream_t st);
-int dx_tc_parts(int T, int N, int C, int nfull, int G);   // parts of the operands, 0: not on the tensor cores
-bool dxa_tc_ok(int T, int k, int C, int nact);
-// dX_act += dZ_act W_act^T (three-term bf16 split on the tensor cores) + H_pre[slot][I_j] d_input
+// terms of the full-state and of the active-state input gradient's product, 0: not on the tensor cores
+int dx_tc_terms(int T, int N, int C, int nfull, int G);
+int dxa_tc_terms(int T, int k, int C, int nact);
+// dX_act += dZ_act W_act^T (in dxa_tc_terms bf16 terms on the tensor cores) + H_pre[slot][I_j] d_input
 //           - cx x_act (the write-back's own term, cx per token in tokmat);
 // in the same pass: dotp[j][g][t] = <x_act_j, d_input> over channels 32 g .. 32 g + 31, and the
 // copy dcopy[slot][t][:] = d_input[t][:]
-// (dz3, w3: the three-part operands, DzPack / WRows with parts 3)
-inline int dxa_ld(int nact) { return (3 * nact + 7) / 8 * 8; }
+// (dzr, wr: the operands in those terms, DzPack / WRows)
 cudaError_t launch_dxa_tc(const Dims& d, int slot, int T, int nact,
-                          const uint16_t* dz3, const uint16_t* w3, const uint16_t* d_input, const float* hpre,
+                          const uint16_t* dzr, const uint16_t* wr, const uint16_t* d_input, const float* hpre,
                           const int* I, const uint16_t* xact, const float* tokmat, float* dxact,
                           float* dotp, uint16_t* dcopy, int* err, cudaStream_t st);
 // dH_pre[t][slot][I_j] = sum over the groups g of 32 channels of dotp[j][g][t] (g in order)
 cudaError_t launch_dots_act(const Dims& d, int slot, int T, const float* dotp, const int* I, float* dhpre,
                             cudaStream_t st);
-// (dz16, w16: the operands in dx_tc_parts parts, K columns altogether)
-inline int dx_ld(int K) { return (K + 7) / 8 * 8; }
+// (dz16, w16: the operands in dx_tc_terms terms)
 cudaError_t launch_dx_tc(const Dims& d, int T, const uint16_t* dz16,
                          const uint16_t* w16, const uint16_t* X, const uint16_t* dinput, const float* hpre,
                          const int* I, const float* dxact, const float* scal, int scal_ld,
