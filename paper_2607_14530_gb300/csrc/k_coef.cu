@@ -67,9 +67,11 @@ __device__ __forceinline__ float slot_sum(const float* p, long long stride, int 
 }
 
 // Two arrays of slot sums into shared memory: dst[0, n0) = sums of p0 + e, dst[n0, n0 + n1) = sums of
-// p1 + e * step1.  The slots of a stream-K plan are added in slot order (any number of tokens gives
-// the same bits for a token, and so the same routing); those of an even split, of which there are
-// many on few tokens, by groups of threads that take interleaved slots (scr: one float per thread).
+// p1 + e * step1.  The slots of a stream-K plan are added in slot order; those of an even split, of which
+// there are many on few tokens, by groups of threads that take interleaved slots (scr: one float per thread),
+// a number of groups that follows from n alone while a block takes one token (below 128 tokens it does).  So a
+// token of a call of fewer than 128 has the same bits whatever the others are; from 128 on the plan, and with it
+// where the sums are cut, depends on the number of tokens.
 // Few elements with many ordered slots pass through shared memory (stage: SS_STAGE floats), so that
 // the whole block loads them: 82 sums over 172 slots took 27 us with a thread each.  Ends with a
 // block barrier.

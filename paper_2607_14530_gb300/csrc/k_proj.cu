@@ -8,6 +8,7 @@
 //   wgrad     dW += A^T dZ, reduced over tokens in a fixed order
 //   colsum    fixed-order partial column sums of W_r (within rowproj below 128 tokens)
 #include <algorithm>
+#include <type_traits>
 
 #include "xhc_internal.cuh"
 
@@ -209,16 +210,39 @@ __global__ void __launch_bounds__(RS_NT) k_rowproj_small(const uint16_t* A, int6
     }
     __syncthreads();
     const int O = n * TT;
+    // (every block of the split folds, however few its rows: V columns an access; with one the decode step above
+    // took 394 us at 127 tokens and 207 at 16, here 340 and 175)
+    using VT = std::conditional_t<V == 4, float4, float>;
+    VT* const sv = reinterpret_cast<VT*>(sm);
     if (work) {
 #pragma unroll
-        for (int c = 0; c < V; ++c)
+        for (int u = 0; u < TT; ++u) {
+            float v[V];
 #pragma unroll
-            for (int u = 0; u < TT; ++u) sm[rl * O + u * n + o + c] = (u & 1) ? acc[c][u / 2].y : acc[c][u / 2].x;
+            for (int c = 0; c < V; ++c) v[c] = (u & 1) ? acc[c][u / 2].y : acc[c][u / 2].x;
+            VT* const dst = sv + (rl * O + u * n + o) / V;
+            if constexpr (V == 4) *dst = make_float4(v[0], v[1], v[2], v[3]);
+            else *dst = v[0];
+        }
     }
     __syncthreads();
     for (int m = nl; m > 1;) {
         const int h = (m + 1) / 2;
-        for (int e = tid; e < (m - h) * O; e += RS_NT) sm[e] += sm[h * O + e];
+        const VT* const hi = sv + h * O / V;
+#pragma unroll 2
+        for (int e = tid; e < (m - h) * O / V; e += RS_NT) {
+            VT a = sv[e];
+            const VT b = hi[e];
+            if constexpr (V == 4) {
+                a.x += b.x;
+                a.y += b.y;
+                a.z += b.z;
+                a.w += b.w;
+            } else {
+                a += b;
+            }
+            sv[e] = a;
+        }
         __syncthreads();
         m = h;
     }
@@ -231,17 +255,21 @@ __global__ void __launch_bounds__(RS_NT) k_rowproj_small(const uint16_t* A, int6
 template <int TT, int V>
 static cudaError_t rowproj_small(const uint16_t* A, int64_t lda, int K, int T, const WSegs& W, int n, int* splits,
                                  float* part, float* pstats, const ColJob& cj, cudaStream_t st) {
-    const int nl = RS_NT / (n / V), ny = (T + TT - 1) / TT;
-    // a block per SM, with at least four rows a row lane
-    int s = std::min(*splits, std::max(1, device_sms() / ny));
-    s = std::max(1, std::min(s, K / (4 * nl)));
+    const int nl = RS_NT / (n / V);
+    // a block per SM for the first tokens, with at least four rows a row lane.  The split follows from K and n
+    // alone, so that a token's projections have the same bits in every batch of fewer than ROWPROJ_SMALL, and a
+    // decoded sequence does not depend on the others of its batch.  (A split that shrinks as the tokens grow, for
+    // one wave of blocks: a decode step of N = 16, C = 4096, four slots takes 331 us at 127 tokens, here 340; N =
+    // 12, C = 1160, k = 8, one slot: 77, here 97.)
+    int s = std::min(device_sms(), K / std::max(256, 4 * nl));
+    s = std::max(1, std::min(s, *splits));   // *splits is no less for these calls
     const int kchunk = ((K + s - 1) / s + 7) / 8 * 8;
     s = (K + kchunk - 1) / kchunk;
     *splits = s;
     const size_t sm = sizeof(float) * std::max((size_t)RS_ROWS * ((TT + 1) / 2 * 2), (size_t)nl * n * TT);
     const cudaError_t e = smem_optin((const void*)k_rowproj_small<TT, V>, sm);
     if (e != cudaSuccess) return e;
-    XHC_LAUNCH(st, dim3(cj.parts + s, ny), RS_NT, sm, (k_rowproj_small<TT, V>), A, lda, K, T, W, n, kchunk, part, pstats, cj);
+    XHC_LAUNCH(st, dim3(cj.parts + s, (T + TT - 1) / TT), RS_NT, sm, (k_rowproj_small<TT, V>), A, lda, K, T, W, n, kchunk, part, pstats, cj);
     return cudaGetLastError();
 }
 

@@ -95,3 +95,36 @@ def test_decode_matches_the_whole_sequence_forward(N, k, m, C, G, B, S):
     assert gd.device_error(ws_d) == 0
     assert torch.equal(pos.cpu(), torch.full((B,), S + ND, dtype=torch.int64)), "pos not advanced"
     assert not errors, "\n".join(errors)
+
+
+@pytest.mark.parametrize("cfg", [Config.flash(16, 4, 2, 1024, 4), Config.full(12, 8, 3, 264, True)], ids=["flash4", "k8"])
+def test_batches_below_a_tile_have_the_same_bits(cfg):
+    """A token decoded in a batch of any size below 128 (the tensor cores' tile) has the same routing,
+    coefficients, sublayer inputs and state, bit by bit, as alone: batches on both sides of the sizes at which
+    the projection takes more tokens a block or more blocks."""
+    dev = torch.device("cuda", 0)
+    n = 127
+    inp = synth.group_inputs(n, cfg.N, cfg.C, cfg.G, 3)
+    P = {k: v.to(dev) for k, v in synth.params(cfg.param_shapes(), 3).items()}
+    g = Group(cfg)
+    R = max(cfg.conv_k) - 1
+    hist = [synth.normal_bf16((n, R, cfg.C), 17 + t).to(dev) for t in range(cfg.G)]
+
+    def decode(rows):
+        B = len(rows)
+        X = inp["X"][rows].to(dev)
+        outs = [o[rows].to(dev) for o in inp["outs"]]
+        rings = g.alloc_rings(B)
+        for t, r in enumerate(rings):
+            if r is not None:
+                r.view(torch.bfloat16).view(B, R, cfg.C).copy_(hist[t][rows])
+        saved, ws = g.alloc(B)
+        pos = torch.full((B,), 40, dtype=torch.int64, device=dev)
+        ins = g.forward_decode(P, X, outs, rings, pos, saved, ws)
+        co = g.coefficients(saved, B)
+        return [X, *ins, *(co[k] for k in ("zfull", "stats", "I", "p", "hpre", "hres")), *co["hpost"]]
+
+    whole = decode(list(range(n)))
+    for first, B in ((0, 1), (126, 1), (3, 2), (5, 9), (0, 16), (40, 17), (1, 33), (20, 64), (9, 100)):
+        for a, b in zip(decode(list(range(first, first + B))), whole):
+            assert torch.equal(a, b[first:first + B]), (first, B)
