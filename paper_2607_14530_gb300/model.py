@@ -68,7 +68,7 @@ class _GroupFn(torch.autograd.Function):
         g, cfg = mod.g, mod.cfg
         T = X.shape[0]
         saved, ws = mod.buffers(T, X.device)
-        P = mod.param_dict()
+        P = mod._params_now()
         pp = g.params(P)
         leaves, outs = [], []
         for t in range(cfg.G):
@@ -105,7 +105,7 @@ class _GroupFn(torch.autograd.Function):
             dX = dX_out
         else:
             dX = dX_out.to(torch.bfloat16).contiguous().clone()
-        P = mod.param_dict()
+        P = mod._params_now()
         # one launch clears them all
         grads = {n: torch.empty_like(v) for n, v in P.items()}
         torch._foreach_zero_(list(grads.values()))
@@ -142,6 +142,12 @@ class XhcGroup(nn.Module):
         self._bufs = {}
 
     def param_dict(self) -> dict:
+        """The group's parameters by their names in the library, detached from autograd (contiguous;
+        they share the parameters' storage wherever those are)."""
+        return {n: v.detach() for n, v in self._params_now().items()}
+
+    def _params_now(self) -> dict:
+        """The same, not detached: for this module's own calls, which only take the pointers."""
         out = {}
         for n, a in zip(self.names, self._attrs):
             v = getattr(self, a)
@@ -176,7 +182,7 @@ class XhcGroup(nn.Module):
         if key not in self._bufs:
             self._bufs[key] = g.alloc_saved(T, device=X.device)
         saved, ws = self._bufs[key], self.buffers_workspace(T, X.device)
-        pp = g.params(self.param_dict())
+        pp = g.params(self._params_now())
         for t in range(cfg.G):
             inp = torch.empty(T, cfg.C, dtype=torch.bfloat16, device=X.device)
             g.pre_fwd(t, pp, X, inp, saved, ws)

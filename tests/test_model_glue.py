@@ -209,3 +209,20 @@ def test_forward_without_grad_records_nothing():
     assert y2.grad_fn is None and not y2.requires_grad
     calls = [e for e in log2 if e[1] in ("pre_fwd", "post_fwd", "sublayer")]
     assert calls == [e for e in log1 if e[1] in ("pre_fwd", "post_fwd", "sublayer")]
+
+
+def test_param_dict_is_detached_and_shares_storage():
+    """What a caller gets may be read into graphs and written in place (an initialisation, a scaling) with grad mode
+    on, and is the parameters' own storage."""
+    cfg = Config.full(4, 2, 1, 8, True, conv_k=(2,))
+    grp = M.XhcGroup(cfg, [nn.Identity()])
+    P = grp.param_dict()
+    assert list(P) == grp.names
+    for n, v in P.items():
+        own = getattr(grp, n.replace(".", "_"))
+        assert not v.requires_grad and v.is_contiguous()
+        assert v.data_ptr() == own.data_ptr()
+        want = own.detach() * 2
+        v.mul_(2)
+        assert torch.equal(own.detach(), want)
+    assert not (P["alpha_pre"] * 3).requires_grad
