@@ -664,7 +664,7 @@ cudaError_t bwd_coef_km(const Dims& d, int slot, int T, const float* red, int ns
                         cudaStream_t st) {
     // 32 tokens a block (k <= 4) fill the fp64 warp, which is what bounds the kernel at many tokens;
     // a quarter of that at few, for more blocks.  (k > 4: 16 and 4.)  The iterates of a long Sinkhorn
-    // run (k > 4, more than 50 iterations) only fit with the small block.
+    // run (k > 4: more than 43 iterations; k <= 4: none of the 64 allowed) only fit with the small block.
     const bool last = (slot == d.G - 1);
     auto smem = [&](int tb) {
         return (size_t)tb * BwdTok<KM>::ROW * 4 + (last ? (size_t)d.iters * KM * tb * KM * 4 : 0);

@@ -20,7 +20,9 @@ CASES = {
     # k > 4: 16-token blocks from 4864 tokens, 4 below; three streams with rows outside the matrix
     "coef_k7_T4867": (Config.full(8, 7, 7, 16, True, seq_len=4867), 4867, {}),
     "coef_k8_T611": (Config.full(8, 8, 8, 16, False), 611, {}),
-    # Sinkhorn iterates that fit only the small block, and none at all
+    # Sinkhorn iterates that just fit the large block, just do not, fit only the small one, and none at all
+    "coef_k8_iters43": (Config.full(8, 8, 8, 8, True, sinkhorn_iters=43, seq_len=4900), 4900, {}),
+    "coef_k8_iters44": (Config.full(8, 8, 8, 8, True, sinkhorn_iters=44, seq_len=4900), 4900, {}),
     "coef_k8_iters64": (Config.full(8, 8, 8, 8, True, sinkhorn_iters=64, seq_len=4900), 4900, {}),
     "coef_k3_iters0": (Config.full(5, 3, 1, 32, True, sinkhorn_iters=0), 130, {}),
     # full-state dX on few blocks: the streams of a block in parts (of 2, 3 or all streams; fixed ones in
