@@ -27,7 +27,8 @@ void PdlScope::set(size_t state_bytes, cudaStream_t st) {
 PdlScope::~PdlScope() { t_pdl = false; }
 
 // ---- shared memory of the kernels -----------------------------------------------------------
-// the limits raised so far, per kernel and device; past the table's end the driver is asked
+// The largest size asked for so far, per kernel and device (past the table's end the driver is asked).  It is set
+// on every call, under the lock: a limit belongs to a context, and a process may have several on a device.
 static std::mutex g_smem_mu;
 static struct {
     const void* fn;
@@ -42,23 +43,20 @@ cudaError_t smem_optin(const void* fn, size_t bytes) {
     std::lock_guard<std::mutex> lk(g_smem_mu);
     int q = 0;
     while (q < g_nsmem && (g_smem[q].fn != fn || g_smem[q].dev != dev)) ++q;
-    int have = 0;
+    int most = (int)bytes;
     if (q < g_nsmem) {
-        have = g_smem[q].bytes;
-    } else {
+        most = std::max(most, g_smem[q].bytes);
+    } else if (q == 1024) {
         cudaFuncAttributes at;
         if ((e = cudaFuncGetAttributes(&at, fn)) != cudaSuccess) return e;
-        have = at.maxDynamicSharedSizeBytes;
+        most = std::max(most, at.maxDynamicSharedSizeBytes);
     }
-    if (have < (int)bytes) {
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        if (e != cudaSuccess) return e;
-        have = (int)bytes;
-    }
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e != cudaSuccess) return e;   // a size the device does not have is not kept
     if (q < 1024) {
         g_smem[q].fn = fn;
         g_smem[q].dev = dev;
-        g_smem[q].bytes = have;
+        g_smem[q].bytes = most;
         if (q == g_nsmem) ++g_nsmem;
     }
     return cudaSuccess;
