@@ -458,7 +458,7 @@ struct BwdTok {
     static constexpr int ROW = (S + KM + 1) | 1;      // odd: a lane per token hits different banks
 };
 
-template <int KM>
+template <int KM, bool SIX>
 __global__ void __launch_bounds__(160) k_bwd_coef(Dims d, int slot, int T, int TB, const float* red,
                                                   int nslice, const float* zact,
                                                   const float* rs, const float* p,
@@ -470,7 +470,7 @@ __global__ void __launch_bounds__(160) k_bwd_coef(Dims d, int slot, int T, int T
                                                   float* __restrict__ colp, DzPack pack, WRows wrows, int nblk) {
     pdl_entry();
     if ((int)blockIdx.x >= nblk) {
-        pack_wrows_of(wrows, (int)blockIdx.x - nblk);
+        pack_wrows_of<SIX>(wrows, (int)blockIdx.x - nblk);
         return;
     }
     using L = BwdTok<KM>;
@@ -632,7 +632,7 @@ __global__ void __launch_bounds__(160) k_bwd_coef(Dims d, int slot, int T, int T
         const int tt = e / n, o = e - tt * n;
         dzs[t0 * n + e] = sm[tt * L::ROW + L::DZ + o];
     }
-    pack_dz_of(pack, sm + L::DZ, L::ROW, n, t0, ntok);
+    pack_dz_of<SIX>(pack, sm + L::DZ, L::ROW, n, t0, ntok);
     if (tid < ntok) {
         // active RMS: z_o = r * zraw_o, r = (sum x^2 / kC + eps)^(-1/2)
         const float* row = sm + tid * L::ROW;
@@ -672,11 +672,11 @@ cudaError_t bwd_coef_km(const Dims& d, int slot, int T, const float* red, int ns
     int TB = 128 / KM;
     if (T < TB * 2 * device_sms() || smem(TB) > 200 * 1024) TB = 32 / KM;
     const size_t sm = smem(TB);
-    const cudaError_t e =
-        smem_optin((const void*)k_bwd_coef<KM>, sm);
+    auto* const kern = wrows.terms == 6 ? &k_bwd_coef<KM, true> : &k_bwd_coef<KM, false>;
+    const cudaError_t e = smem_optin((const void*)kern, sm);
     if (e != cudaSuccess) return e;
     *nblk = (T + TB - 1) / TB;
-    XHC_LAUNCH(st, *nblk + wrows_blocks(wrows, 32 + TB * KM), 32 + TB * KM, sm, (k_bwd_coef<KM>), d, slot, T, TB, red, nslice, zact, rs, p,
+    XHC_LAUNCH(st, *nblk + wrows_blocks(wrows, 32 + TB * KM), 32 + TB * KM, sm, (kern), d, slot, T, TB, red, nslice, zact, rs, p,
                hpost, gram, alpha_post, alpha_res, b_res, tokmat, dz, dp, colp, pack, wrows, *nblk);
     return cudaGetLastError();
 }
@@ -710,6 +710,7 @@ namespace {
 constexpr int FC_NT = 256;
 constexpr int FC_R = 4;   // pre-map columns per lane: G N <= 128
 
+template <bool SIX>
 __global__ void __launch_bounds__(FC_NT) k_full_coef(Dims d, int T, int TB, const float* dhpre,
                                                      const float* hpre,
                                                      const float* zfull,
@@ -722,7 +723,7 @@ __global__ void __launch_bounds__(FC_NT) k_full_coef(Dims d, int T, int TB, cons
     pdl_entry();
     extern __shared__ float dzs[];   // [TB][n] dz, for the packed operands
     if ((int)blockIdx.x >= nblk) {
-        pack_wrows_of(wrows, (int)blockIdx.x - nblk);
+        pack_wrows_of<SIX>(wrows, (int)blockIdx.x - nblk);
         return;
     }
     __shared__ float sh[FC_NT / 32][NCOLP];
@@ -823,7 +824,7 @@ __global__ void __launch_bounds__(FC_NT) k_full_coef(Dims d, int T, int TB, cons
     }
     if (d.hr && lane < N) sh[warp][2 * GN + lane] = srt;
     __syncthreads();
-    pack_dz_of(pack, dzs, n, n, t0, ntok);
+    pack_dz_of<SIX>(pack, dzs, n, n, t0, ntok);
     for (int c = tid; c < 2 * GN + roff; c += FC_NT) {
         float s = 0.f;
 #pragma unroll
@@ -856,7 +857,8 @@ cudaError_t launch_full_coef(const Dims& d, int T, const float* dhpre, const flo
     // 8 tokens a block (a token per warp) at few tokens, 32 at many
     const int TB = (T >= 32 * 2 * device_sms()) ? 32 : 8;
     *nblk = (T + TB - 1) / TB;
-    XHC_LAUNCH(st, *nblk + wrows_blocks(wrows, FC_NT), FC_NT, (size_t)TB * d.nfull * 4, (k_full_coef), d, T, TB, dhpre, hpre, zfull,
+    auto* const kern = wrows.terms == 6 ? &k_full_coef<true> : &k_full_coef<false>;
+    XHC_LAUNCH(st, *nblk + wrows_blocks(wrows, FC_NT), FC_NT, (size_t)TB * d.nfull * 4, (kern), d, T, TB, dhpre, hpre, zfull,
                stats, wsum, I, dp, alpha_pre, dz, scal, colp, pack, wrows, *nblk);
     return cudaGetLastError();
 }

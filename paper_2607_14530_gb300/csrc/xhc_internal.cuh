@@ -453,7 +453,9 @@ struct DzPack {
     uint16_t *hilo, *rows;
     int NB, Tp, ld, terms;
 };
-// dz of a block's ntok tokens from t0 on, in shared memory (row stride rs), into the two operands
+// dz of a block's ntok tokens from t0 on, in shared memory (row stride rs), into the two operands (SIX: terms is
+// 6; a kernel of its own, as a branch cost the others 1 % of a small step)
+template <bool SIX>
 __device__ __forceinline__ void pack_dz_of(const DzPack& p, const float* dz, int rs, int n, long long t0, int ntok) {
     if (p.hilo != nullptr)
         for (int idx = threadIdx.x; idx < p.NB * ntok; idx += blockDim.x) {
@@ -465,20 +467,25 @@ __device__ __forceinline__ void pack_dz_of(const DzPack& p, const float* dz, int
             }
             p.hilo[(long long)r * p.Tp + t0 + tt] = f2bf(v);
         }
-    if (p.rows != nullptr)
+    if (p.rows == nullptr) return;
+    if (SIX) {
+        const int np = split_step(n);
         for (int idx = threadIdx.x; idx < ntok * p.ld; idx += blockDim.x) {
-            const int tt = idx / p.ld, c = idx - tt * p.ld;
-            float v = 0.f;
-            if (p.terms == 6) {
-                const int np = split_step(n), part = c / np, o = c - part * np;
-                if (o < n && part < 3) v = split_part(dz[tt * rs + o], part);
-            } else if (c < p.terms * n) {
-                const int part = c / n;
-                v = dz[tt * rs + c - part * n];
-                if (part == 1) v -= __bfloat162float(__float2bfloat16_rn(v));
-            }
-            p.rows[(t0 + tt) * p.ld + c] = f2bf(v);
+            const int tt = idx / p.ld, c = idx - tt * p.ld, part = c / np, o = c - part * np;
+            p.rows[(t0 + tt) * p.ld + c] = f2bf(o < n && part < 3 ? split_part(dz[tt * rs + o], part) : 0.f);
         }
+        return;
+    }
+    for (int idx = threadIdx.x; idx < ntok * p.ld; idx += blockDim.x) {
+        const int tt = idx / p.ld, c = idx - tt * p.ld;
+        float v = 0.f;
+        if (c < p.terms * n) {
+            const int part = c / n;
+            v = dz[tt * rs + c - part * n];
+            if (part == 1) v -= __bfloat162float(__float2bfloat16_rn(v));
+        }
+        p.rows[(t0 + tt) * p.ld + c] = f2bf(v);
+    }
 }
 // the weight side of the input gradient: dst [rows][ld] bf16, a weight row in the columns of `terms`, zero past
 // them; packed by further blocks of the same launch
@@ -495,6 +502,7 @@ __device__ __forceinline__ int dxa_row(int r) {
 }
 inline int __host__ __device__ dxa_width(int C) { return (C + 31) / 32 * 32; }
 constexpr int WROWS_U = 8;   // elements per thread
+template <bool SIX>
 __device__ __forceinline__ void pack_wrows_of(const WRows& j, int blk) {
     const int at = blk * (int)blockDim.x * WROWS_U + threadIdx.x, tot = j.rows * j.ld;   // < 2^31
     float v[WROWS_U];
@@ -507,24 +515,24 @@ __device__ __forceinline__ void pack_wrows_of(const WRows& j, int blk) {
         if (idx < tot) {
             int r = idx / j.ld;
             const int c = idx - r * j.ld;
-            const int np = j.terms == 6 ? split_step(j.n) : j.n;
-            const int q = c / np, o = c - q * np;
-            bool in = q < (j.terms == 6 ? 3 : j.terms) && o < j.n;
+            const int np = SIX ? split_step(j.n) : j.n;
+            bool in = c < (SIX ? 3 : j.terms) * np;
             if (j.C > 0) {
                 const int slot = r / dxa_width(j.C), ch = dxa_row(r - slot * dxa_width(j.C));
                 in = in && ch < j.C;
                 r = slot * j.C + ch;
             }
             if (in) {
-                part[u] = q;
-                v[u] = seg_elem(j.W, r, o);
+                part[u] = c / np;
+                const int o = c - part[u] * np;
+                if (!SIX || o < j.n) v[u] = seg_elem(j.W, r, o);
             }
         }
     }
 #pragma unroll
     for (int u = 0; u < WROWS_U; ++u) {
         const int idx = at + u * (int)blockDim.x;
-        if (j.terms == 6) v[u] = split_part(v[u], part[u]);
+        if (SIX) v[u] = split_part(v[u], part[u]);
         else if (part[u] == 2) v[u] -= __bfloat162float(__float2bfloat16_rn(v[u]));
         if (idx < tot) j.dst[idx] = f2bf(v[u]);
     }
