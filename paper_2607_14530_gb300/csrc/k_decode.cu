@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(512, 2) k_dec_post(Dims d, int slot, int B, in
     const int t0 = blockIdx.x * DT, ntok = min(DT, B - t0);
     const int rank = blockIdx.y, nr = gridDim.y;     // CTA of the cluster, and their number
     const int s0 = rank * q, sn = min(q, ns - s0);   // this CTA's slices
-    if (tid < ntok) {
+    if ((CONV || rank == 0) && tid < ntok) {
         const long long v = pos[t0 + tid];
         ps[tid] = v;
         rows[tid] = R > 0 ? (int)(v % R) : 0;        // ring row of the position
@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(512, 2) k_dec_post(Dims d, int slot, int B, in
             if (CONV && R > 0) *reinterpret_cast<uint32_t*>(ring + (t * R + rows[tt]) * C + c) = raw;
         }
     }
-    // the conv's CTAs have all read pos (before their last cluster barrier); without conv none but this one does
+    // the conv's CTAs have all read pos (before their last cluster barrier); without conv only this one does
     if (last && rank == 0 && tid < ntok) pos[t0 + tid] = ps[tid] + 1;
 }
 

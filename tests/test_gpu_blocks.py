@@ -64,6 +64,8 @@ DECODE = {
     "B3_N6": (Config.flash(6, 3, 1, 264, 2, conv_k=(2, 5)), 3, 40, False),
     "B9_k8": (Config.full(12, 8, 3, 776, True), 9, 15, False),
     "B17_no_gs": (Config.full(8, 4, 2, 64, True, gram_schmidt=False), 17, 11, False),
+    # no conv in the last slot, several CTAs a token: pos is read and advanced by the first alone
+    "B5_attn_wide": (Config.full(8, 4, 2, 2312, False), 5, 4, False),
     "B31_attn": (Config.full(8, 4, 2, 72, False), 31, 4, False),
     "B127": (Config.flash(8, 4, 2, 2312, 2, conv_k=(16,)), 127, 20, True),
     "B130": (Config.flash(8, 4, 2, 1024, 2), 130, 20, True),
