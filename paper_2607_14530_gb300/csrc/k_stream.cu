@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(256, 3) k_read(Dims d, int T, const uint16_t* 
     if (threadIdx.x < C / 8) {
 #pragma unroll
         for (int ii = 0; ii < 8; ++ii)
-            if (ii < N) ub[ii] = *reinterpret_cast<const uint4*>(xt + (int64_t)ii * C + threadIdx.x * 8);
+            if (ii < N) ub[ii] = ld_stream(xt + (int64_t)ii * C + threadIdx.x * 8);
     }
     for (int q = threadIdx.x; q < G * N; q += blockDim.x) sh[q] = hpre[(int64_t)t * G * N + q];
     for (int i = threadIdx.x; i < N; i += blockDim.x) {
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(256, 3) k_read(Dims d, int T, const uint16_t* 
             if (i0 != 0 || c8 != (int)threadIdx.x) {
 #pragma unroll
                 for (int ii = 0; ii < 8; ++ii)
-                    if (i0 + ii < N) ub[ii] = *reinterpret_cast<const uint4*>(xt + (int64_t)(i0 + ii) * C + c8 * 8);
+                    if (i0 + ii < N) ub[ii] = ld_stream(xt + (int64_t)(i0 + ii) * C + c8 * 8);
             }
 #pragma unroll
             for (int ii = 0; ii < 8; ++ii) {
@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(512) k_full_dots(Dims d, int T, const uint16_t
         for (int u = 0; u < 4; ++u) {
             const int c8 = lane + 32 * u;
             xr[h][u] = make_uint4(0u, 0u, 0u, 0u);
-            if (is[h] >= 0 && c8 < C / 8) xr[h][u] = *reinterpret_cast<const uint4*>(X + row[h] + c8 * 8);
+            if (is[h] >= 0 && c8 < C / 8) xr[h][u] = ld_stream(X + row[h] + c8 * 8);
         }
     for (int idx = threadIdx.x; idx < G * C / 8; idx += blockDim.x) {
         const int q = idx / (C / 8), c8 = idx - q * (C / 8);
@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(512) k_full_dots(Dims d, int T, const uint16_t
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const int c8 = c0 + 32 * u;
-                    if (is[h] >= 0 && c8 < C / 8) xr[h][u] = *reinterpret_cast<const uint4*>(X + row[h] + c8 * 8);
+                    if (is[h] >= 0 && c8 < C / 8) xr[h][u] = ld_stream(X + row[h] + c8 * 8);
                 }
         }
 #pragma unroll

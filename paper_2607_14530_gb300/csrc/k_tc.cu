@@ -765,14 +765,6 @@ constexpr int DX_BN = 128;
 constexpr int DX_EW = 16;                       // epilogue warps: 4 per TMEM lane quarter
 constexpr int DX_THREADS = (2 + DX_EW) * 32;    // + TMA warp + MMA warp
 
-// 16-byte global read (plain LDG: measured faster here than the non-coherent or no-allocate forms)
-__device__ __forceinline__ uint4 ld_stream(const void* p) {
-    uint4 r;
-    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
-    return r;
-}
-
 struct DxArgs {
     int T, C, N, k, G;
     int m;                // full-state epilogue: fixed streams 0..m-1 (active on every token)

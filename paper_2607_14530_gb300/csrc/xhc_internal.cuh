@@ -338,6 +338,13 @@ __device__ __forceinline__ void pdl_entry() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+// A 16-byte read that the compiler leaves where it stands, among the other ones and after the wait.
+__device__ __forceinline__ uint4 ld_stream(const void* p) {
+    uint4 r;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+    return r;
+}
 // Whether the launches of the call that runs on this thread use it.  It takes a microsecond off every
 // kernel of a chain, and costs where the waiting blocks take places from kernels that would still use
 // them: us a pass without / with, N C T bf16 state of 4 MB 221 / 185, 52 MB 600 / 558, 100 MB 332 / 289,
