@@ -60,6 +60,25 @@ OVERLAP = {}
 WINDOWED = ("wgrad_tc_full", "wgrad_tc_active")
 
 
+def bapp_runs(T, S, C, kw):
+    """Runs of tokens of the backward apply (bapp_run of csrc/k_wb.cuh: at most 296 tokens each, fewer where that
+    takes fewer waves of blocks)."""
+    import torch
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    cap, slices, extra = 2 * sms, -(-C // 256), kw + 5
+
+    def runs(tb):
+        return (T // S) * -(-S // tb) + -(-(T % S) // tb)
+
+    def cost(tb):
+        return -(-slices * runs(tb) // cap) * (min(tb, S) + extra)
+
+    if slices * runs(296) >= 4 * cap:
+        return runs(296)
+    return runs(min(range(296, 0, -4), key=cost))   # the longest of the cheapest
+
+
 def kernel_model(cfg, T):
     N, k, C, G = cfg.N, cfg.k, cfg.C, cfg.G
     hr = cfg.m < cfg.k
@@ -83,8 +102,7 @@ def kernel_model(cfg, T):
     row = T * C * b16
     kw = max(cfg.conv_k) if cfg.conv_k else 0
     kw = 0 if kw == 0 else (4 if kw <= 4 else 8 if kw <= 8 else 12 if kw <= 12 else 16)
-    tb = 296 if kw else 0  # tokens per run of the backward apply (bapp_run)
-    runs = (T // S) * -(-S // tb) + -(-(T % S) // tb) if kw else 0
+    runs = bapp_runs(T, S, C, kw) if kw else 0
     cpart = runs * sum(cfg.conv_k) * C * f32
     # forward; the active weights are packed ahead of their projections: slot 0's with the full-state one,
     # later slots' in blocks of the input kernel

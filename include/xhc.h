@@ -153,7 +153,9 @@ typedef struct xhc_handle xhc_handle;
 xhc_status xhc_create(const xhc_config* cfg, xhc_handle** out);
 void xhc_destroy(xhc_handle* h);
 
-/* Bytes of the caller-allocated `saved` and `workspace` buffers for T tokens. */
+/* Bytes of the caller-allocated `saved` and `workspace` buffers for T tokens.  The workspace of fewer tokens may
+ * be the larger one (the work is split according to T, and each split keeps partial sums): a buffer for calls of
+ * several T takes the largest of their sizes. */
 xhc_status xhc_saved_bytes(const xhc_handle* h, int64_t T, size_t* bytes);
 xhc_status xhc_workspace_bytes(const xhc_handle* h, int64_t T, size_t* bytes);
 
@@ -208,7 +210,9 @@ xhc_status xhc_post_fwd(const xhc_handle* h, int slot, int64_t T, const xhc_para
  * bf16, row (s mod R) holding out[s] of position s.  pos [B] int64 (device) is the position of
  * each sequence's current token.  A decode step of a group is, for slot = 0..G-1,
  * xhc_pre_fwd(slot, T = B) then xhc_post_fwd_decode(slot, B); use a handle whose seq_len is 0
- * (or divides B): the conv history comes from the ring, not from the call's tokens.
+ * (or divides B): the conv history comes from the ring, not from the call's tokens.  A token's results in a step of
+ * fewer than 128 sequences do not depend on the others, to the bit; from 128 on the projections' sums are cut
+ * according to B.
  *
  * xhc_ring_bytes: size of one conv slot's ring for B sequences (0 without a conv).
  * xhc_ring_fill: after a prefill of B sequences of S tokens each (rows b*S .. b*S+S-1 of `out`,
@@ -229,8 +233,9 @@ xhc_status xhc_post_fwd_decode(const xhc_handle* h, int slot, int64_t B, const x
 
 /* Backward of post_fwd(slot).  Reads dX (slot G-1: the gradient w.r.t. the group output) or the
  * workspace-held active gradient, leaves the post/res map-logit gradient and its projection
- * weight (both as pre_bwd(slot) multiplies them) in the workspace, writes d_out [T, C] (= dL/d out, including the paths through
- * later sublayer inputs), accumulates the post/res/conv parameter gradients.  slot G-1 also
+ * weight (both as pre_bwd(slot) multiplies them) in the workspace, writes d_out [T, C] (= dL/d out,
+ * including the paths through later sublayer inputs), accumulates the post/res/conv parameter
+ * gradients.  slot G-1 also
  * restores the active rows of X to the group-entry state. */
 xhc_status xhc_post_bwd(const xhc_handle* h, int slot, int64_t T, const xhc_params* P,
                         uint16_t* X, uint16_t* dX, const uint16_t* out, uint16_t* d_out,

@@ -755,8 +755,8 @@ int device_sms() { return num_sms(); }
 //   dX[t][i*C + c] = base + sum_o dZ[t][o] W[i*C + c][o] + a_t + b_t x[t][i*C + c]
 //   base = dX_act[t][j][c]                                  if stream i is active slot j
 //        = dX[t][i*C + c] + sum_q H_pre[t][q][i] d_input_q[t][c]   otherwise
-// MMA K = nfull (dZ and W in bf16: this term is a small share of dX, whose storage is bf16); the
-// tiling is described at the kernel (k_dxf_tc).  The same machinery with "streams" = the k active
+// MMA in dx_tc_terms terms of nfull (one where 64 divides the width: this part is a small share of dX, whose
+// storage is bf16); the tiling is described at the kernel (k_dxf_tc).  The same machinery with "streams" = the k active
 // slots updates dX_act in the backward of each slot's pre-map (k_dx_tc).
 
 namespace {
@@ -831,7 +831,7 @@ __device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Active-state input gradient: tiles of 128 tokens x 128 channels of an active slot j, MMA K = 3 nact,
+// Active-state input gradient: tiles of 128 tokens x 128 channels of an active slot j, MMA in 3 or 6 terms of nact,
 //   dX_act[t][j][c] += acc + H_pre[t][slot][I_j] d_input[t][c] - cx_t x_act[t][j][c]
 // (X = x_act of the slot, scal = the per-token matrices with cx at 112); from the same loads, the dH_pre dot
 // <x_act_j, d_input> of each 32-channel group (dotp) and, in the j = 0 tiles, the workspace copy of
@@ -845,7 +845,7 @@ __device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, float (&v)[16]) {
 // has 4 lanes a row too; the weight's rows are packed in the order that gives lane q of a row the
 // channels 8 q .. 8 q + 7 (dxa_row).  CUT: DX_BN does not divide C, and the lanes
 // past it move nothing (two forms: the test costs registers, and the kernel sits at its 96: T = 8192,
-// C = 2048: 131 -> 135 us with it).  T = 32768, C = 4096, k = 4: 1073 us, 81 % of the copy rate.  With the
+// C = 2048: 131 -> 135 us with it).  T = 32768, C = 4096, k = 4: 1050 us, 84 % of the copy rate.  With the
 // accumulator turned through shared memory instead: the same there, 277 us against 268 at T = 16384,
 // C = 2048 and 72 us against 63 at T = 2103, C = 1536 (the shared-memory pipe was 64 % busy).
 template <bool CUT>
@@ -1436,7 +1436,7 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
 // KB of shared memory).  Below a tile of tokens the CUDA-core pair gemm_dzw + dinput_act stays.  Three terms where
 // DX_BN divides the width and two k-blocks hold them; six elsewhere, where gemm_dzw would take the operands in
 // fp32 and dX_act, which is fp32 and feeds the earlier slots' parameter gradients, shows it.
-// T = 1000, C = 1160, k = 8, nact = 96: gemm_dzw + dinput_act 92 + 29 us, here 38.
+// T = 1000, C = 1160, k = 8, nact = 96: gemm_dzw + dinput_act 92 + 29 us, here 37.
 int dxa_tc_terms(int T, int k, int C, int nact) {
     if (T < BM || split_cols(nact, 6) > 5 * BK ||
         (long long)((T + BM - 1) / BM) * ((C + DX_BN - 1) / DX_BN) * k >= (1LL << 31))   // 32-bit tile indices
@@ -1525,7 +1525,7 @@ static int dxf_stages(int K, int G) { return dxf_smem(K, G, 2) <= 232448 ? 2 : d
 // 192, N = 32 with a router and four pre-maps); in six at other widths, where the CUDA-core full_dx would take
 // both in fp32.  0: full_dx (less than a tile of tokens, or too many columns for the shared memory).
 // T = 1000, N = 12, C = 1160: full_dx 79 us, here 37; T = 4944, N = 16, C = 2840, four
-// slots (G N + N = 80 columns, one stage of weight rows): the step 5.99 -> 3.40 ms with both gradients here.
+// slots (G N + N = 80 columns, one stage of weight rows): the step 5.99 -> 3.60 ms with both gradients here.
 int dx_tc_terms(int T, int N, int C, int nfull, int G) {
     if (T < BM || N < 2 || G < 1 || G > 4 ||
         (long long)((T + BM - 1) / BM) * ((C + DG_BN - 1) / DG_BN) * N >= (1LL << 31))   // 32-bit tile indices

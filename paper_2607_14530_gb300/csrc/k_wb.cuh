@@ -45,8 +45,8 @@ __device__ __forceinline__ float dot2(float2 a, float2 b) { return fmaf(a.x, b.x
 __device__ __forceinline__ float2 fma2(float s, float2 a, float2 acc) {
     return __ffma2_rn(make_float2(s, s), a, acc);
 }
-// the same as two scalar FMAs (measured faster in the backward apply, where the packed form
-// lengthens the schedule)
+// the same as two scalar FMAs, for the backward apply.  (The packed form was slower there while its tokens were
+// parted by branches; it has not been measured since they are not.)
 __device__ __forceinline__ float2 fma2s(float s, float2 a, float2 acc) {
     return make_float2(fmaf(s, a.x, acc.x), fmaf(s, a.y, acc.y));
 }
