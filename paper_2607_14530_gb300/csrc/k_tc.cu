@@ -1160,12 +1160,9 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
     const int nloc = nblk * NU;   // < 2^31: the host checks ntiles * N
     // local tile n: position p of unit `blk` of this CTA (column block unit / nsplit, streams [i0, i0 + NU)).
     // A unit's leading ndin tiles are its streams from m on, which may read d_input, the fixed ones follow.
-    // Each role walks its tiles with a cursor: the divisions run once a unit.  `din` counts the units before
-    // this one that have d_input tiles: only those load the d_input rows and take part in their handshake
-    // (barriers 6 and 7).  A unit of fixed streams alone would load rows that no one waits for, and its CTA
-    // could end, or start the next load, with the copies still in flight.
+    // Each role walks its tiles with a cursor: the divisions run once a unit.
     struct Cursor {
-        int p, blk, tt, cb, i0, ndin, din;
+        int p, blk, tt, cb, i0, ndin;
         __device__ int stream(int NU) const { return p < ndin ? i0 + NU - ndin + p : i0 + p - ndin; }
     };
     auto locate = [&](Cursor& c) {
@@ -1176,19 +1173,20 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
         c.cb = block - c.tt * a.CT;
         c.ndin = min(NU, max(0, c.i0 + NU - a.m));
     };
+    auto start = [&](Cursor& c, int n) {
+        c.blk = n / NU;
+        c.p = n - c.blk * NU;
+        locate(c);
+    };
     auto advance = [&](Cursor& c, int by) {
         c.p += by;
-        while (c.p >= NU) {
-            c.p -= NU;
-            ++c.blk;
-            c.din += c.ndin > 0;
+        if (c.p >= NU) {
+            do {
+                c.p -= NU;
+                ++c.blk;
+            } while (c.p >= NU);
             locate(c);
         }
-    };
-    auto start = [&](Cursor& c, int n) {
-        c.p = c.blk = c.din = 0;
-        locate(c);
-        advance(c, n);
     };
 
     if (warp == 0) {
@@ -1242,16 +1240,23 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
                 unsigned char* xt = sE + (size_t)s * 2 * DG_TILE;
                 tma_load_3d(smem_u32(xt), &tmX, cb * DG_BN, i, tt * BM, fe);
                 if (need_dx) tma_load_3d(smem_u32(xt + DG_TILE), &tmD, cb * DG_BN, i, tt * BM, fe);
-                if (p == 0 && ndin > 0) {
-                    if (cu.din >= 1 && !mbar_wait(smem_u32(&bars[7]), (uint32_t)((cu.din - 1) & 1), a.wait_ns)) {
+                if (p == 0) {
+                    if (blk >= 1 && !mbar_wait(smem_u32(&bars[7]), (uint32_t)((blk - 1) & 1), a.wait_ns)) {
                         atomicExch(a.err, 34);
                         *s_abort = 1;
                         break;
                     }
+                    // a unit of fixed streams alone has no d_input tile, and no one would wait for its rows: the
+                    // CTA could end, or start the next load, with the copies still in flight.  It loads none and
+                    // completes the phase.
                     const uint32_t fg = smem_u32(&bars[6]);
-                    mbar_expect_tx(fg, (uint32_t)a.G * DG_TILE);
-                    for (int q = 0; q < a.G; ++q)
-                        tma_load_2d(smem_u32(sG + q * DG_TILE), &tmG, cb * DG_BN, q * a.T + tt * BM, fg);
+                    if (ndin == 0) {
+                        mbar_arrive(fg);
+                    } else {
+                        mbar_expect_tx(fg, (uint32_t)a.G * DG_TILE);
+                        for (int q = 0; q < a.G; ++q)
+                            tma_load_2d(smem_u32(sG + q * DG_TILE), &tmG, cb * DG_BN, q * a.T + tt * BM, fg);
+                    }
                 }
             }
         }
@@ -1348,7 +1353,7 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
             prefetch(0, pfa);
             bool ok = mbar_wait(smem_u32(&bars[12 + grp]), (uint32_t)((n >> 1) & 1), a.wait_ns);
             ok = ok && mbar_wait(smem_u32(&bars[8 + grp]), (uint32_t)((n >> 1) & 1), a.wait_ns);
-            ok = ok && (!usesg || mbar_wait(smem_u32(&bars[6]), (uint32_t)(cu.din & 1), a.wait_ns));
+            ok = ok && (!usesg || mbar_wait(smem_u32(&bars[6]), (uint32_t)(blk & 1), a.wait_ns));
             if (!ok) {
                 atomicExch(a.err, 36);
                 *s_abort = 1;
@@ -1408,10 +1413,10 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
             fence_async_smem();                                      // results visible to TMA
             if (named_bar_or(1 + grp, (DX_EW / 2) * 32, *s_abort != 0)) break;  // same decision in the group
             if (leader) {
-                // the group's last reader of this block's d_input rows (or, when the block's one d_input
-                // tile is the other group's, its first tile of the block) releases them: one arrival
-                // per group and block that loads them, and at least one after the load is complete
-                if ((usesg && p + 2 >= ndin) || (ndin > 0 && !usesg && p < 2)) mbar_arrive(smem_u32(&bars[7]));
+                // the group's last reader of this block's d_input rows (or, when it has none of the
+                // block's d_input tiles, its first tile of the block) releases them: one arrival per group
+                // and block, and of a block that loads them at least one after the load is complete
+                if ((usesg && p + 2 >= ndin) || (!usesg && p < 2)) mbar_arrive(smem_u32(&bars[7]));
                 tma_store_3d(&tmD, smem_u32(xt), cb * DG_BN, i, tt * BM);
                 bulk_commit();
                 bulk_wait_read0();                                   // the stage may be reloaded
