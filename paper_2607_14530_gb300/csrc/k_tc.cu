@@ -773,7 +773,7 @@ struct DxArgs {
     int NH;               // active epilogue: streams of the H_pre rows
     float* dxa;           // active epilogue: dX_act [T][k][C] fp32, updated in place
     int nkb, ksteps;      // k-blocks of 64, MMA k-steps of 16 of a pair of parts
-    int pr0;              // first pair of parts (6 terms: 0), or 5 for one pass over all columns
+    int pr0;              // 0: the six pairs of parts, 5: one pass over all columns
     int TT, CT;           // token tiles, channel tiles per stream
     long long ntiles;
     int P;
@@ -795,11 +795,22 @@ struct DxArgs {
     int nsplit;           // full-state dX: parts that a column block's streams are cut into (of two streams at least)
 };
 
-// the MMAs of one tile: the k-steps of every pair of parts (see split_cols), from operands in k-blocks of 64 columns
-template <int BN>
+// The MMAs of one tile, from operands in k-blocks of 64 columns: one pass over the columns, or the k-steps of every
+// pair of parts (see split_cols).  ONE, SIX: it is always the former, the latter.  One thread issues them and the
+// tile waits for it, so the first form keeps its simpler loop (the full-state dX of N = 32, ten k-steps, T = 8192:
+// 1696 us, 20 more through the second).
+template <int BN, bool ONE, bool SIX>
 __device__ __forceinline__ void dx_mma(const DxArgs& a, uint32_t d, uint32_t abase, uint32_t bbase, uint32_t idesc) {
+    if (ONE || (!SIX && a.pr0 == 5)) {
+        for (int ks = 0; ks < a.ksteps; ++ks) {
+            const int kb = ks >> 2, kk = ks & 3;
+            mma_bf16(d, sw128_desc(abase + kb * BM * BK * 2 + kk * 32), sw128_desc(bbase + kb * BN * BK * 2 + kk * 32),
+                     idesc, ks > 0 ? 1u : 0u);
+        }
+        return;
+    }
     uint32_t accum = 0;
-    for (int pr = a.pr0; pr < 6; ++pr) {
+    for (int pr = 0; pr < 6; ++pr) {
         const int a0 = split_pair_a(pr) * a.ksteps, b0 = split_pair_b(pr) * a.ksteps;
         for (int ks = 0; ks < a.ksteps; ++ks) {
             const uint32_t ka = (uint32_t)(a0 + ks), kb = (uint32_t)(b0 + ks);
@@ -939,7 +950,7 @@ k_dx_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
                 tc_fence_after();
                 const uint32_t abase = smem_u32(smem);
                 const uint32_t bbase = abase + A_BYTES;
-                dx_mma<DX_BN>(a, tmem + (uint32_t)(s * DX_BN), abase, bbase, idesc);
+                dx_mma<DX_BN, false, CUT>(a, tmem + (uint32_t)(s * DX_BN), abase, bbase, idesc);
                 mma_commit(smem_u32(&bars[1]));      // operands consumed
                 mma_commit(smem_u32(&bars[2 + s]));  // accumulator ready
             }
@@ -1282,7 +1293,7 @@ k_dxf_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
                 tc_fence_after();
                 const uint32_t abase = smem_u32(sA);
                 const uint32_t bbase = smem_u32(sB + b * B_BYTES);
-                dx_mma<DG_BN>(a, tmem + (uint32_t)(s * DG_BN), abase, bbase, idesc);
+                dx_mma<DG_BN, !CUT, CUT>(a, tmem + (uint32_t)(s * DG_BN), abase, bbase, idesc);
                 mma_commit(smem_u32(&bars[4 + b]));              // B stage consumed
                 mma_commit(smem_u32(&bars[8 + s]));              // accumulator ready
                 if (p == NU - 1) mma_commit(smem_u32(&bars[1]));  // the block's A rows consumed
